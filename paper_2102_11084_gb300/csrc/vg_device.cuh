@@ -457,6 +457,32 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* total,
   return __shfl_sync(kFullMask, ws - wt, warp) + inc - v;
 }
 
+// Barrier over every block of a cooperative launch, on an arrival counter that is zero when
+// the launch starts; `target` (thread 0's) grows by the grid each barrier, both modulo 2^32.
+// The wait is bounded: after `spin` polls it records kErrTimeout and goes on.  False (in
+// every thread of the block) when this block's wait ran out.
+__device__ __forceinline__ bool grid_barrier(uint32_t* ctr, uint32_t& target, uint32_t spin,
+                                             int* err) {
+  __syncthreads();
+  bool late = false;
+  if (threadIdx.x == 0) {
+    target += gridDim.x;
+    __threadfence();
+    atomicAdd(ctr, 1u);
+    uint32_t spins = 0;
+    while (static_cast<int32_t>(ld_acquire(ctr) - target) < 0) {
+      if (++spins > spin) {
+        set_error(err, kErrTimeout);
+        late = true;
+        break;
+      }
+      if (spins > 16) __nanosleep(32);
+    }
+    __threadfence();
+  }
+  return __syncthreads_or(late) == 0;
+}
+
 // ---- frame decomposition (chunks of kChunk points inside one frame) -----------------------
 // Loads the frame offsets into s_off[0..F] and the chunk prefix into s_cstart[0..F];
 // returns the number of chunks.  Bad offsets (not starting at 0, not ending at n, or

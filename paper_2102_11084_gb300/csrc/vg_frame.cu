@@ -577,26 +577,11 @@ struct FzArgs {
 // carry count below 2^10.
 static_assert(kFzMaxPointsBits + 21 <= 42 && 42 - 32 < 21, "carry counts fit their fields");
 
-// Grid barrier on an arrival counter the call zeroes; `target` (thread 0's) grows by the
-// grid each barrier.  The wait is bounded.
+// Grid barrier on the arrival counter the call zeroes (a wait that ran out is in the error
+// word; the block goes on).
 __device__ __forceinline__ void fz_grid_sync(uint32_t* ctr, uint32_t& target, uint32_t spin,
                                              int* err) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    target += gridDim.x;
-    __threadfence();
-    atomicAdd(ctr, 1u);
-    uint32_t spins = 0;
-    while (ld_acquire(ctr) < target) {
-      if (++spins > spin) {
-        set_error(err, kErrTimeout);
-        break;
-      }
-      if (spins > 16) __nanosleep(32);
-    }
-    __threadfence();
-  }
-  __syncthreads();
+  (void)grid_barrier(ctr, target, spin, err);
 }
 
 // Ranking the set bits of words [0, nw) in word order takes two steps around a grid

@@ -11,16 +11,24 @@
 // GPU layout of the loop:
 //   grouping   the sort path (wide layout, point_to_voxel on) gives the occupied cells
 //              in key order and the points in cell order;
-//   setup      per point of the sorted table: its coordinates, priority and index; per
-//              cell: its first entry and the rows of its 26 neighbour cells (binary
-//              search in the sorted cell keys, once);
-//   per pass   thin_count_kernel counts and marks; the host reads the number marked;
-//              if it exceeds the batch, a radix select over the 64-bit keys
-//              (priority << 32 | index) of the marked points finds the batch, 8 bits a
-//              round, on 256-bin histograms (thin_hist_kernel); thin_delete_kernel
-//              removes it (or every marked point, in the last pass).
+//   setup      per entry of the sorted table: its coordinates and index in one 16-byte
+//              word; per cell: its first entry and the rows of its 26 neighbour cells
+//              (binary search in the sorted cell keys, once), and how many (point,
+//              candidate) pairs the 27 cells of all points hold.
+// Then one of two forms of the same loop:
+//   counts kept (the usual one)   every point's neighbours are counted once, the points
+//              that start marked are sorted by (priority, index), and one cooperative
+//              launch runs every pass.  A point's count only falls, so the marked set only
+//              shrinks and the batch of every pass is the next `batch` points of the sorted
+//              list that are still marked; the pass then takes one from the count of every
+//              neighbour of a deleted point.  No pass reads the other points again and none
+//              goes through the host.
+//   recounted  where the points are so dense, or the batch so large, that the deleted points
+//              meet more candidates than a fresh count (which stops at the threshold):
+//              thin_count_kernel counts and marks every pass, the host reads the number
+//              marked and finds the batch by a radix select on 256-bin histograms
+//              (thin_hist_kernel), thin_delete_kernel removes it.
 //   output     keep flag per input point and the number kept.
-// The host synchronises the stream once per pass and once per select round.
 #include <cmath>
 
 #include "../../include/vg.h"
@@ -34,9 +42,14 @@ namespace {
 constexpr int kNb = 27;
 constexpr uint32_t kNoCell = 0xffffffffu;
 constexpr uint8_t kAlive = 1, kMarked = 2;
+// Words of the loop: marked points (recounted form), kept points, grid-barrier arrivals, passes
+// run, and the candidate pairs (one 64-bit word).
+constexpr int kCtrMarked = 0, kCtrKept = 1, kCtrBar = 2, kCtrPasses = 3, kCtrPairs = 4;
+constexpr int kCtrGroups = 6;  // groups of entries (counts kept)
+constexpr int kCtrWords = 8;
 
 struct ThinLayout {
-  size_t base, vkeys, vcent, vcnt, vnum, p2v, cstart, nb, sx, sprio, sidx, state, ctr, hist,
+  size_t base, vkeys, pos, cnt, vcnt, vnum, p2v, cstart, nb, sprio, sidx, state, ctr, hist, st2,
       total;
 };
 
@@ -50,18 +63,19 @@ ThinLayout thin_layout(int64_t n) {
     off = align_up(off + bytes, 256);
   };
   take(&L.vkeys, size_t(nn) * sizeof(uint64_t));
-  take(&L.vcent, size_t(nn) * 3 * sizeof(float));
+  take(&L.pos, size_t(nn) * sizeof(float4));  // the grouping's centroids first, then the entries
+  take(&L.cnt, size_t(nn) * sizeof(uint32_t));
   take(&L.vcnt, size_t(nn) * sizeof(uint32_t));
   take(&L.vnum, sizeof(int64_t));
   take(&L.p2v, size_t(nn) * sizeof(int32_t));
   take(&L.cstart, size_t(nn) * sizeof(uint32_t));
   take(&L.nb, size_t(nn) * kNb * sizeof(uint32_t));
-  take(&L.sx, size_t(nn) * 3 * sizeof(float));
   take(&L.sprio, size_t(nn) * sizeof(uint32_t));
   take(&L.sidx, size_t(nn) * sizeof(uint32_t));
   take(&L.state, size_t(nn));
-  take(&L.ctr, 4 * sizeof(uint32_t));  // [0] marked, [1] kept
+  take(&L.ctr, kCtrWords * sizeof(uint32_t));
   take(&L.hist, 256 * sizeof(uint32_t));
+  take(&L.st2, sizeof(State));  // of the sort of the marked points by priority
   L.total = off;
   return L;
 }
@@ -71,12 +85,13 @@ __device__ __forceinline__ const uint32_t* sorted_idx(const State* st, const uin
   return (max(1, sort_passes(st->maxkey)) & 1) ? idx1 : idx0;
 }
 
-// Per sorted entry: gather coordinates, priority and index; mark cell starts.
+// Per sorted entry: gather coordinates, priority and index; mark cell starts; each valid
+// point's entry.
 __global__ void thin_setup_kernel(const State* st, const uint32_t* idx0, const uint32_t* idx1,
                                   const float* __restrict__ xyz, const uint32_t* __restrict__ prio,
-                                  const int32_t* __restrict__ p2v, uint32_t* cstart, float* sx,
-                                  uint32_t* sprio, uint32_t* sidx, uint8_t* state,
-                                  const int* err) {
+                                  const int32_t* __restrict__ p2v, uint32_t* cstart, float4* pos,
+                                  uint32_t* sprio, uint32_t* sidx, uint32_t* entry,
+                                  uint8_t* state, const int* err) {
   if (error_raised(err)) return;  // the grouping failed: point_to_voxel is unwritten
   const int64_t m = st->nitems;
   const uint32_t* I = sorted_idx(st, idx0, idx1);
@@ -86,46 +101,383 @@ __global__ void thin_setup_kernel(const State* st, const uint32_t* idx0, const u
     const int32_t row = p2v[p];
     const int32_t prev = i > 0 ? p2v[I[i - 1]] : -1;
     if (row != prev) cstart[row] = static_cast<uint32_t>(i);
-    sx[3 * i] = xyz[3 * size_t(p)];
-    sx[3 * i + 1] = xyz[3 * size_t(p) + 1];
-    sx[3 * i + 2] = xyz[3 * size_t(p) + 2];
+    pos[i] = make_float4(xyz[3 * size_t(p)], xyz[3 * size_t(p) + 1], xyz[3 * size_t(p) + 2],
+                         __uint_as_float(p));
     sprio[i] = prio[p];
     sidx[i] = p;
+    entry[p] = static_cast<uint32_t>(i);
     state[i] = kAlive;
   }
 }
 
-// Per cell: rows of the 27 cells around it (itself included), kNoCell where empty.
-__global__ void thin_neighbors_kernel(const int64_t* __restrict__ num_cells,
-                                      const uint64_t* __restrict__ vkeys, uint32_t* nb,
-                                      const int* err) {
+// Per cell and neighbour offset: the row of that cell (kNoCell where empty), and the pairs
+// of points the two hold.  A thread a (cell, offset) pair, not a cell: the 27 searches of a
+// cell are independent chains of dependent loads (11,489 cells: 25.8 us one thread a cell).
+__global__ __launch_bounds__(256) void thin_neighbors_kernel(
+    const int64_t* __restrict__ num_cells, const uint64_t* __restrict__ vkeys,
+    const uint32_t* __restrict__ vcnt, uint32_t* nb, unsigned long long* pairs, const int* err) {
   if (error_raised(err)) return;
   const int64_t V = *num_cells;
-  for (int64_t v = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; v < V;
-       v += int64_t(gridDim.x) * blockDim.x) {
+  unsigned long long mine = 0;
+  for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < V * kNb;
+       t += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t v = t / kNb;
+    const int o = static_cast<int>(t - v * kNb);
     const uint64_t key = vkeys[v];
-    const int64_t c[3] = {int64_t(compact3(key)), int64_t(compact3(key >> 1)),
-                          int64_t(compact3(key >> 2))};
-    int o = 0;
-    for (int dx = -1; dx <= 1; ++dx)
-      for (int dy = -1; dy <= 1; ++dy)
-        for (int dz = -1; dz <= 1; ++dz, ++o) {
-          const int64_t a = c[0] + dx, b = c[1] + dy, d = c[2] + dz;
-          uint32_t row = kNoCell;
-          const int64_t lim = int64_t(1) << 21;
-          if (a >= 0 && b >= 0 && d >= 0 && a < lim && b < lim && d < lim) {
-            const uint64_t want = morton3(uint32_t(a), uint32_t(b), uint32_t(d));
-            int64_t lo = 0, hi = V;  // first key >= want
-            while (lo < hi) {
-              const int64_t mid = (lo + hi) >> 1;
-              if (vkeys[mid] < want) lo = mid + 1; else hi = mid;
-            }
-            if (lo < V && vkeys[lo] == want) row = static_cast<uint32_t>(lo);
-          }
-          nb[v * kNb + o] = row;
-        }
+    const int64_t a = int64_t(compact3(key)) + o / 9 - 1;
+    const int64_t b = int64_t(compact3(key >> 1)) + o / 3 % 3 - 1;
+    const int64_t d = int64_t(compact3(key >> 2)) + o % 3 - 1;
+    uint32_t row = kNoCell;
+    const int64_t lim = int64_t(1) << 21;
+    if (a >= 0 && b >= 0 && d >= 0 && a < lim && b < lim && d < lim) {
+      const uint64_t want = morton3(uint32_t(a), uint32_t(b), uint32_t(d));
+      int64_t lo = 0, hi = V;  // first key >= want
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (vkeys[mid] < want) lo = mid + 1; else hi = mid;
+      }
+      if (lo < V && vkeys[lo] == want) row = static_cast<uint32_t>(lo);
+    }
+    nb[t] = row;
+    if (row != kNoCell) mine += (unsigned long long)vcnt[v] * vcnt[row];
+  }
+  for (int off = 16; off; off >>= 1) mine += __shfl_xor_sync(kFullMask, mine, off);
+  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(pairs, mine);
+}
+
+// Squared distance of the definition: binary32, ((dx*dx + dy*dy) + dz*dz), one rounding an
+// operation.  The same value for either point of a pair.
+__device__ __forceinline__ float dist2(const float4& q, float x, float y, float z) {
+  const float ex = __fsub_rn(q.x, x), ey = __fsub_rn(q.y, y), ez = __fsub_rn(q.z, z);
+  return __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
+}
+
+// ---- counts kept ------------------------------------------------------------------------
+
+constexpr int kFullThreads = 128;
+constexpr int kLoopThreads = 1024;
+constexpr int kLoopItems = 2;   // list entries a thread tests per step of the batch search
+constexpr int kLoopSplit = 8;   // warps that share the candidates of one deleted point
+constexpr uint32_t kLoopGroup = 128;  // entries a warp takes at a time (4 a lane)
+
+// Every entry's neighbours, all of them, and its cell; the groups of kLoopGroup entries that
+// the cells are cut into (their first entries, in any order).  A thread an entry, entries in
+// cell order: the lanes of a warp mostly share a cell, so a candidate's 16-byte load is one
+// broadcast.
+__global__ __launch_bounds__(kFullThreads) void thin_full_count_kernel(
+    const State* st, const int32_t* __restrict__ p2v, const uint32_t* __restrict__ cstart,
+    const uint32_t* __restrict__ vcnt, const uint32_t* __restrict__ nb,
+    const float4* __restrict__ pos, uint32_t* __restrict__ cnt, uint32_t* __restrict__ ecell,
+    uint32_t* __restrict__ group, uint32_t* ctr, float r2, const int* err) {
+  if (error_raised(err)) return;
+  const int64_t i = blockIdx.x * int64_t(kFullThreads) + threadIdx.x;
+  if (i >= int64_t(st->nitems)) return;
+  const float4 me = __ldg(pos + i);
+  const uint32_t cell = static_cast<uint32_t>(p2v[__float_as_uint(me.w)]);
+  const uint32_t* row = nb + size_t(cell) * kNb;
+  ecell[i] = cell;
+  if ((uint32_t(i) - __ldg(cstart + cell)) % kLoopGroup == 0)
+    group[atomicAdd(ctr + kCtrGroups, 1u)] = uint32_t(i);
+  uint32_t n = 0;
+  for (int o = 0; o < kNb; ++o) {
+    const uint32_t c = __ldg(row + o);
+    if (c == kNoCell) continue;
+    const uint32_t j0 = __ldg(cstart + c), m = __ldg(vcnt + c);
+    const float4* q = pos + j0;
+    uint32_t j = 0;
+    for (; j + 4 <= m; j += 4) {
+      float4 w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) w[u] = __ldg(q + j + u);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) n += dist2(w[u], me.x, me.y, me.z) <= r2;
+    }
+    for (; j < m; ++j) n += dist2(__ldg(q + j), me.x, me.y, me.z) <= r2;
+  }
+  cnt[i] = n - 1u;  // (the point itself is at distance 0)
+}
+
+// Sort keys of the points that start marked, in point order: their priority (the pass that
+// reads them drops the sentinel rows and keeps equal keys in point order); the first digit's
+// histogram, the number of marked points and the largest key.
+__global__ __launch_bounds__(256) void thin_prio_kernel(int64_t n, const int32_t* __restrict__ p2v,
+                                                        const uint32_t* __restrict__ entry,
+                                                        const uint32_t* __restrict__ cnt,
+                                                        const uint32_t* __restrict__ prio,
+                                                        uint32_t thr, uint64_t* keys, State* st2,
+                                                        const int* err) {
+  __shared__ uint32_t h[kRadix];
+  if (block_error_raised(err)) return;
+  h[threadIdx.x] = 0;
+  __syncthreads();
+  uint32_t mine = 0, big = 0;
+  for (int64_t p = blockIdx.x * int64_t(256) + threadIdx.x; p < n; p += int64_t(gridDim.x) * 256) {
+    const bool in = p2v[p] >= 0 && cnt[entry[p]] > thr;
+    const uint32_t k = in ? prio[p] : 0u;
+    keys[p] = in ? uint64_t(k) : kKeySentinel;
+    if (in) {
+      ++mine;
+      big = max(big, k);
+      atomicAdd(&h[k & (kRadix - 1)], 1u);
+    }
+  }
+  // (the lanes of a warp may leave the loop after different numbers of trips)
+  __syncwarp();
+  mine = __reduce_add_sync(kFullMask, mine);
+  big = __reduce_max_sync(kFullMask, big);
+  if ((threadIdx.x & 31) == 0 && mine) {
+    atomicAdd(&st2->nitems, mine);
+    atomicMax(&st2->maxkey, (unsigned long long)big);
+  }
+  __syncthreads();
+  if (h[threadIdx.x]) atomicAdd(&st2->hist[0][threadIdx.x], h[threadIdx.x]);
+}
+
+// The sorted points as entries.
+__global__ __launch_bounds__(256) void thin_list_kernel(const State* st2, const uint32_t* idx0,
+                                                        const uint32_t* idx1,
+                                                        const uint32_t* __restrict__ entry,
+                                                        uint32_t* __restrict__ list,
+                                                        const int* err) {
+  if (error_raised(err)) return;
+  const uint32_t* I = sorted_idx(st2, idx0, idx1);
+  const int64_t m = st2->nitems;
+  for (int64_t k = blockIdx.x * int64_t(256) + threadIdx.x; k < m; k += int64_t(gridDim.x) * 256)
+    list[k] = entry[I[k]];
+}
+
+struct LoopArgs {
+  const State* st2;
+  const uint32_t* list;  // entries that start marked, by (priority, point index)
+  const uint32_t* ecell;
+  const uint32_t* cstart;
+  const uint32_t* vcnt;
+  const uint32_t* nb;
+  const float4* pos;
+  const uint32_t* group;
+  uint32_t* cnt;
+  uint8_t* dead;
+  uint32_t* sel;            // scattered: the entries a pass deletes
+  unsigned long long* head;  // gathered: pass << 32 | the cell's last deleted entry's rank
+  float4* node;             // gathered: place of the entry of each rank; w = the next rank
+  uint32_t* ctr;
+  float r2;
+  uint32_t thr;
+  uint32_t batch;
+  double pairs_per_point;
+  int64_t max_passes;
+  uint32_t spin_limit;
+  int* err;
+};
+constexpr uint32_t kListEnd = 0xffffffffu;
+
+// Scattered: kLoopSplit warps a deleted entry share the candidates of its 27 cells, in groups
+// of kLoopGroup, and take one from the count of every one within r.  Counts lie in entry
+// order, so the 32 candidates of a warp step are consecutive words and their decrements
+// (which return nothing) a few sectors.
+__device__ __forceinline__ void thin_scatter(const LoopArgs& a, uint32_t taken, uint64_t gw,
+                                             uint64_t gwarps) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t units = uint64_t(taken) * kLoopSplit;
+  for (uint64_t u = gw; u < units; u += gwarps) {
+    const uint32_t part = uint32_t(u % kLoopSplit);
+    const uint32_t i = __ldcg(a.sel + u / kLoopSplit);
+    const float4 me = __ldg(a.pos + i);
+    uint32_t j0 = 0, mm = 0;
+    if (lane < uint32_t(kNb)) {
+      const uint32_t c = __ldg(a.nb + size_t(__ldg(a.ecell + i)) * kNb + lane);
+      if (c != kNoCell) {
+        j0 = __ldg(a.cstart + c);
+        mm = __ldg(a.vcnt + c);
+      }
+    }
+    const uint32_t ng = (mm + kLoopGroup - 1) / kLoopGroup;
+    uint32_t inc = ng;  // groups of the cells up to this one
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFullMask, inc, off);
+      if (lane >= uint32_t(off)) inc += y;
+    }
+    const uint32_t groups = __shfl_sync(kFullMask, inc, 31);
+    for (uint32_t gi = part; gi < groups; gi += kLoopSplit) {
+      const int l = __popc(__ballot_sync(kFullMask, inc <= gi));  // the group's cell
+      const uint32_t off = (gi - __shfl_sync(kFullMask, inc - ng, l)) * kLoopGroup + lane;
+      const uint32_t n = __shfl_sync(kFullMask, mm, l);
+      const uint32_t j = __shfl_sync(kFullMask, j0, l) + off;
+      float4 w[4];
+#pragma unroll
+      for (uint32_t v = 0; v < 4; ++v)
+        if (off + 32u * v < n) w[v] = __ldg(a.pos + j + 32u * v);
+#pragma unroll
+      for (uint32_t v = 0; v < 4; ++v)  // (the counts of dead entries fall too: never read)
+        if (off + 32u * v < n && j + 32u * v != i && dist2(w[v], me.x, me.y, me.z) <= a.r2)
+          atomicSub(a.cnt + j + 32u * v, 1u);
+    }
   }
 }
+
+// Gathered: a warp a group of entries of one cell walks the lists of this pass's deleted
+// entries in the 27 cells around it (lane l the list of cell l) and counts, for the entries
+// still marked (no other count is read again), the ones within r.
+__device__ __forceinline__ void thin_gather(const LoopArgs& a, uint32_t pass, uint32_t groups,
+                                            uint64_t gw, uint64_t gwarps) {
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint64_t u = gw; u < groups; u += gwarps) {
+    const uint32_t i0 = __ldg(a.group + u);
+    const uint32_t cell = __ldg(a.ecell + i0);
+    const uint32_t end = __ldg(a.cstart + cell) + __ldg(a.vcnt + cell);
+    uint32_t r = kListEnd;
+    if (lane < uint32_t(kNb)) {
+      const uint32_t c = __ldg(a.nb + size_t(cell) * kNb + lane);
+      if (c != kNoCell) {
+        const unsigned long long h = __ldcg(a.head + c);
+        if (uint32_t(h >> 32) == pass) r = uint32_t(h);
+      }
+    }
+    uint32_t some = __ballot_sync(kFullMask, r != kListEnd);
+    if (!some) continue;
+    float4 w[4];
+    uint32_t n[4], hit[4];
+    bool any = false;
+#pragma unroll
+    for (uint32_t v = 0; v < 4; ++v) {
+      const uint32_t i = i0 + 32u * v + lane;
+      n[v] = i < end ? __ldcg(a.cnt + i) : 0u;
+      w[v] = i < end ? __ldg(a.pos + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      hit[v] = 0;
+      any = any || n[v] > a.thr;
+    }
+    if (!__any_sync(kFullMask, any)) continue;
+    while (some) {
+      float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (r != kListEnd) {
+        q = __ldcg(a.node + r);
+        r = __float_as_uint(q.w);
+      }
+      for (; some; some &= some - 1) {
+        const int l = __ffs(some) - 1;
+        const float x = __shfl_sync(kFullMask, q.x, l), y = __shfl_sync(kFullMask, q.y, l),
+                    z = __shfl_sync(kFullMask, q.z, l);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) hit[v] += dist2(w[v], x, y, z) <= a.r2;
+      }
+      some = __ballot_sync(kFullMask, r != kListEnd);
+    }
+#pragma unroll
+    for (uint32_t v = 0; v < 4; ++v)  // (a marked entry's count covers every neighbour left)
+      if (n[v] > a.thr && hit[v]) a.cnt[i0 + 32u * v + lane] = n[v] - hit[v];
+  }
+}
+
+// Every pass of the loop, one cooperative launch (a block an SM), two grid barriers a pass:
+//   1. the batch: every block walks the sorted list from where the last pass stopped, tests
+//      kLoopItems entries a thread, and finds the same `batch` entries still marked (one more
+//      tells that this is not the last pass); block b writes those of rank b mod grid;
+//   2. the counts, by the deleted entries (thin_scatter) or by the marked ones (thin_gather).
+// Bound by the latency of the steps and the barriers.  640x480 frame, cell 0.05 m, threshold
+// 20, batches of 1000 (277K points of 3600 candidates each, 2008 cells, 271 passes): a pass
+// takes 23 us scattered (the drain of its 1.8M decrements is 3/4 of it), 13 us gathered,
+// against 570 us for a fresh count and 500 us of host round trips (recounted).  The gathered
+// form touches every group of entries each pass, 9000 cycles a round of the grid's warps; the
+// scattered form 8000 cycles and one per 90 candidates.
+__global__ __launch_bounds__(kLoopThreads, 1) void thin_loop_kernel(const LoopArgs a) {
+  __shared__ uint32_t tmp[kLoopThreads / 32];
+  __shared__ uint32_t s_next;
+  if (block_error_raised(a.err)) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr[kCtrPasses] = 1u;
+    return;
+  }
+  const uint32_t m = a.st2->nitems;
+  const uint32_t groups = a.ctr[kCtrGroups];
+  const uint64_t gwarps = uint64_t(gridDim.x) * (kLoopThreads / 32);
+  const uint64_t gw = uint64_t(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const bool gather = 9000.0 * ceil(double(groups) / double(gwarps)) <=
+                      8000.0 + double(a.batch) * a.pairs_per_point / 90.0;
+  uint32_t target = 0, first = 0;
+  int64_t passes = 0;
+  while (passes < a.max_passes) {
+    ++passes;
+    // 1. the next `batch` marked entries of the list
+    uint32_t found = 0;
+    for (uint32_t k0 = first; found <= a.batch && k0 < m; k0 += kLoopItems * kLoopThreads) {
+      uint32_t e[kLoopItems], mine = 0;
+      bool in[kLoopItems];
+#pragma unroll
+      for (int q = 0; q < kLoopItems; ++q) {
+        const uint32_t k = k0 + kLoopItems * threadIdx.x + q;
+        e[q] = k < m ? __ldg(a.list + k) : 0u;
+        in[q] = k < m;
+      }
+#pragma unroll
+      for (int q = 0; q < kLoopItems; ++q) {
+        in[q] = in[q] && __ldcg(a.cnt + e[q]) > a.thr;
+        mine += in[q];
+      }
+      uint32_t total;
+      uint32_t r = found + block_excl_scan(mine, &total, tmp);
+#pragma unroll
+      for (int q = 0; q < kLoopItems; ++q) {
+        if (!in[q]) continue;
+        if (r < a.batch) {
+          if (r % gridDim.x == blockIdx.x) {
+            a.dead[e[q]] = 1;
+            if (gather) {
+              float4 w = __ldg(a.pos + e[q]);
+              const unsigned long long tag = (unsigned long long)uint32_t(passes) << 32;
+              const unsigned long long old =
+                  atomicExch(a.head + __ldg(a.ecell + e[q]), tag | r);
+              w.w = __uint_as_float((old ^ tag) >> 32 == 0 ? uint32_t(old) : kListEnd);
+              a.node[r] = w;
+            } else {
+              a.sel[r] = e[q];
+            }
+          }
+          if (r + 1 == a.batch) s_next = k0 + kLoopItems * threadIdx.x + q + 1;
+        }
+        ++r;
+      }
+      found += total;
+      if (m - k0 <= uint32_t(kLoopItems * kLoopThreads)) break;  // (k0 stays below 2^32)
+    }
+    // (the same in every block) the last pass: every marked point goes, by its count, in
+    // the output
+    if (found <= a.batch) break;
+    if (!grid_barrier(a.ctr + kCtrBar, target, a.spin_limit, a.err)) return;
+    first = s_next;
+    // 2. the counts
+    if (gather)
+      thin_gather(a, uint32_t(passes), groups, gw, gwarps);
+    else
+      thin_scatter(a, a.batch, gw, gwarps);
+    if (!grid_barrier(a.ctr + kCtrBar, target, a.spin_limit, a.err)) return;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr[kCtrPasses] = static_cast<uint32_t>(passes);
+}
+
+// keep flag per input point (zeroed before: invalid points stay 0): not deleted by a batch
+// (the flags the last pass has set are of marked points: those go anyway),
+// and its count at most the threshold at the end (the last pass deletes the points still
+// marked); number kept.
+__global__ __launch_bounds__(256) void thin_keep_kernel(const State* st,
+                                                        const float4* __restrict__ pos,
+                                                        const uint32_t* __restrict__ cnt,
+                                                        const uint8_t* __restrict__ dead,
+                                                        uint32_t thr, uint8_t* keep,
+                                                        uint32_t* kept, const int* err) {
+  if (error_raised(err)) return;  // every keep flag stays 0, the count 0
+  uint32_t c = 0;
+  const int64_t m = st->nitems;
+  for (int64_t i = blockIdx.x * int64_t(256) + threadIdx.x; i < m; i += int64_t(gridDim.x) * 256) {
+    const bool k = !dead[i] && cnt[i] <= thr;
+    if (k) keep[__float_as_uint(pos[i].w)] = 1;
+    c += k;
+  }
+  __syncwarp();
+  c = __reduce_add_sync(kFullMask, c);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(kept, c);
+}
+
+// ---- recounted --------------------------------------------------------------------------
 
 // One pass: every remaining point counts the other remaining points within r in the 27
 // cells around it (squared distance, binary32, ((dx*dx + dy*dy) + dz*dz)) and is marked
@@ -133,7 +485,7 @@ __global__ void thin_neighbors_kernel(const int64_t* __restrict__ num_cells,
 __global__ __launch_bounds__(256) void thin_count_kernel(
     const State* st, const int32_t* __restrict__ p2v, const uint32_t* __restrict__ sidx,
     const uint32_t* __restrict__ cstart, const uint32_t* __restrict__ vcnt,
-    const uint32_t* __restrict__ nb, const float* __restrict__ sx, uint8_t* state, float r2,
+    const uint32_t* __restrict__ nb, const float4* __restrict__ pos, uint8_t* state, float r2,
     int64_t threshold, uint32_t* marked_count, const int* err) {
   if (error_raised(err)) return;  // nothing marked: the loop ends after one pass
   const int64_t m = st->nitems;
@@ -141,7 +493,7 @@ __global__ __launch_bounds__(256) void thin_count_kernel(
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < m;
        i += int64_t(gridDim.x) * blockDim.x) {
     if (!(state[i] & kAlive)) continue;
-    const float x = sx[3 * i], y = sx[3 * i + 1], z = sx[3 * i + 2];
+    const float4 me = pos[i];
     const uint32_t row = static_cast<uint32_t>(p2v[sidx[i]]);
     int64_t cnt = 0;
     for (int o = 0; o < kNb && cnt <= threshold; ++o) {
@@ -150,12 +502,7 @@ __global__ __launch_bounds__(256) void thin_count_kernel(
       const int64_t j0 = cstart[c], j1 = j0 + vcnt[c];
       for (int64_t j = j0; j < j1 && cnt <= threshold; ++j) {
         if (j == i || !(state[j] & kAlive)) continue;
-        const float ex = __fsub_rn(sx[3 * j], x);
-        const float ey = __fsub_rn(sx[3 * j + 1], y);
-        const float ez = __fsub_rn(sx[3 * j + 2], z);
-        const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)),
-                                   __fmul_rn(ez, ez));
-        if (d2 <= r2) ++cnt;
+        if (dist2(pos[j], me.x, me.y, me.z) <= r2) ++cnt;
       }
     }
     if (cnt > threshold) {
@@ -234,6 +581,26 @@ __global__ void thin_finish_kernel(const uint32_t* kept, int64_t* out_num_kept) 
 
 vg_status thin_status(cudaError_t e) { return e == cudaSuccess ? VG_OK : VG_ERR_CUDA; }
 
+// Blocks of the loop's cooperative launch (one an SM), 0 where it cannot run.
+int thin_loop_grid() {
+  int v = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, thin_loop_kernel, kLoopThreads, 0) !=
+      cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return v > 0 ? num_sms() : 0;
+}
+
+// Whether the loop keeps counts: a pass that deletes `batch` points meets batch * pairs / n
+// candidates; a fresh count of every point tests about three candidates per neighbour it
+// finds, up to threshold + 1 of them, and goes through the host.
+bool keep_counts(int64_t n, unsigned long long pairs, int64_t batch, int64_t threshold) {
+  if (n <= 0) return false;
+  const double per_pass = double(batch < n ? batch : n) * (double(pairs) / double(n));
+  return per_pass <= 3.0 * double(n) * (double(threshold) + 1.0);
+}
+
 int grid_for(int64_t n) {
   const int64_t b = ceil_div(n < 1 ? 1 : n, 256);
   const int64_t cap = int64_t(num_sms()) * 8;
@@ -275,13 +642,16 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
   State* st = reinterpret_cast<State*>(ws + S.state);
   int* err = out_error ? reinterpret_cast<int*>(out_error) : &st->error;
   uint64_t* vkeys = reinterpret_cast<uint64_t*>(ws + L.vkeys);
-  float* vcent = reinterpret_cast<float*>(ws + L.vcent);
+  float* vcent = reinterpret_cast<float*>(ws + L.pos);
+  float4* pos = reinterpret_cast<float4*>(ws + L.pos);
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
   uint32_t* vcnt = reinterpret_cast<uint32_t*>(ws + L.vcnt);
   int64_t* vnum = reinterpret_cast<int64_t*>(ws + L.vnum);
   int32_t* p2v = reinterpret_cast<int32_t*>(ws + L.p2v);
   uint32_t* cstart = reinterpret_cast<uint32_t*>(ws + L.cstart);
   uint32_t* nb = reinterpret_cast<uint32_t*>(ws + L.nb);
-  float* sx = reinterpret_cast<float*>(ws + L.sx);
+  uint32_t* entry = reinterpret_cast<uint32_t*>(ws + L.vkeys);  // (once the cells' keys are read)
+  uint32_t* list = entry + (n < 1 ? 1 : n);
   uint32_t* sprio = reinterpret_cast<uint32_t*>(ws + L.sprio);
   uint32_t* sidx = reinterpret_cast<uint32_t*>(ws + L.sidx);
   uint8_t* state = reinterpret_cast<uint8_t*>(ws + L.state);
@@ -298,24 +668,75 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
                            frames_workspace_bytes(n, 1, VG_METHOD_SORT), VG_METHOD_SORT, stream);
   if (s != VG_OK) return s;
   cudaError_t e = n > 0 ? cudaMemsetAsync(out_keep, 0, size_t(n), stream) : cudaSuccess;
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, 4 * sizeof(uint32_t), stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, kCtrWords * sizeof(uint32_t), stream);
   if (e != cudaSuccess) return VG_ERR_CUDA;
-  const uint32_t* idx0 = reinterpret_cast<const uint32_t*>(ws + S.idx0);
-  const uint32_t* idx1 = reinterpret_cast<const uint32_t*>(ws + S.idx1);
+  uint32_t* idx0 = reinterpret_cast<uint32_t*>(ws + S.idx0);
+  uint32_t* idx1 = reinterpret_cast<uint32_t*>(ws + S.idx1);
   const int g = grid_for(n);
+  unsigned long long pairs = 0;
   if (n > 0) {
-    thin_setup_kernel<<<g, 256, 0, stream>>>(st, idx0, idx1, xyz, priority, p2v, cstart, sx,
-                                             sprio, sidx, state, err);
-    thin_neighbors_kernel<<<g, 256, 0, stream>>>(vnum, vkeys, nb, err);
+    thin_neighbors_kernel<<<num_sms() * 8, 256, 0, stream>>>(
+        vnum, vkeys, vcnt, nb, reinterpret_cast<unsigned long long*>(ctr + kCtrPairs), err);
+    thin_setup_kernel<<<g, 256, 0, stream>>>(st, idx0, idx1, xyz, priority, p2v, cstart, pos,
+                                             sprio, sidx, entry, state, err);
+    e = cudaMemcpyAsync(&pairs, ctr + kCtrPairs, sizeof(pairs), cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) return VG_ERR_CUDA;
   }
-  const float r2 = radius * radius;
   const int64_t max_passes = n / batch + 2;  // every pass but the last deletes `batch` points
+  const float r2 = radius * radius;
   int32_t passes = 0;
+  const int loop_grid = n > 0 ? thin_loop_grid() : 0;
+  if (keep_counts(n, pairs, batch, threshold) && loop_grid > 0) {
+    const uint32_t thr = static_cast<uint32_t>(threshold < 0xfffffffell ? threshold : 0xfffffffell);
+    State* st2 = reinterpret_cast<State*>(ws + L.st2);
+    uint64_t* keys0 = reinterpret_cast<uint64_t*>(ws + S.keys0);
+    uint64_t* keys1 = reinterpret_cast<uint64_t*>(ws + S.keys1);
+    uint32_t* lb_a = reinterpret_cast<uint32_t*>(ws + S.lb_a);
+    uint32_t* lb_b = reinterpret_cast<uint32_t*>(ws + S.lb_b);
+    e = cudaMemsetAsync(st2, 0, sizeof(State), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(state, 0, size_t(n), stream);
+    if (e == cudaSuccess)
+      e = cudaMemsetAsync(lb_a, 0, size_t(S.sort_tiles) * kRadix * sizeof(uint32_t), stream);
+    if (e != cudaSuccess) return VG_ERR_CUDA;
+    uint32_t* ecell = sprio;  // (the recounted form's arrays)
+    uint32_t* group = sidx;
+    thin_full_count_kernel<<<static_cast<int>(ceil_div(n, kFullThreads)), kFullThreads, 0,
+                             stream>>>(st, p2v, cstart, vcnt, nb, pos, cnt, ecell, group, ctr, r2,
+                                       err);
+    thin_prio_kernel<<<g, 256, 0, stream>>>(n, p2v, entry, cnt, priority, thr, keys0, st2, err);
+    for (int p = 0; p < kNarrowPasses && e == cudaSuccess; ++p)  // 32-bit priorities
+      e = launch_sort_pass(st2, keys0, idx0, keys1, idx1, lb_a, lb_b, n, p, false, spin_limit(),
+                           err, stream);
+    if (e != cudaSuccess) return VG_ERR_CUDA;
+    thin_list_kernel<<<g, 256, 0, stream>>>(st2, idx0, idx1, entry, list, err);
+    // the sort's buffers again: the deleted lists' heads (a cell each) and nodes (16 bytes a
+    // point of the batch, in the 16 bytes a point from keys1 to the end of idx1), or `sel`
+    e = cudaMemsetAsync(keys0, 0, size_t(n) * sizeof(uint64_t), stream);
+    if (e != cudaSuccess) return VG_ERR_CUDA;
+    LoopArgs la{st2, list, ecell, cstart, vcnt, nb, pos, group, cnt, state,
+                reinterpret_cast<uint32_t*>(keys0), reinterpret_cast<unsigned long long*>(keys0),
+                reinterpret_cast<float4*>(keys1), ctr, r2, thr,
+                static_cast<uint32_t>(batch < n ? batch : n), double(pairs) / double(n),
+                max_passes, spin_limit(), err};
+    void* args[] = {&la};
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(thin_loop_kernel),
+                                    dim3(loop_grid), dim3(kLoopThreads), args, 0, stream);
+    if (e != cudaSuccess) return VG_ERR_CUDA;
+    thin_keep_kernel<<<g, 256, 0, stream>>>(st, pos, cnt, state, thr, out_keep, ctr + kCtrKept,
+                                            err);
+    thin_finish_kernel<<<1, 1, 0, stream>>>(ctr + kCtrKept, out_num_kept);
+    uint32_t run = 0;
+    e = cudaMemcpyAsync(&run, ctr + kCtrPasses, sizeof(run), cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (out_passes) *out_passes = static_cast<int32_t>(run);
+    return thin_status(e == cudaSuccess ? cudaGetLastError() : e);
+  }
   for (; n > 0 && passes < max_passes; ++passes) {
     uint32_t marked = 0;
     e = cudaMemsetAsync(ctr, 0, sizeof(uint32_t), stream);
     if (e != cudaSuccess) return VG_ERR_CUDA;
-    thin_count_kernel<<<g, 256, 0, stream>>>(st, p2v, sidx, cstart, vcnt, nb, sx, state, r2,
+    thin_count_kernel<<<g, 256, 0, stream>>>(st, p2v, sidx, cstart, vcnt, nb, pos, state, r2,
                                              threshold, ctr, err);
     e = cudaMemcpyAsync(&marked, ctr, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -346,8 +767,8 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
     thin_delete_kernel<<<g, 256, 0, stream>>>(st, state, sprio, sidx, prefix, mask, err);
   }
   if (n > 0) {
-    thin_output_kernel<<<g, 256, 0, stream>>>(st, state, sidx, out_keep, ctr + 1, err);
-    thin_finish_kernel<<<1, 1, 0, stream>>>(ctr + 1, out_num_kept);
+    thin_output_kernel<<<g, 256, 0, stream>>>(st, state, sidx, out_keep, ctr + kCtrKept, err);
+    thin_finish_kernel<<<1, 1, 0, stream>>>(ctr + kCtrKept, out_num_kept);
   } else {
     e = cudaMemsetAsync(out_num_kept, 0, sizeof(int64_t), stream);
   }
