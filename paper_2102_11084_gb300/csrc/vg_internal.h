@@ -412,7 +412,7 @@ cudaError_t launch_hash_p2v(const uint32_t* point_slot, const uint32_t* slot_ran
 // ---- pyramid ----
 constexpr int kMaxLevels = 8;
 constexpr int kMergeThreads = 256;
-constexpr int kMergeItems = 8;
+constexpr int kMergeItems = 4;
 constexpr int kMergeTile = kMergeThreads * kMergeItems;
 // Merges pyramid level k-1 (rows [off[k-1], off[k])) into level k (written from off[k]).
 cudaError_t launch_pyramid_merge(State* st, const FrameState* fs, int level, uint64_t* keys,
