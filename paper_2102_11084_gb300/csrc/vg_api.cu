@@ -12,6 +12,7 @@
 #include "vg_api_internal.h"
 #include "vg_internal.h"
 #include "vg_frame.h"
+#include "vg_trie.h"
 
 namespace vg {
 
@@ -61,6 +62,7 @@ void warm_launch_config() {
   warm_filter_config();
   warm_msd_config();
   warm_frame_config();
+  warm_trie_config();
 }
 
 int persistent_grid(const void* kernel, int threads, size_t dyn_smem, int64_t work_tiles) {
@@ -113,12 +115,23 @@ int method_of(int flags) {
   return m == VG_METHOD_HASH ? VG_METHOD_HASH : VG_METHOD_SORT;
 }
 
+// Whether the flags and the size let a call take the occupancy trie (vg_trie.cu).  AUTO
+// only: the other methods name a grouping.
+bool trie_call(int64_t n, int flags) {
+  return (flags & VG_METHOD_MASK) == VG_METHOD_AUTO &&
+         (flags & (VG_SORT_LSD | VG_SORT_FRAME)) == 0 && n > 0 && n <= kTrSmallPoints;
+}
+
 }  // namespace
 
 size_t frames_workspace_bytes(int64_t n, int frames, int flags) {
   if (n < 0 || frames < 1) return 0;
   if (method_of(flags) == VG_METHOD_HASH) return hash_layout(n, frames).total;
   const SortLayout L = sort_layout(n, frames);
+  if (trie_call(n, flags)) {
+    const size_t t = trie_layout(n, L.lb_a).total;
+    return t > L.total ? t : L.total;
+  }
   if ((flags & VG_SORT_FRAME) == 0) return L.total;
   // the bin grouping after the sort layout, or the one-launch grouping after the frame state
   const size_t a = frame_layout(n, L.total).total, b = fused_layout(n, L.lb_a).total;
@@ -146,7 +159,9 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
   const int F = fr.nframes;
   const int method = method_of(flags);
   const NvtxRange range(method == VG_METHOD_HASH ? "vg: decimate (hash)" : "vg: decimate (sort)");
-  const size_t need = frames_workspace_bytes(n, F, flags);
+  // (a workspace of the sort path alone is enough for a call that may take the trie)
+  const bool trie_ok = trie_call(n, flags);
+  const size_t need = trie_ok ? sort_layout(n, F).total : frames_workspace_bytes(n, F, flags);
   if (!workspace || workspace_bytes < need) return VG_ERR_WORKSPACE;
   char* ws = static_cast<char*>(workspace);
   const uint32_t spins = spin_limit();
@@ -183,6 +198,19 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
     uint64_t* pay_0 = reinterpret_cast<uint64_t*>(ws + L.keys1);
     uint64_t* pay_1 = reinterpret_cast<uint64_t*>(ws + L.idx0);
     int* err = out_error ? reinterpret_cast<int*>(out_error) : &st->error;
+
+    if (trie_ok && trie_available(posed(frn))) {
+      const TrieLayout TL = trie_layout(n, L.lb_a);
+      if (workspace_bytes >= TL.total) {
+        mark(stage, stream);
+        const cudaError_t et = launch_trie(xyz, frn, st, fs, ws, TL, out, spins, err, stream);
+        if (et != cudaErrorCooperativeLaunchTooLarge) {
+          for (int k = 1; k < 1 + 1 + 1 + 3 + kMaxPasses + 1; ++k) mark(stage + k, stream);
+          return cuda_status(et);
+        }
+        (void)cudaGetLastError();  // (SMs withheld from this process: the sort path)
+      }
+    }
 
     // (the frame path needs only the state and frame state cleared: its last kernel
     // writes the voxel count and the frame offsets)
@@ -304,7 +332,7 @@ struct PyramidLayout {
 PyramidLayout pyramid_layout(int64_t n, int levels) {
   PyramidLayout L{};
   const int64_t nn = n < 1 ? 1 : n;
-  L.base = sort_layout(n, 1).total;
+  L.base = frames_workspace_bytes(n, 1, VG_METHOD_AUTO);
   size_t off = L.base;
   L.sums_a = off;
   off = align_up(off + size_t(nn) * 3 * sizeof(long long), 256);
@@ -541,7 +569,7 @@ vg_status vg_pyramid(const float* xyz, int64_t n, float* origin, float leaf, int
   SegOut out{out_keys, out_centroids, out_counts, sums[0], cap_total, out_level_offsets + 1,
              nullptr, out_point_to_voxel};
   // level 0 by the sort method's grouping (the AUTO choice unless the flags name one)
-  s = run_frames(xyz, fr, from_min, out, out_error, workspace, L.total,
+  s = run_frames(xyz, fr, from_min, out, out_error, workspace, P.base,
                  flags & (VG_SORT_BUCKETS | VG_SORT_LSD), stream);
   if (s != VG_OK) return s;
   const uint32_t spins = spin_limit();

@@ -18,6 +18,7 @@
 #include "../../include/vg.h"
 #include "vg_api_internal.h"
 #include "vg_internal.h"
+#include "vg_trie.h"
 
 struct vg_plan {
   int device = 0;
@@ -86,7 +87,11 @@ vg_status vg_plan_create(vg_plan** out, int max_frames, int64_t max_points, int 
   // room for every grouping a later configure may pick
   const size_t a = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_SORT | VG_SORT_FRAME);
   const size_t b = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_HASH);
+  const size_t c = vg::frames_workspace_bytes(
+      max_points < vg::kTrSmallPoints ? max_points : vg::kTrSmallPoints, max_frames,
+      VG_METHOD_AUTO);
   p->ws_bytes = a > b ? a : b;
+  if (c > p->ws_bytes) p->ws_bytes = c;
   if (cudaMalloc(&p->ws, p->ws_bytes) != cudaSuccess) {
     delete p;
     return VG_ERR_CUDA;

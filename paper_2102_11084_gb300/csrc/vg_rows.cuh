@@ -18,7 +18,7 @@ struct RowCtx {
 
 // Row `cur`: cell `key` (the full sort key) with n entries whose offsets sum to s.
 __device__ __forceinline__ void put_row(const RowCtx& rc, const SegOut& out, uint32_t cur,
-                                        uint32_t key, const Acc& a, int* err) {
+                                        uint64_t key, const Acc& a, int* err) {
   if (int64_t(cur) >= out.cap) {
     set_error(err, kErrCapacity);
     return;
