@@ -73,12 +73,16 @@ typedef enum {
 /* flags */
 #define VG_ORIGIN_FROM_MIN 1 /* compute origin = per-axis min of the valid points and
                                 write it to `origin` (else `origin` is read)            */
-#define VG_METHOD_AUTO 0     /* the library's choice: SORT, with the bucket grouping
-                                from 4,194,304 points on and every digit in global radix
-                                passes (VG_SORT_LSD) below.  A single camera frame is
-                                fastest with VG_SORT_FRAME, which AUTO does not take: it
-                                needs 32-bit keys, known only on the device, and AUTO
-                                serves every cloud without a host synchronisation        */
+#define VG_METHOD_AUTO 0     /* the library's choice, without a host synchronisation: up
+                                to 2,097,152 points (in all frames, with or without
+                                point_to_voxel, attributes and poses) an occupancy trie
+                                over the keys, ONE cooperative launch for keys of any
+                                width; the bucket grouping of SORT from 4,194,304 points
+                                on; every digit in global radix passes (VG_SORT_LSD)
+                                between.  The trie needs the workspace of the query; a
+                                smaller one that holds the sort path takes the latter.
+                                One camera frame with 32-bit keys is a little faster
+                                still with VG_SORT_FRAME                                 */
 #define VG_METHOD_SORT 16    /* sort the points by key and reduce each run of equal keys.
                                 32-bit keys (no point_to_voxel, no attributes, extents
                                 bound the keys): the top <= 16 key bits are split by one

@@ -119,7 +119,7 @@ int method_of(int flags) {
 // only: the other methods name a grouping.
 bool trie_call(int64_t n, int flags) {
   return (flags & VG_METHOD_MASK) == VG_METHOD_AUTO &&
-         (flags & (VG_SORT_LSD | VG_SORT_FRAME)) == 0 && n > 0 && n <= kTrSmallPoints;
+         (flags & (VG_SORT_LSD | VG_SORT_FRAME)) == 0 && n > 0 && n <= kTrMaxPoints;
 }
 
 }  // namespace
@@ -129,7 +129,7 @@ size_t frames_workspace_bytes(int64_t n, int frames, int flags) {
   if (method_of(flags) == VG_METHOD_HASH) return hash_layout(n, frames).total;
   const SortLayout L = sort_layout(n, frames);
   if (trie_call(n, flags)) {
-    const size_t t = trie_layout(n, L.lb_a).total;
+    const size_t t = trie_layout(n, frames, L.lb_a).total;
     return t > L.total ? t : L.total;
   }
   if ((flags & VG_SORT_FRAME) == 0) return L.total;
@@ -200,7 +200,7 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
     int* err = out_error ? reinterpret_cast<int*>(out_error) : &st->error;
 
     if (trie_ok && trie_available(posed(frn))) {
-      const TrieLayout TL = trie_layout(n, L.lb_a);
+      const TrieLayout TL = trie_layout(n, F, L.lb_a);
       if (workspace_bytes >= TL.total) {
         mark(stage, stream);
         const cudaError_t et = launch_trie(xyz, frn, st, fs, ws, TL, out, spins, err, stream);

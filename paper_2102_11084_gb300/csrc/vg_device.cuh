@@ -467,8 +467,9 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* ctr, uint32_t& target, ui
   bool late = false;
   if (threadIdx.x == 0) {
     target += gridDim.x;
-    __threadfence();
-    atomicAdd(ctr, 1u);
+    // (the block's writes are ordered before the arrival by the barrier above and the
+    // release; the acquire orders every block's before what follows)
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
     uint32_t spins = 0;
     while (static_cast<int32_t>(ld_acquire(ctr) - target) < 0) {
       if (++spins > spin) {
@@ -476,9 +477,8 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* ctr, uint32_t& target, ui
         late = true;
         break;
       }
-      if (spins > 16) __nanosleep(32);
+      if (spins > 64) __nanosleep(32);
     }
-    __threadfence();
   }
   return __syncthreads_or(late) == 0;
 }

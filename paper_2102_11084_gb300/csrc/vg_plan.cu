@@ -88,7 +88,7 @@ vg_status vg_plan_create(vg_plan** out, int max_frames, int64_t max_points, int 
   const size_t a = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_SORT | VG_SORT_FRAME);
   const size_t b = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_HASH);
   const size_t c = vg::frames_workspace_bytes(
-      max_points < vg::kTrSmallPoints ? max_points : vg::kTrSmallPoints, max_frames,
+      max_points < vg::kTrMaxPoints ? max_points : vg::kTrMaxPoints, max_frames,
       VG_METHOD_AUTO);
   p->ws_bytes = a > b ? a : b;
   if (c > p->ws_bytes) p->ws_bytes = c;

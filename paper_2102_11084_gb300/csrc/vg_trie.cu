@@ -12,22 +12,28 @@
 // Each level is marked by a pass over the points, its set bits counted per block and, after a
 // barrier, ranked: a slot's record holds the set bits before the slot and, as bytes, before
 // each of its 8 words.  Keys of up to 24 bits take one level, each 8 bits more another one.
-// The points are read again by every pass (from L2 for the clouds this is made for) and
-// their keys computed again: that costs less than keeping them.
+// The points are read twice, for the extents and for the first level; that second pass also
+// merges runs of equal keys among a warp's 32 consecutive points (neighbouring pixels of a
+// camera frame often share a cell) and writes each run, 16 bytes, to a dense list of its warp
+// (L2-resident scratch), which every later pass reads instead.  A 1280x720 frame at 0.05 m:
+// 44 us; with every point's run kept in shared memory, undensed, 50 us; computing the keys
+// again in every pass 63 us.
 //
 // Passes, with a grid barrier after each:
 //   extents   per-frame min and max; the first level's bits cleared;
-//   mark      (per level) the bit of every point's prefix: lanes of a warp with the same
-//             word merged, and no atomic where the bit is seen set already;
+//   mark      (per level) the bit of every run's prefix, and no atomic where the bit is seen
+//             set already; the lanes of a warp that set bits of one word merge while that
+//             merges anything (a camera frame's warp meets few words, a shuffled cloud's many);
 //   count, rank
-//   add       runs of equal keys among a warp's 32 consecutive points (neighbouring pixels of a
-//             camera frame often share a cell) summed by a segmented scan; a run adds its points
-//             and sums at its row with two 64-bit atomics whose returned values tell the
-//             carries out of their 32-bit halves; point_to_voxel and attribute sums here too;
+//   add       a run's points and sums at its row, with two 64-bit atomics whose returned
+//             values tell the carries out of their 32-bit halves; attribute sums and, through
+//             the runs, point_to_voxel here too;
 //   rows      one thread a row: the centroid, by the formula and from the integer sums of every
 //             other grouping, so the rows are theirs bit for bit.
-// Bound by the latency of the passes and barriers for a camera frame and by instruction issue
-// for several (every pass computes keys), not by HBM: TRIE_NUMBERS
+// Bound by the latency of the passes and barriers (1.2 us each) for a camera frame, by
+// instruction issue in the first mark pass for several, and by L2's random accesses (80 to 115
+// sectors a cycle) for a shuffled cloud; HBM is idle.  A 640x480 frame at 0.05 m: 33 us, where
+// the radix sort's 15 launches take 105; 1M shuffled points: 110 us against 156.
 // Every wait is bounded (kErrTimeout after the limit, and the block returns), and every index
 // read back from scratch is checked against its buffer.
 #include <cstddef>
@@ -41,6 +47,8 @@
 namespace vg {
 namespace {
 
+constexpr int kTrAdd = 1;  // runs a lane adds at a time
+
 struct TrArgs {
   const float* xyz;
   FramesArg fr;
@@ -50,78 +58,118 @@ struct TrArgs {
   uint4* rootrec;
   char* x;             // buffers of the further levels
   char* y;
-  uint32_t* pslot;     // per point: the slot of its prefix (at the last point of its run)
+  uint4* run;          // a warp's runs: {key, sum x, sum y, sum z | points << 26}
+  uint32_t* runhi;     // the upper key words (keys of more than 32 bits)
+  uint2* runatt;       // the runs' attribute sums, 16 bits a channel
+  uint32_t* pslot;     // the slot of a run's prefix, then its row
+  uint2* mask;         // per 32 points: lanes that end a run, valid lanes (point_to_voxel)
   uint32_t* stat;      // per level (8): the blocks' totals
   SegOut out;
   int64_t slots;       // slots and rows the buffers hold
-  int root_bits;
+  uint32_t chunks;     // chunks of points at most
   uint32_t spin_limit;
   int* err;
 };
 
 struct TrSmem {
-  int64_t off[kMaxFrames + 1];
-  uint32_t cstart[kMaxFrames + 1];
-  float org[kMaxFrames][3];
-  float leaf[kMaxFrames];
-  float rleaf[kMaxFrames];
-  float inv_unit[kMaxFrames];
   uint32_t tmp[kTrThreads / 32];
   float red[kTrThreads / 32][6];
-  unsigned long long kmax[kTrThreads / 32];
   uint32_t bits[kTrThreads / 32];
   uint32_t first;
 };
-static_assert(sizeof(TrSmem) <= 48 * 1024, "static shared memory");
 
-// f(frame, point index, inside, x, y, z) for every point of chunks [c0, c1) (1024 points of
-// one frame each, a thread a point; all threads call f, `inside` false past the frame's end,
-// where the coordinates are NaN).  The next chunk's points are loaded one step ahead.
-template <bool kPosed, typename F>
-__device__ __forceinline__ void tr_points(const TrArgs& a, const TrSmem& sm, uint32_t c0,
-                                          uint32_t c1, F f) {
+// Tables of a call's frames (dynamic shared memory).
+struct TrFrames {
+  float4* pose;      // [F][4]: the rows of [R|t], then the height limits (posed calls)
+  int64_t* off;      // [F + 1]
+  float* org;        // [F][3]
+  float* leaf;       // [F]
+  float* rleaf;
+  float* inv_unit;
+  uint32_t* cstart;  // [F + 1]
+};
+constexpr size_t tr_frames_bytes(int frames, bool posed) {
+  return align_up(size_t(frames + 1) * 12 + size_t(frames) * (posed ? 88 : 24), 16);
+}
+__device__ __forceinline__ TrFrames tr_frames(unsigned char* mem, int F, bool posed) {
+  TrFrames t;
+  t.pose = reinterpret_cast<float4*>(mem);
+  t.off = reinterpret_cast<int64_t*>(t.pose + (posed ? 4 * F : 0));
+  t.org = reinterpret_cast<float*>(t.off + F + 1);
+  t.leaf = t.org + 3 * F;
+  t.rleaf = t.leaf + F;
+  t.inv_unit = t.rleaf + F;
+  t.cstart = reinterpret_cast<uint32_t*>(t.inv_unit + F);
+  return t;
+}
+
+// U points of a thread (one of each of U chunks): frame, index, whether inside the frame, and
+// coordinates (NaN outside).
+template <int U>
+struct TrPoints {
+  int f[U];
+  int64_t p[U];
+  bool in[U];
+  float q[U][3];
+};
+
+// fn(points) for every U chunks of this block: chunk c (1024 points of one frame, a thread a
+// point) belongs to block c mod grid, so that the blocks share the dense parts of a cloud.  All
+// threads call fn the same number of times.  The next points are loaded one step ahead.
+template <bool kPosed, int U, typename Fn>
+__device__ __forceinline__ void tr_points(const TrArgs& a, const TrFrames& fm, uint32_t T, Fn fn) {
   const int nf = a.fr.nframes;
   const float nan = __int_as_float(0x7fc00000);
-  int fn = 0;
-  int64_t pn = 0;
-  bool inn = false;
-  float nx = nan, ny = nan, nz = nan;
-  auto load = [&](uint32_t c) {
-    fn = nf > 1 ? chunk_frame(sm.cstart, nf, c) : 0;
-    pn = sm.off[fn] + int64_t(c - sm.cstart[fn]) * kChunk + threadIdx.x;
-    inn = pn < sm.off[fn + 1];
-    const float* q = a.xyz + 3 * pn;
-    nx = inn ? __ldg(q) : nan;
-    ny = inn ? __ldg(q + 1) : nan;
-    nz = inn ? __ldg(q + 2) : nan;
-  };
-  if (c0 < c1) load(c0);
-  Pose P;
-  int pose_f = -1;
-  for (uint32_t c = c0; c < c1; ++c) {
-    float x = nx, y = ny, z = nz;
-    const int fr = fn;
-    const int64_t p = pn;
-    const bool in = inn;
-    if (c + 1 < c1) load(c + 1);
-    if (kPosed) {
-      if (fr != pose_f) {
-        load_pose(a.fr, fr, P);
-        pose_f = fr;
+  TrPoints<U> next;
+  auto load = [&](uint64_t c0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint64_t c = c0 + uint64_t(u) * gridDim.x;
+      next.f[u] = 0;
+      next.p[u] = 0;
+      next.in[u] = false;
+      if (c < T) {
+        const int f = nf > 1 ? chunk_frame(fm.cstart, nf, uint32_t(c)) : 0;
+        next.f[u] = f;
+        next.p[u] = fm.off[f] + (int64_t(c) - fm.cstart[f]) * kChunk + threadIdx.x;
+        next.in[u] = next.p[u] < fm.off[f + 1];
       }
-      pose_point(P, x, y, z);
+      const float* q = a.xyz + 3 * next.p[u];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) next.q[u][k] = next.in[u] ? __ldg(q + k) : nan;
     }
-    f(fr, p, in, x, y, z);
+  };
+  const uint64_t step = uint64_t(U) * gridDim.x;
+  load(blockIdx.x);
+  for (uint64_t c = blockIdx.x; c < T; c += step) {
+    TrPoints<U> now = next;
+    if (c + step < T) load(c + step);
+    if (kPosed) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float4* t = fm.pose + 4 * now.f[u];
+        const float4 r0 = t[0], r1 = t[1], r2 = t[2], z = t[3];
+        Pose P;
+        P.r[0] = r0.x, P.r[1] = r0.y, P.r[2] = r0.z, P.r[3] = r0.w;
+        P.r[4] = r1.x, P.r[5] = r1.y, P.r[6] = r1.z, P.r[7] = r1.w;
+        P.r[8] = r2.x, P.r[9] = r2.y, P.r[10] = r2.z, P.r[11] = r2.w;
+        P.zlo = z.x;
+        P.zhi = z.y;
+        P.rigid = a.fr.poses != nullptr;
+        pose_point(P, now.q[u][0], now.q[u][1], now.q[u][2]);
+      }
+    }
+    fn(now);
   }
 }
 
 // The sort key of a point of frame f (indices in ijk); false for an invalid point or one out
 // of range (*range_bad set).
-__device__ __forceinline__ bool tr_key(const TrSmem& sm, int f, float x, float y, float z,
+__device__ __forceinline__ bool tr_key(const TrFrames& fm, int f, float x, float y, float z,
                                        bool wide, uint32_t key_shift, uint64_t* key,
                                        uint32_t ijk[3], bool* range_bad) {
-  const float o[3] = {sm.org[f][0], sm.org[f][1], sm.org[f][2]};
-  if (!point_index(x, y, z, o, sm.leaf[f], sm.rleaf[f], ijk, range_bad)) return false;
+  const float o[3] = {fm.org[3 * f], fm.org[3 * f + 1], fm.org[3 * f + 2]};
+  if (!point_index(x, y, z, o, fm.leaf[f], fm.rleaf[f], ijk, range_bad)) return false;
   if (wide)
     *key = key_compose(uint32_t(f), morton3(ijk[0], ijk[1], ijk[2]), key_shift);
   else  // per-frame keys of at most 32 bits
@@ -144,29 +192,43 @@ __device__ __forceinline__ uint32_t tr_run(uint64_t key, bool ok, uint32_t* head
   return later ? lane + __ffs(later) - 1u : 31u;
 }
 
-// Sets bit d (0..255) of slot s for the lanes of `em`: one atomic a word among the warp's
-// lanes that do not see their bit set (kCached: through L1, where a stale line can only
-// lack bits).
-template <bool kCached>
-__device__ __forceinline__ void tr_mark(uint32_t* bits, uint32_t s, uint32_t d, bool emit) {
-  const uint32_t word = s * kTrWords + (d >> 5);
-  const uint32_t bit = 1u << (d & 31u);
-  bool need = false;
-  if (emit) need = ((kCached ? __ldca(bits + word) : __ldcg(bits + word)) & bit) == 0u;
-  const uint32_t m = __ballot_sync(kFullMask, need);
-  if (need) {
-    const uint32_t peers = __match_any_sync(m, word);
-    const uint32_t v = __reduce_or_sync(peers, bit);
-    if (int(threadIdx.x & 31u) == __ffs(peers) - 1) atomicOr(bits + word, v);
+// Sets bit id & 255 of slot id >> 8 for every lane with `emit` that does not see its bit set
+// (`seen`: the word as loaded before; a stale one can only lack bits).  Up to half a warp of
+// lanes (a camera frame's runs, which meet a few words) merges them word by word: the
+// atomics of all warps on the few words took 8,500 cycles more of a 640x480 frame.  More
+// lanes (a shuffled cloud's points, a word each) merge the first two words' only: match.any
+// and a redux a group cost a full warp 2,000 cycles.
+__device__ __forceinline__ void tr_set(uint32_t* bits, uint32_t id, bool emit, uint32_t seen) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t bit = 1u << (id & 31u), word = id >> 5;
+  bool need = emit && (seen & bit) == 0u;
+  uint32_t m = __ballot_sync(kFullMask, need);
+  if (__popc(m) <= 16) {
+    if (need) {
+      const uint32_t peers = __match_any_sync(m, word);
+      const uint32_t v = __reduce_or_sync(peers, bit);
+      if (int(lane) == __ffs(peers) - 1) atomicOr(bits + word, v);
+    }
+    return;
   }
+#pragma unroll 1
+  for (int k = 0; k < 2 && m; ++k) {
+    const uint32_t w = __shfl_sync(kFullMask, word, __ffs(m) - 1);
+    const bool mine = need && word == w;
+    const uint32_t same = __ballot_sync(kFullMask, mine);
+    const uint32_t v = __reduce_or_sync(kFullMask, mine ? bit : 0u);
+    if (mine) {
+      if (int(lane) == __ffs(same) - 1) atomicOr(bits + w, v);
+      need = false;
+    }
+    m &= ~same;
+  }
+  if (need) atomicOr(bits + word, bit);
 }
 
-// Rank of bit d of slot s (the slots' records and bits).
-__device__ __forceinline__ uint32_t tr_rank(const uint4* rec, const uint32_t* bits, uint32_t s,
-                                            uint32_t d) {
+// Rank of bit d of a slot, from its record r and the word v that holds the bit.
+__device__ __forceinline__ uint32_t tr_rank(uint4 r, uint32_t v, uint32_t d) {
   const uint32_t w = d >> 5;
-  const uint32_t v = __ldcg(bits + s * kTrWords + w);
-  const uint4 r = __ldcg(rec + s);
   const uint32_t before = ((w & 4u ? r.z : r.y) >> (8u * (w & 3u))) & 255u;
   return r.x + before + __popc(v & ((1u << (d & 31u)) - 1u));
 }
@@ -272,38 +334,116 @@ __device__ __forceinline__ void tr_flush_extent(float mn[3], float mx[3], FrameS
   }
 }
 
+// Biased corner offsets of a point; sums of N words over the lanes of a run, at its last lane
+// (32 offsets of 21 bits fit 32 bits).
+__device__ __forceinline__ void tr_offsets(const TrFrames& fm, int f, const float q[3],
+                                           const uint32_t ijk[3], uint32_t w[3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    w[c] = uint32_t(quant_offset(q[c], voxel_corner(ijk[c], fm.org[3 * f + c], fm.leaf[f]),
+                                 fm.inv_unit[f]) -
+                    kQMin);
+}
+template <int N>
+__device__ __forceinline__ void tr_scan(uint32_t w[N], uint32_t head) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+  for (uint32_t d = 1; d < 32; d <<= 1) {
+    if (!__any_sync(kFullMask, lane >= head + d)) break;  // no run is longer
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      const uint32_t y = __shfl_up_sync(kFullMask, w[c], d);
+      if (lane >= head + d) w[c] += y;
+    }
+  }
+}
+
+// A level in use: its slots' bits and records.
+struct TrLevel {
+  uint32_t* bits;
+  uint4* rec;
+  uint32_t ns;  // slots
+};
+
+// The rows' sums (arrays of `cap` entries): A = x + y 2^32 and B = z + points 2^32 (mod 2^64),
+// C = the carries out of A's and B's low halves and out of A, 21 bits each (a cell of n < 2^30
+// points carries at most n / 2^11 times); the row's key; attribute sums of channels 0, 1 and
+// 2, 3 in 32 bits each.
+struct TrRows {
+  unsigned long long *A, *B, *C, *key, *att;
+  int64_t cap;
+  uint32_t rows;
+};
+
 template <bool kPosed>
 __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
+  extern __shared__ __align__(16) unsigned char tr_smem[];
   __shared__ TrSmem sm;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const uint32_t gt = blockIdx.x * kTrThreads + threadIdx.x, gthreads = gridDim.x * kTrThreads;
   const int F = a.fr.nframes;
+  const TrFrames fm = tr_frames(tr_smem, F, kPosed);
+  // this warp's runs (their number, the same in every lane) and masks
+  const uint32_t cq = a.chunks / gridDim.x, cr = a.chunks % gridDim.x;
+  const uint32_t steps = cq + (blockIdx.x < cr ? 1u : 0u);  // chunks of this block at most
+  const size_t w0 = size_t(blockIdx.x * cq + min(blockIdx.x, cr)) * (kTrThreads / 32) +
+                    size_t(warp) * steps;
+  uint4* run = a.run + w0 * 32;
+  uint32_t* pslot = a.pslot + w0 * 32;
+  uint32_t nruns = 0;
   int* err = a.err;
   uint32_t* bar = &a.st->fz_bar;
   uint32_t target = 0;
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
 
   // ---- extents; the first level's bits cleared ----
-  for (uint32_t i = gt; i < (1u << (a.root_bits - 7)); i += gthreads)
+  for (uint32_t i = gt; i < (1u << (kTrRootBits - 7)); i += gthreads)
     reinterpret_cast<uint4*>(a.root)[i] = zero4;
-  const uint32_t T = build_chunk_map(a.fr, sm.off, sm.cstart, sm.tmp, err);
-  uint32_t c0, c1;
-  block_range(T, &c0, &c1);
+  if (kPosed)
+    for (int f = threadIdx.x; f < F; f += kTrThreads) {
+      Pose P;
+      load_pose(a.fr, f, P);
+      for (int r = 0; r < 3; ++r)
+        fm.pose[4 * f + r] = make_float4(P.r[4 * r], P.r[4 * r + 1], P.r[4 * r + 2], P.r[4 * r + 3]);
+      fm.pose[4 * f + 3] = make_float4(P.zlo, P.zhi, 0.0f, 0.0f);
+    }
+  uint32_t T;
+  if (F > 1) {
+    T = build_chunk_map(a.fr, fm.off, fm.cstart, sm.tmp, err);
+  } else {
+    const bool bad =
+        a.fr.offsets && (__ldg(a.fr.offsets) != 0 || __ldg(a.fr.offsets + 1) != a.fr.n);
+    T = bad ? 0u : static_cast<uint32_t>(ceil_div(a.fr.n, kChunk));
+    if (threadIdx.x == 0) {
+      fm.off[0] = 0;
+      fm.off[1] = a.fr.n;
+      fm.cstart[0] = 0u;
+      fm.cstart[1] = T;
+      if (bad && blockIdx.x == 0) set_error(err, kErrInvalidArg);
+    }
+    __syncthreads();
+  }
   {
+    constexpr int U = kPosed ? 2 : 4;
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
     int cur = -1;
-    tr_points<kPosed>(a, sm, c0, c1, [&](int f, int64_t, bool, float x, float y, float z) {
-      if (f != cur) {
-        if (cur >= 0) tr_flush_extent(mn, mx, a.fs, cur, sm);
-        cur = f;
-      }
-      if (point_valid(x, y, z)) {
-        mn[0] = fminf(mn[0], x), mx[0] = fmaxf(mx[0], x);
-        mn[1] = fminf(mn[1], y), mx[1] = fmaxf(mx[1], y);
-        mn[2] = fminf(mn[2], z), mx[2] = fmaxf(mx[2], z);
+    tr_points<kPosed, U>(a, fm, T, [&](const TrPoints<U>& t) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (F > 1 && t.f[u] != cur) {
+          if (cur >= 0) tr_flush_extent(mn, mx, a.fs, cur, sm);
+          cur = t.f[u];
+        }
+        if (point_valid(t.q[u][0], t.q[u][1], t.q[u][2])) {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            mn[c] = fminf(mn[c], t.q[u][c]);
+            mx[c] = fmaxf(mx[c], t.q[u][c]);
+          }
+        }
       }
     });
-    if (cur >= 0) tr_flush_extent(mn, mx, a.fs, cur, sm);
+    tr_flush_extent(mn, mx, a.fs, cur < 0 ? 0 : cur, sm);
   }
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
 
@@ -326,11 +466,11 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
           const uint32_t u = __ldcg(&a.fs[f].ord_min_inv[c]);
           o[c] = u == 0u ? 0.0f : ordered_to_float(~u);
         }
-        sm.org[f][c] = o[c];
+        fm.org[3 * f + c] = o[c];
       }
-      sm.leaf[f] = leaf;
-      sm.rleaf[f] = fast_leaf(leaf) ? __fdiv_rn(1.0f, leaf) : 0.0f;
-      sm.inv_unit[f] = quant_inv_unit(leaf);
+      fm.leaf[f] = leaf;
+      fm.rleaf[f] = fast_leaf(leaf) ? __fdiv_rn(1.0f, leaf) : 0.0f;
+      fm.inv_unit[f] = quant_inv_unit(leaf);
       if (blockIdx.x == 0) {
         for (int c = 0; c < 3; ++c) {
           a.fs[f].origin[c] = o[c];
@@ -375,36 +515,73 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   }
   const bool wide = local_bits > 32u;
   // levels, and the key bits below level 1
-  const uint32_t root_bits = static_cast<uint32_t>(a.root_bits);
+  constexpr uint32_t root_bits = kTrRootBits;
   const int levels =
       kb <= root_bits ? 1 : 1 + int((kb - root_bits + kTrDigitBits - 1) / kTrDigitBits);
   const uint32_t below = uint32_t(levels - 1) * kTrDigitBits;
   const uint32_t top = max(kb - below, uint32_t(kTrDigitBits));
-  uint32_t ns = 1u << (top - kTrDigitBits);  // slots of the level
+  TrLevel lv{a.root, a.rootrec, 1u << (top - kTrDigitBits)};
   const int64_t cap = a.slots;
+  const bool with_attrs = a.out.attrs_in != nullptr;
 
-  // ---- level 1 marked ----
+  // ---- runs; level 1 marked ----
   bool range_bad = false;
-  tr_points<kPosed>(a, sm, c0, c1, [&](int f, int64_t, bool, float x, float y, float z) {
-    uint64_t key = 0;
-    uint32_t ijk[3];
-    const bool ok = tr_key(sm, f, x, y, z, wide, key_shift, &key, ijk, &range_bad);
-    const uint64_t pre = key >> below;
-    const uint32_t s = static_cast<uint32_t>(pre >> kTrDigitBits);
-    tr_mark<true>(a.root, s, uint32_t(pre) & 255u, ok && s < ns);
-  });
+  {
+    uint32_t s = 0;
+    tr_points<kPosed, 2>(a, fm, T, [&](const TrPoints<2>& t) {
+      uint32_t id[2], seen[2];
+      bool tail[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        uint64_t key = 0;
+        uint32_t ijk[3], head, w[3] = {0u, 0u, 0u};
+        const bool ok = tr_key(fm, t.f[u], t.q[u][0], t.q[u][1], t.q[u][2], wide, key_shift, &key,
+                               ijk, &range_bad);
+        const uint32_t last = tr_run(key, ok, &head);
+        tail[u] = ok && last == lane;
+        id[u] = static_cast<uint32_t>(key >> below);  // (at most 28 bits)
+        seen[u] =
+            tail[u] && (id[u] >> kTrDigitBits) < lv.ns ? __ldca(a.root + (id[u] >> 5)) : ~0u;
+        if (ok) tr_offsets(fm, t.f[u], t.q[u], ijk, w);
+        tr_scan<3>(w, head);
+        const uint32_t tm = __ballot_sync(kFullMask, tail[u]);
+        const uint32_t i = nruns + __popc(tm & ((1u << lane) - 1u));
+        if (tail[u]) {
+          run[i] = make_uint4(uint32_t(key), w[0], w[1], w[2] | ((lane - head + 1u) << 26));
+          if (wide || kb > 32u) a.runhi[w0 * 32 + i] = static_cast<uint32_t>(key >> 32);
+        }
+        if (with_attrs) {
+          uint32_t at[2] = {0u, 0u};
+          if (ok) {
+            const uint8_t* b = a.out.attrs_in + size_t(t.p[u]) * a.out.channels;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)  // two 16-bit sums a word (32 x 255 fit)
+              if (c < a.out.channels) at[c >> 1] |= uint32_t(__ldg(b + c)) << (16 * (c & 1));
+          }
+          tr_scan<2>(at, head);
+          if (tail[u]) a.runatt[w0 * 32 + i] = make_uint2(at[0], at[1]);
+        }
+        if (a.out.p2v) {
+          const uint32_t vm = __ballot_sync(kFullMask, ok);
+          if (lane == 0 && s < steps) a.mask[w0 + s] = make_uint2(tm, vm);
+        }
+        nruns += __popc(tm);
+        ++s;
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) tr_set(a.root, id[u], tail[u], seen[u]);
+    });
+  }
   if (__any_sync(kFullMask, range_bad) && lane == 0) set_error(err, kErrRange);
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
 
   // ---- every level ranked, the next one marked ----
-  uint32_t* bits = a.root;
-  uint4* rec = a.rootrec;
   uint32_t rows = 0;
   for (int j = 1;; ++j) {
     uint32_t* agg = a.stat + size_t(j - 1) * kTrMaxGrid;
-    tr_count(bits, ns, agg, sm.tmp);
+    tr_count(lv.bits, lv.ns, agg, sm.tmp);
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
-    const uint32_t set = tr_rank_slots(bits, rec, ns, agg, sm);
+    const uint32_t set = tr_rank_slots(lv.bits, lv.rec, lv.ns, agg, sm);
     const uint32_t n1 = static_cast<uint32_t>(min(int64_t(set), cap));
     if (set > n1 && blockIdx.x == 0 && threadIdx.x == 0) set_error(err, kErrInvalidArg);
     if (j == levels) {
@@ -414,50 +591,68 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     // the buffers alternate so that the last level lies in x
     char* nb = ((levels - j - 1) & 1) ? a.y : a.x;
     uint32_t* nbits = reinterpret_cast<uint32_t*>(nb);
-    uint4* nrec = reinterpret_cast<uint4*>(nb + size_t(cap) * 32);
     for (uint32_t i = gt; i < n1 * 2u; i += gthreads) reinterpret_cast<uint4*>(nbits)[i] = zero4;
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
     const uint32_t sh = below - uint32_t(j) * kTrDigitBits;  // key bits below the next level
-    tr_points<kPosed>(a, sm, c0, c1, [&](int f, int64_t p, bool, float x, float y, float z) {
-      uint64_t key = 0;
-      uint32_t ijk[3], head;
-      bool bad = false;
-      const bool ok = tr_key(sm, f, x, y, z, wide, key_shift, &key, ijk, &bad);
-      const bool tail = tr_run(key, ok, &head) == lane && ok;
-      uint32_t s = 0;
-      bool good = false;
-      if (tail) {
-        const uint64_t pre = key >> (sh + kTrDigitBits);
-        const uint32_t s0 = j == 1 ? static_cast<uint32_t>(pre >> kTrDigitBits) : a.pslot[p];
-        if (s0 < ns) {
-          s = tr_rank(rec, bits, s0, uint32_t(pre) & 255u);
-          good = s < n1;
+    for (uint32_t i0 = 0; i0 < nruns; i0 += 64) {
+      uint32_t id[2], seen[2], v[2];
+      uint4 r[2];
+      bool in[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t i = i0 + 32u * u + lane;
+        in[u] = i < nruns;
+        id[u] = 0u;
+        v[u] = 0u;
+        r[u] = make_uint4(~0u, 0u, 0u, 0u);
+        if (!in[u]) continue;
+        uint64_t key = run[i].x;
+        if (kb > 32u) key |= uint64_t(a.runhi[w0 * 32 + i]) << 32;
+        id[u] = static_cast<uint32_t>(key >> sh) & 0xffffu;  // this level's digit and the next
+        const uint32_t s0 =
+            j == 1 ? static_cast<uint32_t>(key >> (sh + 2 * kTrDigitBits)) : pslot[i];
+        if (s0 < lv.ns) {
+          v[u] = __ldcg(lv.bits + s0 * kTrWords + (id[u] >> 13));
+          r[u] = __ldcg(lv.rec + s0);
         }
-        a.pslot[p] = good ? s : ~0u;
-        if (!good) set_error(err, kErrInvalidArg);
       }
-      tr_mark<false>(nbits, s, uint32_t(key >> sh) & 255u, good);
-    });
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        seen[u] = 0u;
+        if (!in[u]) continue;
+        const uint32_t s = r[u].x == ~0u ? ~0u : tr_rank(r[u], v[u], id[u] >> kTrDigitBits);
+        pslot[i0 + 32u * u + lane] = s;
+        if (s >= n1) {
+          set_error(err, kErrInvalidArg);
+          in[u] = false;
+          continue;
+        }
+        id[u] = (s << kTrDigitBits) | (id[u] & 255u);
+        seen[u] = __ldcg(nbits + (id[u] >> 5));
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) tr_set(nbits, id[u], in[u], seen[u]);
+    }
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
-    bits = nbits;
-    rec = nrec;
-    ns = n1;
+    lv = TrLevel{nbits, reinterpret_cast<uint4*>(nb + size_t(cap) * 32), n1};
   }
 
   // ---- the rows' sums cleared ----
-  unsigned long long* accA = reinterpret_cast<unsigned long long*>(a.y);
-  unsigned long long* accB = accA + cap;
-  unsigned long long* accC = accB + cap;
-  unsigned long long* rowkey = accC + cap;
-  unsigned long long* att = rowkey + cap;  // two a row: channels 0, 1 and 2, 3 in 32 bits each
-  const bool with_attrs = a.out.attrs_in != nullptr;
+  TrRows R;
+  R.A = reinterpret_cast<unsigned long long*>(a.y);
+  R.B = R.A + cap;
+  R.C = R.B + cap;
+  R.key = R.C + cap;
+  R.att = R.key + cap;
+  R.cap = cap;
+  R.rows = rows;
   for (uint32_t i = gt; i < rows; i += gthreads) {
-    accA[i] = 0ull;
-    accB[i] = 0ull;
-    accC[i] = 0ull;
+    R.A[i] = 0ull;
+    R.B[i] = 0ull;
+    R.C[i] = 0ull;
     if (with_attrs) {
-      att[i] = 0ull;
-      att[i + cap] = 0ull;
+      R.att[i] = 0ull;
+      R.att[i + cap] = 0ull;
     }
   }
   if (blockIdx.x == 0) {
@@ -473,78 +668,78 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
 
   // ---- every run's points and sums at its row ----
-  tr_points<kPosed>(a, sm, c0, c1, [&](int f, int64_t p, bool in, float x, float y, float z) {
-    uint64_t key = 0;
-    uint32_t ijk[3], head;
-    bool bad = false;
-    const bool ok = tr_key(sm, f, x, y, z, wide, key_shift, &key, ijk, &bad);
-    const uint32_t last = tr_run(key, ok, &head);
-    const bool tail = ok && last == lane;
-    uint32_t row = ~0u;
-    if (tail) {
-      const uint32_t s0 = levels == 1 ? static_cast<uint32_t>(key >> kTrDigitBits) : a.pslot[p];
-      if (s0 < ns) row = tr_rank(rec, bits, s0, uint32_t(key) & 255u);
-      if (row >= rows) {
+  for (uint32_t i0 = 0; i0 < nruns; i0 += 32u * kTrAdd) {
+    uint4 e[kTrAdd], r[kTrAdd];
+    uint32_t v[kTrAdd], row[kTrAdd];
+    unsigned long long oa[kTrAdd], ob[kTrAdd], va[kTrAdd], vb[kTrAdd];
+#pragma unroll
+    for (int u = 0; u < kTrAdd; ++u) {
+      const uint32_t i = i0 + 32u * u + lane;
+      v[u] = 0u;
+      r[u] = make_uint4(~0u, 0u, 0u, 0u);
+      e[u] = zero4;
+      if (i >= nruns) continue;
+      e[u] = run[i];
+      const uint32_t s0 = levels == 1 ? e[u].x >> kTrDigitBits : pslot[i];
+      if (s0 < lv.ns) {
+        v[u] = __ldcg(lv.bits + s0 * kTrWords + ((e[u].x >> 5) & 7u));
+        r[u] = __ldcg(lv.rec + s0);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kTrAdd; ++u) {
+      const uint32_t i = i0 + 32u * u + lane;
+      row[u] = ~0u;
+      oa[u] = ob[u] = va[u] = vb[u] = 0ull;
+      if (i >= nruns) continue;
+      if (r[u].x != ~0u) row[u] = tr_rank(r[u], v[u], e[u].x & 255u);
+      if (row[u] >= rows) {
         set_error(err, kErrInvalidArg);
-        row = ~0u;
-      }
-    }
-    // biased offsets, summed over the run (32 offsets of 21 bits fit 32 bits)
-    uint32_t v[3] = {0u, 0u, 0u}, at[2] = {0u, 0u};
-    if (ok) {
-      const float q[3] = {x, y, z};
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        v[c] = uint32_t(quant_offset(q[c], voxel_corner(ijk[c], sm.org[f][c], sm.leaf[f]),
-                                     sm.inv_unit[f]) -
-                        kQMin);
-      if (with_attrs) {
-        const uint8_t* b = a.out.attrs_in + size_t(p) * a.out.channels;
-#pragma unroll
-        for (int c = 0; c < 4; ++c)  // two 16-bit sums a word (32 x 255 fit)
-          if (c < a.out.channels) at[c >> 1] |= uint32_t(__ldg(b + c)) << (16 * (c & 1));
-      }
-    }
-#pragma unroll
-    for (uint32_t d = 1; d < 32; d <<= 1) {
-      if (!__any_sync(kFullMask, lane >= head + d)) break;  // no run is longer
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const uint32_t u = __shfl_up_sync(kFullMask, v[c], d);
-        if (lane >= head + d) v[c] += u;
-      }
-      if (with_attrs) {
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const uint32_t u = __shfl_up_sync(kFullMask, at[c], d);
-          if (lane >= head + d) at[c] += u;
+        row[u] = ~0u;
+      } else {
+        uint64_t key = e[u].x;
+        if (kb > 32u) key |= uint64_t(a.runhi[w0 * 32 + i]) << 32;
+        R.key[row[u]] = key;  // (every run of the row stores the same key)
+        va[u] = e[u].y | ((unsigned long long)e[u].z << 32);
+        vb[u] = (e[u].w & 0x3ffffffu) | ((unsigned long long)(e[u].w >> 26) << 32);
+        oa[u] = atomicAdd(R.A + row[u], va[u]);
+        ob[u] = atomicAdd(R.B + row[u], vb[u]);
+        if (with_attrs) {
+          const uint2 t = a.runatt[w0 * 32 + i];
+          atomicAdd(R.att + row[u],
+                    (unsigned long long)(t.x & 0xffffu) | ((unsigned long long)(t.x >> 16) << 32));
+          if (a.out.channels > 2)
+            atomicAdd(R.att + cap + row[u], (unsigned long long)(t.y & 0xffffu) |
+                                                ((unsigned long long)(t.y >> 16) << 32));
         }
       }
+      if (a.out.p2v) pslot[i] = row[u];
     }
-    if (row != ~0u) {
-      rowkey[row] = key;  // (every run of the row stores the same key)
-      const unsigned long long va = v[0] | ((unsigned long long)v[1] << 32);
-      const unsigned long long vb = v[2] | ((unsigned long long)(lane - head + 1u) << 32);
-      const unsigned long long oa = atomicAdd(accA + row, va);
-      const unsigned long long ob = atomicAdd(accB + row, vb);
-      if (with_attrs) {
-        atomicAdd(att + row, (unsigned long long)(at[0] & 0xffffu) |
-                                 ((unsigned long long)(at[0] >> 16) << 32));
-        if (a.out.channels > 2)
-          atomicAdd(att + cap + row, (unsigned long long)(at[1] & 0xffffu) |
-                                         ((unsigned long long)(at[1] >> 16) << 32));
-      }
+#pragma unroll
+    for (int u = 0; u < kTrAdd; ++u) {
+      if (row[u] == ~0u) continue;
       // carries out of a 32-bit half: x into y, A out of 64 bits, z into the points
-      const unsigned long long cx = ((oa & 0xffffffffull) + (va & 0xffffffffull)) >> 32;
-      const unsigned long long cy = oa + va < oa ? 1ull : 0ull;
-      const unsigned long long cz = ((ob & 0xffffffffull) + (vb & 0xffffffffull)) >> 32;
-      if (cx | cy | cz) atomicAdd(accC + row, cx | (cy << 21) | (cz << 42));
+      const unsigned long long cx = ((oa[u] & 0xffffffffull) + (va[u] & 0xffffffffull)) >> 32;
+      const unsigned long long cy = oa[u] + va[u] < oa[u] ? 1ull : 0ull;
+      const unsigned long long cz = ((ob[u] & 0xffffffffull) + (vb[u] & 0xffffffffull)) >> 32;
+      if (cx | cy | cz) atomicAdd(R.C + row[u], cx | (cy << 21) | (cz << 42));
     }
-    if (a.out.p2v) {
-      const uint32_t r = __shfl_sync(kFullMask, row, last);
-      if (in) a.out.p2v[p] = ok && r != ~0u ? static_cast<int32_t>(r) : -1;
+  }
+  if (a.out.p2v) {  // a point's row is its run's
+    __syncwarp();
+    uint32_t first = 0;
+    for (uint32_t s = 0; s < steps; ++s) {
+      const uint64_t c = uint64_t(s) * gridDim.x + blockIdx.x;
+      if (c >= T) break;
+      const int f = F > 1 ? chunk_frame(fm.cstart, F, uint32_t(c)) : 0;
+      const int64_t p = fm.off[f] + (int64_t(c) - fm.cstart[f]) * kChunk + threadIdx.x;
+      const uint2 m = a.mask[w0 + s];
+      uint32_t q = ~0u;
+      if ((m.y >> lane) & 1u) q = pslot[first + __popc(m.x & ((1u << lane) - 1u))];
+      if (p < fm.off[f + 1]) a.out.p2v[p] = static_cast<int32_t>(q);
+      first += __popc(m.x);
     }
-  });
+  }
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
 
   // ---- rows (a thread a row), the first out.cap of them ----
@@ -556,22 +751,21 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   RowCtx rc;
   rc.fs = a.fs;
   rc.key_shift = key_shift;
-  rc.o1[0] = sm.org[0][0];
-  rc.o1[1] = sm.org[0][1];
-  rc.o1[2] = sm.org[0][2];
-  rc.leaf1 = sm.leaf[0];
+  rc.o1[0] = fm.org[0];
+  rc.o1[1] = fm.org[1];
+  rc.o1[2] = fm.org[2];
+  rc.leaf1 = fm.leaf[0];
   for (uint32_t row = gt; row < rows; row += gthreads) {
-    const unsigned long long key = __ldcg(rowkey + row);
+    const unsigned long long key = __ldcg(R.key + row);
     if (F > 1 && a.out.frame_offsets) {
       const uint32_t fk = key_frame(key, key_shift);
-      const uint32_t f0 = row > 0 ? key_frame(__ldcg(rowkey + row - 1), key_shift) + 1u : 0u;
+      const uint32_t f0 = row > 0 ? key_frame(__ldcg(R.key + row - 1), key_shift) + 1u : 0u;
       for (uint32_t f = f0; f <= fk; ++f) a.out.frame_offsets[f] = row;
       if (row + 1u == rows)
         for (uint32_t f = fk + 1u; f <= uint32_t(F); ++f) a.out.frame_offsets[f] = rows;
     }
     if (int64_t(row) >= a.out.cap) continue;
-    const unsigned long long A = __ldcg(accA + row), B = __ldcg(accB + row),
-                             C = __ldcg(accC + row);
+    const unsigned long long A = __ldcg(R.A + row), B = __ldcg(R.B + row), C = __ldcg(R.C + row);
     const unsigned long long cx = C & 0x1fffffull, cy = (C >> 21) & 0x1fffffull, cz = C >> 42;
     // x = low(A) + cx 2^32; y = high(A) + cy 2^32 - cx; z = low(B) + cz 2^32;
     // points = high(B) - cz
@@ -591,12 +785,12 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     else
       put_row(rc, a.out, row, key, r, err);
     if (with_attrs) {
-      const unsigned long long w[2] = {__ldcg(att + row), __ldcg(att + cap + row)};
+      const unsigned long long t[2] = {__ldcg(R.att + row), __ldcg(R.att + cap + row)};
 #pragma unroll
       for (int c = 0; c < 4; ++c)  // exact sums, one FP64 division each
         if (c < a.out.channels)
           a.out.attrs_out[size_t(row) * a.out.channels + c] = __double2float_rn(
-              __ddiv_rn(static_cast<double>(uint32_t(w[c >> 1] >> (32 * (c & 1)))),
+              __ddiv_rn(static_cast<double>(uint32_t(t[c >> 1] >> (32 * (c & 1)))),
                         static_cast<double>(r.n)));
     }
   }
@@ -609,6 +803,10 @@ __global__ __launch_bounds__(1024) void trie_clear_kernel(uint32_t* st, uint32_t
   if (threadIdx.x == 0) *err = 0;
 }
 
+// Dynamic shared memory of a block at most: the tables of kMaxFrames frames.
+constexpr size_t kTrSmem = tr_frames_bytes(kMaxFrames, true);
+static_assert(kTrSmem + sizeof(TrSmem) <= 227 * 1024, "block shared memory");
+
 // Blocks an SM holds of the kernel (0: it cannot run there), per device.
 int trie_blocks_per_sm(bool posed) {
   static int cache[64][2];
@@ -619,7 +817,10 @@ int trie_blocks_per_sm(bool posed) {
     const void* fn = posed ? reinterpret_cast<const void*>(trie_kernel<true>)
                            : reinterpret_cast<const void*>(trie_kernel<false>);
     int v = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, fn, kTrThreads, 0) != cudaSuccess) v = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kTrSmem)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, fn, kTrThreads, kTrSmem) != cudaSuccess)
+      v = 0;
     (void)cudaGetLastError();
     b = v > 0 ? v : -1;
   }
@@ -647,26 +848,29 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   a.rootrec = reinterpret_cast<uint4*>(ws + L.rootrec);
   a.x = ws + L.x;
   a.y = ws + L.y;
+  a.run = reinterpret_cast<uint4*>(ws + L.run);
+  a.runhi = reinterpret_cast<uint32_t*>(ws + L.runhi);
+  a.runatt = reinterpret_cast<uint2*>(ws + L.runatt);
   a.pslot = reinterpret_cast<uint32_t*>(ws + L.pslot);
+  a.mask = reinterpret_cast<uint2*>(ws + L.mask);
   a.stat = reinterpret_cast<uint32_t*>(ws + L.stat);
   a.out = out;
   a.slots = L.slots;
-  a.root_bits = trie_root_bits(fr.n);
   a.spin_limit = spin_limit;
   a.err = err;
   // one block a chunk of points, but enough of them to clear and rank the first level
-  const int64_t sms = num_sms() < kTrMaxGrid ? num_sms() : kTrMaxGrid;
   const int64_t chunks = max_chunks(fr.n, fr.nframes);
-  const int64_t half = sms > 1 ? sms / 2 : 1;
-  const int64_t g = chunks < half ? half : (chunks < sms ? chunks : sms);
+  const int64_t g = trie_grid(chunks, num_sms());
+  a.chunks = static_cast<uint32_t>(chunks);
   const size_t head = reinterpret_cast<char*>(fs + fr.nframes) - reinterpret_cast<char*>(st);
   trie_clear_kernel<<<1, 1024, 0, stream>>>(reinterpret_cast<uint32_t*>(st),
                                            static_cast<uint32_t>(head / sizeof(uint32_t)), err);
   void* args[] = {&a};
   const void* fn = posed(fr) ? reinterpret_cast<const void*>(trie_kernel<true>)
                              : reinterpret_cast<const void*>(trie_kernel<false>);
-  return cudaLaunchCooperativeKernel(fn, dim3(static_cast<unsigned>(g)), dim3(kTrThreads), args, 0,
-                                     stream);
+  return cudaLaunchCooperativeKernel(fn, dim3(static_cast<unsigned>(g)), dim3(kTrThreads), args,
+                                     
+                                     tr_frames_bytes(fr.nframes, posed(fr)), stream);
 }
 
 }  // namespace vg

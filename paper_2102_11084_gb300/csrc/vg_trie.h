@@ -8,40 +8,52 @@ constexpr int kTrThreads = 1024;    // threads of a block (one block an SM)
 constexpr int kTrDigitBits = 8;     // a slot of the trie: 2^8 children, one bit each
 constexpr int kTrWords = (1 << kTrDigitBits) / 32;
 constexpr int kTrMaxGrid = 1024;    // blocks of the launch at most
-// Bits of the first level (one bit per key prefix, cleared by every call): 2 MB up to
-// kTrSmallPoints points, where clearing and ranking more costs as much as another level's
-// three barriers; 32 MB above, where another level is another pass over the points.
+// Bits of the first level (one bit per key prefix, cleared by every call): 2 MB.
 constexpr int kTrRootBits = 24;
-constexpr int kTrRootBitsLarge = 28;
-constexpr int64_t kTrSmallPoints = int64_t(1) << 22;
+// Largest call: the trie's accesses miss L2 beyond, and a shuffled cloud of 2.5M points takes
+// 268 us at 0.02 m where the radix sort takes 247 (2.0M: 206 against 224).
+constexpr int64_t kTrMaxPoints = int64_t(1) << 21;
 
-constexpr int trie_root_bits(int64_t n) {
-  return n <= kTrSmallPoints ? kTrRootBits : kTrRootBitsLarge;
+// Blocks of the launch for so many chunks of points: one a chunk, but enough of them to clear
+// and rank the first level, and at most one an SM.
+constexpr int64_t trie_grid(int64_t chunks, int sms) {
+  const int64_t most = sms < kTrMaxGrid ? sms : kTrMaxGrid;
+  const int64_t least = most > 1 ? most / 2 : 1;
+  return chunks < least ? least : (chunks < most ? chunks : most);
 }
 
 // Scratch, from `base` on: the first level's bits and records, two buffers of slots (32 B of
 // bits and a 16 B record each; the second one holds the rows' sums, keys and attribute sums
-// once the rows are known), a word per point, the blocks' totals.
+// once the rows are known), the runs of every warp (each warp's list has a place for every
+// point it may read), the blocks' totals.
 struct TrieLayout {
-  size_t root, rootrec, x, y, pslot, stat, total;
+  size_t root, rootrec, x, y, run, runhi, runatt, pslot, mask, stat, total;
   int64_t slots;  // slots (and rows) the buffers hold
 };
-constexpr TrieLayout trie_layout(int64_t n, size_t base) {
+constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base) {
   TrieLayout L{};
   const int64_t nn = n < 1 ? 1 : n;
-  const int rb = trie_root_bits(nn);
   L.slots = nn;
   size_t off = align_up(base, 256);
   L.root = off;
-  off = align_up(off + (size_t(1) << (rb - 3)), 256);
+  off = align_up(off + (size_t(1) << (kTrRootBits - 3)), 256);
   L.rootrec = off;
-  off = align_up(off + (size_t(1) << (rb - kTrDigitBits)) * 16, 256);
+  off = align_up(off + (size_t(1) << (kTrRootBits - kTrDigitBits)) * 16, 256);
   L.x = off;
   off = align_up(off + size_t(L.slots) * 48, 256);
   L.y = off;
   off = align_up(off + size_t(L.slots) * 48, 256);
+  const size_t places = size_t(max_chunks(nn, frames)) * kChunk;
+  L.run = off;
+  off = align_up(off + places * 16, 256);
+  L.runhi = off;
+  off = align_up(off + places * 4, 256);
+  L.runatt = off;
+  off = align_up(off + places * 8, 256);
   L.pslot = off;
-  off = align_up(off + size_t(nn) * sizeof(uint32_t), 256);
+  off = align_up(off + places * 4, 256);
+  L.mask = off;
+  off = align_up(off + places / 32 * 8, 256);
   L.stat = off;
   off = align_up(off + 8 * size_t(kTrMaxGrid) * sizeof(uint32_t), 256);
   L.total = off;

@@ -1,4 +1,4 @@
-"""The occupancy trie (AUTO up to 2^22 points): keys, counts, order, frame offsets,
+"""The occupancy trie (AUTO up to 2^21 points): keys, counts, order, frame offsets,
 point_to_voxel and origins equal to the oracle's, and every output bit for bit that of the
 global radix sort ("sort_lsd"), over the forms the route accepts: key widths from one level
 to six, ragged sizes, runs across warps, cells of many points (carries of the packed sums),
@@ -63,7 +63,7 @@ def test_key_widths(bits):
     check(x, 0.015625, np.zeros(3, np.float32))
 
 
-@pytest.mark.parametrize("n", [(1 << 22) - 1, 1 << 22, (1 << 22) + 1])
+@pytest.mark.parametrize("n", [(1 << 21) - 1, 1 << 21, (1 << 21) + 1, (1 << 22) - 1, 1 << 22])
 def test_threshold_of_the_route(n):
     x = cuda(synth.fused_map(n, seed=3, extent=(20.0, 20.0, 5.0)))
     same(vg.downsample(x, 0.05), vg.downsample(x, 0.05, method="sort_lsd"))
