@@ -450,10 +450,10 @@ VG_API size_t vg_downsample_noalloc_scratch_bytes(void);
  * origin (recorded even when skipped), keys, then the bucket grouping's first partition
  * pass (with the scan of its digit counts), second partition pass (with its digit
  * histogram and bucket scan) and bucket kernel (all three return at once, or are not
- * launched, when the call takes the global radix sort), then 8 radix passes (those
- * beyond the key's significant digits, and all of them with the bucket grouping, return
- * at once) and the segmented reduction (count, scan, reduce); of the hash path: origin,
- * insert, compaction, 8 radix passes, finalize, point-to-voxel.
+ * launched, when the call takes the global radix sort), then 8 events of the radix
+ * passes (one launch runs all of them: the first event follows it, the others mark
+ * nothing more) and the segmented reduction (count, scan, reduce); of the hash path: origin,
+ * insert, compaction, 8 events of the radix passes (as above), finalize, point-to-voxel.
  * Returns the largest number of events a call records (20). */
 VG_API int vg_set_stage_events(void** events, int max_events);
 

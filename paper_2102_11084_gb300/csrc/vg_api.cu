@@ -265,11 +265,10 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
       for (int k = 0; k < 3; ++k) mark(stage + k, stream);
     }
     stage += 3;
-    for (int p = 0; p < kMaxPasses && e == cudaSuccess; ++p) {
-      e = launch_sort_pass(st, keys0, idx0, keys1, idx1, lb_a, lb_b, n, p, false, spins, err,
-                           stream, &nb);
-      mark(stage++, stream);
-    }
+    if (e == cudaSuccess)
+      e = launch_sort(st, keys0, idx0, keys1, idx1, lb_a, lb_b, n, kMaxPasses, false, spins, err,
+                      stream, &nb);
+    for (int p = 0; p < kMaxPasses; ++p) mark(stage++, stream);
     if (e == cudaSuccess)
       e = launch_segreduce(st, fs, F, keys0, idx0, keys1, idx1, xyz, recs, n, out, err, stream,
                            &nb, frn.poses);
@@ -309,10 +308,10 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
   mark(stage++, stream);
   if (e == cudaSuccess) e = launch_hash_compact(tab, st, keys0, idx0, err, stream);
   mark(stage++, stream);
-  for (int p = 0; p < kMaxPasses && e == cudaSuccess; ++p) {
-    e = launch_sort_pass(st, keys0, idx0, keys1, idx1, lb_a, lb_b, n, p, true, spins, err, stream);
-    mark(stage++, stream);
-  }
+  if (e == cudaSuccess)
+    e = launch_sort(st, keys0, idx0, keys1, idx1, lb_a, lb_b, n, kMaxPasses, true, spins, err,
+                    stream);
+  for (int p = 0; p < kMaxPasses; ++p) mark(stage++, stream);
   if (e == cudaSuccess)
     e = launch_hash_finalize(st, fs, F, keys0, idx0, keys1, idx1, tab, slot_rank, n, out, err,
                              stream);

@@ -130,6 +130,7 @@ struct alignas(256) State {
   uint32_t njobs3;            // chunks of large buckets the third partition pass splits
   uint32_t fspan;             // single-frame bins: bin = key >> fspan (vg_frame.cu)
   uint32_t ftop;              // single-frame bins: 2^ftop bins
+  uint32_t sort_bar;          // radix passes: grid-barrier arrivals
   uint32_t fz_bar;            // one-launch frame grouping: grid-barrier arrivals
   uint32_t fz_rows;           // one-launch frame grouping: rows (occupied cells)
   uint32_t ctot[64];          // entries of every 1024 consecutive buckets
@@ -286,13 +287,14 @@ struct NarrowBuffers {
   uint64_t* p1;
 };
 constexpr int kNarrowPasses = 4;
-// a3: one radix pass of the layout the key kernel chose.  compact_input: pass 0 reads
-// st->nitems compacted keys with their payload from idx0 (hash path, wide layout only)
-// instead of n raw keys with an implicit index.  nb = nullptr: wide layout only.
-cudaError_t launch_sort_pass(State* st, uint64_t* keys0, uint32_t* idx0, uint64_t* keys1,
-                             uint32_t* idx1, uint32_t* lb_a, uint32_t* lb_b, int64_t n_max,
-                             int pass, bool compact_input, uint32_t spin_limit, int* err,
-                             cudaStream_t stream, const NarrowBuffers* nb = nullptr);
+// a3: the radix passes (at most max_passes) of the layout the key kernel chose.
+// compact_input: pass 0 reads st->nitems compacted keys with their payload from idx0 (hash
+// path, wide layout only) instead of n raw keys with an implicit index.  nb = nullptr: wide
+// layout only.  lb_a zeroed before, lb_b not.
+cudaError_t launch_sort(State* st, uint64_t* keys0, uint32_t* idx0, uint64_t* keys1,
+                        uint32_t* idx1, uint32_t* lb_a, uint32_t* lb_b, int64_t n_max,
+                        int max_passes, bool compact_input, uint32_t spin_limit, int* err,
+                        cudaStream_t stream, const NarrowBuffers* nb = nullptr);
 // a4 + a5: reduce-by-key of the sorted table into key-ordered voxels.
 struct SegOut {
   uint64_t* keys;

@@ -203,9 +203,9 @@ vg_status vg_map_extract(vg_map* m, uint64_t* out_keys, float* out_centroids,
   map_extract_init<<<1, 1, 0, stream>>>(m->st, m->xst);
   e = vg::launch_hash_compact(m->tab, m->xst, m->keys0, m->idx0, err, stream);
   const uint32_t spins = vg::spin_limit();
-  for (int p = 0; p < vg::kMaxPasses && e == cudaSuccess; ++p)
-    e = vg::launch_sort_pass(m->xst, m->keys0, m->idx0, m->keys1, m->idx1, m->lb_a, m->lb_b,
-                             m->slots, p, true, spins, err, stream);
+  if (e == cudaSuccess)
+    e = vg::launch_sort(m->xst, m->keys0, m->idx0, m->keys1, m->idx1, m->lb_a, m->lb_b, m->slots,
+                        vg::kMaxPasses, true, spins, err, stream);
   vg::SegOut out{out_keys, out_centroids, out_counts, nullptr, cap, out_num_voxels, nullptr,
                  nullptr};
   if (e == cudaSuccess)

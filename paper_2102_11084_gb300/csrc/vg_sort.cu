@@ -12,6 +12,9 @@
 //   * pass 0 reads the raw per-point keys, drops invalid rows (sentinel keys) and
 //     generates the payload index itself, so compaction costs nothing extra;
 //   * every pass also histograms the next digit, so no separate upsweep pass exists;
+//   * all passes run in one cooperative launch with a grid barrier between them: eight
+//     launches, half of them empty for 32-bit keys, cost 2.3 us each (300,000
+//     points: 106 -> 85 us a call, 2.5M: 256 -> 239);
 //   * tile ids come from an atomic ticket (a waiting tile only waits on tiles that have
 //     already started), and every wait is bounded: after the limit the kernel records
 //     a timeout status and carries on, so a fault can never hang the GPU.
@@ -74,16 +77,15 @@ struct SortSmem {
 };
 
 // One radix pass.  KeyT/PayT: (uint64, uint32 point index) for the wide layout, or
-// (uint32, uint64 packed offsets) for the narrow one.  A pass beyond the needed ones
-// returns before taking a tile ticket.  Keys are loaded, ranked and written first; the
+// (uint32, uint64 packed offsets) for the narrow one.  (The buffers are written and read in
+// turn by the passes of one launch: loads go to L2.)  Keys are loaded, ranked and written first; the
 // payloads are loaded only once the keys sit in shared memory (their loads overlap the
 // key write-out), so the ranking holds no payload registers.
 template <typename KeyT, typename PayT, bool kNarrow>
 __device__ __forceinline__ void onesweep_body(
-    const KeyT* __restrict__ keys_in, const PayT* __restrict__ pay_in,
-    KeyT* __restrict__ keys_out, PayT* __restrict__ pay_out, State* st, uint32_t* lb_cur,
-    uint32_t* lb_next, int pass, int64_t n_host, int compact_input, uint32_t spin_limit,
-    int* err, SortSmem& sm) {
+    const KeyT* keys_in, const PayT* pay_in, KeyT* keys_out, PayT* pay_out, State* st,
+    uint32_t* lb_cur, uint32_t* lb_next, int pass, int64_t n_host, int compact_input,
+    uint32_t spin_limit, int* err, SortSmem& sm) {
   uint32_t (&warp_hist)[kSortThreads / 32][kRadix] = sm.warp_hist;
   uint32_t* digit_start = sm.digit_start;
   int32_t* gofs = sm.gofs;
@@ -94,8 +96,6 @@ __device__ __forceinline__ void onesweep_body(
   int& s_tile = sm.s_tile;
   uint32_t& s_tile_n = sm.s_tile_n;
 
-  const int passes = pass_count(st);
-  if (pass >= passes) return;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   // Pass 0 of the sort path reads all n raw entries and drops the invalid rows (sentinel
   // keys); every other pass, and pass 0 of compacted input, reads st->nitems entries.
@@ -138,7 +138,7 @@ __device__ __forceinline__ void onesweep_body(
   for (int j = 0; j < kSortItems; ++j) {
     const int64_t i = my_base + j * 32;
     const bool in = i < n_items;
-    key[j] = in ? __ldcs(keys_in + i) : KeyT(0);
+    key[j] = in ? __ldcg(keys_in + i) : KeyT(0);
     bool ok = in;
     // raw rows: the sentinel key (all ones, in either width) marks an invalid point; the
     // narrow layout is chosen only when no valid key can be all ones
@@ -222,7 +222,7 @@ __device__ __forceinline__ void onesweep_body(
     if (!kNarrow && raw)
       pay[j] = static_cast<PayT>(i);
     else
-      pay[j] = ((vmask >> j) & 1u) ? __ldcs(pay_in + i) : PayT(0);
+      pay[j] = ((vmask >> j) & 1u) ? __ldcg(pay_in + i) : PayT(0);
   }
   const uint32_t tile_n = s_tile_n;
   for (uint32_t i = t; i < tile_n; i += kSortThreads) {
@@ -265,20 +265,46 @@ __device__ __forceinline__ void onesweep_body(
     atomicAdd(&st->hist[pass + 1][t], next_hist[t]);
 }
 
-// One radix pass of whichever layout the key kernel chose (read on the device).
-__global__ __launch_bounds__(kSortThreads, kSortMinBlocks) void onesweep_kernel(
-    const uint64_t* kw_in, const uint32_t* iw_in, uint64_t* kw_out, uint32_t* iw_out,
-    const uint32_t* kn_in, const uint64_t* pn_in, uint32_t* kn_out, uint64_t* pn_out, State* st,
-    uint32_t* lb_cur, uint32_t* lb_next, int pass, int64_t n_host, int compact_input,
-    uint32_t spin_limit, int* err) {
+struct SortArgs {
+  uint64_t *kw0, *kw1;  // wide layout: keys and point indices, even passes read the first
+  uint32_t *iw0, *iw1;
+  uint32_t *kn0, *kn1;  // narrow layout: keys and packed offsets
+  uint64_t *pn0, *pn1;
+  uint32_t *lb0, *lb1;  // status rows, even passes use the first and clear the other
+  State* st;
+  int64_t n_host;
+  int compact_input;
+  uint32_t spin_limit;
+  int* err;
+};
+
+// Radix passes [first, last) of whichever layout the key kernel chose (read on the device),
+// those beyond the key's significant digits left out.  With more than one pass a cooperative
+// launch: a grid barrier separates them.
+__global__ __launch_bounds__(kSortThreads, kSortMinBlocks) void onesweep_kernel(const SortArgs a,
+                                                                                int first,
+                                                                                int last) {
   __shared__ SortSmem sm;
-  if (block_error_raised(err)) return;  // an earlier step failed
-  if (st->narrow)
-    onesweep_body<uint32_t, uint64_t, true>(kn_in, pn_in, kn_out, pn_out, st, lb_cur, lb_next, pass,
-                                            n_host, compact_input, spin_limit, err, sm);
-  else
-    onesweep_body<uint64_t, uint32_t, false>(kw_in, iw_in, kw_out, iw_out, st, lb_cur, lb_next,
-                                             pass, n_host, compact_input, spin_limit, err, sm);
+  if (block_error_raised(a.err)) return;  // an earlier step failed
+  const bool narrow = a.st->narrow != 0;
+  const int passes = min(last, pass_count(a.st));
+  uint32_t target = 0;
+  for (int p = first; p < passes; ++p) {
+    const bool odd = (p & 1) != 0;
+    uint32_t* lb = odd ? a.lb1 : a.lb0;
+    uint32_t* lb_next = odd ? a.lb0 : a.lb1;
+    if (narrow)
+      onesweep_body<uint32_t, uint64_t, true>(odd ? a.kn1 : a.kn0, odd ? a.pn1 : a.pn0,
+                                              odd ? a.kn0 : a.kn1, odd ? a.pn0 : a.pn1, a.st, lb,
+                                              lb_next, p, a.n_host, a.compact_input, a.spin_limit,
+                                              a.err, sm);
+    else
+      onesweep_body<uint64_t, uint32_t, false>(odd ? a.kw1 : a.kw0, odd ? a.iw1 : a.iw0,
+                                               odd ? a.kw0 : a.kw1, odd ? a.iw0 : a.iw1, a.st, lb,
+                                               lb_next, p, a.n_host, a.compact_input, a.spin_limit,
+                                               a.err, sm);
+    if (p + 1 < passes && !grid_barrier(&a.st->sort_bar, target, a.spin_limit, a.err)) return;
+  }
 }
 
 // Test kernel: one chained-scan wait of tile `tile` on status words nobody publishes; it
@@ -295,24 +321,24 @@ cudaError_t launch_debug_wait(const uint32_t* status, int tile, uint32_t limit, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_sort_pass(State* st, uint64_t* keys0, uint32_t* idx0, uint64_t* keys1,
-                             uint32_t* idx1, uint32_t* lb_a, uint32_t* lb_b, int64_t n_max,
-                             int pass, bool compact_input, uint32_t spin_limit, int* err,
-                             cudaStream_t stream, const NarrowBuffers* nb) {
+cudaError_t launch_sort(State* st, uint64_t* keys0, uint32_t* idx0, uint64_t* keys1,
+                        uint32_t* idx1, uint32_t* lb_a, uint32_t* lb_b, int64_t n_max,
+                        int max_passes, bool compact_input, uint32_t spin_limit, int* err,
+                        cudaStream_t stream, const NarrowBuffers* nb) {
   if (n_max == 0) return cudaSuccess;
   const int tiles = persistent_grid(reinterpret_cast<const void*>(onesweep_kernel), kSortThreads,
                                     0, ceil_div(n_max, kSortTile));
-  const bool even = (pass & 1) == 0;
-  // pass p reads buffer (p odd ? 1 : 0) and writes the other; pass 0 reads raw keys.
-  const bool raw = pass == 0 && !compact_input;
-  const uint32_t* kn_in = nb ? (even ? nb->k0 : nb->k1) : nullptr;
-  const uint64_t* pn_in = nb ? (even ? nb->p0 : nb->p1) : nullptr;
-  uint32_t* kn_out = nb ? (even ? nb->k1 : nb->k0) : nullptr;
-  uint64_t* pn_out = nb ? (even ? nb->p1 : nb->p0) : nullptr;
-  onesweep_kernel<<<tiles, kSortThreads, 0, stream>>>(
-      even ? keys0 : keys1, raw ? nullptr : (even ? idx0 : idx1), even ? keys1 : keys0,
-      even ? idx1 : idx0, kn_in, pn_in, kn_out, pn_out, st, even ? lb_a : lb_b,
-      even ? lb_b : lb_a, pass, n_max, compact_input ? 1 : 0, spin_limit, err);
+  SortArgs a{keys0, keys1, idx0, idx1, nb ? nb->k0 : nullptr, nb ? nb->k1 : nullptr,
+             nb ? nb->p0 : nullptr, nb ? nb->p1 : nullptr, lb_a, lb_b, st, n_max,
+             compact_input ? 1 : 0, spin_limit, err};
+  int first = 0, last = max_passes;
+  void* args[] = {&a, &first, &last};
+  cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(onesweep_kernel),
+                                              dim3(tiles), dim3(kSortThreads), args, 0, stream);
+  if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+  (void)cudaGetLastError();  // (SMs withheld from this process: a launch a pass)
+  for (int p = 0; p < max_passes; ++p)
+    onesweep_kernel<<<tiles, kSortThreads, 0, stream>>>(a, p, p + 1);
   return cudaGetLastError();
 }
 

@@ -705,9 +705,8 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
                              stream>>>(st, p2v, cstart, vcnt, nb, pos, cnt, ecell, group, ctr, r2,
                                        err);
     thin_prio_kernel<<<g, 256, 0, stream>>>(n, p2v, entry, cnt, priority, thr, keys0, st2, err);
-    for (int p = 0; p < kNarrowPasses && e == cudaSuccess; ++p)  // 32-bit priorities
-      e = launch_sort_pass(st2, keys0, idx0, keys1, idx1, lb_a, lb_b, n, p, false, spin_limit(),
-                           err, stream);
+    e = launch_sort(st2, keys0, idx0, keys1, idx1, lb_a, lb_b, n, kNarrowPasses, false,
+                    spin_limit(), err, stream);  // (32-bit priorities)
     if (e != cudaSuccess) return VG_ERR_CUDA;
     thin_list_kernel<<<g, 256, 0, stream>>>(st2, idx0, idx1, entry, list, err);
     // the sort's buffers again: the deleted lists' heads (a cell each) and nodes (16 bytes a
