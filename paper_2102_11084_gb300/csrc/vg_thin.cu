@@ -500,7 +500,19 @@ __global__ __launch_bounds__(256) void thin_count_kernel(
       const uint32_t c = nb[size_t(row) * kNb + o];
       if (c == kNoCell) continue;
       const int64_t j0 = cstart[c], j1 = j0 + vcnt[c];
-      for (int64_t j = j0; j < j1 && cnt <= threshold; ++j) {
+      int64_t j = j0;
+      for (; j + 4 <= j1 && cnt <= threshold; j += 4) {  // four at a time: their loads overlap
+        float4 q[4];
+        bool alive[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          alive[u] = (state[j + u] & kAlive) != 0 && j + u != i;
+          q[u] = pos[j + u];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cnt += alive[u] && dist2(q[u], me.x, me.y, me.z) <= r2;
+      }
+      for (; j < j1 && cnt <= threshold; ++j) {
         if (j == i || !(state[j] & kAlive)) continue;
         if (dist2(pos[j], me.x, me.y, me.z) <= r2) ++cnt;
       }
@@ -592,13 +604,17 @@ int thin_loop_grid() {
   return v > 0 ? num_sms() : 0;
 }
 
-// Whether the loop keeps counts: a pass that deletes `batch` points meets batch * pairs / n
-// candidates; a fresh count of every point tests about three candidates per neighbour it
-// finds, up to threshold + 1 of them, and goes through the host.
+// Whether the loop keeps counts, by estimated microseconds.  Kept: every candidate pair is
+// tested about twice in all (the count, then the deletions; 1.5e12 tests a second) and a pass
+// takes 10 us.  Recounted: a pass takes 100 us of host round trips and about 100 ps a point and
+// neighbour it looks for (640x480 frame, threshold 20: 570 us).  Passes: where the candidates
+// of a point are many times the threshold, most points are deleted.
 bool keep_counts(int64_t n, unsigned long long pairs, int64_t batch, int64_t threshold) {
   if (n <= 0) return false;
-  const double per_pass = double(batch < n ? batch : n) * (double(pairs) / double(n));
-  return per_pass <= 3.0 * double(n) * (double(threshold) + 1.0);
+  const double nn = double(n), pp = double(pairs), want = double(threshold) + 1.0;
+  const double gone = pp > 0.0 ? 1.0 - 3.0 * want * nn / pp : 0.0;
+  const double passes = gone > 0.0 && gone * nn > double(batch) ? gone * nn / double(batch) : 1.0;
+  return 2.0 * pp / 1.5e6 + 10.0 * passes <= passes * (100.0 + nn * want * 1e-4);
 }
 
 int grid_for(int64_t n) {

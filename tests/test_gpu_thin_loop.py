@@ -2,7 +2,7 @@
 afresh every pass) against the oracle: keep flags, number kept and passes are whole numbers
 and must be equal.  The sizes lie at the edges of the batch search (2048 list entries a step,
 one list entry more or less than a batch) and on both sides of the rule that picks the form
-(batch * candidates against 3 * points * (threshold + 1))."""
+(all candidate pairs against the passes a fresh count would take)."""
 import numpy as np
 import pytest
 import torch
@@ -38,6 +38,13 @@ def test_dense_clouds_both_sides_of_the_rule(n, t, batch):
     rng = np.random.Generator(np.random.PCG64(n + t))
     x = (1.0 + rng.uniform(0, 0.11, (n, 3))).astype(np.float32)
     check(x, 0.05, t, rng.permutation(n).astype(np.uint32), batch, radius=0.04)
+
+
+def test_recounted_form():
+    # 24,000 points of a few cells, two passes: a fresh count stops at the third neighbour
+    rng = np.random.Generator(np.random.PCG64(11))
+    x = (1.0 + rng.uniform(0, 0.04, (24_000, 3))).astype(np.float32)
+    check(x, 0.05, 2, rng.permutation(24_000).astype(np.uint32), 23_000)
 
 
 def test_equal_and_large_priorities():
