@@ -115,11 +115,17 @@ int method_of(int flags) {
   return m == VG_METHOD_HASH ? VG_METHOD_HASH : VG_METHOD_SORT;
 }
 
-// Whether the flags and the size let a call take the occupancy trie (vg_trie.cu).  AUTO
-// only: the other methods name a grouping.
+// Whether the flags let a call take the occupancy trie (vg_trie.cu).  AUTO only: the other
+// methods name a grouping.
 bool trie_call(int64_t n, int flags) {
   return (flags & VG_METHOD_MASK) == VG_METHOD_AUTO &&
-         (flags & (VG_SORT_LSD | VG_SORT_FRAME)) == 0 && n > 0 && n <= kTrMaxPoints;
+         (flags & (VG_SORT_LSD | VG_SORT_FRAME)) == 0 && n > 0;
+}
+
+// The trie's scratch: in the place of the sort path's, or, where the sort path may follow,
+// after what that clears before the trie runs.
+TrieLayout trie_scratch(int64_t n, int frames, const SortLayout& L) {
+  return trie_layout(n, frames, n <= kTrMaxPoints ? L.lb_a : L.lb_b);
 }
 
 }  // namespace
@@ -129,7 +135,7 @@ size_t frames_workspace_bytes(int64_t n, int frames, int flags) {
   if (method_of(flags) == VG_METHOD_HASH) return hash_layout(n, frames).total;
   const SortLayout L = sort_layout(n, frames);
   if (trie_call(n, flags)) {
-    const size_t t = trie_layout(n, frames, L.lb_a).total;
+    const size_t t = trie_scratch(n, frames, L).total;
     return t > L.total ? t : L.total;
   }
   if ((flags & VG_SORT_FRAME) == 0) return L.total;
@@ -181,8 +187,13 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
     const bool frame_path = (flags & VG_SORT_FRAME) != 0 && F == 1 && frn.allow_narrow && n > 0;
     // a frame that one cooperative launch holds: that launch alone (it finds the extents)
     const bool fused = frame_path && frame_fused_fits(n, posed(frn));
-    const bool have_extent = from_min || F > 1 || frn.allow_narrow;
     const SortLayout L = sort_layout(n, F);
+    // The trie: every call of up to kTrMaxPoints points; above, those whose sample shows few
+    // cells (decided on the device).  Its 32-bit channel sums bound the points with attributes.
+    const TrieLayout TL = trie_scratch(n, F, L);
+    const bool trie = trie_ok && trie_available(posed(frn)) && workspace_bytes >= TL.total &&
+                      !(out.attrs_in && n > (int64_t(1) << 24));
+    const bool have_extent = from_min || F > 1 || frn.allow_narrow || trie;
     State* st = reinterpret_cast<State*>(ws + L.state);
     FrameState* fs = reinterpret_cast<FrameState*>(ws + L.frames);
     uint64_t* keys0 = reinterpret_cast<uint64_t*>(ws + L.keys0);
@@ -199,18 +210,16 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
     uint64_t* pay_1 = reinterpret_cast<uint64_t*>(ws + L.idx0);
     int* err = out_error ? reinterpret_cast<int*>(out_error) : &st->error;
 
-    if (trie_ok && trie_available(posed(frn))) {
-      const TrieLayout TL = trie_layout(n, F, L.lb_a);
-      if (workspace_bytes >= TL.total) {
-        mark(stage, stream);
-        const cudaError_t et = launch_trie(xyz, frn, st, fs, ws, TL, out, spins, err, stream);
-        if (et != cudaErrorCooperativeLaunchTooLarge) {
-          for (int k = 1; k < 1 + 1 + 1 + 3 + kMaxPasses + 1; ++k) mark(stage + k, stream);
-          return cuda_status(et);
-        }
-        (void)cudaGetLastError();  // (SMs withheld from this process: the sort path)
+    if (trie && n <= kTrMaxPoints) {
+      mark(stage, stream);
+      const cudaError_t et = launch_trie(xyz, frn, st, fs, ws, TL, out, spins, err, stream);
+      if (et != cudaErrorCooperativeLaunchTooLarge) {
+        for (int k = 1; k < 1 + 1 + 1 + 3 + kMaxPasses + 1; ++k) mark(stage + k, stream);
+        return cuda_status(et);
       }
+      (void)cudaGetLastError();  // (SMs withheld from this process: the sort path)
     }
+    const bool try_trie = trie && n > kTrMaxPoints;
 
     // (the frame path needs only the state and frame state cleared: its last kernel
     // writes the voxel count and the frame offsets)
@@ -240,10 +249,17 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
         const FrameLayout FL = frame_layout(n, L.total);
         e = launch_origin(xyz, frn, st, fs, err, stream, ws + FL.zero, FL.zero_bytes);
       } else {
-        e = launch_origin(xyz, frn, st, fs, err, stream);
+        e = launch_origin(xyz, frn, st, fs, err, stream, nullptr, 0, try_trie);
       }
     }
     mark(stage++, stream);
+    if (e == cudaSuccess && try_trie) {
+      e = launch_trie(xyz, frn, st, fs, ws, TL, out, spins, err, stream);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {  // (SMs withheld from this process)
+        (void)cudaGetLastError();
+        e = cudaSuccess;
+      }
+    }
     if (e == cudaSuccess && !frame_path)
       e = launch_keys_any(xyz, frn, have_extent, st, fs, keys0, k32_0, pay_0, err, stream);
     if (!frame_path) mark(stage++, stream);

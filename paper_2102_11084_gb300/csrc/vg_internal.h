@@ -108,6 +108,10 @@ struct FrameState {
   uint32_t pad[2];
 };
 
+// st->msd (with st->narrow = 1, which every later kernel reads anyway) once the occupancy trie
+// has written the rows: nothing is left to do for the sort path's kernels.
+constexpr uint32_t kRowsWritten = 2;
+
 // Per-call device state, at the start of the workspace.  Zeroed by the call.
 struct alignas(256) State {
   unsigned long long maxkey;  // largest sort key
@@ -118,7 +122,7 @@ struct alignas(256) State {
   uint32_t nchunks;           // chunks of the frame decomposition
   uint32_t narrow;            // 1: 32-bit sort keys + packed-offset payload (no gather)
   int32_t error;              // internal error word when the caller passes none
-  uint32_t msd;               // 1: narrow layout grouped by buckets (vg_msd.cu)
+  uint32_t msd;               // 1: narrow layout grouped by buckets (vg_msd.cu); kRowsWritten
   uint32_t lowbits;           // bucket = key >> lowbits; the low bits are reduced on chip
   uint32_t levels;            // partition passes over the bucket bits (1 or 2)
   uint32_t b1, b2;            // digit widths of the two passes (b2 = 0 with one pass)
@@ -133,6 +137,8 @@ struct alignas(256) State {
   uint32_t sort_bar;          // radix passes: grid-barrier arrivals
   uint32_t fz_bar;            // one-launch frame grouping: grid-barrier arrivals
   uint32_t fz_rows;           // one-launch frame grouping: rows (occupied cells)
+  unsigned long long smp;     // sampled pairs of consecutive points: valid ones, and (upper
+                              // 32 bits) those of one cell
   uint32_t ctot[64];          // entries of every 1024 consecutive buckets
   uint32_t nztot[64];         // non-empty buckets of every 1024 consecutive buckets
   uint32_t vtot[64];          // cells of every 1024 consecutive non-empty buckets
@@ -273,9 +279,10 @@ void warm_reduce_config();
 // Launchers (all asynchronous on `stream`).
 // a1: per-frame min (and max) of the valid points into FrameState.
 // `zero`/`zero_bytes` (16-byte multiple, or 0): a region the kernel also clears.
+// `sample`: also count, in some chunks, the pairs of consecutive points and those of one cell.
 cudaError_t launch_origin(const float* xyz, const FramesArg& fr, State* st, FrameState* fs,
                           int* err, cudaStream_t stream, void* zero = nullptr,
-                          size_t zero_bytes = 0);
+                          size_t zero_bytes = 0, bool sample = false);
 // a2: per-point sort keys (frame id above a key_shift-bit Morton field; ~0 = invalid).
 cudaError_t launch_keys(const float* xyz, const FramesArg& fr, bool have_extent, State* st,
                         FrameState* fs, uint64_t* keys, int* err, cudaStream_t stream);

@@ -54,12 +54,32 @@ __device__ __forceinline__ void flush_extent(float mn[3], float mx[3], FrameStat
   }
 }
 
-// a1: per-frame minimum and maximum over the valid points.
+// Pairs of consecutive points among a warp's 128 (4 a thread in v, NaN rows invalid) and those
+// of one cell, added to st->smp (lattice through 0: the origin is not known yet).
+__device__ __forceinline__ void sample_pairs(const float v[12], float leaf, State* st) {
+  const float r = __fdiv_rn(1.0f, leaf);
+  uint32_t pairs = 0, same = 0;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const float* a = v + 3 * j;
+    if (!point_valid(a[0], a[1], a[2]) || !point_valid(a[3], a[4], a[5])) continue;
+    ++pairs;
+    same += floorf(a[0] * r) == floorf(a[3] * r) && floorf(a[1] * r) == floorf(a[4] * r) &&
+            floorf(a[2] * r) == floorf(a[5] * r);
+  }
+  pairs = __reduce_add_sync(kFullMask, pairs);
+  same = __reduce_add_sync(kFullMask, same);
+  if ((threadIdx.x & 31) == 0 && pairs)
+    atomicAdd(&st->smp, (unsigned long long)pairs | ((unsigned long long)same << 32));
+}
+
+// a1: per-frame minimum and maximum over the valid points.  With st, the first 128 points of
+// every eighth block are sampled (one atomic a sampled block).
 template <bool kPosed>
-__global__ __launch_bounds__(kStreamThreads) void origin_kernel(const float* __restrict__ xyz,
+__global__ __launch_bounds__(kStreamThreads, kPosed ? 1 : 8) void origin_kernel(const float* __restrict__ xyz,
                                                                 FramesArg fr, FrameState* fs,
                                                                 int* err, uint4* zero,
-                                                                size_t zero16) {
+                                                                size_t zero16, State* st) {
   // only the frame/chunk map (no per-frame origin or leaf is needed here)
   __shared__ struct {
     int64_t off[kMaxFrames + 1];
@@ -74,6 +94,22 @@ __global__ __launch_bounds__(kStreamThreads) void origin_kernel(const float* __r
   uint32_t c0, c1;
   block_range(T, &c0, &c1);
   const bool xyz_vec = (reinterpret_cast<uintptr_t>(xyz) & 15) == 0;
+  // (loaded apart from the loop's points: kept among them it cost the loop registers, and two
+  // of its eight blocks an SM)
+  if (st && (blockIdx.x & 7u) == 0u && threadIdx.x < 32 && c0 < c1) {
+    const int f = chunk_frame(sm.cstart, fr.nframes, c0);
+    const int64_t start = sm.off[f] + int64_t(c0 - sm.cstart[f]) * kChunk;
+    float v[12];
+    load4(xyz, start + int64_t(threadIdx.x) * kStreamPoints, min(start + kChunk, sm.off[f + 1]),
+          xyz_vec && (start & 3) == 0, v);
+    if (kPosed) {
+      Pose P;
+      load_pose(fr, f, P);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) pose_point(P, v[3 * j], v[3 * j + 1], v[3 * j + 2]);
+    }
+    sample_pairs(v, fr.leaves ? __ldg(fr.leaves + f) : fr.leaf, st);
+  }
   float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
   int cur = -1;
   Pose P;
@@ -231,6 +267,7 @@ __global__ __launch_bounds__(kStreamThreads, kPosed ? 1 : VG_KEY_MINB) void key_
   __shared__ unsigned long long wmax[kStreamThreads / 32];
   __shared__ uint32_t wcount[kStreamThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (st->msd == kRowsWritten) return;  // (the same in every block)
   for (int d = threadIdx.x; d < kRadix; d += kStreamThreads) hist[d] = 0;
   const uint32_t T = build_chunk_map(fr, sm.off, sm.cstart, sm.tmp, err);
   bool narrow = false;
@@ -287,17 +324,20 @@ int stream_grid(const FramesArg& fr) {
 }
 
 cudaError_t launch_origin(const float* xyz, const FramesArg& fr, State* st, FrameState* fs,
-                          int* err, cudaStream_t stream, void* zero, size_t zero_bytes) {
-  (void)st;
+                          int* err, cudaStream_t stream, void* zero, size_t zero_bytes,
+                          bool sample) {
+  State* smp = sample ? st : nullptr;
   if (fr.n == 0) {
     return zero_bytes ? cudaMemsetAsync(zero, 0, zero_bytes, stream) : cudaSuccess;
   }
   uint4* z = static_cast<uint4*>(zero);
   const size_t z16 = zero ? zero_bytes / 16 : 0;
   if (posed(fr))
-    origin_kernel<true><<<stream_grid(fr), kStreamThreads, 0, stream>>>(xyz, fr, fs, err, z, z16);
+    origin_kernel<true><<<stream_grid(fr), kStreamThreads, 0, stream>>>(xyz, fr, fs, err, z, z16,
+                                                                          smp);
   else
-    origin_kernel<false><<<stream_grid(fr), kStreamThreads, 0, stream>>>(xyz, fr, fs, err, z, z16);
+    origin_kernel<false><<<stream_grid(fr), kStreamThreads, 0, stream>>>(xyz, fr, fs, err, z, z16,
+                                                                          smp);
   return cudaGetLastError();
 }
 

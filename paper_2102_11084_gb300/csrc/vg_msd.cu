@@ -38,7 +38,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-__device__ __forceinline__ bool msd_on(const State* st) { return st->narrow && st->msd; }
+__device__ __forceinline__ bool msd_on(const State* st) { return st->narrow && st->msd == 1u; }
 
 // ---- scan of the first digit ----------------------------------------------------------
 

@@ -87,11 +87,12 @@ vg_status vg_plan_create(vg_plan** out, int max_frames, int64_t max_points, int 
   // room for every grouping a later configure may pick
   const size_t a = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_SORT | VG_SORT_FRAME);
   const size_t b = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_HASH);
-  const size_t c = vg::frames_workspace_bytes(
-      max_points < vg::kTrMaxPoints ? max_points : vg::kTrMaxPoints, max_frames,
-      VG_METHOD_AUTO);
-  p->ws_bytes = a > b ? a : b;
-  if (c > p->ws_bytes) p->ws_bytes = c;
+  const size_t small = vg::frames_workspace_bytes(
+      max_points < vg::kTrMaxPoints ? max_points : vg::kTrMaxPoints, max_frames, VG_METHOD_AUTO);
+  const size_t large = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_AUTO);
+  p->ws_bytes = 0;
+  for (const size_t w : {a, b, small, large})
+    if (w > p->ws_bytes) p->ws_bytes = w;
   if (cudaMalloc(&p->ws, p->ws_bytes) != cudaSuccess) {
     delete p;
     return VG_ERR_CUDA;

@@ -67,6 +67,8 @@ struct TrArgs {
   SegOut out;
   int64_t slots;       // slots and rows the buffers hold
   uint32_t chunks;     // chunks of points at most
+  int root_bits;
+  int large;           // after the extent kernel; the call may be left to the sort path
   uint32_t spin_limit;
   int* err;
 };
@@ -396,9 +398,14 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   uint32_t target = 0;
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
 
+  if (a.large) {  // (the same in every block)
+    const unsigned long long smp = a.st->smp;
+    if (kTrSameOf * uint32_t(smp >> 32) < kTrSame * uint32_t(smp)) return;
+  }
   // ---- extents; the first level's bits cleared ----
-  for (uint32_t i = gt; i < (1u << (kTrRootBits - 7)); i += gthreads)
-    reinterpret_cast<uint4*>(a.root)[i] = zero4;
+  if (!a.large)
+    for (uint32_t i = gt; i < (1u << (kTrRootBits - 7)); i += gthreads)
+      reinterpret_cast<uint4*>(a.root)[i] = zero4;
   if (kPosed)
     for (int f = threadIdx.x; f < F; f += kTrThreads) {
       Pose P;
@@ -423,7 +430,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     }
     __syncthreads();
   }
-  {
+  if (!a.large) {
     constexpr int U = kPosed ? 2 : 4;
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
     int cur = -1;
@@ -444,8 +451,8 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
       }
     });
     tr_flush_extent(mn, mx, a.fs, cur < 0 ? 0 : cur, sm);
+    if (!grid_barrier(bar, target, a.spin_limit, err)) return;
   }
-  if (!grid_barrier(bar, target, a.spin_limit, err)) return;
 
   // ---- every frame's origin and leaf, the width of the keys (the same in every block) ----
   uint32_t key_shift = 64, kb, local_bits;
@@ -506,7 +513,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     }
   }
   if (!go) {  // (the same in every block)
-    if (blockIdx.x == 0) {
+    if (blockIdx.x == 0 && !a.large) {
       if (a.out.frame_offsets)
         for (int f = threadIdx.x; f <= F; f += kTrThreads) a.out.frame_offsets[f] = 0;
       if (threadIdx.x == 0) *a.out.num_voxels = 0;
@@ -515,7 +522,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   }
   const bool wide = local_bits > 32u;
   // levels, and the key bits below level 1
-  constexpr uint32_t root_bits = kTrRootBits;
+  const uint32_t root_bits = static_cast<uint32_t>(a.root_bits);
   const int levels =
       kb <= root_bits ? 1 : 1 + int((kb - root_bits + kTrDigitBits - 1) / kTrDigitBits);
   const uint32_t below = uint32_t(levels - 1) * kTrDigitBits;
@@ -523,6 +530,12 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   TrLevel lv{a.root, a.rootrec, 1u << (top - kTrDigitBits)};
   const int64_t cap = a.slots;
   const bool with_attrs = a.out.attrs_in != nullptr;
+
+  if (a.large) {  // the bits of the first level
+    for (uint32_t i = gt; i < lv.ns * 2u; i += gthreads)
+      reinterpret_cast<uint4*>(a.root)[i] = zero4;
+    if (!grid_barrier(bar, target, a.spin_limit, err)) return;
+  }
 
   // ---- runs; level 1 marked ----
   bool range_bad = false;
@@ -540,8 +553,9 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
         const uint32_t last = tr_run(key, ok, &head);
         tail[u] = ok && last == lane;
         id[u] = static_cast<uint32_t>(key >> below);  // (at most 28 bits)
-        seen[u] =
-            tail[u] && (id[u] >> kTrDigitBits) < lv.ns ? __ldca(a.root + (id[u] >> 5)) : ~0u;
+        seen[u] = ~0u;
+        if (tail[u] && (id[u] >> kTrDigitBits) < lv.ns)
+          seen[u] = a.large ? __ldcg(a.root + (id[u] >> 5)) : __ldca(a.root + (id[u] >> 5));
         if (ok) tr_offsets(fm, t.f[u], t.q[u], ijk, w);
         tr_scan<3>(w, head);
         const uint32_t tm = __ballot_sync(kFullMask, tail[u]);
@@ -583,7 +597,10 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
     const uint32_t set = tr_rank_slots(lv.bits, lv.rec, lv.ns, agg, sm);
     const uint32_t n1 = static_cast<uint32_t>(min(int64_t(set), cap));
-    if (set > n1 && blockIdx.x == 0 && threadIdx.x == 0) set_error(err, kErrInvalidArg);
+    if (set > n1) {  // (the same in every block)
+      if (a.large) return;  // more cells than the buffers hold: the sort path
+      if (blockIdx.x == 0 && threadIdx.x == 0) set_error(err, kErrInvalidArg);
+    }
     if (j == levels) {
       rows = n1;
       break;
@@ -660,6 +677,10 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
       // more cells than output rows: recorded once, here; the first cap rows are written
       if (int64_t(rows) > a.out.cap) set_error(err, kErrCapacity);
       *a.out.num_voxels = rows;
+      if (a.large) {
+        a.st->narrow = 1u;
+        a.st->msd = kRowsWritten;
+      }
     }
     if (a.out.frame_offsets && (F == 1 || rows == 0))
       for (int f = threadIdx.x; f <= F; f += kTrThreads)
@@ -862,9 +883,13 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   const int64_t chunks = max_chunks(fr.n, fr.nframes);
   const int64_t g = trie_grid(chunks, num_sms());
   a.chunks = static_cast<uint32_t>(chunks);
-  const size_t head = reinterpret_cast<char*>(fs + fr.nframes) - reinterpret_cast<char*>(st);
-  trie_clear_kernel<<<1, 1024, 0, stream>>>(reinterpret_cast<uint32_t*>(st),
-                                           static_cast<uint32_t>(head / sizeof(uint32_t)), err);
+  a.large = fr.n > kTrMaxPoints ? 1 : 0;
+  a.root_bits = a.large ? kTrRootBitsLarge : kTrRootBits;
+  if (!a.large) {
+    const size_t head = reinterpret_cast<char*>(fs + fr.nframes) - reinterpret_cast<char*>(st);
+    trie_clear_kernel<<<1, 1024, 0, stream>>>(reinterpret_cast<uint32_t*>(st),
+                                             static_cast<uint32_t>(head / sizeof(uint32_t)), err);
+  }
   void* args[] = {&a};
   const void* fn = posed(fr) ? reinterpret_cast<const void*>(trie_kernel<true>)
                              : reinterpret_cast<const void*>(trie_kernel<false>);

@@ -8,11 +8,19 @@ constexpr int kTrThreads = 1024;    // threads of a block (one block an SM)
 constexpr int kTrDigitBits = 8;     // a slot of the trie: 2^8 children, one bit each
 constexpr int kTrWords = (1 << kTrDigitBits) / 32;
 constexpr int kTrMaxGrid = 1024;    // blocks of the launch at most
-// Bits of the first level (one bit per key prefix, cleared by every call): 2 MB.
+// Bits of the first level (one bit per key prefix): 2 MB up to kTrMaxPoints points, where
+// clearing and ranking more costs as much as another level's three barriers; up to 32 MB
+// above, where another level is another pass over the runs.
 constexpr int kTrRootBits = 24;
-// Largest call: the trie's accesses miss L2 beyond, and a shuffled cloud of 2.5M points takes
-// 268 us at 0.02 m where the radix sort takes 247 (2.0M: 206 against 224).
+constexpr int kTrRootBitsLarge = 28;
+// Up to so many points every call takes the trie.  Above, its accesses miss L2 where the cells
+// are many (a shuffled cloud of 2.5M points: 268 us at 0.02 m, the radix sort 247; 2.0M: 206
+// against 224), so the cells must be few: 2 of 5 sampled pairs of consecutive points share a
+// cell (camera frames at 5 mm to 0.1 m: 2 of 5 come with cells for at most a quarter of the
+// points, 1 of 5 with more than half), and the cells fit a quarter of the points.
 constexpr int64_t kTrMaxPoints = int64_t(1) << 21;
+constexpr int64_t kTrCellShare = 4;
+constexpr uint32_t kTrSame = 2, kTrSameOf = 5;
 
 // Blocks of the launch for so many chunks of points: one a chunk, but enough of them to clear
 // and rank the first level, and at most one an SM.
@@ -33,12 +41,13 @@ struct TrieLayout {
 constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base) {
   TrieLayout L{};
   const int64_t nn = n < 1 ? 1 : n;
-  L.slots = nn;
+  const int root_bits = nn <= kTrMaxPoints ? kTrRootBits : kTrRootBitsLarge;
+  L.slots = nn <= kTrMaxPoints ? nn : nn / kTrCellShare;
   size_t off = align_up(base, 256);
   L.root = off;
-  off = align_up(off + (size_t(1) << (kTrRootBits - 3)), 256);
+  off = align_up(off + (size_t(1) << (root_bits - 3)), 256);
   L.rootrec = off;
-  off = align_up(off + (size_t(1) << (kTrRootBits - kTrDigitBits)) * 16, 256);
+  off = align_up(off + (size_t(1) << (root_bits - kTrDigitBits)) * 16, 256);
   L.x = off;
   off = align_up(off + size_t(L.slots) * 48, 256);
   L.y = off;
@@ -60,7 +69,10 @@ constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base) {
   return L;
 }
 
-// Whether the grouping runs on this device, and its launch (two kernels).
+// Whether the grouping runs on this device, and its launch.  Up to kTrMaxPoints points it
+// needs nothing before it and writes every row (two kernels).  Above, it follows the extent
+// kernel (with its sample) on a cleared state, and either writes every row (kRowsWritten)
+// or leaves the call to the kernels behind it.
 bool trie_available(bool posed);
 cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameState* fs, char* ws,
                         const TrieLayout& L, const SegOut& out, uint32_t spin_limit, int* err,

@@ -121,6 +121,36 @@ def test_many_frames():
     same(a, b)
 
 
+@pytest.mark.parametrize("frames,w,h,leaf", [(3, 1280, 720, 0.02), (9, 800, 600, 0.01),
+                                             (5, 1280, 720, 0.0005)])
+def test_large_coherent_and_incoherent_frames(frames, w, h, leaf):
+    # above the size every call takes: camera frames (the sample admits them), and at 0.5 mm
+    # more cells than the share of points the buffers hold (left to the sort path), with
+    # and without the options, and the sort path after a refusal
+    x = cuda(np.concatenate([synth.rgbd_frame(w, h, seed=60 + f) for f in range(frames)]))
+    n = w * h
+    offs = [f * n for f in range(frames + 1)]
+    leaves = [leaf * (1 + f % 2) for f in range(frames)]
+    rgb = (torch.arange(3 * x.shape[0], device="cuda") * 37 % 256).to(torch.uint8).reshape(-1, 3)
+    for kw in ({}, {"point_to_voxel": True}, {"attrs": rgb, "min_count": 2}):
+        a = vg.downsample_frames((x, offs), leaves, **kw)
+        b = vg.downsample_frames((x, offs), leaves, method="sort_lsd", **kw)
+        assert a.offsets == b.offsets and torch.equal(a.origins, b.origins)
+        same(a, b)
+
+
+@pytest.mark.parametrize("p2v", [False, True])
+@pytest.mark.parametrize("origin", [None, (-1.0, -1.0, -1.0)])
+def test_large_cloud_that_the_sample_refuses(p2v, origin):
+    x = cuda(synth.fused_map(2_300_001, seed=5, extent=(20.0, 20.0, 5.0)))
+    o = None if origin is None else cuda(origin)
+    same(vg.downsample(x, 0.02, o, point_to_voxel=p2v),
+         vg.downsample(x, 0.02, o, point_to_voxel=p2v, method="sort_lsd"))
+    few = (x * 0.02).contiguous()  # the same shuffle, a few thousand cells: admitted
+    same(vg.downsample(few, 0.02, point_to_voxel=p2v),
+         vg.downsample(few, 0.02, point_to_voxel=p2v, method="sort_lsd"))
+
+
 def test_short_output_and_short_workspace():
     x = cuda(synth.rgbd_frame(640, 480, seed=0))
     n = x.shape[0]
