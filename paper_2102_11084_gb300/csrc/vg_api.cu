@@ -59,6 +59,7 @@ void warm_launch_config() {
   num_sms();
   warm_sort_config();
   warm_reduce_config();
+  warm_hash_config();
   warm_filter_config();
   warm_msd_config();
   warm_frame_config();
@@ -74,7 +75,9 @@ int persistent_grid(const void* kernel, int threads, size_t dyn_smem, int64_t wo
     for (int i = 0; i < g_occ_n; ++i)
       if (g_occ[i].fn == kernel && g_occ[i].dev == dev) blocks = g_occ[i].blocks;
     if (blocks == 0) {
-      if (dyn_smem > 48 * 1024 - 4096)
+      cudaFuncAttributes attr{};
+      if (cudaFuncGetAttributes(&attr, kernel) != cudaSuccess ||
+          dyn_smem + attr.sharedSizeBytes > 48 * 1024)
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(dyn_smem));
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, threads, dyn_smem) !=
@@ -304,7 +307,7 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
   uint32_t* lb_a = reinterpret_cast<uint32_t*>(ws + L.lb_a);
   uint32_t* lb_b = reinterpret_cast<uint32_t*>(ws + L.lb_b);
   HashTable tab{reinterpret_cast<unsigned long long*>(ws + L.tkeys),
-                reinterpret_cast<HashAcc*>(ws + L.tacc), static_cast<uint32_t>(L.slots - 1)};
+                reinterpret_cast<HashAcc*>(ws + L.tacc), static_cast<uint32_t>(L.slots - 1), 0};
   uint32_t* slot_rank = out.p2v ? reinterpret_cast<uint32_t*>(ws + L.slot_rank) : nullptr;
   uint32_t* point_slot = out.p2v ? reinterpret_cast<uint32_t*>(ws + L.point_slot) : nullptr;
   int* err = out_error ? reinterpret_cast<int*>(out_error) : &st->error;

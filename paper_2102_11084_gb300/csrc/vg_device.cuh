@@ -53,9 +53,11 @@ __device__ __forceinline__ bool axis_index(float p, float o, float leaf, uint32_
 }
 
 // The same index as axis_index, cheaper: q1 = fl(fl(p-o) * r) with r = fl(1/leaf) is
-// within 1.5*2^-23*|q| of fl((p-o)/leaf), so whenever q1 lies farther than |q1|*2^-20 from
-// every integer both have the same floor (and the same side of 0 and 2^21, which are
-// integers); otherwise the exact division decides.  Valid for 2^-100 < leaf < 2^100
+// within 3*2^-24*|q|*(1+2^-22) of fl((p-o)/leaf) (one rounding of r, one of the product, one of
+// the quotient), so whenever q1 lies farther than |q1|*2^-22 from every integer both have the
+// same floor (and the same side of 0 and 2^21, which are integers); otherwise the exact
+// division decides (at q = 1000 one point in 700 on some axis, a warp step in 25; with 2^-20,
+// one in seven).  Valid for 2^-100 < leaf < 2^100
 // (r is then a normal number); callers check that range.
 __device__ __forceinline__ bool axis_index_fast(float p, float o, float leaf, float r,
                                                 uint32_t* i) {
@@ -63,7 +65,7 @@ __device__ __forceinline__ bool axis_index_fast(float p, float o, float leaf, fl
   const float q1 = __fmul_rn(t, r);
   const float fl = floorf(q1);
   const float d = q1 - fl;
-  const float margin = fabsf(q1) * 9.5367431640625e-07f;  // 2^-20
+  const float margin = fabsf(q1) * 2.384185791015625e-07f;  // 2^-22
   if (d > margin && 1.0f - d > margin) {
     if (!(fl >= 0.0f) || !(fl < kAxisLimitF)) return false;
     *i = static_cast<uint32_t>(fl);
@@ -81,18 +83,7 @@ __device__ __forceinline__ bool point_valid(float x, float y, float z) {
   return isfinite(x) && isfinite(y) && isfinite(z);
 }
 
-// Spread the low 21 bits of v so that bit b lands on bit 3b.
-__device__ __forceinline__ uint64_t spread3(uint32_t v) {
-  uint64_t x = v & 0x1fffffu;
-  x = (x | (x << 32)) & 0x001f00000000ffffull;
-  x = (x | (x << 16)) & 0x001f0000ff0000ffull;
-  x = (x | (x << 8)) & 0x100f00f00f00f00full;
-  x = (x | (x << 4)) & 0x10c30c30c30c30c3ull;
-  x = (x | (x << 2)) & 0x1249249249249249ull;
-  return x;
-}
-
-// Inverse of spread3: gather bits 0, 3, 6, ... into the low 21 bits.
+// Gather bits 0, 3, 6, ... into the low 21 bits.
 __device__ __forceinline__ uint32_t compact3(uint64_t x) {
   x &= 0x1249249249249249ull;
   x = (x | (x >> 2)) & 0x10c30c30c30c30c3ull;
@@ -103,7 +94,7 @@ __device__ __forceinline__ uint32_t compact3(uint64_t x) {
   return static_cast<uint32_t>(x);
 }
 
-// spread3 for indices below 2^11, with 32-bit operations (bit b -> bit 3b, up to bit 30).
+// Spread the bits of an index below 2^11 so that bit b lands on bit 3b, up to bit 30.
 __device__ __forceinline__ uint32_t spread3_32(uint32_t x) {
   x &= 0x7ffu;
   x = (x | (x << 16)) & 0x070000ffu;
@@ -111,6 +102,18 @@ __device__ __forceinline__ uint32_t spread3_32(uint32_t x) {
   x = (x | (x << 4)) & 0x430c30c3u;
   x = (x | (x << 2)) & 0x49249249u;
   return x;
+}
+
+// The low ten bits of each index on 32-bit words; the rest, which most points do not have, on
+// its own (three 64-bit spreads took half again as long).
+__device__ __forceinline__ uint64_t morton3(uint32_t ix, uint32_t iy, uint32_t iz) {
+  uint64_t key = spread3_32(ix & 1023u) | (spread3_32(iy & 1023u) << 1) |
+                 (spread3_32(iz & 1023u) << 2);
+  if ((ix | iy | iz) >> 10)
+    key |= (uint64_t(spread3_32(ix >> 10)) | (uint64_t(spread3_32(iy >> 10)) << 1) |
+            (uint64_t(spread3_32(iz >> 10)) << 2))
+           << 30;
+  return key;
 }
 
 // compact3 for keys below 2^32 (11 bits of x and y, 10 of z), with 32-bit operations.
@@ -128,9 +131,6 @@ __device__ __forceinline__ uint32_t key_axis(uint64_t key, int axis) {
   return (key >> 32) == 0 ? compact3_32(static_cast<uint32_t>(key) >> axis) : compact3(key >> axis);
 }
 
-__device__ __forceinline__ uint64_t morton3(uint32_t ix, uint32_t iy, uint32_t iz) {
-  return spread3(ix) | (spread3(iy) << 1) | (spread3(iz) << 2);
-}
 
 // Validity and voxel indices of a point (no key); *range_bad set when out of range.
 __device__ __forceinline__ bool point_index(float x, float y, float z, const float o[3],

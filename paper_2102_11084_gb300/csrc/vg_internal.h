@@ -275,6 +275,7 @@ int persistent_grid(const void* kernel, int threads, size_t dyn_smem, int64_t wo
 void warm_launch_config();
 void warm_sort_config();
 void warm_reduce_config();
+void warm_hash_config();
 
 // Launchers (all asynchronous on `stream`).
 // a1: per-frame min (and max) of the valid points into FrameState.
@@ -345,15 +346,17 @@ cudaError_t launch_keys_any(const float* xyz, const FramesArg& fr, bool have_ext
                             uint64_t* payload, int* err, cudaStream_t stream);
 
 // ---- hash path ----
+// A cell's three sums of biased offsets and its points: a = x + y 2^32, b = z + points 2^32
+// (mod 2^64), c = the carries out of a's and b's low halves and out of a, 21 bits each (n
+// points carry at most n / 2^11 times), so that a run of points is added by two atomics.
 struct alignas(32) HashAcc {
-  uint32_t n;
-  uint32_t pad;
-  long long s[3];
+  unsigned long long a, b, c, pad;
 };
 struct HashTable {
   unsigned long long* keys;  // [H], ~0 = empty
   HashAcc* acc;              // [H]
   uint32_t mask;             // H - 1, H a power of two
+  int zeroed;                // 1: the accumulators of empty slots are zero
 };
 
 // Slot count of the hash table for n points: a power of two >= 2n (never fills).
@@ -408,6 +411,8 @@ constexpr HashLayout hash_layout(int64_t n, int frames = 1) {
 cudaError_t launch_hash_insert(const float* xyz, const FramesArg& fr, bool have_extent, State* st,
                                FrameState* fs, const HashTable& tab, uint32_t* point_slot,
                                uint32_t spin_limit, int* err, cudaStream_t stream);
+// Empties a zeroed table: its occupied slots cleared, keys and accumulators.
+cudaError_t launch_hash_clear(const HashTable& tab, cudaStream_t stream);
 cudaError_t launch_hash_compact(const HashTable& tab, State* st, uint64_t* keys, uint32_t* slots,
                                 const int* err, cudaStream_t stream);
 cudaError_t launch_hash_finalize(const State* st, const FrameState* fs, int nframes,

@@ -116,7 +116,7 @@ vg_status vg_map_create(vg_map** out, int64_t capacity, const float* origin, flo
   m->leaves = reinterpret_cast<float*>(base + L.leaves);
   m->tab = vg::HashTable{reinterpret_cast<unsigned long long*>(base + L.tkeys),
                          reinterpret_cast<vg::HashAcc*>(base + L.tacc),
-                         static_cast<uint32_t>(m->slots - 1)};
+                         static_cast<uint32_t>(m->slots - 1), 1};
   m->lb_a = reinterpret_cast<uint32_t*>(base + L.lb_a);
   m->lb_b = reinterpret_cast<uint32_t*>(base + L.lb_b);
   m->keys0 = reinterpret_cast<uint64_t*>(base + L.keys0);
@@ -138,6 +138,7 @@ vg_status vg_map_create(vg_map** out, int64_t capacity, const float* origin, flo
                    size_t(vg::kMaxFrames) * sizeof(float), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemset(m->tab.keys, 0xff, size_t(m->slots) * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMemset(m->tab.acc, 0, size_t(m->slots) * sizeof(vg::HashAcc));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     cudaFree(m->mem);
@@ -161,8 +162,7 @@ vg_status vg_map_clear(vg_map* m, vg_stream_t stream_) {
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
   cudaError_t e = cudaMemsetAsync(m->st, 0, sizeof(vg::State), stream);
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(m->tab.keys, 0xff, size_t(m->slots) * sizeof(unsigned long long),
-                        stream);
+    e = vg::launch_hash_clear(m->tab, stream);
   return cuda_status(e);
 }
 
