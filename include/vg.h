@@ -418,12 +418,12 @@ VG_API vg_status vg_downsample_backward(const float* grad_centroids, const uint3
  *
  * Arguments are those of vg_downsample minus workspace/workspace_bytes; the caller still
  * passes (and owns) the input cloud and all outputs.  The scratch is a static device
- * array of vg_downsample_noalloc_scratch_bytes() bytes (about 25 MB, the workspace of
- * VG_NOALLOC_MAX_POINTS points) that every GPU loading the library keeps until the
+ * array of vg_downsample_noalloc_scratch_bytes() bytes (about 88 MB, AUTO's workspace
+ * for VG_NOALLOC_MAX_POINTS points) that every GPU loading the library keeps until the
  * process exits.  The call allocates nothing.
  *   * n > VG_NOALLOC_MAX_POINTS is rejected with VG_ERR_INVALID_ARG before any launch.
  *   * Only the sort method runs here (VG_METHOD_AUTO, VG_METHOD_SORT, with or without
- *     VG_SORT_BUCKETS or VG_SORT_LSD): the array holds the sort path's workspace, so
+ *     VG_SORT_BUCKETS or VG_SORT_LSD): the array holds AUTO's and SORT's workspace, so
  *     VG_METHOD_HASH and VG_SORT_FRAME are rejected with VG_ERR_INVALID_ARG before any
  *     launch.
  *   * The device address of the array is cached per device; cudaDeviceReset invalidates

@@ -127,9 +127,12 @@ bool trie_call(int64_t n, int flags) {
 
 // The trie's scratch: in the place of the sort path's, or, where the sort path may follow,
 // after what that clears before the trie runs.
-TrieLayout trie_scratch(int64_t n, int frames, const SortLayout& L) {
-  return trie_layout(n, frames, n <= kTrMaxPoints ? L.lb_a : L.lb_b);
+TrieLayout trie_scratch(int64_t n, int frames, const SortLayout& L, size_t att_base = 0) {
+  return trie_layout(n, frames, n <= kTrMaxPoints ? L.lb_a : L.lb_b, att_base);
 }
+
+// Points whose attribute sums a row's 32-bit words hold, whatever their cells.
+constexpr int64_t kTrieAttrPoints = int64_t(1) << 24;
 
 }  // namespace
 
@@ -193,9 +196,11 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
     const SortLayout L = sort_layout(n, F);
     // The trie: every call of up to kTrMaxPoints points; above, those whose sample shows few
     // cells (decided on the device).  Its 32-bit channel sums bound the points with attributes.
-    const TrieLayout TL = trie_scratch(n, F, L);
-    const bool trie = trie_ok && trie_available(posed(frn)) && workspace_bytes >= TL.total &&
-                      !(out.attrs_in && n > (int64_t(1) << 24));
+    const size_t all = frames_workspace_bytes(n, F, flags);
+    const TrieLayout TL = trie_scratch(n, F, L, all);
+    const bool trie = trie_ok && trie_available(posed(frn)) &&
+                      workspace_bytes >= (out.attrs_in ? TL.att_total : all) &&
+                      !(out.attrs_in && n > kTrieAttrPoints);
     const bool have_extent = from_min || F > 1 || frn.allow_narrow || trie;
     State* st = reinterpret_cast<State*>(ws + L.state);
     FrameState* fs = reinterpret_cast<FrameState*>(ws + L.frames);
@@ -347,10 +352,10 @@ struct PyramidLayout {
   int64_t merge_tiles;
 };
 
-PyramidLayout pyramid_layout(int64_t n, int levels) {
+PyramidLayout pyramid_layout(int64_t n, int levels, size_t base) {
   PyramidLayout L{};
   const int64_t nn = n < 1 ? 1 : n;
-  L.base = frames_workspace_bytes(n, 1, VG_METHOD_AUTO);
+  L.base = base;
   size_t off = L.base;
   L.sums_a = off;
   off = align_up(off + size_t(nn) * 3 * sizeof(long long), 256);
@@ -483,10 +488,18 @@ vg_status vg_downsample_frames_posed(const float* xyz, int64_t n_total,
                                  workspace, workspace_bytes, flags, stream);
 }
 
+// Workspace of a call with extras before the minimum-count filter's: with attributes, the
+// trie's sums of them follow.
+static size_t ex_base(int64_t n, int frames, int flags, bool attrs) {
+  const size_t base = frames_workspace_bytes(n, frames, flags);
+  if (!attrs || !trie_call(n, flags) || n > kTrieAttrPoints) return base;
+  return trie_scratch(n, frames, sort_layout(n, frames), base).att_total;
+}
+
 size_t vg_downsample_ex_workspace_bytes(int64_t n_total, int n_frames, int flags,
                                         const vg_voxel_extras* extras) {
   if (n_total < 0 || n_frames < 1 || n_frames > kMaxFrames) return 0;
-  const size_t base = frames_workspace_bytes(n_total, n_frames, flags);
+  const size_t base = ex_base(n_total, n_frames, flags, extras && extras->attrs);
   if (!extras || extras->min_count <= 1) return base;
   return filter_layout(n_total, base).total;
 }
@@ -529,14 +542,19 @@ vg_status vg_downsample_frames_ex(const float* xyz, int64_t n_total,
   SegOut out{out_keys, out_centroids, out_counts, nullptr, cap, out_frame_offsets + n_frames,
              out_frame_offsets, out_point_to_voxel, attrs, channels,
              attrs ? extras->out_attrs : nullptr};
-  const size_t base = frames_workspace_bytes(n_total, n_frames, flags);
+  size_t base = ex_base(n_total, n_frames, flags, attrs != nullptr);
   FilterLayout FL{};
   if (filtered) {
     FL = filter_layout(n_total, base);
+    if (workspace && workspace_bytes < FL.total) {  // (the sort path's workspace is enough)
+      base = trie_call(n_total, flags) ? sort_layout(n_total, n_frames).total : base;
+      FL = filter_layout(n_total, base);
+    }
     if (!workspace || workspace_bytes < FL.total) return VG_ERR_WORKSPACE;
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  s = run_frames(xyz, fr, from_min, out, out_error, workspace, workspace_bytes, flags, st);
+  s = run_frames(xyz, fr, from_min, out, out_error, workspace, filtered ? base : workspace_bytes,
+                 flags, st);
   if (s != VG_OK || !filtered) return s;
   char* ws = static_cast<char*>(workspace);
   int* err = out_error ? reinterpret_cast<int*>(out_error) : &reinterpret_cast<State*>(ws)->error;
@@ -547,7 +565,7 @@ vg_status vg_downsample_frames_ex(const float* xyz, int64_t n_total,
 size_t vg_pyramid_workspace_bytes(int64_t n_points, int levels, int flags) {
   (void)flags;
   if (n_points < 0 || levels < 1 || levels > kMaxLevels) return 0;
-  return pyramid_layout(n_points, levels).total;
+  return pyramid_layout(n_points, levels, frames_workspace_bytes(n_points, 1, VG_METHOD_AUTO)).total;
 }
 
 vg_status vg_pyramid(const float* xyz, int64_t n, float* origin, float leaf, int levels,
@@ -566,7 +584,9 @@ vg_status vg_pyramid(const float* xyz, int64_t n, float* origin, float leaf, int
                               out_level_offsets, out_point_to_voxel, out_error, workspace);
   if (s != VG_OK) return s;
   if (!aligned(origin, 4)) return VG_ERR_ALIGN;
-  const PyramidLayout P = pyramid_layout(n, levels);
+  PyramidLayout P = pyramid_layout(n, levels, frames_workspace_bytes(n, 1, VG_METHOD_AUTO));
+  if (workspace_bytes < P.total)  // (level 0 by the sort path)
+    P = pyramid_layout(n, levels, sort_layout(n, 1).total);
   if (!workspace || workspace_bytes < P.total) return VG_ERR_WORKSPACE;
   char* ws = static_cast<char*>(workspace);
   const SortLayout L = sort_layout(n, 1);

@@ -5,20 +5,25 @@
 // that has no way to hand the library a workspace.
 //
 // The scratch lives in a file-scope __device__ array sized for VG_NOALLOC_MAX_POINTS
-// points (the sort-path workspace for that many points, about 25 MB).  Every GPU that
-// loads this module keeps the array until the process exits.  Nothing here allocates:
-// the call looks up the array's device address once per device and then runs the
-// ordinary vg_downsample (sort path only) on it.  A cudaDeviceReset unloads the module;
+// points (AUTO's workspace for that many points, the occupancy trie's, about 88 MB).  Every
+// GPU that loads this module keeps the array until the process exits.  Nothing here
+// allocates: the call looks up the array's device address once per device and then runs the
+// ordinary vg_downsample (AUTO and the sort path only) on it.  A cudaDeviceReset unloads the module;
 // the cached address is then stale, so the entry point is not for use after a reset.
 #include <mutex>
 
 #include "../../include/vg.h"
 #include "vg_internal.h"
+#include "vg_trie.h"
 
 namespace {
 
 constexpr int64_t kMaxPoints = VG_NOALLOC_MAX_POINTS;
-constexpr size_t kScratchBytes = vg::sort_layout(kMaxPoints).total;
+constexpr size_t kSortBytes = vg::sort_layout(kMaxPoints).total;
+constexpr size_t kTrieBytes =
+    vg::trie_layout(kMaxPoints, 1, vg::sort_layout(kMaxPoints).lb_a).total;
+constexpr size_t kScratchBytes = kTrieBytes > kSortBytes ? kTrieBytes : kSortBytes;
+static_assert(kMaxPoints <= vg::kTrMaxPoints, "the trie's scratch for every cloud accepted here");
 
 // Device scratch shared by every call on a device.
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
@@ -51,8 +56,8 @@ vg_status vg_downsample_noalloc(const float* xyz, int64_t n, float* origin, floa
                                 int64_t cap, int64_t* out_num_voxels, int32_t* out_point_to_voxel,
                                 int32_t* out_error, int flags, vg_stream_t stream) {
   if (n < 0 || n > kMaxPoints) return VG_ERR_INVALID_ARG;
-  // The array is sized for the sort path's workspace; the hash path and the single-frame
-  // bin grouping need more.
+  // The array is sized for AUTO's workspace; the hash path and the single-frame method need
+  // more.
   if ((flags & VG_METHOD_MASK) == VG_METHOD_HASH || (flags & VG_SORT_FRAME) != 0)
     return VG_ERR_INVALID_ARG;
   void* scratch = nullptr;

@@ -6,12 +6,12 @@
 // among the occupied keys is its row, and the points add their offsets at the row (exact
 // integers, so in any order).  The ranks come from a trie of bitmaps over the keys:
 //   level 1   one bit per prefix of up to 24 key bits (28 for large clouds), grouped in slots
-//             of 2^8 bits;
-//   level j   one slot of 2^8 bits per occupied prefix of level j - 1, numbered by its rank
-//             there, for the next 8 key bits.
+//             of 2^7 bits;
+//   level j   one slot of 2^7 bits per occupied prefix of level j - 1, numbered by its rank
+//             there, for the next 7 key bits.
 // Each level is marked by a pass over the points, its set bits counted per block and, after a
 // barrier, ranked: a slot's record holds the set bits before the slot and, as bytes, before
-// each of its 8 words.  Keys of up to 24 bits take one level, each 8 bits more another one.
+// each of its words.  Keys of up to 24 bits take one level, each 7 bits more another one.
 // The points are read twice, for the extents and for the first level; that second pass also
 // merges runs of equal keys among a warp's 32 consecutive points (neighbouring pixels of a
 // camera frame often share a cell) and writes each run, 16 bytes, to a dense list of its warp
@@ -55,12 +55,13 @@ struct TrArgs {
   State* st;
   FrameState* fs;
   uint32_t* root;      // first level: bits, then records (below)
-  uint4* rootrec;
+  uint2* rootrec;
   char* x;             // buffers of the further levels
   char* y;
   uint4* run;          // a warp's runs: {key, sum x, sum y, sum z | points << 26}
   uint32_t* runhi;     // the upper key words (keys of more than 32 bits)
   uint2* runatt;       // the runs' attribute sums, 16 bits a channel
+  unsigned long long* rowatt;  // the rows', two words a row
   uint32_t* pslot;     // the slot of a run's prefix, then its row
   uint2* mask;         // per 32 points: lanes that end a run, valid lanes (point_to_voxel)
   uint32_t* stat;      // per level (8): the blocks' totals
@@ -194,7 +195,7 @@ __device__ __forceinline__ uint32_t tr_run(uint64_t key, bool ok, uint32_t* head
   return later ? lane + __ffs(later) - 1u : 31u;
 }
 
-// Sets bit id & 255 of slot id >> 8 for every lane with `emit` that does not see its bit set
+// Sets bit id mod 2^7 of slot id >> 7 for every lane with `emit` that does not see its bit set
 // (`seen`: the word as loaded before; a stale one can only lack bits).  Up to half a warp of
 // lanes (a camera frame's runs, which meet a few words) merges them word by word: the
 // atomics of all warps on the few words took 8,500 cycles more of a 640x480 frame.  More
@@ -229,16 +230,14 @@ __device__ __forceinline__ void tr_set(uint32_t* bits, uint32_t id, bool emit, u
 }
 
 // Rank of bit d of a slot, from its record r and the word v that holds the bit.
-__device__ __forceinline__ uint32_t tr_rank(uint4 r, uint32_t v, uint32_t d) {
+__device__ __forceinline__ uint32_t tr_rank(uint2 r, uint32_t v, uint32_t d) {
   const uint32_t w = d >> 5;
-  const uint32_t before = ((w & 4u ? r.z : r.y) >> (8u * (w & 3u))) & 255u;
+  const uint32_t before = (r.y >> (8u * w)) & 255u;
   return r.x + before + __popc(v & ((1u << (d & 31u)) - 1u));
 }
 
-__device__ __forceinline__ void tr_slot_words(const uint32_t* bits, uint32_t s, uint4 v[2]) {
-  const uint4* q = reinterpret_cast<const uint4*>(bits) + 2 * size_t(s);
-  v[0] = __ldcg(q);
-  v[1] = __ldcg(q + 1);
+__device__ __forceinline__ uint4 tr_slot_words(const uint32_t* bits, uint32_t s) {
+  return __ldcg(reinterpret_cast<const uint4*>(bits) + s);
 }
 
 // Ranking the set bits of slots [0, ns) takes two steps around a grid barrier: block b takes a
@@ -254,17 +253,15 @@ __device__ __forceinline__ void tr_count(const uint32_t* bits, uint32_t ns, uint
   uint32_t s0, s1, mine = 0;
   tr_slice(ns, &s0, &s1);
   for (uint32_t s = s0 + threadIdx.x; s < s1; s += kTrThreads) {
-    uint4 v[2];
-    tr_slot_words(bits, s, v);
-    mine += __popc(v[0].x) + __popc(v[0].y) + __popc(v[0].z) + __popc(v[0].w) + __popc(v[1].x) +
-            __popc(v[1].y) + __popc(v[1].z) + __popc(v[1].w);
+    const uint4 v = tr_slot_words(bits, s);
+    mine += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
   }
   uint32_t total;
   (void)block_excl_scan(mine, &total, tmp);
   if (threadIdx.x == 0) agg[blockIdx.x] = total;
 }
 // Returns the grand total (the same in every block).  Contains __syncthreads.
-__device__ __forceinline__ uint32_t tr_rank_slots(const uint32_t* bits, uint4* rec, uint32_t ns,
+__device__ __forceinline__ uint32_t tr_rank_slots(const uint32_t* bits, uint2* rec, uint32_t ns,
                                                   const uint32_t* agg, TrSmem& sm) {
   uint32_t s0, s1;
   tr_slice(ns, &s0, &s1);
@@ -276,19 +273,13 @@ __device__ __forceinline__ uint32_t tr_rank_slots(const uint32_t* bits, uint4* r
   uint32_t base = sm.first;
   for (uint32_t t0 = s0; t0 < s1; t0 += kTrThreads) {  // (the same trips in every thread)
     const uint32_t s = t0 + threadIdx.x;
-    uint4 v[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
-    if (s < s1) tr_slot_words(bits, s, v);
-    const uint32_t w[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
-    uint32_t run = 0, lo = 0, hi = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {  // set bits before word i: at most 224
-      if (i < 4) lo |= run << (8 * i);
-      else hi |= run << (8 * (i - 4));
-      run += __popc(w[i]);
-    }
+    const uint4 v = s < s1 ? tr_slot_words(bits, s) : make_uint4(0u, 0u, 0u, 0u);
+    // set bits before each word: at most 96
+    const uint32_t b1 = __popc(v.x), b2 = b1 + __popc(v.y), b3 = b2 + __popc(v.z);
+    const uint32_t run = b3 + __popc(v.w);
     uint32_t tot;
     const uint32_t r = base + block_excl_scan(run, &tot, sm.tmp);
-    if (s < s1) rec[s] = make_uint4(r, lo, hi, 0u);
+    if (s < s1) rec[s] = make_uint2(r, (b1 << 8) | (b2 << 16) | (b3 << 24));
     base += tot;
   }
   return all;
@@ -363,7 +354,7 @@ __device__ __forceinline__ void tr_scan(uint32_t w[N], uint32_t head) {
 // A level in use: its slots' bits and records.
 struct TrLevel {
   uint32_t* bits;
-  uint4* rec;
+  uint2* rec;
   uint32_t ns;  // slots
 };
 
@@ -532,7 +523,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   const bool with_attrs = a.out.attrs_in != nullptr;
 
   if (a.large) {  // the bits of the first level
-    for (uint32_t i = gt; i < lv.ns * 2u; i += gthreads)
+    for (uint32_t i = gt; i < lv.ns; i += gthreads)
       reinterpret_cast<uint4*>(a.root)[i] = zero4;
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
   }
@@ -608,12 +599,12 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     // the buffers alternate so that the last level lies in x
     char* nb = ((levels - j - 1) & 1) ? a.y : a.x;
     uint32_t* nbits = reinterpret_cast<uint32_t*>(nb);
-    for (uint32_t i = gt; i < n1 * 2u; i += gthreads) reinterpret_cast<uint4*>(nbits)[i] = zero4;
+    for (uint32_t i = gt; i < n1; i += gthreads) reinterpret_cast<uint4*>(nbits)[i] = zero4;
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
     const uint32_t sh = below - uint32_t(j) * kTrDigitBits;  // key bits below the next level
     for (uint32_t i0 = 0; i0 < nruns; i0 += 64) {
       uint32_t id[2], seen[2], v[2];
-      uint4 r[2];
+      uint2 r[2];
       bool in[2];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
@@ -621,15 +612,15 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
         in[u] = i < nruns;
         id[u] = 0u;
         v[u] = 0u;
-        r[u] = make_uint4(~0u, 0u, 0u, 0u);
+        r[u] = make_uint2(~0u, 0u);
         if (!in[u]) continue;
         uint64_t key = run[i].x;
         if (kb > 32u) key |= uint64_t(a.runhi[w0 * 32 + i]) << 32;
-        id[u] = static_cast<uint32_t>(key >> sh) & 0xffffu;  // this level's digit and the next
+        id[u] = static_cast<uint32_t>(key >> sh) & ((kTrDigit << kTrDigitBits) | kTrDigit);  // two digits
         const uint32_t s0 =
             j == 1 ? static_cast<uint32_t>(key >> (sh + 2 * kTrDigitBits)) : pslot[i];
         if (s0 < lv.ns) {
-          v[u] = __ldcg(lv.bits + s0 * kTrWords + (id[u] >> 13));
+          v[u] = __ldcg(lv.bits + s0 * kTrWords + (id[u] >> (kTrDigitBits + 5)));
           r[u] = __ldcg(lv.rec + s0);
         }
       }
@@ -644,14 +635,14 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
           in[u] = false;
           continue;
         }
-        id[u] = (s << kTrDigitBits) | (id[u] & 255u);
+        id[u] = (s << kTrDigitBits) | (id[u] & kTrDigit);
         seen[u] = __ldcg(nbits + (id[u] >> 5));
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) tr_set(nbits, id[u], in[u], seen[u]);
     }
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
-    lv = TrLevel{nbits, reinterpret_cast<uint4*>(nb + size_t(cap) * 32), n1};
+    lv = TrLevel{nbits, reinterpret_cast<uint2*>(nb + size_t(cap) * (kTrWords * 4)), n1};
   }
 
   // ---- the rows' sums cleared ----
@@ -660,7 +651,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   R.B = R.A + cap;
   R.C = R.B + cap;
   R.key = R.C + cap;
-  R.att = R.key + cap;
+  R.att = a.rowatt;
   R.cap = cap;
   R.rows = rows;
   for (uint32_t i = gt; i < rows; i += gthreads) {
@@ -690,20 +681,21 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
 
   // ---- every run's points and sums at its row ----
   for (uint32_t i0 = 0; i0 < nruns; i0 += 32u * kTrAdd) {
-    uint4 e[kTrAdd], r[kTrAdd];
+    uint4 e[kTrAdd];
+    uint2 r[kTrAdd];
     uint32_t v[kTrAdd], row[kTrAdd];
     unsigned long long oa[kTrAdd], ob[kTrAdd], va[kTrAdd], vb[kTrAdd];
 #pragma unroll
     for (int u = 0; u < kTrAdd; ++u) {
       const uint32_t i = i0 + 32u * u + lane;
       v[u] = 0u;
-      r[u] = make_uint4(~0u, 0u, 0u, 0u);
+      r[u] = make_uint2(~0u, 0u);
       e[u] = zero4;
       if (i >= nruns) continue;
       e[u] = run[i];
       const uint32_t s0 = levels == 1 ? e[u].x >> kTrDigitBits : pslot[i];
       if (s0 < lv.ns) {
-        v[u] = __ldcg(lv.bits + s0 * kTrWords + ((e[u].x >> 5) & 7u));
+        v[u] = __ldcg(lv.bits + s0 * kTrWords + ((e[u].x >> 5) & (kTrWords - 1u)));
         r[u] = __ldcg(lv.rec + s0);
       }
     }
@@ -713,7 +705,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
       row[u] = ~0u;
       oa[u] = ob[u] = va[u] = vb[u] = 0ull;
       if (i >= nruns) continue;
-      if (r[u].x != ~0u) row[u] = tr_rank(r[u], v[u], e[u].x & 255u);
+      if (r[u].x != ~0u) row[u] = tr_rank(r[u], v[u], e[u].x & kTrDigit);
       if (row[u] >= rows) {
         set_error(err, kErrInvalidArg);
         row[u] = ~0u;
@@ -866,12 +858,13 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   a.st = st;
   a.fs = fs;
   a.root = reinterpret_cast<uint32_t*>(ws + L.root);
-  a.rootrec = reinterpret_cast<uint4*>(ws + L.rootrec);
+  a.rootrec = reinterpret_cast<uint2*>(ws + L.rootrec);
   a.x = ws + L.x;
   a.y = ws + L.y;
   a.run = reinterpret_cast<uint4*>(ws + L.run);
   a.runhi = reinterpret_cast<uint32_t*>(ws + L.runhi);
   a.runatt = reinterpret_cast<uint2*>(ws + L.runatt);
+  a.rowatt = reinterpret_cast<unsigned long long*>(ws + L.rowatt);
   a.pslot = reinterpret_cast<uint32_t*>(ws + L.pslot);
   a.mask = reinterpret_cast<uint2*>(ws + L.mask);
   a.stat = reinterpret_cast<uint32_t*>(ws + L.stat);

@@ -5,8 +5,12 @@
 namespace vg {
 
 constexpr int kTrThreads = 1024;    // threads of a block (one block an SM)
-constexpr int kTrDigitBits = 8;     // a slot of the trie: 2^8 children, one bit each
+constexpr int kTrDigitBits = 7;     // a slot of the trie: 2^7 children, one bit each
+constexpr uint32_t kTrDigit = (1u << kTrDigitBits) - 1u;
 constexpr int kTrWords = (1 << kTrDigitBits) / 32;
+constexpr size_t kTrSlotBytes = kTrWords * 4 + 8;  // bits and record
+constexpr size_t kTrRowBytes = 32;                 // sums, carries and key
+static_assert(kTrWords == 4, "a slot's bits are one 16-byte word, its record three prefixes");
 constexpr int kTrMaxGrid = 1024;    // blocks of the launch at most
 // Bits of the first level (one bit per key prefix): 2 MB up to kTrMaxPoints points, where
 // clearing and ranking more costs as much as another level's three barriers; up to 32 MB
@@ -30,35 +34,34 @@ constexpr int64_t trie_grid(int64_t chunks, int sms) {
   return chunks < least ? least : (chunks < most ? chunks : most);
 }
 
-// Scratch, from `base` on: the first level's bits and records, two buffers of slots (32 B of
-// bits and a 16 B record each; the second one holds the rows' sums, keys and attribute sums
-// once the rows are known), the runs of every warp (each warp's list has a place for every
-// point it may read), the blocks' totals.
+// Scratch, from `base` on: the first level's bits and records, two buffers of slots (16 B of
+// bits and an 8 B record each; the second one holds the rows' sums and keys once the rows are
+// known), the runs of every warp (each warp's list has a place for every point it may read),
+// the blocks' totals; with attributes, from `att_base` on, the runs' and the rows' sums.
 struct TrieLayout {
-  size_t root, rootrec, x, y, run, runhi, runatt, pslot, mask, stat, total;
+  size_t root, rootrec, x, y, run, runhi, pslot, mask, stat, total;
+  size_t runatt, rowatt, att_total;
   int64_t slots;  // slots (and rows) the buffers hold
 };
-constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base) {
+constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base, size_t att_base = 0) {
   TrieLayout L{};
   const int64_t nn = n < 1 ? 1 : n;
   const int root_bits = nn <= kTrMaxPoints ? kTrRootBits : kTrRootBitsLarge;
   L.slots = nn <= kTrMaxPoints ? nn : nn / kTrCellShare;
+  const size_t places = size_t(max_chunks(nn, frames)) * kChunk;
   size_t off = align_up(base, 256);
   L.root = off;
   off = align_up(off + (size_t(1) << (root_bits - 3)), 256);
   L.rootrec = off;
-  off = align_up(off + (size_t(1) << (root_bits - kTrDigitBits)) * 16, 256);
+  off = align_up(off + (size_t(1) << (root_bits - kTrDigitBits)) * 8, 256);
   L.x = off;
-  off = align_up(off + size_t(L.slots) * 48, 256);
+  off = align_up(off + size_t(L.slots) * kTrSlotBytes, 256);
   L.y = off;
-  off = align_up(off + size_t(L.slots) * 48, 256);
-  const size_t places = size_t(max_chunks(nn, frames)) * kChunk;
+  off = align_up(off + size_t(L.slots) * kTrRowBytes, 256);
   L.run = off;
   off = align_up(off + places * 16, 256);
   L.runhi = off;
   off = align_up(off + places * 4, 256);
-  L.runatt = off;
-  off = align_up(off + places * 8, 256);
   L.pslot = off;
   off = align_up(off + places * 4, 256);
   L.mask = off;
@@ -66,8 +69,16 @@ constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base) {
   L.stat = off;
   off = align_up(off + 8 * size_t(kTrMaxGrid) * sizeof(uint32_t), 256);
   L.total = off;
+  off = align_up(att_base, 256);
+  L.runatt = off;
+  off = align_up(off + places * 8, 256);
+  L.rowatt = off;
+  off = align_up(off + size_t(L.slots) * 16, 256);
+  L.att_total = off;
   return L;
 }
+static_assert(kTrRowBytes >= kTrSlotBytes, "the second buffer holds slots too");
+static_assert((63 - kTrRootBits + kTrDigitBits - 1) / kTrDigitBits + 1 <= 8, "levels");
 
 // Whether the grouping runs on this device, and its launch.  Up to kTrMaxPoints points it
 // needs nothing before it and writes every row (two kernels).  Above, it follows the extent
