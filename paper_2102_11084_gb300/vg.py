@@ -180,9 +180,37 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
 
+def _raw_stream(stream: Optional[torch.cuda.Stream]) -> int:
+    # (the handle itself: a torch.cuda.Stream object of the current stream costs 10 us)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
 def _stream_ptr(stream: Optional[torch.cuda.Stream]):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return ctypes.c_void_p(_raw_stream(stream))
+
+
+def _wait(stream: Optional[torch.cuda.Stream], device: torch.device) -> None:
+    """Waits for the stream a call was launched on, unless a copy of `device`'s tensors to the
+    host waits for it anyway (it is that device's current stream)."""
+    cur = torch._C._cuda_getDevice()
+    if device.index not in (None, cur) or \
+            _raw_stream(stream) != torch._C._cuda_getCurrentRawStream(cur):
+        (stream or torch.cuda.current_stream()).synchronize()
+
+
+def _scalars(device) -> torch.Tensor:
+    """Voxel count (int64) and error word (int32, the low half of the second entry) of a call,
+    written by it: one allocation and one copy to the host."""
+    return torch.empty(2, dtype=torch.int64, device=device)
+
+
+def _read_scalars(scal: torch.Tensor, stream, where: str) -> int:
+    _wait(stream, scal.device)
+    v, err = scal.tolist()
+    _check(err & 0xffffffff, where)
+    return v
 
 
 def _cuda_cloud(xyz: torch.Tensor) -> torch.Tensor:
@@ -293,16 +321,24 @@ def downsample(xyz: torch.Tensor, leaf: float, origin: Optional[torch.Tensor] = 
     org = None
     if origin is not None:
         org = torch.as_tensor(origin, dtype=torch.float32, device=xyz.device).reshape(3).contiguous()
-    buf = alloc_buffers(n, xyz.device, point_to_voxel=point_to_voxel,
-                        flags=method_flag(method), origin=org)
-    downsample_into(xyz, leaf, buf, origin_from_min=origin is None, method=method, stream=stream,
-                    cap=n)
-    (stream or torch.cuda.current_stream()).synchronize()
-    err = int(buf.error.item())
-    _check(err, "vg_downsample (device)")
-    v = int(buf.num_voxels.item())
-    return Decimation(buf.keys[:v], buf.centroids[:v], buf.counts[:v], buf.origin,
-                      buf.point_to_voxel[:n] if point_to_voxel else None)
+    dev = xyz.device
+    flags = method_flag(method) | (ORIGIN_FROM_MIN if origin is None else 0)
+    if org is None:
+        org = torch.empty(3, dtype=torch.float32, device=dev)  # (the call writes it)
+    cap = max(n, 1)
+    keys = torch.empty(cap, dtype=torch.int64, device=dev)
+    cents = torch.empty((cap, 3), dtype=torch.float32, device=dev)
+    counts = torch.empty(cap, dtype=torch.int32, device=dev)
+    p2v = torch.empty(cap, dtype=torch.int32, device=dev) if point_to_voxel else None
+    ws = torch.empty(max(workspace_bytes(n, flags), 256), dtype=torch.uint8, device=dev)
+    scal = _scalars(dev)
+    st = lib().vg_downsample(
+        xyz.data_ptr(), n, org.data_ptr(), leaf, keys.data_ptr(), cents.data_ptr(),
+        counts.data_ptr(), n, scal.data_ptr(), None if p2v is None else p2v.data_ptr(),
+        scal.data_ptr() + 8, ws.data_ptr(), ws.numel(), flags, _raw_stream(stream))
+    _check(st, "vg_downsample")
+    v = _read_scalars(scal, stream, "vg_downsample (device)")
+    return Decimation(keys[:v], cents[:v], counts[:v], org, p2v[:n] if point_to_voxel else None)
 
 
 NOALLOC_MAX_POINTS = 1 << 20
@@ -318,23 +354,20 @@ def downsample_noalloc(xyz: torch.Tensor, leaf: float, origin: Optional[torch.Te
     xyz = _cuda_cloud(xyz)
     n = xyz.shape[0]
     dev = xyz.device
-    org = (torch.zeros(3, dtype=torch.float32, device=dev) if origin is None else
+    org = (torch.empty(3, dtype=torch.float32, device=dev) if origin is None else
            torch.as_tensor(origin, dtype=torch.float32, device=dev).reshape(3).contiguous())
     cap = max(n, 1)
     keys = torch.empty(cap, dtype=torch.int64, device=dev)
     cents = torch.empty((cap, 3), dtype=torch.float32, device=dev)
     counts = torch.empty(cap, dtype=torch.int32, device=dev)
-    nv = torch.zeros(1, dtype=torch.int64, device=dev)
-    err = torch.zeros(1, dtype=torch.int32, device=dev)
+    scal = _scalars(dev)
     p2v = torch.empty(cap, dtype=torch.int32, device=dev) if point_to_voxel else None
     flags = method_flag(method) | (ORIGIN_FROM_MIN if origin is None else 0)
     st = lib().vg_downsample_noalloc(
         _ptr(xyz), n, _ptr(org), ctypes.c_float(leaf), _ptr(keys), _ptr(cents), _ptr(counts), n,
-        _ptr(nv), _ptr(p2v), _ptr(err), flags, _stream_ptr(stream))
+        scal.data_ptr(), _ptr(p2v), scal.data_ptr() + 8, flags, _stream_ptr(stream))
     _check(st, "vg_downsample_noalloc")
-    (stream or torch.cuda.current_stream()).synchronize()
-    _check(int(err.item()), "vg_downsample_noalloc (device)")
-    v = int(nv.item())
+    v = _read_scalars(scal, stream, "vg_downsample_noalloc (device)")
     return Decimation(keys[:v], cents[:v], counts[:v], org, p2v[:n] if point_to_voxel else None)
 
 
@@ -367,7 +400,7 @@ def _is_cat_form(frames) -> bool:
             and not (isinstance(frames[1], torch.Tensor) and frames[1].dim() == 2))
 
 
-def _frame_inputs(frames, leaves, origins, device):
+def _frame_clouds(frames, device):
     """Concatenate a list of [N_f,3] clouds (or take (xyz, offsets) as given)."""
     if not _is_cat_form(frames):
         sizes = [int(f.shape[0]) for f in frames]
@@ -379,12 +412,15 @@ def _frame_inputs(frames, leaves, origins, device):
     else:
         xyz, offs = frames
         offs = [int(v) for v in offs]
-    F = len(offs) - 1
-    off_t = torch.tensor(offs, dtype=torch.int64, device=device)
+    return _cuda_cloud(xyz), torch.tensor(offs, dtype=torch.int64, device=device), len(offs) - 1
+
+
+def _frame_inputs(frames, leaves, origins, device):
+    xyz, off_t, F = _frame_clouds(frames, device)
     lv = torch.as_tensor(leaves, dtype=torch.float32).reshape(F).to(device)
-    og = (torch.zeros((F, 3), dtype=torch.float32, device=device) if origins is None else
-          _per_frame(origins, F, 3, device))
-    return _cuda_cloud(xyz), off_t, F, lv, og
+    og = (torch.empty((F, 3), dtype=torch.float32, device=device) if origins is None else
+          _per_frame(origins, F, 3, device))  # (without origins the call writes them)
+    return xyz, off_t, F, lv, og
 
 
 def _per_frame(values, F: int, width: int, device) -> Optional[torch.Tensor]:
@@ -429,8 +465,9 @@ def downsample_frames(frames, leaves, origins=None, *, method="auto", point_to_v
     keys = torch.empty(cap, dtype=torch.int64, device=dev)
     cents = torch.empty((cap, 3), dtype=torch.float32, device=dev)
     counts = torch.empty(cap, dtype=torch.int32, device=dev)
-    out_off = torch.zeros(F + 1, dtype=torch.int64, device=dev)
-    err = torch.zeros(1, dtype=torch.int32, device=dev)
+    # row offsets, then the error word (low half of the last entry): written by the call
+    out_off = torch.empty(F + 2, dtype=torch.int64, device=dev)
+    err = out_off.data_ptr() + 8 * (F + 1)
     p2v = torch.empty(cap, dtype=torch.int32, device=dev) if point_to_voxel else None
     out_at = (torch.empty((cap, at.shape[1]), dtype=torch.float32, device=dev)
               if at is not None else None)
@@ -444,18 +481,18 @@ def downsample_frames(frames, leaves, origins=None, *, method="auto", point_to_v
     if pz is None and zl is None and ex is None:
         st = lib().vg_downsample_frames(
             _ptr(xyz), n, _ptr(off_t), F, _ptr(og), _ptr(lv), _ptr(keys), _ptr(cents),
-            _ptr(counts), n, _ptr(out_off), _ptr(p2v), _ptr(err), _ptr(ws), ws.numel(), flags,
+            _ptr(counts), n, _ptr(out_off), _ptr(p2v), err, _ptr(ws), ws.numel(), flags,
             _stream_ptr(stream))
     else:
         st = lib().vg_downsample_frames_ex(
             _ptr(xyz), n, _ptr(off_t), F, _ptr(pz), _ptr(zl), _ptr(og), _ptr(lv), _ptr(keys),
             _ptr(cents), _ptr(counts), n, _ptr(out_off), _ptr(p2v),
-            ctypes.byref(ex) if ex else None, _ptr(err), _ptr(ws), ws.numel(), flags,
+            ctypes.byref(ex) if ex else None, err, _ptr(ws), ws.numel(), flags,
             _stream_ptr(stream))
     _check(st, "vg_downsample_frames")
-    (stream or torch.cuda.current_stream()).synchronize()
-    _check(int(err.item()), "vg_downsample_frames (device)")
-    offs = out_off.cpu().tolist()
+    _wait(stream, dev)
+    offs = out_off.tolist()
+    _check(offs.pop() & 0xffffffff, "vg_downsample_frames (device)")
     v = offs[-1]
     return Frames(keys[:v], cents[:v], counts[:v], offs, og, p2v[:n] if point_to_voxel else None,
                   None if out_at is None else out_at[:v])
@@ -527,20 +564,18 @@ def thin(xyz: torch.Tensor, cell: float, threshold: int, priority: torch.Tensor,
     org = (torch.zeros(3, dtype=torch.float32, device=dev) if origin is None else
            torch.as_tensor(origin, dtype=torch.float32, device=dev).reshape(3).contiguous())
     keep = torch.zeros(max(n, 1), dtype=torch.uint8, device=dev)
-    kept = torch.zeros(1, dtype=torch.int64, device=dev)
-    err = torch.zeros(1, dtype=torch.int32, device=dev)
+    scal = _scalars(dev)
     ws = torch.empty(max(int(lib().vg_thin_workspace_bytes(n)), 256), dtype=torch.uint8,
                      device=dev)
     passes = ctypes.c_int32(0)
     st = lib().vg_thin(_ptr(xyz), n, _ptr(org), ctypes.c_float(cell),
                        ctypes.c_float(cell if radius is None else radius), int(threshold),
-                       int(batch), _ptr(pr), _ptr(keep), _ptr(kept), ctypes.byref(passes),
-                       _ptr(err), _ptr(ws), ws.numel(), ORIGIN_FROM_MIN if origin is None else 0,
-                       _stream_ptr(stream))
+                       int(batch), _ptr(pr), _ptr(keep), scal.data_ptr(), ctypes.byref(passes),
+                       scal.data_ptr() + 8, _ptr(ws), ws.numel(),
+                       ORIGIN_FROM_MIN if origin is None else 0, _stream_ptr(stream))
     _check(st, "vg_thin")
-    (stream or torch.cuda.current_stream()).synchronize()
-    _check(int(err.item()), "vg_thin (device)")
-    return Thinned(keep[:n].bool(), int(kept.item()), int(passes.value), org)
+    kept = _read_scalars(scal, stream, "vg_thin (device)")
+    return Thinned(keep[:n].bool(), kept, int(passes.value), org)
 
 
 class VoxelMap:
@@ -567,8 +602,7 @@ class VoxelMap:
         (xyz, offsets) tuple; asynchronous."""
         if isinstance(frames, torch.Tensor):
             frames = [frames]
-        xyz, off_t, F, _, _ = _frame_inputs(frames, [self.leaf] * (
-            len(frames) if not _is_cat_form(frames) else len(frames[1]) - 1), None, self.device)
+        xyz, off_t, F = _frame_clouds(frames, self.device)
         pz = _per_frame(poses, F, 12, self.device)
         zl = _per_frame(z_limits, F, 2, self.device)
         self._keep = (xyz, off_t, pz, zl)  # alive until the launch has read them
@@ -584,10 +618,10 @@ class VoxelMap:
         keys = torch.empty(max(cap, 1), dtype=torch.int64, device=d)
         cents = torch.empty((max(cap, 1), 3), dtype=torch.float32, device=d)
         counts = torch.empty(max(cap, 1), dtype=torch.int32, device=d)
-        nv = torch.zeros(1, dtype=torch.int64, device=d)
+        nv = torch.empty(1, dtype=torch.int64, device=d)  # (the call writes it)
         _check(lib().vg_map_extract(self._h, _ptr(keys), _ptr(cents), _ptr(counts), cap, _ptr(nv),
                                     _ptr(self.error), _stream_ptr(stream)), "vg_map_extract")
-        (stream or torch.cuda.current_stream(d)).synchronize()
+        _wait(stream, d)
         _check(int(self.error.item()), "vg_map (device)")
         v = int(nv.item())
         return Decimation(keys[:v], cents[:v], counts[:v],
@@ -715,8 +749,9 @@ def pyramid(xyz: torch.Tensor, leaf: float, levels: int, origin: Optional[torch.
     keys = torch.empty(cap, dtype=torch.int64, device=dev)
     cents = torch.empty((cap, 3), dtype=torch.float32, device=dev)
     counts = torch.empty(cap, dtype=torch.int32, device=dev)
-    loff = torch.zeros(levels + 1, dtype=torch.int64, device=dev)
-    err = torch.zeros(1, dtype=torch.int32, device=dev)
+    # level offsets, then the error word (low half of the last entry): written by the call
+    loff = torch.empty(levels + 2, dtype=torch.int64, device=dev)
+    err = loff.data_ptr() + 8 * (levels + 1)
     p2v = torch.empty(max(n, 1), dtype=torch.int32, device=dev) if point_to_voxel else None
     if method_flag(method) & ~(METHOD_SORT | SORT_BUCKETS | SORT_LSD):  # (auto = 0 passes)
         raise ValueError("vg_pyramid groups level 0 by sorting")
@@ -725,12 +760,12 @@ def pyramid(xyz: torch.Tensor, leaf: float, levels: int, origin: Optional[torch.
     ws = torch.empty(max(int(lib().vg_pyramid_workspace_bytes(n, levels, flags)), 256),
                      dtype=torch.uint8, device=dev)
     st = lib().vg_pyramid(_ptr(xyz), n, _ptr(org), ctypes.c_float(leaf), int(levels), _ptr(keys),
-                          _ptr(cents), _ptr(counts), cap, _ptr(loff), _ptr(p2v), _ptr(err),
+                          _ptr(cents), _ptr(counts), cap, _ptr(loff), _ptr(p2v), err,
                           _ptr(ws), ws.numel(), flags, _stream_ptr(stream))
     _check(st, "vg_pyramid")
-    (stream or torch.cuda.current_stream()).synchronize()
-    _check(int(err.item()), "vg_pyramid (device)")
-    o = loff.cpu().tolist()
+    _wait(stream, dev)
+    o = loff.tolist()
+    _check(o.pop() & 0xffffffff, "vg_pyramid (device)")
     out = []
     for k in range(levels):
         a, b = o[k], o[k + 1]
@@ -747,13 +782,14 @@ def backward(grad_centroids: torch.Tensor, counts: torch.Tensor, point_to_voxel:
     v = g.shape[0]
     n = point_to_voxel.shape[0]
     out = torch.empty((n, 3), dtype=torch.float32, device=g.device)
-    err = torch.zeros(1, dtype=torch.int32, device=g.device)
+    err = torch.empty(1, dtype=torch.int32, device=g.device) if n else \
+        torch.zeros(1, dtype=torch.int32, device=g.device)  # (a call of no points writes nothing)
     st = lib().vg_downsample_backward(_ptr(g), _ptr(counts.contiguous()),
                                       _ptr(point_to_voxel.contiguous()), n, v, _ptr(out), _ptr(err),
                                       _stream_ptr(stream))
     _check(st, "vg_downsample_backward")
     if check:
-        (stream or torch.cuda.current_stream()).synchronize()
+        _wait(stream, g.device)
         _check(int(err.item()), "vg_downsample_backward (device)")
     return out
 
