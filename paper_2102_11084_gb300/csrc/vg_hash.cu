@@ -213,17 +213,18 @@ __global__ __launch_bounds__(kStreamThreads, 3) void hash_insert_kernel(
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       uint32_t ijk[3];
+      float fi[3];
       key[j] = 0;
       n[j] = 0;
       w[j][0] = w[j][1] = w[j][2] = 0;
-      ok[j] = point_index(v[3 * j], v[3 * j + 1], v[3 * j + 2], o, leaf, rleaf, ijk, &range_bad);
+      ok[j] = point_index(v[3 * j], v[3 * j + 1], v[3 * j + 2], o, leaf, rleaf, ijk, fi,
+                          &range_bad);
       if (!ok[j]) continue;
       key[j] = key_compose(static_cast<uint32_t>(f), morton3(ijk[0], ijk[1], ijk[2]), key_shift);
       n[j] = 1;
 #pragma unroll
       for (int a = 0; a < 3; ++a)
-        w[j][a] = uint32_t(quant_offset(v[3 * j + a], voxel_corner(ijk[a], o[a], leaf), inv_unit) -
-                           kQMin);
+        w[j][a] = quant_biased(v[3 * j + a], voxel_corner(fi[a], o[a], leaf), inv_unit);
       ++nvalid;
       kmax = key[j] > kmax ? key[j] : kmax;
       if (j > 0 && ok[j - 1] && key[j - 1] == key[j]) {
@@ -301,7 +302,11 @@ __global__ __launch_bounds__(kStreamThreads) void hash_insert_p2v_kernel(
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       uint64_t local = 0;
-      const bool ok = point_key(v[3 * j], v[3 * j + 1], v[3 * j + 2], o, leaf, rleaf, &local, &range_bad);
+      uint32_t ijk[3];
+      float fi[3];
+      const bool ok = point_index(v[3 * j], v[3 * j + 1], v[3 * j + 2], o, leaf, rleaf, ijk, fi,
+                                  &range_bad);
+      if (ok) local = morton3(ijk[0], ijk[1], ijk[2]);
       const uint64_t key = ok ? key_compose(static_cast<uint32_t>(f), local, key_shift) : 0;
       uint32_t slot = kNoSlot;
       const uint32_t vm = __ballot_sync(kFullMask, ok);

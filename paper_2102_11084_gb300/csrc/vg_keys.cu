@@ -213,7 +213,8 @@ __device__ __forceinline__ void key_loop(const float* __restrict__ xyz, const Fr
         k[j] = ok ? static_cast<KeyT>(k32) : static_cast<KeyT>(kKeySentinel);
       } else {
         uint32_t ijk[3];
-        ok = point_index(v[3 * j], v[3 * j + 1], v[3 * j + 2], o, leaf, rleaf, ijk, &range_bad);
+        float fi[3];
+        ok = point_index(v[3 * j], v[3 * j + 1], v[3 * j + 2], o, leaf, rleaf, ijk, fi, &range_bad);
         k[j] = ok ? key_compose(static_cast<uint32_t>(f), morton3(ijk[0], ijk[1], ijk[2]),
                                 key_shift)
                   : kKeySentinel;

@@ -61,15 +61,16 @@ __device__ __forceinline__ bool narrow_entry(float x, float y, float z, const fl
                                              uint32_t f, uint32_t key_shift, uint32_t* key,
                                              uint64_t* pay, bool* range_bad) {
   uint32_t ijk[3];
-  if (!point_index(x, y, z, o, leaf, rleaf, ijk, range_bad)) return false;
+  float fi[3];
+  if (!point_index(x, y, z, o, leaf, rleaf, ijk, fi, range_bad)) return false;
   // the indices have at most 11 bits: the interleave runs on 32-bit words
   const uint32_t local =
       spread3_32(ijk[0]) | (spread3_32(ijk[1]) << 1) | (spread3_32(ijk[2]) << 2);
   *key = static_cast<uint32_t>(key_compose(f, local, key_shift));
   const float v[3] = {x, y, z};
-  int qq[3];
+  uint32_t qq[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) qq[a] = quant_offset(v[a], voxel_corner(ijk[a], o[a], leaf), inv_unit);
+  for (int a = 0; a < 3; ++a) qq[a] = quant_biased(v[a], voxel_corner(fi[a], o[a], leaf), inv_unit);
   *pay = pack_offsets(qq[0], qq[1], qq[2]);
   return true;
 }

@@ -166,13 +166,14 @@ __device__ __forceinline__ void tr_points(const TrArgs& a, const TrFrames& fm, u
   }
 }
 
-// The sort key of a point of frame f (indices in ijk); false for an invalid point or one out
+// The sort key of a point of frame f (its indices as floats in fi); false for an invalid point or one out
 // of range (*range_bad set).
 __device__ __forceinline__ bool tr_key(const TrFrames& fm, int f, float x, float y, float z,
                                        bool wide, uint32_t key_shift, uint64_t* key,
-                                       uint32_t ijk[3], bool* range_bad) {
+                                       float fi[3], bool* range_bad) {
+  uint32_t ijk[3];
   const float o[3] = {fm.org[3 * f], fm.org[3 * f + 1], fm.org[3 * f + 2]};
-  if (!point_index(x, y, z, o, fm.leaf[f], fm.rleaf[f], ijk, range_bad)) return false;
+  if (!point_index(x, y, z, o, fm.leaf[f], fm.rleaf[f], ijk, fi, range_bad)) return false;
   if (wide)
     *key = key_compose(uint32_t(f), morton3(ijk[0], ijk[1], ijk[2]), key_shift);
   else  // per-frame keys of at most 32 bits
@@ -330,12 +331,10 @@ __device__ __forceinline__ void tr_flush_extent(float mn[3], float mx[3], FrameS
 // Biased corner offsets of a point; sums of N words over the lanes of a run, at its last lane
 // (32 offsets of 21 bits fit 32 bits).
 __device__ __forceinline__ void tr_offsets(const TrFrames& fm, int f, const float q[3],
-                                           const uint32_t ijk[3], uint32_t w[3]) {
+                                           const float fi[3], uint32_t w[3]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c)
-    w[c] = uint32_t(quant_offset(q[c], voxel_corner(ijk[c], fm.org[3 * f + c], fm.leaf[f]),
-                                 fm.inv_unit[f]) -
-                    kQMin);
+    w[c] = quant_biased(q[c], voxel_corner(fi[c], fm.org[3 * f + c], fm.leaf[f]), fm.inv_unit[f]);
 }
 template <int N>
 __device__ __forceinline__ void tr_scan(uint32_t w[N], uint32_t head) {
@@ -538,16 +537,17 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         uint64_t key = 0;
-        uint32_t ijk[3], head, w[3] = {0u, 0u, 0u};
+        uint32_t head, w[3] = {0u, 0u, 0u};
+        float fi[3];
         const bool ok = tr_key(fm, t.f[u], t.q[u][0], t.q[u][1], t.q[u][2], wide, key_shift, &key,
-                               ijk, &range_bad);
+                               fi, &range_bad);
         const uint32_t last = tr_run(key, ok, &head);
         tail[u] = ok && last == lane;
         id[u] = static_cast<uint32_t>(key >> below);  // (at most 28 bits)
         seen[u] = ~0u;
         if (tail[u] && (id[u] >> kTrDigitBits) < lv.ns)
           seen[u] = a.large ? __ldcg(a.root + (id[u] >> 5)) : __ldca(a.root + (id[u] >> 5));
-        if (ok) tr_offsets(fm, t.f[u], t.q[u], ijk, w);
+        if (ok) tr_offsets(fm, t.f[u], t.q[u], fi, w);
         tr_scan<3>(w, head);
         const uint32_t tm = __ballot_sync(kFullMask, tail[u]);
         const uint32_t i = nruns + __popc(tm & ((1u << lane) - 1u));
