@@ -74,15 +74,17 @@ typedef enum {
 #define VG_ORIGIN_FROM_MIN 1 /* compute origin = per-axis min of the valid points and
                                 write it to `origin` (else `origin` is read)            */
 #define VG_METHOD_AUTO 0     /* the library's choice, without a host synchronisation: up
-                                to 2,097,152 points (in all frames, with or without
+                                to 2,621,440 points (in all frames, with or without
                                 point_to_voxel, attributes and poses) an occupancy trie
                                 over the keys, ONE cooperative launch for keys of any
-                                width; the bucket grouping of SORT from 4,194,304 points
-                                on; every digit in global radix passes (VG_SORT_LSD)
-                                between.  The trie needs the workspace of the query; a
-                                smaller one that holds the sort path takes the latter.
-                                One camera frame with 32-bit keys is a little faster
-                                still with VG_SORT_FRAME                                 */
+                                width; above, the trie where the device finds few cells
+                                (or, up to 4,194,304 points, keys that suit it), else the
+                                bucket grouping of SORT from 4,194,304 points on and every
+                                digit in global radix passes (VG_SORT_LSD) below.  The
+                                trie needs the workspace of the query; a smaller one that
+                                holds the sort path takes the latter.  One camera frame
+                                with 32-bit keys is a little faster still with
+                                VG_SORT_FRAME                                            */
 #define VG_METHOD_SORT 16    /* sort the points by key and reduce each run of equal keys.
                                 32-bit keys (no point_to_voxel, no attributes, extents
                                 bound the keys): the top <= 16 key bits are split by one
@@ -418,7 +420,7 @@ VG_API vg_status vg_downsample_backward(const float* grad_centroids, const uint3
  *
  * Arguments are those of vg_downsample minus workspace/workspace_bytes; the caller still
  * passes (and owns) the input cloud and all outputs.  The scratch is a static device
- * array of vg_downsample_noalloc_scratch_bytes() bytes (about 88 MB, AUTO's workspace
+ * array of vg_downsample_noalloc_scratch_bytes() bytes (about 97 MB, AUTO's workspace
  * for VG_NOALLOC_MAX_POINTS points) that every GPU loading the library keeps until the
  * process exits.  The call allocates nothing.
  *   * n > VG_NOALLOC_MAX_POINTS is rejected with VG_ERR_INVALID_ARG before any launch.

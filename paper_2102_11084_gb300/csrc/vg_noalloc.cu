@@ -5,7 +5,7 @@
 // that has no way to hand the library a workspace.
 //
 // The scratch lives in a file-scope __device__ array sized for VG_NOALLOC_MAX_POINTS
-// points (AUTO's workspace for that many points, the occupancy trie's, about 88 MB).  Every
+// points (AUTO's workspace for that many points, the occupancy trie's, about 97 MB).  Every
 // GPU that loads this module keeps the array until the process exits.  Nothing here
 // allocates: the call looks up the array's device address once per device and then runs the
 // ordinary vg_downsample (AUTO and the sort path only) on it.  A cudaDeviceReset unloads the module;

@@ -88,7 +88,7 @@ vg_status vg_plan_create(vg_plan** out, int max_frames, int64_t max_points, int 
   const size_t a = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_SORT | VG_SORT_FRAME);
   const size_t b = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_HASH);
   const size_t small = vg::frames_workspace_bytes(
-      max_points < vg::kTrMaxPoints ? max_points : vg::kTrMaxPoints, max_frames, VG_METHOD_AUTO);
+      max_points < vg::kTrMidPoints ? max_points : vg::kTrMidPoints, max_frames, VG_METHOD_AUTO);
   const size_t large = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_AUTO);
   p->ws_bytes = 0;
   for (const size_t w : {a, b, small, large})

@@ -5,13 +5,13 @@
 // points to get there; the occupied cells alone give the order: the rank of a cell's key
 // among the occupied keys is its row, and the points add their offsets at the row (exact
 // integers, so in any order).  The ranks come from a trie of bitmaps over the keys:
-//   level 1   one bit per prefix of up to 24 key bits (28 for large clouds), grouped in slots
+//   level 1   one bit per prefix of up to 26 key bits (28 for large clouds), grouped in slots
 //             of 2^7 bits;
 //   level j   one slot of 2^7 bits per occupied prefix of level j - 1, numbered by its rank
 //             there, for the next 7 key bits.
 // Each level is marked by a pass over the points, its set bits counted per block and, after a
 // barrier, ranked: a slot's record holds the set bits before the slot and, as bytes, before
-// each of its words.  Keys of up to 24 bits take one level, each 7 bits more another one.
+// each of its words.  Keys of up to 26 bits take one level, each 7 bits more another one.
 // The points are read twice, for the extents and for the first level; that second pass also
 // merges runs of equal keys among a warp's 32 consecutive points (neighbouring pixels of a
 // camera frame often share a cell) and writes each run, 16 bytes, to a dense list of its warp
@@ -388,13 +388,15 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   uint32_t target = 0;
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
 
-  if (a.large) {  // (the same in every block)
+  bool few = true;  // (the same in every block)
+  if (a.large) {
     const unsigned long long smp = a.st->smp;
-    if (kTrSameOf * uint32_t(smp >> 32) < kTrSame * uint32_t(smp)) return;
+    few = kTrSameOf * uint32_t(smp >> 32) >= kTrSame * uint32_t(smp);
+    if (!few && a.fr.n > kTrMidPoints) return;
   }
   // ---- extents; the first level's bits cleared ----
   if (!a.large)
-    for (uint32_t i = gt; i < (1u << (kTrRootBits - 7)); i += gthreads)
+    for (uint32_t i = gt; i < (1u << (kTrRootClear - 7)); i += gthreads)
       reinterpret_cast<uint4*>(a.root)[i] = zero4;
   if (kPosed)
     for (int f = threadIdx.x; f < F; f += kTrThreads) {
@@ -510,6 +512,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     }
     return;
   }
+  if (!few && kb > kTrMidBits && kb <= 32u) return;
   const bool wide = local_bits > 32u;
   // levels, and the key bits below level 1
   const uint32_t root_bits = static_cast<uint32_t>(a.root_bits);
@@ -521,8 +524,10 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   const int64_t cap = a.slots;
   const bool with_attrs = a.out.attrs_in != nullptr;
 
-  if (a.large) {  // the bits of the first level
-    for (uint32_t i = gt; i < lv.ns; i += gthreads)
+  // the bits of the first level not cleared yet
+  const uint32_t clean = a.large ? 0u : 1u << (kTrRootClear - kTrDigitBits);
+  if (lv.ns > clean) {  // (the same in every block)
+    for (uint32_t i = clean + gt; i < lv.ns; i += gthreads)
       reinterpret_cast<uint4*>(a.root)[i] = zero4;
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
   }
@@ -877,7 +882,7 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   const int64_t g = trie_grid(chunks, num_sms());
   a.chunks = static_cast<uint32_t>(chunks);
   a.large = fr.n > kTrMaxPoints ? 1 : 0;
-  a.root_bits = a.large ? kTrRootBitsLarge : kTrRootBits;
+  a.root_bits = trie_root_bits(fr.n);
   if (!a.large) {
     const size_t head = reinterpret_cast<char*>(fs + fr.nframes) - reinterpret_cast<char*>(st);
     trie_clear_kernel<<<1, 1024, 0, stream>>>(reinterpret_cast<uint32_t*>(st),

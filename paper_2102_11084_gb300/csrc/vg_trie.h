@@ -12,19 +12,34 @@ constexpr size_t kTrSlotBytes = kTrWords * 4 + 8;  // bits and record
 constexpr size_t kTrRowBytes = 32;                 // sums, carries and key
 static_assert(kTrWords == 4, "a slot's bits are one 16-byte word, its record three prefixes");
 constexpr int kTrMaxGrid = 1024;    // blocks of the launch at most
-// Bits of the first level (one bit per key prefix): 2 MB up to kTrMaxPoints points, where
-// clearing and ranking more costs as much as another level's three barriers; up to 32 MB
-// above, where another level is another pass over the runs.
-constexpr int kTrRootBits = 24;
+// Bits of the first level at most (one bit per key prefix).  Up to kTrMidPoints points 2^26,
+// 2^24 of which (2 MB) every call of at most kTrMaxPoints clears while the extents are found
+// and the rest, where the keys' width calls for more, with a barrier of its own: less than
+// another level's three barriers and pass over the runs (1M shuffled points of 32-bit keys: 155
+// us with 24 bits and two further levels, 106 with 25 and one).  Above, 32 MB where the keys
+// are that wide.
+constexpr int kTrRootClear = 24;
+constexpr int kTrRootBits = 26;
 constexpr int kTrRootBitsLarge = 28;
-// Up to so many points every call takes the trie.  Above, its accesses miss L2 where the cells
-// are many (a shuffled cloud of 2.5M points: 268 us at 0.02 m, the radix sort 247; 2.0M: 206
-// against 224), so the cells must be few: 2 of 5 sampled pairs of consecutive points share a
-// cell (camera frames at 5 mm to 0.1 m: 2 of 5 come with cells for at most a quarter of the
-// points, 1 of 5 with more than half), and the cells fit a quarter of the points.
-constexpr int64_t kTrMaxPoints = int64_t(1) << 21;
+// Up to kTrMaxPoints points every call takes the trie.  Above, its accesses miss L2 where the
+// cells are many: a shuffled cloud takes 213 to 237 us at 2.5M points (0.05 to 0.02 m), the
+// radix sort 236; at 3.5M 308 to 386 against 293.  So the kernel looks, on the device, and
+// takes the calls
+//   * whose cells are few: 2 of 5 sampled pairs of consecutive points share a cell (camera
+//     frames at 5 mm to 0.1 m: 2 of 5 come with cells for at most a quarter of the points, 1
+//     of 5 with more than half); above kTrMidPoints they must fit a quarter of the points;
+//   * up to kTrMidPoints points, whose keys have at most 27 bits (one level or a nearly empty
+//     second: 4M points of 26-bit keys 210 us, the radix sort 316) or more than 32 (the radix
+//     sort's wide layout: a scan of 4M points 401 us against 450).
+constexpr int64_t kTrMaxPoints = int64_t(5) << 19;
+constexpr int64_t kTrMidPoints = int64_t(1) << 22;
 constexpr int64_t kTrCellShare = 4;
+constexpr uint32_t kTrMidBits = 27;
 constexpr uint32_t kTrSame = 2, kTrSameOf = 5;
+
+constexpr int trie_root_bits(int64_t n) {
+  return n <= kTrMidPoints ? kTrRootBits : kTrRootBitsLarge;
+}
 
 // Blocks of the launch for so many chunks of points: one a chunk, but enough of them to clear
 // and rank the first level, and at most one an SM.
@@ -46,8 +61,8 @@ struct TrieLayout {
 constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base, size_t att_base = 0) {
   TrieLayout L{};
   const int64_t nn = n < 1 ? 1 : n;
-  const int root_bits = nn <= kTrMaxPoints ? kTrRootBits : kTrRootBitsLarge;
-  L.slots = nn <= kTrMaxPoints ? nn : nn / kTrCellShare;
+  const int root_bits = trie_root_bits(nn);
+  L.slots = nn <= kTrMidPoints ? nn : nn / kTrCellShare;
   const size_t places = size_t(max_chunks(nn, frames)) * kChunk;
   size_t off = align_up(base, 256);
   L.root = off;

@@ -30,8 +30,8 @@ SORT_LSD = 4
 USE_GRAPH = 64
 SORT_FRAME = 128
 GRID_SHIFT = 8
-# "auto" (the default): an occupancy trie in one cooperative launch up to 2,097,152 points,
-# "sort" from 4,194,304 points on, else "sort_lsd";
+# "auto" (the default): an occupancy trie in one cooperative launch up to 2,621,440 points and
+# for larger clouds of few cells, else "sort" from 4,194,304 points on and "sort_lsd" below;
 # "sort": 32-bit keys grouped by buckets (partition passes over the top key bits, every
 # bucket reduced on chip), otherwise a global radix sort; "sort_lsd": every key digit in a
 # global radix pass and the segmented reduction; "sort_bucket": the same as "sort" (kept

@@ -1,4 +1,4 @@
-"""The occupancy trie (AUTO up to 2^21 points): keys, counts, order, frame offsets,
+"""The occupancy trie (AUTO): keys, counts, order, frame offsets,
 point_to_voxel and origins equal to the oracle's, and every output bit for bit that of the
 global radix sort ("sort_lsd"), over the forms the route accepts: key widths from one level
 to six, ragged sizes, runs across warps, cells of many points (carries of the packed sums),
@@ -63,10 +63,14 @@ def test_key_widths(bits):
     check(x, 0.015625, np.zeros(3, np.float32))
 
 
-@pytest.mark.parametrize("n", [(1 << 21) - 1, 1 << 21, (1 << 21) + 1, (1 << 22) - 1, 1 << 22])
+@pytest.mark.parametrize("n", [(1 << 21) + 1, 5 << 19, (5 << 19) + 1, (1 << 22) - 1, 1 << 22,
+                               (1 << 22) + 1])
 def test_threshold_of_the_route(n):
+    # shuffled: keys of 26 and 29 bits (either side of what the kernel takes between the
+    # sizes), and of more than 32
     x = cuda(synth.fused_map(n, seed=3, extent=(20.0, 20.0, 5.0)))
-    same(vg.downsample(x, 0.05), vg.downsample(x, 0.05, method="sort_lsd"))
+    for leaf in (0.1, 0.05, 0.008):
+        same(vg.downsample(x, leaf), vg.downsample(x, leaf, method="sort_lsd"))
 
 
 def test_cells_of_many_points():
@@ -142,7 +146,7 @@ def test_large_coherent_and_incoherent_frames(frames, w, h, leaf):
 @pytest.mark.parametrize("p2v", [False, True])
 @pytest.mark.parametrize("origin", [None, (-1.0, -1.0, -1.0)])
 def test_large_cloud_that_the_sample_refuses(p2v, origin):
-    x = cuda(synth.fused_map(2_300_001, seed=5, extent=(20.0, 20.0, 5.0)))
+    x = cuda(synth.fused_map(2_900_001, seed=5, extent=(20.0, 20.0, 5.0)))
     o = None if origin is None else cuda(origin)
     same(vg.downsample(x, 0.02, o, point_to_voxel=p2v),
          vg.downsample(x, 0.02, o, point_to_voxel=p2v, method="sort_lsd"))
