@@ -90,8 +90,9 @@ __device__ __forceinline__ const uint32_t* sorted_idx(const State* st, const uin
 __global__ void thin_setup_kernel(const State* st, const uint32_t* idx0, const uint32_t* idx1,
                                   const float* __restrict__ xyz, const uint32_t* __restrict__ prio,
                                   const int32_t* __restrict__ p2v, uint32_t* cstart, float4* pos,
-                                  uint32_t* sprio, uint32_t* sidx, uint32_t* entry,
-                                  uint8_t* state, const int* err) {
+                                  float* sx, float* sy, float* sz, uint32_t* sprio,
+                                  uint32_t* sidx, uint32_t* entry, uint8_t* state,
+                                  const int* err) {
   if (error_raised(err)) return;  // the grouping failed: point_to_voxel is unwritten
   const int64_t m = st->nitems;
   const uint32_t* I = sorted_idx(st, idx0, idx1);
@@ -101,8 +102,11 @@ __global__ void thin_setup_kernel(const State* st, const uint32_t* idx0, const u
     const int32_t row = p2v[p];
     const int32_t prev = i > 0 ? p2v[I[i - 1]] : -1;
     if (row != prev) cstart[row] = static_cast<uint32_t>(i);
-    pos[i] = make_float4(xyz[3 * size_t(p)], xyz[3 * size_t(p) + 1], xyz[3 * size_t(p) + 2],
-                         __uint_as_float(p));
+    const float x = xyz[3 * size_t(p)], y = xyz[3 * size_t(p) + 1], z = xyz[3 * size_t(p) + 2];
+    pos[i] = make_float4(x, y, z, __uint_as_float(p));
+    sx[i] = x;
+    sy[i] = y;
+    sz[i] = z;
     sprio[i] = prio[p];
     sidx[i] = p;
     entry[p] = static_cast<uint32_t>(i);
@@ -160,14 +164,33 @@ constexpr int kLoopItems = 2;   // list entries a thread tests per step of the b
 constexpr int kLoopSplit = 8;   // warps that share the candidates of one deleted point
 constexpr uint32_t kLoopGroup = 128;  // entries a warp takes at a time (4 a lane)
 
+// Two binary32 operations in one instruction, each with its own rounding.
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long both(float v) {
+  const unsigned long long b = __float_as_uint(v);
+  return b | (b << 32);
+}
+
 // Every entry's neighbours, all of them, and its cell; the groups of kLoopGroup entries that
 // the cells are cut into (their first entries, in any order).  A thread an entry, entries in
-// cell order: the lanes of a warp mostly share a cell, so a candidate's 16-byte load is one
-// broadcast.
+// cell order: the lanes of a warp mostly share a cell, so a candidate's load is a broadcast.
+// Bound by FP32 issue: candidates are tested two to an instruction (dist2's operations, q + (-x)
+// being q - x), four to three 16-byte loads of the coordinates' own arrays, where a candidate a
+// time from 16-byte entries took 705 us of a 640x480 frame (1e9 pairs); 507 us.
 __global__ __launch_bounds__(kFullThreads) void thin_full_count_kernel(
     const State* st, const int32_t* __restrict__ p2v, const uint32_t* __restrict__ cstart,
     const uint32_t* __restrict__ vcnt, const uint32_t* __restrict__ nb,
-    const float4* __restrict__ pos, uint32_t* __restrict__ cnt, uint32_t* __restrict__ ecell,
+    const float4* __restrict__ pos, const float* __restrict__ sx, const float* __restrict__ sy,
+    const float* __restrict__ sz, uint32_t* __restrict__ cnt, uint32_t* __restrict__ ecell,
     uint32_t* __restrict__ group, uint32_t* ctr, float r2, const int* err) {
   if (error_raised(err)) return;
   const int64_t i = blockIdx.x * int64_t(kFullThreads) + threadIdx.x;
@@ -178,21 +201,33 @@ __global__ __launch_bounds__(kFullThreads) void thin_full_count_kernel(
   ecell[i] = cell;
   if ((uint32_t(i) - __ldg(cstart + cell)) % kLoopGroup == 0)
     group[atomicAdd(ctr + kCtrGroups, 1u)] = uint32_t(i);
+  const unsigned long long mx = both(-me.x), my = both(-me.y), mz = both(-me.z);
   uint32_t n = 0;
   for (int o = 0; o < kNb; ++o) {
     const uint32_t c = __ldg(row + o);
     if (c == kNoCell) continue;
-    const uint32_t j0 = __ldg(cstart + c), m = __ldg(vcnt + c);
-    const float4* q = pos + j0;
-    uint32_t j = 0;
-    for (; j + 4 <= m; j += 4) {
-      float4 w[4];
+    uint32_t j = __ldg(cstart + c);
+    const uint32_t end = j + __ldg(vcnt + c);
+    auto one = [&](uint32_t k) {
+      const float4 q = make_float4(__ldg(sx + k), __ldg(sy + k), __ldg(sz + k), 0.0f);
+      n += dist2(q, me.x, me.y, me.z) <= r2;
+    };
+    for (; j < end && (j & 3u) != 0; ++j) one(j);  // up to a 16-byte boundary
+#pragma unroll 2
+    for (; j + 4 <= end; j += 4) {
+      const ulonglong2 x = __ldg(reinterpret_cast<const ulonglong2*>(sx + j));
+      const ulonglong2 y = __ldg(reinterpret_cast<const ulonglong2*>(sy + j));
+      const ulonglong2 z = __ldg(reinterpret_cast<const ulonglong2*>(sz + j));
 #pragma unroll
-      for (int u = 0; u < 4; ++u) w[u] = __ldg(q + j + u);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) n += dist2(w[u], me.x, me.y, me.z) <= r2;
+      for (int h = 0; h < 2; ++h) {
+        const unsigned long long ex = add2(h ? x.y : x.x, mx), ey = add2(h ? y.y : y.x, my),
+                                 ez = add2(h ? z.y : z.x, mz);
+        const unsigned long long d = add2(add2(mul2(ex, ex), mul2(ey, ey)), mul2(ez, ez));
+        n += __uint_as_float(uint32_t(d)) <= r2;
+        n += __uint_as_float(uint32_t(d >> 32)) <= r2;
+      }
     }
-    for (; j < m; ++j) n += dist2(__ldg(q + j), me.x, me.y, me.z) <= r2;
+    for (; j < end; ++j) one(j);
   }
   cnt[i] = n - 1u;  // (the point itself is at distance 0)
 }
@@ -319,64 +354,71 @@ __device__ __forceinline__ void thin_scatter(const LoopArgs& a, uint32_t taken, 
 // Gathered: a warp a group of entries of one cell walks the lists of this pass's deleted
 // entries in the 27 cells around it (lane l the list of cell l) and counts, for the entries
 // still marked (no other count is read again), the ones within r.
-__device__ __forceinline__ void thin_gather(const LoopArgs& a, uint32_t pass, uint32_t groups,
-                                            uint64_t gw, uint64_t gwarps) {
+struct ThinGroup {
+  uint32_t i0;       // first entry
+  uint32_t nb;       // lane l: the l-th cell around, or kNoCell
+  float x[4], y[4], z[4];  // the lane's entries
+  uint32_t n[4];           // and their counts (0 past the cell's end)
+};
+__device__ __forceinline__ void thin_group_load(const LoopArgs& a, uint64_t u, ThinGroup& g) {
   const uint32_t lane = threadIdx.x & 31u;
-  for (uint64_t u = gw; u < groups; u += gwarps) {
-    const uint32_t i0 = __ldg(a.group + u);
-    const uint32_t cell = __ldg(a.ecell + i0);
-    const uint32_t end = __ldg(a.cstart + cell) + __ldg(a.vcnt + cell);
-    uint32_t r = kListEnd;
-    if (lane < uint32_t(kNb)) {
-      const uint32_t c = __ldg(a.nb + size_t(cell) * kNb + lane);
-      if (c != kNoCell) {
-        const unsigned long long h = __ldcg(a.head + c);
-        if (uint32_t(h >> 32) == pass) r = uint32_t(h);
-      }
-    }
-    uint32_t some = __ballot_sync(kFullMask, r != kListEnd);
-    if (!some) continue;
-    float4 w[4];
-    uint32_t n[4], hit[4];
-    bool any = false;
+  g.i0 = __ldg(a.group + u);
+  const uint32_t cell = __ldg(a.ecell + g.i0);
+  const uint32_t end = __ldg(a.cstart + cell) + __ldg(a.vcnt + cell);
+  g.nb = lane < uint32_t(kNb) ? __ldg(a.nb + size_t(cell) * kNb + lane) : kNoCell;
 #pragma unroll
-    for (uint32_t v = 0; v < 4; ++v) {
-      const uint32_t i = i0 + 32u * v + lane;
-      n[v] = i < end ? __ldcg(a.cnt + i) : 0u;
-      w[v] = i < end ? __ldg(a.pos + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      hit[v] = 0;
-      any = any || n[v] > a.thr;
-    }
-    if (!__any_sync(kFullMask, any)) continue;
-    while (some) {
-      float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (r != kListEnd) {
-        q = __ldcg(a.node + r);
-        r = __float_as_uint(q.w);
-      }
-      for (; some; some &= some - 1) {
-        const int l = __ffs(some) - 1;
-        const float x = __shfl_sync(kFullMask, q.x, l), y = __shfl_sync(kFullMask, q.y, l),
-                    z = __shfl_sync(kFullMask, q.z, l);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) hit[v] += dist2(w[v], x, y, z) <= a.r2;
-      }
-      some = __ballot_sync(kFullMask, r != kListEnd);
-    }
-#pragma unroll
-    for (uint32_t v = 0; v < 4; ++v)  // (a marked entry's count covers every neighbour left)
-      if (n[v] > a.thr && hit[v]) a.cnt[i0 + 32u * v + lane] = n[v] - hit[v];
+  for (uint32_t v = 0; v < 4; ++v) {
+    const uint32_t i = g.i0 + 32u * v + lane;
+    g.n[v] = i < end ? __ldcg(a.cnt + i) : 0u;
+    const float4 w = i < end ? __ldg(a.pos + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    g.x[v] = w.x;
+    g.y[v] = w.y;
+    g.z[v] = w.z;
   }
+}
+__device__ __forceinline__ void thin_gather(const LoopArgs& a, uint32_t pass, ThinGroup& g) {
+  const uint32_t lane = threadIdx.x & 31u;
+  if (!__any_sync(kFullMask, g.n[0] > a.thr || g.n[1] > a.thr || g.n[2] > a.thr || g.n[3] > a.thr))
+    return;
+  uint32_t r = kListEnd;
+  if (g.nb != kNoCell) {
+    const unsigned long long h = __ldcg(a.head + g.nb);
+    if (uint32_t(h >> 32) == pass) r = uint32_t(h);
+  }
+  uint32_t hit[4] = {0u, 0u, 0u, 0u};
+  for (uint32_t some; (some = __ballot_sync(kFullMask, r != kListEnd)) != 0u;) {
+    float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (r != kListEnd) {
+      q = __ldcg(a.node + r);
+      r = __float_as_uint(q.w);
+    }
+    for (; some; some &= some - 1) {
+      const int l = __ffs(some) - 1;
+      const float x = __shfl_sync(kFullMask, q.x, l), y = __shfl_sync(kFullMask, q.y, l),
+                  z = __shfl_sync(kFullMask, q.z, l);
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        hit[v] += dist2(make_float4(g.x[v], g.y[v], g.z[v], 0.0f), x, y, z) <= a.r2;
+    }
+  }
+#pragma unroll
+  for (uint32_t v = 0; v < 4; ++v)  // (a marked entry's count covers every neighbour left)
+    if (g.n[v] > a.thr && hit[v]) {
+      g.n[v] -= hit[v];
+      a.cnt[g.i0 + 32u * v + lane] = g.n[v];
+    }
 }
 
 // Every pass of the loop, one cooperative launch (a block an SM), two grid barriers a pass:
 //   1. the batch: every block walks the sorted list from where the last pass stopped, tests
 //      kLoopItems entries a thread, and finds the same `batch` entries still marked (one more
-//      tells that this is not the last pass); block b writes those of rank b mod grid;
-//   2. the counts, by the deleted entries (thin_scatter) or by the marked ones (thin_gather).
+//      tells that this is not the last pass); the block that a list entry belongs to writes it.
+//      The list's next entries are loaded before the barrier;
+//   2. the counts, by the deleted entries (thin_scatter) or by the marked ones (thin_gather: a
+//      warp keeps its first group in registers through all passes).
 // Bound by the latency of the steps and the barriers.  640x480 frame, cell 0.05 m, threshold
 // 20, batches of 1000 (277K points of 3600 candidates each, 2008 cells, 271 passes): a pass
-// takes 23 us scattered (the drain of its 1.8M decrements is 3/4 of it), 13 us gathered,
+// takes 23 us scattered (the drain of its 1.8M decrements is 3/4 of it), 12 us gathered,
 // against 570 us for a fresh count and 500 us of host round trips (recounted).  The gathered
 // form touches every group of entries each pass, 9000 cycles a round of the grid's warps; the
 // scattered form 8000 cycles and one per 90 candidates.
@@ -395,39 +437,51 @@ __global__ __launch_bounds__(kLoopThreads, 1) void thin_loop_kernel(const LoopAr
                       8000.0 + double(a.batch) * a.pairs_per_point / 90.0;
   uint32_t target = 0, first = 0;
   int64_t passes = 0;
+  ThinGroup mine{};  // (no entries: no count is above the threshold)
+  mine.nb = kNoCell;
+  if (gather && gw < groups) thin_group_load(a, gw, mine);
+  uint32_t e[kLoopItems];  // the list entries this thread tests next
+  auto fetch = [&](uint32_t k0) {
+#pragma unroll
+    for (int q = 0; q < kLoopItems; ++q) {
+      const uint32_t k = k0 + kLoopItems * threadIdx.x + q;
+      e[q] = k < m ? __ldg(a.list + k) : kListEnd;
+    }
+  };
+  fetch(0);
   while (passes < a.max_passes) {
     ++passes;
     // 1. the next `batch` marked entries of the list
     uint32_t found = 0;
-    for (uint32_t k0 = first; found <= a.batch && k0 < m; k0 += kLoopItems * kLoopThreads) {
-      uint32_t e[kLoopItems], mine = 0;
-      bool in[kLoopItems];
+    for (uint32_t k0 = first;;) {
+      uint32_t some = 0, cell[kLoopItems];
+      float4 w[kLoopItems];
+      bool in[kLoopItems], own[kLoopItems];
 #pragma unroll
       for (int q = 0; q < kLoopItems; ++q) {
-        const uint32_t k = k0 + kLoopItems * threadIdx.x + q;
-        e[q] = k < m ? __ldg(a.list + k) : 0u;
-        in[q] = k < m;
-      }
-#pragma unroll
-      for (int q = 0; q < kLoopItems; ++q) {
-        in[q] = in[q] && __ldcg(a.cnt + e[q]) > a.thr;
-        mine += in[q];
+        in[q] = e[q] != kListEnd && __ldcg(a.cnt + e[q]) > a.thr;
+        // (its place and cell beside its count: one latency)
+        own[q] = e[q] != kListEnd &&
+                 ((k0 + kLoopItems * threadIdx.x + q) >> 5) % gridDim.x == blockIdx.x;
+        if (gather && own[q]) {
+          cell[q] = __ldg(a.ecell + e[q]);
+          w[q] = __ldg(a.pos + e[q]);
+        }
+        some += in[q];
       }
       uint32_t total;
-      uint32_t r = found + block_excl_scan(mine, &total, tmp);
+      uint32_t r = found + block_excl_scan(some, &total, tmp);
 #pragma unroll
       for (int q = 0; q < kLoopItems; ++q) {
         if (!in[q]) continue;
         if (r < a.batch) {
-          if (r % gridDim.x == blockIdx.x) {
+          if (own[q]) {
             a.dead[e[q]] = 1;
             if (gather) {
-              float4 w = __ldg(a.pos + e[q]);
               const unsigned long long tag = (unsigned long long)uint32_t(passes) << 32;
-              const unsigned long long old =
-                  atomicExch(a.head + __ldg(a.ecell + e[q]), tag | r);
-              w.w = __uint_as_float((old ^ tag) >> 32 == 0 ? uint32_t(old) : kListEnd);
-              a.node[r] = w;
+              const unsigned long long old = atomicExch(a.head + cell[q], tag | r);
+              w[q].w = __uint_as_float((old ^ tag) >> 32 == 0 ? uint32_t(old) : kListEnd);
+              a.node[r] = w[q];
             } else {
               a.sel[r] = e[q];
             }
@@ -437,18 +491,28 @@ __global__ __launch_bounds__(kLoopThreads, 1) void thin_loop_kernel(const LoopAr
         ++r;
       }
       found += total;
-      if (m - k0 <= uint32_t(kLoopItems * kLoopThreads)) break;  // (k0 stays below 2^32)
+      if (found > a.batch || m - k0 <= uint32_t(kLoopItems * kLoopThreads)) break;
+      k0 += kLoopItems * kLoopThreads;  // (stays below m)
+      fetch(k0);
     }
     // (the same in every block) the last pass: every marked point goes, by its count, in
     // the output
     if (found <= a.batch) break;
-    if (!grid_barrier(a.ctr + kCtrBar, target, a.spin_limit, a.err)) return;
+    __syncthreads();
     first = s_next;
+    fetch(first);
+    if (!grid_barrier(a.ctr + kCtrBar, target, a.spin_limit, a.err)) return;
     // 2. the counts
-    if (gather)
-      thin_gather(a, uint32_t(passes), groups, gw, gwarps);
-    else
+    if (gather) {
+      thin_gather(a, uint32_t(passes), mine);
+      for (uint64_t u = gw + gwarps; u < groups; u += gwarps) {
+        ThinGroup more;
+        thin_group_load(a, u, more);
+        thin_gather(a, uint32_t(passes), more);
+      }
+    } else {
       thin_scatter(a, a.batch, gw, gwarps);
+    }
     if (!grid_barrier(a.ctr + kCtrBar, target, a.spin_limit, a.err)) return;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr[kCtrPasses] = static_cast<uint32_t>(passes);
@@ -689,12 +753,16 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
   uint32_t* idx0 = reinterpret_cast<uint32_t*>(ws + S.idx0);
   uint32_t* idx1 = reinterpret_cast<uint32_t*>(ws + S.idx1);
   const int g = grid_for(n);
+  // the entries' coordinates, an array each (16-byte boundaries), in the sort's key buffers
+  float* sx = reinterpret_cast<float*>(ws + S.keys0);
+  float* sy = sx + align_up(size_t(n < 1 ? 1 : n), 4);
+  float* sz = sy + align_up(size_t(n < 1 ? 1 : n), 4);
   unsigned long long pairs = 0;
   if (n > 0) {
     thin_neighbors_kernel<<<num_sms() * 8, 256, 0, stream>>>(
         vnum, vkeys, vcnt, nb, reinterpret_cast<unsigned long long*>(ctr + kCtrPairs), err);
-    thin_setup_kernel<<<g, 256, 0, stream>>>(st, idx0, idx1, xyz, priority, p2v, cstart, pos,
-                                             sprio, sidx, entry, state, err);
+    thin_setup_kernel<<<g, 256, 0, stream>>>(st, idx0, idx1, xyz, priority, p2v, cstart, pos, sx,
+                                             sy, sz, sprio, sidx, entry, state, err);
     e = cudaMemcpyAsync(&pairs, ctr + kCtrPairs, sizeof(pairs), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return VG_ERR_CUDA;
@@ -718,8 +786,8 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
     uint32_t* ecell = sprio;  // (the recounted form's arrays)
     uint32_t* group = sidx;
     thin_full_count_kernel<<<static_cast<int>(ceil_div(n, kFullThreads)), kFullThreads, 0,
-                             stream>>>(st, p2v, cstart, vcnt, nb, pos, cnt, ecell, group, ctr, r2,
-                                       err);
+                             stream>>>(st, p2v, cstart, vcnt, nb, pos, sx, sy, sz, cnt, ecell, group,
+                                       ctr, r2, err);
     thin_prio_kernel<<<g, 256, 0, stream>>>(n, p2v, entry, cnt, priority, thr, keys0, st2, err);
     e = launch_sort(st2, keys0, idx0, keys1, idx1, lb_a, lb_b, n, kNarrowPasses, false,
                     spin_limit(), err, stream);  // (32-bit priorities)
