@@ -13,11 +13,15 @@
 // barrier, ranked: a slot's record holds the set bits before the slot and, as bytes, before
 // each of its words.  Keys of up to 26 bits take one level, each 7 bits more another one.
 // The points are read twice, for the extents and for the first level; that second pass also
-// merges runs of equal keys among a warp's 32 consecutive points (neighbouring pixels of a
-// camera frame often share a cell) and writes each run, 16 bytes, to a dense list of its warp
-// (L2-resident scratch), which every later pass reads instead.  A 1280x720 frame at 0.05 m:
-// 44 us; with every point's run kept in shared memory, undensed, 50 us; computing the keys
-// again in every pass 63 us.
+// merges runs of equal keys among 32 consecutive points (neighbouring pixels of a camera
+// frame often share a cell) and writes each run, 16 bytes, to a dense list of its block
+// (L2-resident scratch), which every later pass reads instead, its lanes evenly filled.  A
+// 1280x720 frame at 0.05 m: 44 us; with every point's run kept in shared memory, undensed, 50
+// us; computing the keys again in every pass 63 us.  A lane takes 2 or 4 consecutive points, so
+// that it merges within itself and the warp's shuffles, ballots and scans run once for 64 or
+// 128 points: 64 frames of 20k to 920k points 905 -> 771 us with 4; calls of at most
+// kTrMaxPoints points, bound by latency and L2, take 2 (one frame's runs are added in 28,900
+// cycles, not 40,000; with 4 a shuffled cloud's first pass took 91,000 cycles, not 79,000).
 //
 // Passes, with a grid barrier after each:
 //   extents   per-frame min and max; the first level's bits cleared;
@@ -48,6 +52,11 @@ namespace vg {
 namespace {
 
 constexpr int kTrAdd = 1;  // runs a lane adds at a time
+// Consecutive points of a lane in the marking pass: calls of up to kTrMaxPoints points, larger
+// ones.
+constexpr int kTrLane = 2, kTrLaneLarge = 4;
+
+static_assert(32ull * 0x1fffffu < (1ull << 26), "a run of 32 points in its fields");
 
 struct TrArgs {
   const float* xyz;
@@ -58,12 +67,13 @@ struct TrArgs {
   uint2* rootrec;
   char* x;             // buffers of the further levels
   char* y;
-  uint4* run;          // a warp's runs: {key, sum x, sum y, sum z | points << 26}
+  uint4* run;          // a block's runs: {key, sum x, sum y, sum z | points << 26}
   uint32_t* runhi;     // the upper key words (keys of more than 32 bits)
   uint2* runatt;       // the runs' attribute sums, 16 bits a channel
   unsigned long long* rowatt;  // the rows', two words a row
   uint32_t* pslot;     // the slot of a run's prefix, then its row
-  uint2* mask;         // per 32 points: lanes that end a run, valid lanes (point_to_voxel)
+  uint2* mask;         // per warp's points of one place in their lanes: ends of runs, valid points
+  uint32_t* first;     // per warp's points: its first run (both for point_to_voxel)
   uint32_t* stat;      // per level (8): the blocks' totals
   SegOut out;
   int64_t slots;       // slots and rows the buffers hold
@@ -79,6 +89,7 @@ struct TrSmem {
   float red[kTrThreads / 32][6];
   uint32_t bits[kTrThreads / 32];
   uint32_t first;
+  uint32_t nruns;
 };
 
 // Tables of a call's frames (dynamic shared memory).
@@ -104,6 +115,19 @@ __device__ __forceinline__ TrFrames tr_frames(unsigned char* mem, int F, bool po
   t.inv_unit = t.rleaf + F;
   t.cstart = reinterpret_cast<uint32_t*>(t.inv_unit + F);
   return t;
+}
+
+__device__ __forceinline__ Pose tr_pose(const TrArgs& a, const TrFrames& fm, int f) {
+  const float4* t = fm.pose + 4 * f;
+  const float4 r0 = t[0], r1 = t[1], r2 = t[2], z = t[3];
+  Pose P;
+  P.r[0] = r0.x, P.r[1] = r0.y, P.r[2] = r0.z, P.r[3] = r0.w;
+  P.r[4] = r1.x, P.r[5] = r1.y, P.r[6] = r1.z, P.r[7] = r1.w;
+  P.r[8] = r2.x, P.r[9] = r2.y, P.r[10] = r2.z, P.r[11] = r2.w;
+  P.zlo = z.x;
+  P.zhi = z.y;
+  P.rigid = a.fr.poses != nullptr;
+  return P;
 }
 
 // U points of a thread (one of each of U chunks): frame, index, whether inside the frame, and
@@ -150,19 +174,94 @@ __device__ __forceinline__ void tr_points(const TrArgs& a, const TrFrames& fm, u
     if (kPosed) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const float4* t = fm.pose + 4 * now.f[u];
-        const float4 r0 = t[0], r1 = t[1], r2 = t[2], z = t[3];
-        Pose P;
-        P.r[0] = r0.x, P.r[1] = r0.y, P.r[2] = r0.z, P.r[3] = r0.w;
-        P.r[4] = r1.x, P.r[5] = r1.y, P.r[6] = r1.z, P.r[7] = r1.w;
-        P.r[8] = r2.x, P.r[9] = r2.y, P.r[10] = r2.z, P.r[11] = r2.w;
-        P.zlo = z.x;
-        P.zhi = z.y;
-        P.rigid = a.fr.poses != nullptr;
+        const Pose P = tr_pose(a, fm, now.f[u]);
         pose_point(P, now.q[u][0], now.q[u][1], now.q[u][2]);
       }
     }
     fn(now);
+  }
+}
+
+// A lane's points in the marking pass: K consecutive ones from p on, m of them in frame f.
+// Chunk k of the block is the cloud's k * grid + blockIdx.x; kChunk / 32K warps take it.
+template <int K>
+struct TrLanePoints {
+  int f, m;
+  int64_t p;
+  float q[K][3];
+};
+template <int K>
+constexpr uint32_t tr_chunk_warps() {
+  return kChunk / (32 * K);
+}
+template <int K>
+__device__ __forceinline__ void tr_lane_load(const TrArgs& a, TrLanePoints<K>& t) {
+  const float* src = a.xyz + 3 * t.p;
+  const uint32_t low = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(src));
+  if (K == 4 && t.m == K && (low & 15u) == 0u) {
+    const float4* v = reinterpret_cast<const float4*>(src);
+#pragma unroll
+    for (int i = 0; i < 3 * K / 4; ++i) {
+      const float4 x = __ldg(v + i);
+      t.q[(4 * i) / 3][(4 * i) % 3] = x.x;
+      t.q[(4 * i + 1) / 3][(4 * i + 1) % 3] = x.y;
+      t.q[(4 * i + 2) / 3][(4 * i + 2) % 3] = x.z;
+      t.q[(4 * i + 3) / 3][(4 * i + 3) % 3] = x.w;
+    }
+  } else if (K == 2 && t.m == K && (low & 7u) == 0u) {
+    const float2* v = reinterpret_cast<const float2*>(src);
+#pragma unroll
+    for (int i = 0; i < 3 * K / 2; ++i) {
+      const float2 x = __ldg(v + i);
+      t.q[(2 * i) / 3][(2 * i) % 3] = x.x;
+      t.q[(2 * i + 1) / 3][(2 * i + 1) % 3] = x.y;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        t.q[j][c] = j < t.m ? __ldg(src + 3 * j + c) : __int_as_float(0x7fc00000);
+  }
+}
+// fn(part, points) for every part of this block's chunks that this warp takes; with kLoad the
+// coordinates too (one step ahead where a lane has few), posed in a posed call.
+template <bool kPosed, int K, bool kLoad, typename Fn>
+__device__ __forceinline__ void tr_lanes(const TrArgs& a, const TrFrames& fm, uint32_t T, Fn fn) {
+  constexpr uint32_t kWarps = tr_chunk_warps<K>();
+  constexpr bool kAhead = kLoad && K <= 2;
+  static_assert(kTrThreads / 32 % kWarps == 0, "whole chunks of points");
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+  const int nf = a.fr.nframes;
+  TrLanePoints<K> next;
+  auto find = [&](uint32_t k) {
+    const uint64_t c = uint64_t(k) * gridDim.x + blockIdx.x;
+    if (c >= T) return false;
+    next.f = nf > 1 ? chunk_frame(fm.cstart, nf, uint32_t(c)) : 0;
+    next.p = fm.off[next.f] + (int64_t(c) - fm.cstart[next.f]) * kChunk +
+             ((warp % kWarps) * 32u + lane) * K;
+    const int64_t left = fm.off[next.f + 1] - next.p;
+    next.m = left < K ? (left < 0 ? 0 : static_cast<int>(left)) : K;
+    if (kAhead) tr_lane_load<K>(a, next);
+    return true;
+  };
+  uint32_t k = warp / kWarps;
+  bool more = find(k);
+  while (more) {
+    TrLanePoints<K> t = next;
+    const uint32_t part = k * kWarps + warp % kWarps;
+    k += kTrThreads / 32 / kWarps;
+    if (kAhead) more = find(k);
+    if (kAhead || __any_sync(kFullMask, t.m != 0)) {
+      if (kLoad && !kAhead) tr_lane_load<K>(a, t);
+      if (kLoad && kPosed) {
+        const Pose P = tr_pose(a, fm, t.f);
+#pragma unroll
+        for (int j = 0; j < K; ++j) pose_point(P, t.q[j][0], t.q[j][1], t.q[j][2]);
+      }
+      fn(part, t);
+    }
+    if (!kAhead) more = find(k);
   }
 }
 
@@ -183,29 +282,52 @@ __device__ __forceinline__ bool tr_key(const TrFrames& fm, int f, float x, float
   return true;
 }
 
-// Last lane of the calling lane's run of equal keys among the valid lanes of the warp; the
-// run's first lane in *head.
-__device__ __forceinline__ uint32_t tr_run(uint64_t key, bool ok, uint32_t* head) {
+// Runs of equal keys in a warp's points, K consecutive ones a lane.  A run ends within its
+// group of 32 points (32 / K lanes), so that its sums fit their fields.
+struct TrRun {
+  uint32_t same;  // bit j: the lane's point j has the key of its point j - 1 (bit 0: of the lane before's last)
+  uint32_t head;  // first lane of the chain of whole lanes that ends in the lane's last point
+  uint32_t tail;  // bit j: point j is valid and ends its run
+};
+constexpr uint64_t kTrNoKey = ~0ull;  // an invalid point's
+template <int K>
+__device__ __forceinline__ TrRun tr_run(const uint64_t key[K]) {
   const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t prev = __shfl_up_sync(kFullMask, key, 1);
-  const uint32_t okm = __ballot_sync(kFullMask, ok);
-  const uint32_t heads =
-      __ballot_sync(kFullMask, lane == 0 || !ok || !((okm >> (lane - 1u)) & 1u) || key != prev);
-  *head = 31u - __clz(heads & (kFullMask >> (31u - lane)));
-  const uint32_t later = lane == 31u ? 0u : heads >> (lane + 1u);
-  return later ? lane + __ffs(later) - 1u : 31u;
+  const uint64_t prev = __shfl_up_sync(kFullMask, key[K - 1], 1);
+  TrRun r;
+  r.same = (lane & (32u / K - 1u)) != 0u && prev == key[0] ? 1u : 0u;
+#pragma unroll
+  for (int j = 1; j < K; ++j) r.same |= key[j] == key[j - 1] ? 1u << j : 0u;
+  const uint32_t heads = __ballot_sync(kFullMask, r.same != (1u << K) - 1u);
+  r.head = 31u - __clz(heads & (kFullMask >> (31u - lane)));
+  const uint32_t links = __ballot_sync(kFullMask, (r.same & 1u) != 0u);
+  const uint32_t next = (r.same >> 1) | (((links >> 1 >> lane) & 1u) << (K - 1));
+  r.tail = 0u;
+#pragma unroll
+  for (int j = 0; j < K; ++j)
+    r.tail |= key[j] != kTrNoKey && !((next >> j) & 1u) ? 1u << j : 0u;
+  return r;
 }
 
-// Sets bit id mod 2^7 of slot id >> 7 for every lane with `emit` that does not see its bit set
-// (`seen`: the word as loaded before; a stale one can only lack bits).  Up to half a warp of
+// Place of the lane's first run among the warp's, in the points' order, from the ballots of the
+// points that end one.
+template <int K>
+__device__ __forceinline__ uint32_t tr_place(const uint32_t tails[K]) {
+  uint32_t i = 0u;
+#pragma unroll
+  for (int j = 0; j < K; ++j) i += __popc(tails[j] & ((1u << (threadIdx.x & 31u)) - 1u));
+  return i;
+}
+
+// Sets the bits `bit` of a word for every lane that has some (those it did not see set in the
+// word as loaded before; a stale one can only lack bits).  Up to half a warp of
 // lanes (a camera frame's runs, which meet a few words) merges them word by word: the
 // atomics of all warps on the few words took 8,500 cycles more of a 640x480 frame.  More
 // lanes (a shuffled cloud's points, a word each) merge the first two words' only: match.any
 // and a redux a group cost a full warp 2,000 cycles.
-__device__ __forceinline__ void tr_set(uint32_t* bits, uint32_t id, bool emit, uint32_t seen) {
+__device__ __forceinline__ void tr_set(uint32_t* bits, uint32_t word, uint32_t bit) {
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t bit = 1u << (id & 31u), word = id >> 5;
-  bool need = emit && (seen & bit) == 0u;
+  bool need = bit != 0u;
   uint32_t m = __ballot_sync(kFullMask, need);
   if (__popc(m) <= 16) {
     if (need) {
@@ -328,24 +450,43 @@ __device__ __forceinline__ void tr_flush_extent(float mn[3], float mx[3], FrameS
   }
 }
 
-// Biased corner offsets of a point; sums of N words over the lanes of a run, at its last lane
-// (32 offsets of 21 bits fit 32 bits).
+// Biased corner offsets of a point, in the form of a run's sums: z carries the number of points
+// above its 26 bits (32 offsets of 21 bits fit them).
 __device__ __forceinline__ void tr_offsets(const TrFrames& fm, int f, const float q[3],
                                            const float fi[3], uint32_t w[3]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c)
     w[c] = quant_biased(q[c], voxel_corner(fi[c], fm.org[3 * f + c], fm.leaf[f]), fm.inv_unit[f]);
+  w[2] |= 1u << 26;
 }
-template <int N>
-__device__ __forceinline__ void tr_scan(uint32_t w[N], uint32_t head) {
+// Sums of N words over a run, at every point that ends one: within the lane, along the chain of
+// whole lanes, and the part before the lane added to its first run.
+template <int K, int N>
+__device__ __forceinline__ void tr_sums(uint32_t w[K][N], const TrRun& r) {
   const uint32_t lane = threadIdx.x & 31u;
 #pragma unroll
-  for (uint32_t d = 1; d < 32; d <<= 1) {
-    if (!__any_sync(kFullMask, lane >= head + d)) break;  // no run is longer
+  for (int j = 1; j < K; ++j)
+#pragma unroll
+    for (int c = 0; c < N; ++c) w[j][c] += (r.same >> j) & 1u ? w[j - 1][c] : 0u;
+#pragma unroll
+  for (uint32_t d = 1; d < 32u / K; d <<= 1) {
+    if (!__any_sync(kFullMask, lane >= r.head + d)) break;  // no chain is longer
 #pragma unroll
     for (int c = 0; c < N; ++c) {
-      const uint32_t y = __shfl_up_sync(kFullMask, w[c], d);
-      if (lane >= head + d) w[c] += y;
+      const uint32_t y = __shfl_up_sync(kFullMask, w[K - 1][c], d);
+      if (lane >= r.head + d) w[K - 1][c] += y;
+    }
+  }
+  if (!__any_sync(kFullMask, (r.same & 1u) != 0u)) return;  // no run crosses lanes
+#pragma unroll
+  for (int c = 0; c < N; ++c) {
+    uint32_t y = __shfl_up_sync(kFullMask, w[K - 1][c], 1);
+    if (!(r.same & 1u)) y = 0u;
+    bool on = true;
+#pragma unroll
+    for (int j = 0; j < K - 1; ++j) {  // (the last point's sum has it already)
+      on = on && (j == 0 || ((r.same >> j) & 1u));
+      w[j][c] += on ? y : 0u;
     }
   }
 }
@@ -367,7 +508,7 @@ struct TrRows {
   uint32_t rows;
 };
 
-template <bool kPosed>
+template <bool kPosed, int K>
 __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   extern __shared__ __align__(16) unsigned char tr_smem[];
   __shared__ TrSmem sm;
@@ -375,19 +516,22 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   const uint32_t gt = blockIdx.x * kTrThreads + threadIdx.x, gthreads = gridDim.x * kTrThreads;
   const int F = a.fr.nframes;
   const TrFrames fm = tr_frames(tr_smem, F, kPosed);
-  // this warp's runs (their number, the same in every lane) and masks
+  // this block's places (for its chunks at most) and runs in them
   const uint32_t cq = a.chunks / gridDim.x, cr = a.chunks % gridDim.x;
-  const uint32_t steps = cq + (blockIdx.x < cr ? 1u : 0u);  // chunks of this block at most
-  const size_t w0 = size_t(blockIdx.x * cq + min(blockIdx.x, cr)) * (kTrThreads / 32) +
-                    size_t(warp) * steps;
-  uint4* run = a.run + w0 * 32;
-  uint32_t* pslot = a.pslot + w0 * 32;
-  uint32_t nruns = 0;
+  const uint32_t places = (cq + (blockIdx.x < cr ? 1u : 0u)) * kChunk;
+  const size_t w0 = size_t(blockIdx.x * cq + min(blockIdx.x, cr)) * kChunk;
+  uint4* run = a.run + w0;
+  uint32_t* runhi = a.runhi + w0;
+  uint2* runatt = a.runatt + w0;
+  uint32_t* pslot = a.pslot + w0;
+  uint2* mask = a.mask + w0 / 32;
+  uint32_t* firsts = a.first + w0 / (32 * K);
   int* err = a.err;
   uint32_t* bar = &a.st->fz_bar;
   uint32_t target = 0;
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
 
+  if (threadIdx.x == 0) sm.nruns = 0u;  // (barriers below come before its first use)
   bool few = true;  // (the same in every block)
   if (a.large) {
     const unsigned long long smp = a.st->smp;
@@ -534,56 +678,87 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
 
   // ---- runs; level 1 marked ----
   bool range_bad = false;
-  {
-    uint32_t s = 0;
-    tr_points<kPosed, 2>(a, fm, T, [&](const TrPoints<2>& t) {
-      uint32_t id[2], seen[2];
-      bool tail[2];
+  tr_lanes<kPosed, K, true>(a, fm, T, [&](uint32_t part, const TrLanePoints<K>& t) {
+    uint64_t key[K];
+    uint32_t w[K][3];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        uint64_t key = 0;
-        uint32_t head, w[3] = {0u, 0u, 0u};
-        float fi[3];
-        const bool ok = tr_key(fm, t.f[u], t.q[u][0], t.q[u][1], t.q[u][2], wide, key_shift, &key,
-                               fi, &range_bad);
-        const uint32_t last = tr_run(key, ok, &head);
-        tail[u] = ok && last == lane;
-        id[u] = static_cast<uint32_t>(key >> below);  // (at most 28 bits)
-        seen[u] = ~0u;
-        if (tail[u] && (id[u] >> kTrDigitBits) < lv.ns)
-          seen[u] = a.large ? __ldcg(a.root + (id[u] >> 5)) : __ldca(a.root + (id[u] >> 5));
-        if (ok) tr_offsets(fm, t.f[u], t.q[u], fi, w);
-        tr_scan<3>(w, head);
-        const uint32_t tm = __ballot_sync(kFullMask, tail[u]);
-        const uint32_t i = nruns + __popc(tm & ((1u << lane) - 1u));
-        if (tail[u]) {
-          run[i] = make_uint4(uint32_t(key), w[0], w[1], w[2] | ((lane - head + 1u) << 26));
-          if (wide || kb > 32u) a.runhi[w0 * 32 + i] = static_cast<uint32_t>(key >> 32);
-        }
-        if (with_attrs) {
-          uint32_t at[2] = {0u, 0u};
-          if (ok) {
-            const uint8_t* b = a.out.attrs_in + size_t(t.p[u]) * a.out.channels;
+    for (int j = 0; j < K; ++j) {
+      float fi[3];
+      key[j] = kTrNoKey;
+      w[j][0] = w[j][1] = w[j][2] = 0u;
+      if (tr_key(fm, t.f, t.q[j][0], t.q[j][1], t.q[j][2], wide, key_shift, &key[j], fi,
+                 &range_bad))
+        tr_offsets(fm, t.f, t.q[j], fi, w[j]);
+    }
+    const TrRun r = tr_run<K>(key);
+    tr_sums<K, 3>(w, r);
+    uint32_t tails[K], total = 0u, base = 0u;
 #pragma unroll
-            for (int c = 0; c < 4; ++c)  // two 16-bit sums a word (32 x 255 fit)
-              if (c < a.out.channels) at[c >> 1] |= uint32_t(__ldg(b + c)) << (16 * (c & 1));
-          }
-          tr_scan<2>(at, head);
-          if (tail[u]) a.runatt[w0 * 32 + i] = make_uint2(at[0], at[1]);
-        }
-        if (a.out.p2v) {
-          const uint32_t vm = __ballot_sync(kFullMask, ok);
-          if (lane == 0 && s < steps) a.mask[w0 + s] = make_uint2(tm, vm);
-        }
-        nruns += __popc(tm);
-        ++s;
+    for (int j = 0; j < K; ++j) {
+      tails[j] = __ballot_sync(kFullMask, (r.tail >> j) & 1u);
+      total += __popc(tails[j]);
+    }
+    if (lane == 0) base = atomicAdd(&sm.nruns, total);
+    base = __shfl_sync(kFullMask, base, 0);
+    const uint32_t place = tr_place<K>(tails);
+    if (a.out.p2v) {
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        const uint32_t valid = __ballot_sync(kFullMask, key[j] != kTrNoKey);
+        if (lane == 0) mask[part * K + j] = make_uint2(tails[j], valid);
       }
+      if (lane == 0) firsts[part] = base;
+    }
+    uint32_t word[K], bit[K], seen[K];
+    uint32_t i = base + place;
 #pragma unroll
-      for (int u = 0; u < 2; ++u) tr_set(a.root, id[u], tail[u], seen[u]);
-    });
-  }
+    for (int j = 0; j < K; ++j) {
+      const bool tail = (r.tail >> j) & 1u;
+      const uint32_t id = static_cast<uint32_t>(key[j] >> below);  // (at most 28 bits)
+      word[j] = id >> 5;
+      bit[j] = seen[j] = 0u;
+      if (tail) {
+        run[i] = make_uint4(uint32_t(key[j]), w[j][0], w[j][1], w[j][2]);
+        if (wide || kb > 32u) runhi[i] = static_cast<uint32_t>(key[j] >> 32);
+        ++i;
+      }
+      if (tail && (id >> kTrDigitBits) < lv.ns) {
+        bit[j] = 1u << (id & 31u);
+        seen[j] = __ldca(a.root + word[j]);
+      }
+    }
+    if (with_attrs) {
+      uint32_t at[K][2];
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        at[j][0] = at[j][1] = 0u;
+        if (key[j] == kTrNoKey) continue;
+        const uint8_t* b = a.out.attrs_in + size_t(t.p + j) * a.out.channels;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)  // two 16-bit sums a word (32 x 255 fit)
+          if (c < a.out.channels) at[j][c >> 1] |= uint32_t(__ldg(b + c)) << (16 * (c & 1));
+      }
+      tr_sums<K, 2>(at, r);
+      uint32_t i = base + place;
+#pragma unroll
+      for (int j = 0; j < K; ++j)
+        if ((r.tail >> j) & 1u) runatt[i++] = make_uint2(at[j][0], at[j][1]);
+    }
+    // the bits not seen set; of two points a lane's in one word together (a scan of 1M points,
+    // whose runs are single points: 10 us less; large calls mostly see them set)
+#pragma unroll
+    for (int j = 0; j < K; ++j) bit[j] &= ~seen[j];
+    if (K == 2 && word[0] == word[K - 1]) {
+      bit[K - 1] |= bit[0];
+      bit[0] = 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+      if (__any_sync(kFullMask, bit[j] != 0u)) tr_set(a.root, word[j], bit[j]);
+  });
   if (__any_sync(kFullMask, range_bad) && lane == 0) set_error(err, kErrRange);
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
+  const uint32_t nruns = min(sm.nruns, places);
 
   // ---- every level ranked, the next one marked ----
   uint32_t rows = 0;
@@ -607,20 +782,20 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     for (uint32_t i = gt; i < n1; i += gthreads) reinterpret_cast<uint4*>(nbits)[i] = zero4;
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
     const uint32_t sh = below - uint32_t(j) * kTrDigitBits;  // key bits below the next level
-    for (uint32_t i0 = 0; i0 < nruns; i0 += 64) {
+    for (uint32_t i0 = 0; i0 < nruns; i0 += 2 * kTrThreads) {
       uint32_t id[2], seen[2], v[2];
       uint2 r[2];
       bool in[2];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const uint32_t i = i0 + 32u * u + lane;
+        const uint32_t i = i0 + kTrThreads * u + threadIdx.x;
         in[u] = i < nruns;
         id[u] = 0u;
         v[u] = 0u;
         r[u] = make_uint2(~0u, 0u);
         if (!in[u]) continue;
         uint64_t key = run[i].x;
-        if (kb > 32u) key |= uint64_t(a.runhi[w0 * 32 + i]) << 32;
+        if (kb > 32u) key |= uint64_t(runhi[i]) << 32;
         id[u] = static_cast<uint32_t>(key >> sh) & ((kTrDigit << kTrDigitBits) | kTrDigit);  // two digits
         const uint32_t s0 =
             j == 1 ? static_cast<uint32_t>(key >> (sh + 2 * kTrDigitBits)) : pslot[i];
@@ -634,7 +809,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
         seen[u] = 0u;
         if (!in[u]) continue;
         const uint32_t s = r[u].x == ~0u ? ~0u : tr_rank(r[u], v[u], id[u] >> kTrDigitBits);
-        pslot[i0 + 32u * u + lane] = s;
+        pslot[i0 + kTrThreads * u + threadIdx.x] = s;
         if (s >= n1) {
           set_error(err, kErrInvalidArg);
           in[u] = false;
@@ -644,7 +819,8 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
         seen[u] = __ldcg(nbits + (id[u] >> 5));
       }
 #pragma unroll
-      for (int u = 0; u < 2; ++u) tr_set(nbits, id[u], in[u], seen[u]);
+      for (int u = 0; u < 2; ++u)
+        tr_set(nbits, id[u] >> 5, in[u] ? (1u << (id[u] & 31u)) & ~seen[u] : 0u);
     }
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
     lv = TrLevel{nbits, reinterpret_cast<uint2*>(nb + size_t(cap) * (kTrWords * 4)), n1};
@@ -685,14 +861,14 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
 
   // ---- every run's points and sums at its row ----
-  for (uint32_t i0 = 0; i0 < nruns; i0 += 32u * kTrAdd) {
+  for (uint32_t i0 = 0; i0 < nruns; i0 += kTrThreads * kTrAdd) {
     uint4 e[kTrAdd];
     uint2 r[kTrAdd];
     uint32_t v[kTrAdd], row[kTrAdd];
     unsigned long long oa[kTrAdd], ob[kTrAdd], va[kTrAdd], vb[kTrAdd];
 #pragma unroll
     for (int u = 0; u < kTrAdd; ++u) {
-      const uint32_t i = i0 + 32u * u + lane;
+      const uint32_t i = i0 + kTrThreads * u + threadIdx.x;
       v[u] = 0u;
       r[u] = make_uint2(~0u, 0u);
       e[u] = zero4;
@@ -706,7 +882,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     }
 #pragma unroll
     for (int u = 0; u < kTrAdd; ++u) {
-      const uint32_t i = i0 + 32u * u + lane;
+      const uint32_t i = i0 + kTrThreads * u + threadIdx.x;
       row[u] = ~0u;
       oa[u] = ob[u] = va[u] = vb[u] = 0ull;
       if (i >= nruns) continue;
@@ -716,14 +892,14 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
         row[u] = ~0u;
       } else {
         uint64_t key = e[u].x;
-        if (kb > 32u) key |= uint64_t(a.runhi[w0 * 32 + i]) << 32;
+        if (kb > 32u) key |= uint64_t(runhi[i]) << 32;
         R.key[row[u]] = key;  // (every run of the row stores the same key)
         va[u] = e[u].y | ((unsigned long long)e[u].z << 32);
         vb[u] = (e[u].w & 0x3ffffffu) | ((unsigned long long)(e[u].w >> 26) << 32);
         oa[u] = atomicAdd(R.A + row[u], va[u]);
         ob[u] = atomicAdd(R.B + row[u], vb[u]);
         if (with_attrs) {
-          const uint2 t = a.runatt[w0 * 32 + i];
+          const uint2 t = runatt[i];
           atomicAdd(R.att + row[u],
                     (unsigned long long)(t.x & 0xffffu) | ((unsigned long long)(t.x >> 16) << 32));
           if (a.out.channels > 2)
@@ -743,20 +919,41 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
       if (cx | cy | cz) atomicAdd(R.C + row[u], cx | (cy << 21) | (cz << 42));
     }
   }
-  if (a.out.p2v) {  // a point's row is its run's
-    __syncwarp();
-    uint32_t first = 0;
-    for (uint32_t s = 0; s < steps; ++s) {
-      const uint64_t c = uint64_t(s) * gridDim.x + blockIdx.x;
-      if (c >= T) break;
-      const int f = F > 1 ? chunk_frame(fm.cstart, F, uint32_t(c)) : 0;
-      const int64_t p = fm.off[f] + (int64_t(c) - fm.cstart[f]) * kChunk + threadIdx.x;
-      const uint2 m = a.mask[w0 + s];
-      uint32_t q = ~0u;
-      if ((m.y >> lane) & 1u) q = pslot[first + __popc(m.x & ((1u << lane) - 1u))];
-      if (p < fm.off[f + 1]) a.out.p2v[p] = static_cast<int32_t>(q);
-      first += __popc(m.x);
-    }
+  if (a.out.p2v) {  // a point's row is its run's: that of the next point to end one
+    __syncthreads();
+    tr_lanes<kPosed, K, false>(a, fm, T, [&](uint32_t part, const TrLanePoints<K>& t) {
+      uint32_t row[K], tails[K], m = 0u, valid = 0u, first = ~0u;
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        const uint2 b = mask[part * K + j];
+        tails[j] = b.x;
+        m |= ((b.x >> lane) & 1u) << j;
+        valid |= ((b.y >> lane) & 1u) << j;
+      }
+      const uint32_t place = firsts[part] + tr_place<K>(tails);
+#pragma unroll
+      for (int j = K - 1; j >= 0; --j) {
+        row[j] = ~0u;
+        if (!((m >> j) & 1u)) continue;
+        const uint32_t i = place + __popc(m & ((1u << j) - 1u));
+        first = row[j] = i < nruns ? pslot[i] : ~0u;
+      }
+      const uint32_t later = (__ballot_sync(kFullMask, m != 0u) >> 1) >> lane;
+      uint32_t cur = __shfl_sync(kFullMask, first, later ? int(lane) + __ffs(later) : int(lane));
+#pragma unroll
+      for (int j = K - 1; j >= 0; --j) {
+        if ((m >> j) & 1u) cur = row[j];
+        row[j] = (valid >> j) & 1u ? cur : ~0u;
+      }
+      int32_t* dst = a.out.p2v + t.p;
+      if (K == 4 && t.m == K && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0u) {
+        *reinterpret_cast<uint4*>(dst) = make_uint4(row[0], row[1 % K], row[2 % K], row[3 % K]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+          if (j < t.m) dst[j] = static_cast<int32_t>(row[j]);
+      }
+    });
   }
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
 
@@ -826,14 +1023,18 @@ constexpr size_t kTrSmem = tr_frames_bytes(kMaxFrames, true);
 static_assert(kTrSmem + sizeof(TrSmem) <= 227 * 1024, "block shared memory");
 
 // Blocks an SM holds of the kernel (0: it cannot run there), per device.
-int trie_blocks_per_sm(bool posed) {
-  static int cache[64][2];
+using TrKernel = void (*)(const TrArgs);
+TrKernel trie_kernel_of(bool posed, bool large) {
+  if (posed) return large ? trie_kernel<true, kTrLaneLarge> : trie_kernel<true, kTrLane>;
+  return large ? trie_kernel<false, kTrLaneLarge> : trie_kernel<false, kTrLane>;
+}
+int trie_blocks_per_sm(bool posed, bool large) {
+  static int cache[64][2][2];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  int& b = cache[dev][posed ? 1 : 0];
+  int& b = cache[dev][posed ? 1 : 0][large ? 1 : 0];
   if (b == 0) {
-    const void* fn = posed ? reinterpret_cast<const void*>(trie_kernel<true>)
-                           : reinterpret_cast<const void*>(trie_kernel<false>);
+    const void* fn = reinterpret_cast<const void*>(trie_kernel_of(posed, large));
     int v = 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kTrSmem)) != cudaSuccess ||
@@ -847,11 +1048,12 @@ int trie_blocks_per_sm(bool posed) {
 
 }  // namespace
 
-bool trie_available(bool posed) { return trie_blocks_per_sm(posed) > 0; }
+bool trie_available(bool posed) {
+  return trie_blocks_per_sm(posed, false) > 0 && trie_blocks_per_sm(posed, true) > 0;
+}
 
 void warm_trie_config() {
-  (void)trie_blocks_per_sm(false);
-  (void)trie_blocks_per_sm(true);
+  for (int i = 0; i < 4; ++i) (void)trie_blocks_per_sm((i & 1) != 0, (i & 2) != 0);
 }
 
 cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameState* fs, char* ws,
@@ -872,6 +1074,7 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   a.rowatt = reinterpret_cast<unsigned long long*>(ws + L.rowatt);
   a.pslot = reinterpret_cast<uint32_t*>(ws + L.pslot);
   a.mask = reinterpret_cast<uint2*>(ws + L.mask);
+  a.first = reinterpret_cast<uint32_t*>(ws + L.first);
   a.stat = reinterpret_cast<uint32_t*>(ws + L.stat);
   a.out = out;
   a.slots = L.slots;
@@ -889,8 +1092,7 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
                                              static_cast<uint32_t>(head / sizeof(uint32_t)), err);
   }
   void* args[] = {&a};
-  const void* fn = posed(fr) ? reinterpret_cast<const void*>(trie_kernel<true>)
-                             : reinterpret_cast<const void*>(trie_kernel<false>);
+  const void* fn = reinterpret_cast<const void*>(trie_kernel_of(posed(fr), a.large != 0));
   return cudaLaunchCooperativeKernel(fn, dim3(static_cast<unsigned>(g)), dim3(kTrThreads), args,
                                      
                                      tr_frames_bytes(fr.nframes, posed(fr)), stream);

@@ -51,10 +51,10 @@ constexpr int64_t trie_grid(int64_t chunks, int sms) {
 
 // Scratch, from `base` on: the first level's bits and records, two buffers of slots (16 B of
 // bits and an 8 B record each; the second one holds the rows' sums and keys once the rows are
-// known), the runs of every warp (each warp's list has a place for every point it may read),
+// known), the runs of every block (each block's list has a place for every point it may read),
 // the blocks' totals; with attributes, from `att_base` on, the runs' and the rows' sums.
 struct TrieLayout {
-  size_t root, rootrec, x, y, run, runhi, pslot, mask, stat, total;
+  size_t root, rootrec, x, y, run, runhi, pslot, mask, first, stat, total;
   size_t runatt, rowatt, att_total;
   int64_t slots;  // slots (and rows) the buffers hold
 };
@@ -80,7 +80,9 @@ constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base, size_t att_
   L.pslot = off;
   off = align_up(off + places * 4, 256);
   L.mask = off;
-  off = align_up(off + places / 32 * 8, 256);
+  off = align_up(off + places / 4, 256);
+  L.first = off;
+  off = align_up(off + places / 32 * 4, 256);
   L.stat = off;
   off = align_up(off + 8 * size_t(kTrMaxGrid) * sizeof(uint32_t), 256);
   L.total = off;
