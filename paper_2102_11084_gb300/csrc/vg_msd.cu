@@ -725,7 +725,7 @@ constexpr int kSlotMax = 256;  // keys of an oversized window (one coarse range)
 // its cells has more; their further entries go into one 64-bit sum per axis.
 constexpr uint32_t kSumSplit = 2048;
 static_assert(kBkStage % kBkThreads == 0, "bucket stage");
-static_assert(kBkWords % kBkThreads == 0, "bucket bitmap");
+static_assert(kBkPer == 4 && kBkWords % kBkThreads == 0, "a thread's words are one 16-byte load");
 static_assert(kBkStage < 2 * int(kSumSplit), "at most one cell per job above the 32-bit sums");
 static_assert(uint64_t(kSumSplit) * 0x1fffffu <= 0xffffffffull, "32-bit sums");
 static_assert(kBkStage < 65536, "16-bit ranks and key offsets");
@@ -754,6 +754,8 @@ static_assert(offsetof(BkSmem, pay) % 16 == 0 && (8 * (kBkStage + 2)) % 16 == 0,
               "payload stage buffer on a 16-byte boundary");
 static_assert(offsetof(BkSmem, sum) % 8 == 0, "oversized windows sum in 64 bits there");
 static_assert(offsetof(BkSmem, bar) % 8 == 0, "mbarrier alignment");
+static_assert(offsetof(BkSmem, bits) % 16 == 0 && offsetof(BkSmem, rank) % 8 == 0,
+              "a thread's bitmap words and ranks are one access each");
 static_assert(offsetof(BkSmem, job) % 16 == 0 && offsetof(BkSmem, ahd) % 16 == 0 &&
                   sizeof(Job) == 32,
               "descriptors copied in 16-byte pieces");
@@ -892,6 +894,11 @@ __device__ __forceinline__ void slot_window(BkSmem& sm, const Bufs& bf, const Jo
 //      per-axis sums (shared-memory atomics; integers, so the order does not matter);
 //   4. one thread per cell writes its row and clears its counter and sums.
 // Four barriers a job; counters, sums and bitmaps are left clean for the next one.
+// Bound by shared-memory wavefronts (64 % of their rate) and issue (54 %).  A job's bitmap is 2048
+// words where its bucket spans 2^16 keys, whatever its entries (some 500 of a 14M-point map at
+// 0.02 m), so a thread reads, ranks and clears its four words with one access each, where
+// scalar ones took four wavefronts for one: 50M points 580 -> 532 us, the 14M map 331 -> 287.
+// Storing a cell's first entry and adding only the others (no clearing, a barrier more): 581.
 __global__ __launch_bounds__(kBkThreads, VG_BK_MINB) void msd_bucket_kernel(
     State* st, const FrameState* __restrict__ fs, const uint32_t* k0, const uint64_t* p0,
     const uint32_t* k1, const uint64_t* p1, const uint32_t* __restrict__ jobsw,
@@ -989,13 +996,11 @@ __global__ __launch_bounds__(kBkThreads, VG_BK_MINB) void msd_bucket_kernel(
       if (nxt_copy) issue_keys(sm, bf, nxt);
 
       // 2. cells before every word (exclusive prefix of the popcounts) and the cell count
-      uint32_t pc[kBkPer], mine = 0;
-#pragma unroll
-      for (int q2 = 0; q2 < kBkPer; ++q2) {
-        const int w = kBkPer * t + q2;
-        pc[q2] = w < nw ? __popc(bits[w]) : 0u;
-        mine += pc[q2];
-      }
+      const bool any = kBkPer * t < nw;
+      uint4 bw = make_uint4(0u, 0u, 0u, 0u);
+      if (any) bw = reinterpret_cast<const uint4*>(bits)[t];  // (words past nw are zero)
+      const uint32_t p1 = __popc(bw.x), p2 = p1 + __popc(bw.y), p3 = p2 + __popc(bw.z);
+      const uint32_t mine = p3 + __popc(bw.w);
       uint32_t inc = mine;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
@@ -1004,21 +1009,12 @@ __global__ __launch_bounds__(kBkThreads, VG_BK_MINB) void msd_bucket_kernel(
       }
       if (lane == 31) sm.tmp[warp] = inc;
       __syncthreads();
-      uint32_t wt = lane < kBkWarps ? sm.tmp[lane] : 0u;
-#pragma unroll
-      for (int off = 1; off < kBkWarps; off <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, wt, off);
-        if (lane >= off) wt += y;
-      }
-      const uint32_t V = __shfl_sync(kFull, wt, kBkWarps - 1);
-      const uint32_t wex = __shfl_sync(kFull, wt, (warp + 31) & 31);
-      uint32_t run = (warp ? wex : 0u) + inc - mine;
-#pragma unroll
-      for (int q2 = 0; q2 < kBkPer; ++q2) {
-        const int w = kBkPer * t + q2;
-        if (w < nw) sm.rank[w] = static_cast<uint16_t>(run);
-        run += pc[q2];
-      }
+      const uint32_t wt = lane < kBkWarps ? sm.tmp[lane] : 0u;
+      const uint32_t V = __reduce_add_sync(kFull, wt);
+      const uint32_t run = __reduce_add_sync(kFull, lane < warp ? wt : 0u) + inc - mine;
+      if (any)
+        reinterpret_cast<uint2*>(sm.rank)[t] =
+            make_uint2(run | ((run + p1) << 16), (run + p2) | ((run + p3) << 16));
       __syncthreads();
 
       // 3. the payloads, into their cells' counters and sums
@@ -1091,11 +1087,7 @@ __global__ __launch_bounds__(kBkThreads, VG_BK_MINB) void msd_bucket_kernel(
         }
         put_row32(rc, out, row0 + r, d.key_lo + sm.vkey[r], n, sf, s64, err);
       }
-#pragma unroll
-      for (int q2 = 0; q2 < kBkPer; ++q2) {
-        const int w = kBkPer * t + q2;
-        if (w < nw) bits[w] = 0;
-      }
+      if (any) reinterpret_cast<uint4*>(bits)[t] = make_uint4(0u, 0u, 0u, 0u);
       jb ^= 1;
     }
     if (t == 0) {  // slot s takes the job after the next; every thread has read this one
