@@ -8,9 +8,9 @@
 // points -- are then radix-sorted into key order.  Same key, same accumulator and same
 // centroid formula as the sort path, so both paths give identical bits.
 //
-//   hash_insert_kernel   key per point; runs of equal keys among a thread's four consecutive
-//                        points merged and queued by warp; 32 queued runs at a time claim or
-//                        find their slots and add to them
+//   hash_insert_kernel   key per point; runs of equal keys within 32 consecutive points (eight
+//                        threads' four) merged and queued by warp; 32 queued runs at a time
+//                        claim or find their slots and add to them
 //   hash_insert_p2v_kernel  the same for calls that want point_to_voxel: points of a warp with
 //                        equal keys are merged (match.any) and their leader claims/updates one
 //                        slot, which every point of the group records
@@ -25,8 +25,8 @@
 // LOCKED wait (bounded) and then add with atomics after an acquire load of the key.
 //
 // The insert is bound by instruction issue (keys, offsets) and by L2's atomics: 64 posed
-// frames (29M points) 511 us; merging by match.any lane group by lane group with four
-// atomics a group took 954.
+// frames (29M points) 417 us; runs within a thread's four points only, 475; merging by
+// match.any lane group by lane group with four atomics a group, 954.
 #include "vg_device.cuh"
 #include "vg_internal.h"
 #include "vg_stream.cuh"
@@ -151,7 +151,7 @@ constexpr int kQueue = 160;
 struct InsertQueue {
   unsigned long long key[kQueue];
   unsigned long long xy[kQueue];  // sum x | sum y << 32
-  uint32_t zn[kQueue];            // sum z | points << 28
+  uint32_t zn[kQueue];            // sum z | points << 26
 };
 constexpr size_t kInsertSmem = (kStreamThreads / 32) * sizeof(InsertQueue);
 
@@ -206,42 +206,36 @@ __global__ __launch_bounds__(kStreamThreads, 3) void hash_insert_kernel(
     const float leaf = sm.leaf[f];
     const float rleaf = sm.rleaf[f];
     const float inv_unit = sm.inv_unit[f];
-    // a thread's points and their runs: key, and the sums of a run up to each point
+    // a thread's points and their runs (z carries the points above its 26 bits)
     uint64_t key[4];
-    uint32_t w[4][3], n[4];
-    bool ok[4];
+    uint32_t w[4][3];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       uint32_t ijk[3];
       float fi[3];
-      key[j] = 0;
-      n[j] = 0;
+      key[j] = kNoKey;
       w[j][0] = w[j][1] = w[j][2] = 0;
-      ok[j] = point_index(v[3 * j], v[3 * j + 1], v[3 * j + 2], o, leaf, rleaf, ijk, fi,
-                          &range_bad);
-      if (!ok[j]) continue;
+      if (!point_index(v[3 * j], v[3 * j + 1], v[3 * j + 2], o, leaf, rleaf, ijk, fi, &range_bad))
+        continue;
       key[j] = key_compose(static_cast<uint32_t>(f), morton3(ijk[0], ijk[1], ijk[2]), key_shift);
-      n[j] = 1;
 #pragma unroll
       for (int a = 0; a < 3; ++a)
         w[j][a] = quant_biased(v[3 * j + a], voxel_corner(fi[a], o[a], leaf), inv_unit);
+      w[j][2] |= 1u << 26;
       ++nvalid;
       kmax = key[j] > kmax ? key[j] : kmax;
-      if (j > 0 && ok[j - 1] && key[j - 1] == key[j]) {
-        n[j] += n[j - 1];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) w[j][a] += w[j - 1][a];
-      }
     }
+    const LaneRuns r = lane_runs<4>(key);
+    run_sums<4, 3>(w, r);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const bool end = ok[j] && (j == 3 || !ok[j + 1] || key[j + 1] != key[j]);
+      const bool end = (r.tail >> j) & 1u;
       const uint32_t m = __ballot_sync(kFullMask, end);
       if (end) {
         const uint32_t i = qn + __popc(m & ((1u << lane) - 1u));
         q.key[i] = key[j];
         q.xy[i] = w[j][0] | ((unsigned long long)w[j][1] << 32);
-        q.zn[i] = w[j][2] | (n[j] << 28);  // (four offsets of 21 bits)
+        q.zn[i] = w[j][2];
       }
       qn += __popc(m);
     }
@@ -253,7 +247,7 @@ __global__ __launch_bounds__(kStreamThreads, 3) void hash_insert_kernel(
       if (uint32_t(lane) < take) {
         const uint32_t b = q.zn[qn + lane];
         (void)table_add(tab, q.key[qn + lane], q.xy[qn + lane],
-                        (b & 0xfffffffu) | ((unsigned long long)(b >> 28) << 32), spin_limit, err);
+                        (b & 0x3ffffffu) | ((unsigned long long)(b >> 26) << 32), spin_limit, err);
       }
     }
     __syncwarp();

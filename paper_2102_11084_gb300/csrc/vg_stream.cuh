@@ -207,4 +207,65 @@ __device__ __forceinline__ uint32_t frame_prologue(const FramesArg& fr, bool hav
   return key_shift;
 }
 
+// ---- runs of equal keys in consecutive points ----------------------------------------------
+// Runs of equal keys in a warp's points, K consecutive ones a lane.  A run ends within its
+// group of 32 points (32 / K lanes), so that its sums fit their fields (26 bits an offset).
+struct LaneRuns {
+  uint32_t same;  // bit j: the lane's point j has the key of its point j - 1 (bit 0: of the lane before's last)
+  uint32_t head;  // first lane of the chain of whole lanes that ends in the lane's last point
+  uint32_t tail;  // bit j: point j is valid and ends its run
+};
+constexpr uint64_t kNoKey = ~0ull;  // an invalid point's
+static_assert(32ull * 0x1fffffu < (1ull << 26), "a run of 32 points in its fields");
+template <int K>
+__device__ __forceinline__ LaneRuns lane_runs(const uint64_t key[K]) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t prev = __shfl_up_sync(kFullMask, key[K - 1], 1);
+  LaneRuns r;
+  r.same = (lane & (32u / K - 1u)) != 0u && prev == key[0] ? 1u : 0u;
+#pragma unroll
+  for (int j = 1; j < K; ++j) r.same |= key[j] == key[j - 1] ? 1u << j : 0u;
+  const uint32_t heads = __ballot_sync(kFullMask, r.same != (1u << K) - 1u);
+  r.head = 31u - __clz(heads & (kFullMask >> (31u - lane)));
+  const uint32_t links = __ballot_sync(kFullMask, (r.same & 1u) != 0u);
+  const uint32_t next = (r.same >> 1) | (((links >> 1 >> lane) & 1u) << (K - 1));
+  r.tail = 0u;
+#pragma unroll
+  for (int j = 0; j < K; ++j)
+    r.tail |= key[j] != kNoKey && !((next >> j) & 1u) ? 1u << j : 0u;
+  return r;
+}
+
+// Sums of N words over a run, at every point that ends one: within the lane, along the chain of
+// whole lanes, and the part before the lane added to its first run.
+template <int K, int N>
+__device__ __forceinline__ void run_sums(uint32_t w[K][N], const LaneRuns& r) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+  for (int j = 1; j < K; ++j)
+#pragma unroll
+    for (int c = 0; c < N; ++c) w[j][c] += (r.same >> j) & 1u ? w[j - 1][c] : 0u;
+#pragma unroll
+  for (uint32_t d = 1; d < 32u / K; d <<= 1) {
+    if (!__any_sync(kFullMask, lane >= r.head + d)) break;  // no chain is longer
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      const uint32_t y = __shfl_up_sync(kFullMask, w[K - 1][c], d);
+      if (lane >= r.head + d) w[K - 1][c] += y;
+    }
+  }
+  if (!__any_sync(kFullMask, (r.same & 1u) != 0u)) return;  // no run crosses lanes
+#pragma unroll
+  for (int c = 0; c < N; ++c) {
+    uint32_t y = __shfl_up_sync(kFullMask, w[K - 1][c], 1);
+    if (!(r.same & 1u)) y = 0u;
+    bool on = true;
+#pragma unroll
+    for (int j = 0; j < K - 1; ++j) {  // (the last point's sum has it already)
+      on = on && (j == 0 || ((r.same >> j) & 1u));
+      w[j][c] += on ? y : 0u;
+    }
+  }
+}
+
 }  // namespace vg

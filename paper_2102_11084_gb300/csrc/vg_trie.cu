@@ -56,8 +56,6 @@ constexpr int kTrAdd = 1;  // runs a lane adds at a time
 // ones.
 constexpr int kTrLane = 2, kTrLaneLarge = 4;
 
-static_assert(32ull * 0x1fffffu < (1ull << 26), "a run of 32 points in its fields");
-
 struct TrArgs {
   const float* xyz;
   FramesArg fr;
@@ -282,33 +280,6 @@ __device__ __forceinline__ bool tr_key(const TrFrames& fm, int f, float x, float
   return true;
 }
 
-// Runs of equal keys in a warp's points, K consecutive ones a lane.  A run ends within its
-// group of 32 points (32 / K lanes), so that its sums fit their fields.
-struct TrRun {
-  uint32_t same;  // bit j: the lane's point j has the key of its point j - 1 (bit 0: of the lane before's last)
-  uint32_t head;  // first lane of the chain of whole lanes that ends in the lane's last point
-  uint32_t tail;  // bit j: point j is valid and ends its run
-};
-constexpr uint64_t kTrNoKey = ~0ull;  // an invalid point's
-template <int K>
-__device__ __forceinline__ TrRun tr_run(const uint64_t key[K]) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t prev = __shfl_up_sync(kFullMask, key[K - 1], 1);
-  TrRun r;
-  r.same = (lane & (32u / K - 1u)) != 0u && prev == key[0] ? 1u : 0u;
-#pragma unroll
-  for (int j = 1; j < K; ++j) r.same |= key[j] == key[j - 1] ? 1u << j : 0u;
-  const uint32_t heads = __ballot_sync(kFullMask, r.same != (1u << K) - 1u);
-  r.head = 31u - __clz(heads & (kFullMask >> (31u - lane)));
-  const uint32_t links = __ballot_sync(kFullMask, (r.same & 1u) != 0u);
-  const uint32_t next = (r.same >> 1) | (((links >> 1 >> lane) & 1u) << (K - 1));
-  r.tail = 0u;
-#pragma unroll
-  for (int j = 0; j < K; ++j)
-    r.tail |= key[j] != kTrNoKey && !((next >> j) & 1u) ? 1u << j : 0u;
-  return r;
-}
-
 // Place of the lane's first run among the warp's, in the points' order, from the ballots of the
 // points that end one.
 template <int K>
@@ -459,38 +430,6 @@ __device__ __forceinline__ void tr_offsets(const TrFrames& fm, int f, const floa
     w[c] = quant_biased(q[c], voxel_corner(fi[c], fm.org[3 * f + c], fm.leaf[f]), fm.inv_unit[f]);
   w[2] |= 1u << 26;
 }
-// Sums of N words over a run, at every point that ends one: within the lane, along the chain of
-// whole lanes, and the part before the lane added to its first run.
-template <int K, int N>
-__device__ __forceinline__ void tr_sums(uint32_t w[K][N], const TrRun& r) {
-  const uint32_t lane = threadIdx.x & 31u;
-#pragma unroll
-  for (int j = 1; j < K; ++j)
-#pragma unroll
-    for (int c = 0; c < N; ++c) w[j][c] += (r.same >> j) & 1u ? w[j - 1][c] : 0u;
-#pragma unroll
-  for (uint32_t d = 1; d < 32u / K; d <<= 1) {
-    if (!__any_sync(kFullMask, lane >= r.head + d)) break;  // no chain is longer
-#pragma unroll
-    for (int c = 0; c < N; ++c) {
-      const uint32_t y = __shfl_up_sync(kFullMask, w[K - 1][c], d);
-      if (lane >= r.head + d) w[K - 1][c] += y;
-    }
-  }
-  if (!__any_sync(kFullMask, (r.same & 1u) != 0u)) return;  // no run crosses lanes
-#pragma unroll
-  for (int c = 0; c < N; ++c) {
-    uint32_t y = __shfl_up_sync(kFullMask, w[K - 1][c], 1);
-    if (!(r.same & 1u)) y = 0u;
-    bool on = true;
-#pragma unroll
-    for (int j = 0; j < K - 1; ++j) {  // (the last point's sum has it already)
-      on = on && (j == 0 || ((r.same >> j) & 1u));
-      w[j][c] += on ? y : 0u;
-    }
-  }
-}
-
 // A level in use: its slots' bits and records.
 struct TrLevel {
   uint32_t* bits;
@@ -684,14 +623,14 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
 #pragma unroll
     for (int j = 0; j < K; ++j) {
       float fi[3];
-      key[j] = kTrNoKey;
+      key[j] = kNoKey;
       w[j][0] = w[j][1] = w[j][2] = 0u;
       if (tr_key(fm, t.f, t.q[j][0], t.q[j][1], t.q[j][2], wide, key_shift, &key[j], fi,
                  &range_bad))
         tr_offsets(fm, t.f, t.q[j], fi, w[j]);
     }
-    const TrRun r = tr_run<K>(key);
-    tr_sums<K, 3>(w, r);
+    const LaneRuns r = lane_runs<K>(key);
+    run_sums<K, 3>(w, r);
     uint32_t tails[K], total = 0u, base = 0u;
 #pragma unroll
     for (int j = 0; j < K; ++j) {
@@ -704,7 +643,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     if (a.out.p2v) {
 #pragma unroll
       for (int j = 0; j < K; ++j) {
-        const uint32_t valid = __ballot_sync(kFullMask, key[j] != kTrNoKey);
+        const uint32_t valid = __ballot_sync(kFullMask, key[j] != kNoKey);
         if (lane == 0) mask[part * K + j] = make_uint2(tails[j], valid);
       }
       if (lane == 0) firsts[part] = base;
@@ -732,13 +671,13 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
 #pragma unroll
       for (int j = 0; j < K; ++j) {
         at[j][0] = at[j][1] = 0u;
-        if (key[j] == kTrNoKey) continue;
+        if (key[j] == kNoKey) continue;
         const uint8_t* b = a.out.attrs_in + size_t(t.p + j) * a.out.channels;
 #pragma unroll
         for (int c = 0; c < 4; ++c)  // two 16-bit sums a word (32 x 255 fit)
           if (c < a.out.channels) at[j][c >> 1] |= uint32_t(__ldg(b + c)) << (16 * (c & 1));
       }
-      tr_sums<K, 2>(at, r);
+      run_sums<K, 2>(at, r);
       uint32_t i = base + place;
 #pragma unroll
       for (int j = 0; j < K; ++j)

@@ -1,5 +1,5 @@
-"""The hash insert's queue of runs (a warp's pieces of 128 points, runs of up to four of a
-thread's points, 32 added at a time) and the voxel map's packed sums, against the radix sort
+"""The hash insert's queue of runs (a warp's pieces of 128 points, runs within 32 points, 32
+added at a time) and the voxel map's packed sums, against the radix sort
 and the oracle: ragged sizes around a piece and a chunk, runs that end at every place of a
 thread, cells of many points (every carry), frames of all sizes, clearing and refilling."""
 import numpy as np
@@ -30,6 +30,25 @@ def test_ragged_sizes(n):
     got = vg.downsample(cuda(x), 0.05, method="hash")
     assert_decimation_equal(got, oracle.downsample(x, 0.05), check_p2v=False)
     same(got, vg.downsample(cuda(x), 0.05, method="sort_lsd"))
+
+
+@pytest.mark.parametrize("method", ["hash", "auto"])
+@pytest.mark.parametrize("posed", [False, True])
+def test_runs_of_every_length(method, posed):
+    # runs of 1 to 97 points, some of them invalid, from every place of a lane and across
+    # lanes, groups of 32 points, warps and chunks; frames that start off a 16-byte boundary
+    sizes = [1, 30_002, 129, 50_001, 3]
+    x = synth.random_cloud(8_000, seed=9, extent=1.0, nan_frac=0.1)
+    x = np.repeat(x, np.arange(len(x)) * 13 % 97 + 1, axis=0)[: sum(sizes)]
+    offs = [0] + [int(v) for v in np.cumsum(sizes)]
+    kw = {"poses": synth.sensor_poses(len(sizes), seed=2)[0]} if posed else {}
+    for p2v in (False, True):
+        a = vg.downsample_frames((cuda(x), offs), [0.05] * 5, method=method, point_to_voxel=p2v, **kw)
+        b = vg.downsample_frames((cuda(x), offs), [0.05] * 5, method="sort_lsd", point_to_voxel=p2v,
+                                 **kw)
+        assert a.offsets == b.offsets
+        same(a, b)
+        assert not p2v or torch.equal(a.point_to_voxel, b.point_to_voxel)
 
 
 @pytest.mark.parametrize("bits", [9, 10, 11, 14, 20])
