@@ -40,12 +40,14 @@ namespace vg {
 namespace {
 
 constexpr int kNb = 27;
+constexpr uint32_t kLoopGroup = 128;  // entries a warp takes at a time (4 a lane)
 constexpr uint32_t kNoCell = 0xffffffffu;
 constexpr uint8_t kAlive = 1, kMarked = 2;
 // Words of the loop: marked points (recounted form), kept points, grid-barrier arrivals, passes
-// run, and the candidate pairs (one 64-bit word).
-constexpr int kCtrMarked = 0, kCtrKept = 1, kCtrBar = 2, kCtrPasses = 3, kCtrPairs = 4;
-constexpr int kCtrGroups = 6;  // groups of entries (counts kept)
+// run, the candidate pairs (one 64-bit word), groups of entries (at most kLoopGroup of one cell:
+// how many there are, and how many are listed).
+constexpr int kCtrMarked = 0, kCtrKept = 1, kCtrBar = 2, kCtrPasses = 3, kCtrPairs = 4,
+              kCtrAll = 6, kCtrGroups = 7;
 constexpr int kCtrWords = 8;
 
 struct ThinLayout {
@@ -119,10 +121,11 @@ __global__ void thin_setup_kernel(const State* st, const uint32_t* idx0, const u
 // cell are independent chains of dependent loads (11,489 cells: 25.8 us one thread a cell).
 __global__ __launch_bounds__(256) void thin_neighbors_kernel(
     const int64_t* __restrict__ num_cells, const uint64_t* __restrict__ vkeys,
-    const uint32_t* __restrict__ vcnt, uint32_t* nb, unsigned long long* pairs, const int* err) {
+    const uint32_t* __restrict__ vcnt, uint32_t* nb, uint32_t* ctr, const int* err) {
   if (error_raised(err)) return;
   const int64_t V = *num_cells;
   unsigned long long mine = 0;
+  uint32_t groups = 0;
   for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < V * kNb;
        t += int64_t(gridDim.x) * blockDim.x) {
     const int64_t v = t / kNb;
@@ -143,10 +146,14 @@ __global__ __launch_bounds__(256) void thin_neighbors_kernel(
       if (lo < V && vkeys[lo] == want) row = static_cast<uint32_t>(lo);
     }
     nb[t] = row;
+    if (o == 0) groups += (vcnt[v] + kLoopGroup - 1) / kLoopGroup;
     if (row != kNoCell) mine += (unsigned long long)vcnt[v] * vcnt[row];
   }
   for (int off = 16; off; off >>= 1) mine += __shfl_xor_sync(kFullMask, mine, off);
-  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(pairs, mine);
+  groups = __reduce_add_sync(kFullMask, groups);
+  if ((threadIdx.x & 31) == 0 && mine)
+    atomicAdd(reinterpret_cast<unsigned long long*>(ctr + kCtrPairs), mine);
+  if ((threadIdx.x & 31) == 0 && groups) atomicAdd(ctr + kCtrAll, groups);
 }
 
 // Squared distance of the definition: binary32, ((dx*dx + dy*dy) + dz*dz), one rounding an
@@ -162,7 +169,6 @@ constexpr int kFullThreads = 128;
 constexpr int kLoopThreads = 1024;
 constexpr int kLoopItems = 2;   // list entries a thread tests per step of the batch search
 constexpr int kLoopSplit = 8;   // warps that share the candidates of one deleted point
-constexpr uint32_t kLoopGroup = 128;  // entries a warp takes at a time (4 a lane)
 
 // Two binary32 operations in one instruction, each with its own rounding.
 __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
@@ -295,6 +301,12 @@ struct LoopArgs {
   uint32_t* sel;            // scattered: the entries a pass deletes
   unsigned long long* head;  // gathered: pass << 32 | the cell's last deleted entry's rank
   float4* node;             // gathered: place of the entry of each rank; w = the next rank
+  // in the block's own memory: per list position its place (negated; w = its cell), the pass
+  // that unmarked it (0: none yet) and whether a pass deleted it; per entry its position
+  float4* lnode;
+  uint32_t* off;
+  uint8_t* gone;
+  uint32_t* rank;
   uint32_t* ctr;
   float r2;
   uint32_t thr;
@@ -409,7 +421,8 @@ __device__ __forceinline__ void thin_gather(const LoopArgs& a, uint32_t pass, Th
     }
 }
 
-// Every pass of the loop, one cooperative launch (a block an SM), two grid barriers a pass:
+// Every pass of the loop where local_lists leaves it (few candidates, or a batch of more than
+// kLocalBatch), one cooperative launch (a block an SM), two grid barriers a pass:
 //   1. the batch: every block walks the sorted list from where the last pass stopped, tests
 //      kLoopItems entries a thread, and finds the same `batch` entries still marked (one more
 //      tells that this is not the last pass); the block that a list entry belongs to writes it.
@@ -418,7 +431,8 @@ __device__ __forceinline__ void thin_gather(const LoopArgs& a, uint32_t pass, Th
 //      warp keeps its first group in registers through all passes).
 // Bound by the latency of the steps and the barriers.  640x480 frame, cell 0.05 m, threshold
 // 20, batches of 1000 (277K points of 3600 candidates each, 2008 cells, 271 passes): a pass
-// takes 23 us scattered (the drain of its 1.8M decrements is 3/4 of it), 12 us gathered,
+// takes 23 us scattered (the drain of its 1.8M decrements is 3/4 of it), 12 us gathered
+// (thin_local_kernel, which takes it for batches of this size, 7.0 us),
 // against 570 us for a fresh count and 500 us of host round trips (recounted).  The gathered
 // form touches every group of entries each pass, 9000 cycles a round of the grid's warps; the
 // scattered form 8000 cycles and one per 90 candidates.
@@ -516,6 +530,182 @@ __global__ __launch_bounds__(kLoopThreads, 1) void thin_loop_kernel(const LoopAr
     if (!grid_barrier(a.ctr + kCtrBar, target, a.spin_limit, a.err)) return;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr[kCtrPasses] = static_cast<uint32_t>(passes);
+}
+
+// The same loop for batches of at most kLocalBatch points, one grid barrier a pass: every block
+// finds the same batch by itself and keeps its own copy, in lists by cell in shared memory, for
+// thin_gather's walk.  What a pass reads to find its batch lies in list order, and a thread's
+// first place is loaded ahead of the barrier.  A marked entry whose count falls to the
+// threshold records the pass; one that a faster block records in this pass still counts as
+// marked, so that no barrier is needed between finding the batch and counting.
+// Bound by the walk of the densest groups (8000 of a pass's 14,500 cycles in the frame of
+// thin_loop_kernel's comment; the barrier 2500, finding the batch 3000): 7.0 us a pass, where
+// gathering from lists in global memory, two barriers a pass, took 12.  Three or four points at
+// a time, or fewer warps with more registers, were no faster.
+constexpr uint32_t kLocalBatch = 4096;
+constexpr uint32_t kLocalHeads = 4096;  // lists (a power of two): a cell's by its low bits
+constexpr int kLocalAtOnce = 2;  // deleted points a warp tests at a time
+struct LocalSmem {
+  float4 node[kLocalBatch + 1];  // place (negated); w = the next rank of the list; a far point
+  uint32_t cell[kLocalBatch];
+  uint32_t head[kLocalHeads];
+};
+struct LocalGroup {
+  uint32_t i0, nb;                         // as ThinGroup
+  unsigned long long x[2], y[2], z[2];     // the lane's entries, two to a word
+  uint32_t n[4];
+  uint32_t changed;                        // bit v: n[v] is not the one in memory
+};
+__device__ __forceinline__ void local_group_load(const LoopArgs& a, uint64_t u, LocalGroup& g) {
+  ThinGroup t;
+  thin_group_load(a, u, t);
+  g.i0 = t.i0;
+  g.nb = t.nb;
+  g.changed = 0u;
+  auto two = [](float lo, float hi) {
+    return __float_as_uint(lo) | ((unsigned long long)__float_as_uint(hi) << 32);
+  };
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    g.x[h] = two(t.x[2 * h], t.x[2 * h + 1]);
+    g.y[h] = two(t.y[2 * h], t.y[2 * h + 1]);
+    g.z[h] = two(t.z[2 * h], t.z[2 * h + 1]);
+  }
+#pragma unroll
+  for (int v = 0; v < 4; ++v) g.n[v] = t.n[v];
+}
+__device__ __forceinline__ void local_gather(const LoopArgs& a, const LocalSmem& sm, uint32_t pass,
+                                             LocalGroup& g) {
+  const uint32_t lane = threadIdx.x & 31u;
+  if (!__any_sync(kFullMask, g.n[0] > a.thr || g.n[1] > a.thr || g.n[2] > a.thr || g.n[3] > a.thr))
+    return;
+  uint32_t r = g.nb != kNoCell ? sm.head[g.nb & (kLocalHeads - 1u)] : kListEnd;
+  uint32_t hit[4] = {0u, 0u, 0u, 0u};
+  for (;;) {
+    while (r != kListEnd && sm.cell[r] != g.nb) r = __float_as_uint(sm.node[r].w);
+    uint32_t some = __ballot_sync(kFullMask, r != kListEnd);
+    if (some == 0u) break;
+    while (some) {
+      float4 q[kLocalAtOnce];
+#pragma unroll
+      for (int b = 0; b < kLocalAtOnce; ++b) {
+        const uint32_t at = __shfl_sync(kFullMask, r, (__ffs(some) - 1) & 31);
+        q[b] = sm.node[some ? at : kLocalBatch];
+        some &= some - 1;
+      }
+#pragma unroll
+      for (int b = 0; b < kLocalAtOnce; ++b) {
+        const unsigned long long x = both(q[b].x), y = both(q[b].y), z = both(q[b].z);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const unsigned long long ex = add2(g.x[h], x), ey = add2(g.y[h], y), ez = add2(g.z[h], z);
+          const unsigned long long d = add2(add2(mul2(ex, ex), mul2(ey, ey)), mul2(ez, ez));
+          hit[2 * h] += __uint_as_float(uint32_t(d)) <= a.r2;
+          hit[2 * h + 1] += __uint_as_float(uint32_t(d >> 32)) <= a.r2;
+        }
+      }
+    }
+    if (r != kListEnd) r = __float_as_uint(sm.node[r].w);
+  }
+#pragma unroll
+  for (uint32_t v = 0; v < 4; ++v)
+    if (g.n[v] > a.thr && hit[v]) {
+      g.n[v] -= hit[v];
+      g.changed |= 1u << v;
+      if (g.n[v] <= a.thr) a.off[__ldca(a.rank + g.i0 + 32u * v + lane)] = pass;
+    }
+}
+__device__ __forceinline__ void local_group_store(const LoopArgs& a, const LocalGroup& g) {
+#pragma unroll
+  for (uint32_t v = 0; v < 4; ++v)
+    if ((g.changed >> v) & 1u) a.cnt[g.i0 + 32u * v + (threadIdx.x & 31u)] = g.n[v];
+}
+
+__global__ __launch_bounds__(kLoopThreads, 1) void thin_local_kernel(const LoopArgs a) {
+  extern __shared__ __align__(16) unsigned char local_smem[];
+  LocalSmem& sm = *reinterpret_cast<LocalSmem*>(local_smem);
+  __shared__ uint32_t tmp[2][32];
+  __shared__ uint32_t s_next;
+  if (block_error_raised(a.err)) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr[kCtrPasses] = 1u;
+    return;
+  }
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t m = a.st2->nitems;
+  const uint32_t groups = a.ctr[kCtrGroups];
+  const uint64_t gwarps = uint64_t(gridDim.x) * (kLoopThreads / 32);
+  const uint64_t gw = uint64_t(warp) * gridDim.x + blockIdx.x;
+  const uint32_t gt = blockIdx.x * kLoopThreads + threadIdx.x, gthreads = gridDim.x * kLoopThreads;
+  for (uint64_t k = gt; k < m; k += gthreads) {
+    const uint32_t e = __ldg(a.list + k);
+    const float4 w = __ldg(a.pos + e);
+    a.lnode[k] = make_float4(-w.x, -w.y, -w.z, __uint_as_float(__ldg(a.ecell + e)));
+    a.off[k] = 0u;
+    a.gone[k] = 0;
+    a.rank[e] = static_cast<uint32_t>(k);
+  }
+  if (threadIdx.x == 0)  // (at no finite distance)
+    sm.node[kLocalBatch] = make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(kListEnd));
+  LocalGroup mine{};  // (no entries: no count is above the threshold)
+  mine.nb = kNoCell;
+  if (gw < groups) local_group_load(a, gw, mine);
+  uint32_t target = 0, first = 0, pass = 0, writer = 0, buf = 0;
+  if (!grid_barrier(a.ctr + kCtrBar, target, a.spin_limit, a.err)) return;
+  float4 ahead = make_float4(0.0f, 0.0f, 0.0f, 0.0f);  // the place of list entry first + thread
+  if (threadIdx.x < m) ahead = __ldcg(a.lnode + threadIdx.x);
+  while (int64_t(pass) < a.max_passes) {
+    ++pass;
+    const bool writes = blockIdx.x == writer;  // the block that writes this pass's deletions
+    writer = writer + 1u < gridDim.x ? writer + 1u : 0u;
+    // 1. the next `batch` marked entries of the list
+    for (uint32_t h = threadIdx.x; h < kLocalHeads; h += kLoopThreads) sm.head[h] = kListEnd;
+    uint32_t found = 0;
+    auto take = [&](bool in, uint32_t r, uint32_t k, bool fresh) {
+      if (!in || r >= a.batch) return;
+      const float4 w = fresh ? __ldcg(a.lnode + k) : ahead;
+      const uint32_t c = __float_as_uint(w.w);
+      const uint32_t old = atomicExch(&sm.head[c & (kLocalHeads - 1u)], r);
+      sm.cell[r] = c;
+      sm.node[r] = make_float4(w.x, w.y, w.z, __uint_as_float(old));
+      if (writes) a.gone[k] = 1;
+      if (r + 1 == a.batch) s_next = k + 1;
+    };
+    for (uint32_t k0 = first;;) {
+      const uint32_t ka = k0 + threadIdx.x, kb = ka + kLoopThreads;
+      const uint32_t fa = ka < m ? __ldcg(a.off + ka) : ~0u, fb = kb < m ? __ldcg(a.off + kb) : ~0u;
+      const bool ina = fa == 0u || fa == pass, inb = fb == 0u || fb == pass;
+      const uint32_t ba = __ballot_sync(kFullMask, ina), bb = __ballot_sync(kFullMask, inb);
+      if (lane == 0) tmp[buf][warp] = __popc(ba) | (__popc(bb) << 16);
+      __syncthreads();
+      const uint32_t v = tmp[buf][lane];
+      buf ^= 1u;
+      const uint32_t tot = __reduce_add_sync(kFullMask, v);
+      const uint32_t pre = __reduce_add_sync(kFullMask, lane < warp ? v : 0u);
+      const uint32_t lt = (1u << lane) - 1u;
+      take(ina, found + (pre & 0xffffu) + __popc(ba & lt), ka, k0 != first);
+      take(inb, found + (tot & 0xffffu) + (pre >> 16) + __popc(bb & lt), kb, true);
+      found += (tot & 0xffffu) + (tot >> 16);
+      if (found > a.batch || m - k0 <= 2u * kLoopThreads) break;
+      k0 += 2u * kLoopThreads;  // (stays below m)
+    }
+    if (found <= a.batch) break;  // (the same in every block) the last pass
+    __syncthreads();
+    first = s_next;
+    // 2. the counts
+    local_gather(a, sm, pass, mine);
+    for (uint64_t u = gw + gwarps; u < groups; u += gwarps) {
+      LocalGroup more;
+      local_group_load(a, u, more);
+      local_gather(a, sm, pass, more);
+      local_group_store(a, more);
+    }
+    if (first + threadIdx.x < m) ahead = __ldcg(a.lnode + first + threadIdx.x);
+    if (!grid_barrier(a.ctr + kCtrBar, target, a.spin_limit, a.err)) return;
+  }
+  local_group_store(a, mine);
+  for (uint64_t k = gt; k < m; k += gthreads)
+    if (__ldcg(a.gone + k)) a.dead[__ldg(a.list + k)] = 1;
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr[kCtrPasses] = pass;
 }
 
 // keep flag per input point (zeroed before: invalid points stay 0): not deleted by a batch
@@ -668,6 +858,19 @@ int thin_loop_grid() {
   return v > 0 ? num_sms() : 0;
 }
 
+// The same of thin_local_kernel.
+int thin_local_grid() {
+  int v = 0;
+  if (cudaFuncSetAttribute(thin_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(sizeof(LocalSmem))) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, thin_local_kernel, kLoopThreads,
+                                                    sizeof(LocalSmem)) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return v > 0 ? num_sms() : 0;
+}
+
 // Whether the loop keeps counts, by estimated microseconds.  Kept: every candidate pair is
 // tested about twice in all (the count, then the deletions; 1.5e12 tests a second) and a pass
 // takes 10 us.  Recounted: a pass takes 100 us of host round trips and about 100 ps a point and
@@ -679,6 +882,18 @@ bool keep_counts(int64_t n, unsigned long long pairs, int64_t batch, int64_t thr
   const double gone = pp > 0.0 ? 1.0 - 3.0 * want * nn / pp : 0.0;
   const double passes = gone > 0.0 && gone * nn > double(batch) ? gone * nn / double(batch) : 1.0;
   return 2.0 * pp / 1.5e6 + 10.0 * passes <= passes * (100.0 + nn * want * 1e-4);
+}
+
+// Whether a pass is thin_local_kernel's, by estimated cycles: 6000 and, for every round of the
+// grid's warps over the groups, 2500 and 500 a deleted point that a group meets; scattered, 18,000
+// and one per 90 candidates.  Both sides measured: 640x480 frame at 0.05 m, batches of 1000 (one
+// round, 13 points a group, 3600 candidates): 7.0 us a pass against 23; 200K points of 84
+// candidates (13 rounds): 25 against 14; 1280x720 at 0.02 m (several rounds of small cells): 18
+// against 11.
+bool local_lists(uint32_t groups, uint32_t batch, double pairs, double n, int grid) {
+  const double rounds = std::ceil(double(groups) / (double(grid) * (kLoopThreads / 32)));
+  const double met = double(batch) * pairs / n;  // candidates of a batch
+  return batch <= kLocalBatch && 6000.0 + rounds * (2500.0 + 500.0 * met / n) <= 18000.0 + met / 90.0;
 }
 
 int grid_for(int64_t n) {
@@ -758,14 +973,19 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
   float* sy = sx + align_up(size_t(n < 1 ? 1 : n), 4);
   float* sz = sy + align_up(size_t(n < 1 ? 1 : n), 4);
   unsigned long long pairs = 0;
+  uint32_t groups = 0;
   if (n > 0) {
     thin_neighbors_kernel<<<num_sms() * 8, 256, 0, stream>>>(
-        vnum, vkeys, vcnt, nb, reinterpret_cast<unsigned long long*>(ctr + kCtrPairs), err);
+        vnum, vkeys, vcnt, nb, ctr, err);
     thin_setup_kernel<<<g, 256, 0, stream>>>(st, idx0, idx1, xyz, priority, p2v, cstart, pos, sx,
                                              sy, sz, sprio, sidx, entry, state, err);
-    e = cudaMemcpyAsync(&pairs, ctr + kCtrPairs, sizeof(pairs), cudaMemcpyDeviceToHost, stream);
+    uint32_t c[4];
+    static_assert(kCtrAll == kCtrPairs + 2, "read together");
+    e = cudaMemcpyAsync(c, ctr + kCtrPairs, sizeof(c), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return VG_ERR_CUDA;
+    pairs = c[0] | ((unsigned long long)c[1] << 32);
+    groups = c[2];
   }
   const int64_t max_passes = n / batch + 2;  // every pass but the last deletes `batch` points
   const float r2 = radius * radius;
@@ -793,18 +1013,49 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
                     spin_limit(), err, stream);  // (32-bit priorities)
     if (e != cudaSuccess) return VG_ERR_CUDA;
     thin_list_kernel<<<g, 256, 0, stream>>>(st2, idx0, idx1, entry, list, err);
-    // the sort's buffers again: the deleted lists' heads (a cell each) and nodes (16 bytes a
-    // point of the batch, in the 16 bytes a point from keys1 to the end of idx1), or `sel`
-    e = cudaMemsetAsync(keys0, 0, size_t(n) * sizeof(uint64_t), stream);
-    if (e != cudaSuccess) return VG_ERR_CUDA;
-    LoopArgs la{st2, list, ecell, cstart, vcnt, nb, pos, group, cnt, state,
-                reinterpret_cast<uint32_t*>(keys0), reinterpret_cast<unsigned long long*>(keys0),
-                reinterpret_cast<float4*>(keys1), ctr, r2, thr,
-                static_cast<uint32_t>(batch < n ? batch : n), double(pairs) / double(n),
-                max_passes, spin_limit(), err};
+    LoopArgs la{};
+    la.st2 = st2;
+    la.list = list;
+    la.ecell = ecell;
+    la.cstart = cstart;
+    la.vcnt = vcnt;
+    la.nb = nb;
+    la.pos = pos;
+    la.group = group;
+    la.cnt = cnt;
+    la.dead = state;
+    la.ctr = ctr;
+    la.r2 = r2;
+    la.thr = thr;
+    la.batch = static_cast<uint32_t>(batch < n ? batch : n);
+    la.pairs_per_point = double(pairs) / double(n);
+    la.max_passes = max_passes;
+    la.spin_limit = spin_limit();
+    la.err = err;
     void* args[] = {&la};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(thin_loop_kernel),
-                                    dim3(loop_grid), dim3(kLoopThreads), args, 0, stream);
+    // the sort's buffers again
+    const int local_grid =
+        local_lists(groups, la.batch, double(pairs), double(n), loop_grid) ? thin_local_grid() : 0;
+    if (local_grid > 0) {
+      // 16 bytes a point from keys1 to the end of idx1, 5 in keys0, 4 in the entries of points
+      la.lnode = reinterpret_cast<float4*>(keys1);
+      la.off = reinterpret_cast<uint32_t*>(keys0);
+      la.gone = reinterpret_cast<uint8_t*>(la.off + align_up(size_t(n), 4));
+      la.rank = entry;
+      e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(thin_local_kernel),
+                                      dim3(local_grid), dim3(kLoopThreads), args,
+                                      sizeof(LocalSmem), stream);
+    } else {
+      // the deleted lists' heads (a cell each) and nodes (16 bytes a point of the batch, in
+      // the 16 bytes a point from keys1 to the end of idx1), or `sel`
+      e = cudaMemsetAsync(keys0, 0, size_t(n) * sizeof(uint64_t), stream);
+      if (e != cudaSuccess) return VG_ERR_CUDA;
+      la.sel = reinterpret_cast<uint32_t*>(keys0);
+      la.head = reinterpret_cast<unsigned long long*>(keys0);
+      la.node = reinterpret_cast<float4*>(keys1);
+      e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(thin_loop_kernel),
+                                      dim3(loop_grid), dim3(kLoopThreads), args, 0, stream);
+    }
     if (e != cudaSuccess) return VG_ERR_CUDA;
     thin_keep_kernel<<<g, 256, 0, stream>>>(st, pos, cnt, state, thr, out_keep, ctr + kCtrKept,
                                             err);

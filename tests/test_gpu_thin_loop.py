@@ -53,3 +53,17 @@ def test_equal_and_large_priorities():
     check(x, 0.05, 3, np.zeros(3000, np.uint32), 50)
     check(x, 0.05, 3, rng.integers(0xfffffff0, 1 << 32, 3000, dtype=np.uint64).astype(np.uint32),
           50)
+
+
+@pytest.mark.parametrize("n,ext,t,batch", [
+    (20_000, 0.4, 10, 4096), (20_000, 0.4, 10, 4097),  # either side of a block's own lists
+    (1_500, 0.14, 3, 1), (6_000, 0.2, 0, 33),          # most list entries unmarked at the end
+    (60_000, 1.0, 20, 4000),                           # groups of several rounds, lists shared
+    (40_000, 1.6, 1, 500),                             # few candidates: scattered
+])
+def test_forms_of_the_kept_counts(n, ext, t, batch):
+    rng = np.random.Generator(np.random.PCG64(n + batch))
+    x = rng.uniform(0, ext, (n, 3)).astype(np.float32)
+    x[: n // 8] *= 0.3  # crowded cells among sparse ones
+    x[::211] = np.inf
+    check(x, 0.05, t, rng.permutation(n).astype(np.uint32), batch)
