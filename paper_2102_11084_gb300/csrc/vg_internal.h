@@ -46,10 +46,10 @@ constexpr int kMsdBuckets = 1 << kMsdMaxTop;   // bucket ids
 #define VG_MSD_TARGET 2048
 #endif
 constexpr int kMsdTarget = VG_MSD_TARGET;               // average points per bucket the split aims at
-// Clouds from this many points on take the bucket grouping under VG_METHOD_AUTO; smaller
-// ones (camera frames, whose dense surfaces make large buckets of few cells) take the
-// global radix sort, which is faster there (measured: a 640x480 frame 0.10 vs 0.20 ms,
-// the 50M-point map 2.78 vs 2.24 ms).
+// Clouds from this many points on that the occupancy trie (vg_trie.h) leaves take the bucket
+// grouping under VG_METHOD_AUTO; smaller ones take the global radix sort (4M shuffled points
+// 0.32 ms both; where dense surfaces make large buckets of few cells it is faster, a 640x480
+// frame 0.10 vs 0.20 ms; the 50M-point map takes 2.8 ms sorted and 1.79 in buckets).
 constexpr int64_t kAutoBucketMinPoints = int64_t(1) << 22;
 constexpr int kPartThreads = 256;              // partition pass: 256 threads x 16 records
 constexpr int kPartItems = 16;
