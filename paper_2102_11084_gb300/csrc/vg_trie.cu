@@ -84,7 +84,6 @@ struct TrArgs {
 
 struct TrSmem {
   uint32_t tmp[kTrThreads / 32];
-  float red[kTrThreads / 32][6];
   uint32_t bits[kTrThreads / 32];
   uint32_t first;
   uint32_t nruns;
@@ -99,9 +98,10 @@ struct TrFrames {
   float* rleaf;
   float* inv_unit;
   uint32_t* cstart;  // [F + 1]
+  uint32_t* ext;     // [F][6]: the block's extents, as the frames' (ord_min_inv, ord_max)
 };
 constexpr size_t tr_frames_bytes(int frames, bool posed) {
-  return align_up(size_t(frames + 1) * 12 + size_t(frames) * (posed ? 88 : 24), 16);
+  return align_up(size_t(frames + 1) * 12 + size_t(frames) * (posed ? 112 : 48), 16);
 }
 __device__ __forceinline__ TrFrames tr_frames(unsigned char* mem, int F, bool posed) {
   TrFrames t;
@@ -112,6 +112,7 @@ __device__ __forceinline__ TrFrames tr_frames(unsigned char* mem, int F, bool po
   t.rleaf = t.leaf + F;
   t.inv_unit = t.rleaf + F;
   t.cstart = reinterpret_cast<uint32_t*>(t.inv_unit + F);
+  t.ext = t.cstart + F + 1;
   return t;
 }
 
@@ -128,59 +129,7 @@ __device__ __forceinline__ Pose tr_pose(const TrArgs& a, const TrFrames& fm, int
   return P;
 }
 
-// U points of a thread (one of each of U chunks): frame, index, whether inside the frame, and
-// coordinates (NaN outside).
-template <int U>
-struct TrPoints {
-  int f[U];
-  int64_t p[U];
-  bool in[U];
-  float q[U][3];
-};
-
-// fn(points) for every U chunks of this block: chunk c (1024 points of one frame, a thread a
-// point) belongs to block c mod grid, so that the blocks share the dense parts of a cloud.  All
-// threads call fn the same number of times.  The next points are loaded one step ahead.
-template <bool kPosed, int U, typename Fn>
-__device__ __forceinline__ void tr_points(const TrArgs& a, const TrFrames& fm, uint32_t T, Fn fn) {
-  const int nf = a.fr.nframes;
-  const float nan = __int_as_float(0x7fc00000);
-  TrPoints<U> next;
-  auto load = [&](uint64_t c0) {
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint64_t c = c0 + uint64_t(u) * gridDim.x;
-      next.f[u] = 0;
-      next.p[u] = 0;
-      next.in[u] = false;
-      if (c < T) {
-        const int f = nf > 1 ? chunk_frame(fm.cstart, nf, uint32_t(c)) : 0;
-        next.f[u] = f;
-        next.p[u] = fm.off[f] + (int64_t(c) - fm.cstart[f]) * kChunk + threadIdx.x;
-        next.in[u] = next.p[u] < fm.off[f + 1];
-      }
-      const float* q = a.xyz + 3 * next.p[u];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) next.q[u][k] = next.in[u] ? __ldg(q + k) : nan;
-    }
-  };
-  const uint64_t step = uint64_t(U) * gridDim.x;
-  load(blockIdx.x);
-  for (uint64_t c = blockIdx.x; c < T; c += step) {
-    TrPoints<U> now = next;
-    if (c + step < T) load(c + step);
-    if (kPosed) {
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const Pose P = tr_pose(a, fm, now.f[u]);
-        pose_point(P, now.q[u][0], now.q[u][1], now.q[u][2]);
-      }
-    }
-    fn(now);
-  }
-}
-
-// A lane's points in the marking pass: K consecutive ones from p on, m of them in frame f.
+// A lane's points: K consecutive ones from p on, m of them in frame f (NaN past them).
 // Chunk k of the block is the cloud's k * grid + blockIdx.x; kChunk / 32K warps take it.
 template <int K>
 struct TrLanePoints {
@@ -379,43 +328,21 @@ __device__ __forceinline__ uint32_t tr_rank_slots(const uint32_t* bits, uint2* r
   return all;
 }
 
-// Folds the block's min and max of the valid points of frame f into its state.  Contains
-// __syncthreads.
-__device__ __forceinline__ void tr_flush_extent(float mn[3], float mx[3], FrameState* fs, int f,
-                                                TrSmem& sm) {
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int off = 16; off; off >>= 1) {
-      mn[c] = fminf(mn[c], __shfl_xor_sync(kFullMask, mn[c], off));
-      mx[c] = fmaxf(mx[c], __shfl_xor_sync(kFullMask, mx[c], off));
-    }
-  __syncthreads();
-  if (lane == 0)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      sm.red[warp][c] = mn[c];
-      sm.red[warp][3 + c] = mx[c];
-    }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      float m = sm.red[lane][c], M = sm.red[lane][3 + c];
-#pragma unroll
-      for (int off = 16; off; off >>= 1) {
-        m = fminf(m, __shfl_xor_sync(kFullMask, m, off));
-        M = fmaxf(M, __shfl_xor_sync(kFullMask, M, off));
-      }
-      if (lane == 0 && m != INFINITY) {
-        atomicMax(&fs[f].ord_min_inv[c], ~float_to_ordered(m));
-        atomicMax(&fs[f].ord_max[c], float_to_ordered(M));
-      }
-    }
-  }
+// Folds the warp's min and max of the valid points of a frame into the block's (no barrier: a
+// block meets every frame of a call, and folding the block's six values in two barriers a frame
+// took a third of the pass over 8 posed frames).
+__device__ __forceinline__ void tr_fold_extent(float mn[3], float mx[3], uint32_t* ext) {
+  const uint32_t lane = threadIdx.x & 31u;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
+    const uint32_t lo =
+        __reduce_max_sync(kFullMask, mn[c] == INFINITY ? 0u : ~float_to_ordered(mn[c]));
+    const uint32_t hi =
+        __reduce_max_sync(kFullMask, mx[c] == -INFINITY ? 0u : float_to_ordered(mx[c]));
+    if (lane == 0 && lo) {
+      atomicMax(ext + c, lo);
+      atomicMax(ext + 3 + c, hi);
+    }
     mn[c] = INFINITY;
     mx[c] = -INFINITY;
   }
@@ -470,7 +397,9 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   uint32_t target = 0;
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
 
-  if (threadIdx.x == 0) sm.nruns = 0u;  // (barriers below come before its first use)
+  // (barriers below come before their first use)
+  if (threadIdx.x == 0) sm.nruns = 0u;
+  for (int i = threadIdx.x; i < 6 * F; i += kTrThreads) fm.ext[i] = 0u;
   bool few = true;  // (the same in every block)
   if (a.large) {
     const unsigned long long smp = a.st->smp;
@@ -506,26 +435,33 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     __syncthreads();
   }
   if (!a.large) {
-    constexpr int U = kPosed ? 2 : 4;
+    // four points a lane: 48 bytes in flight a lane, and a frame looked up for 128 points, not
+    // 32 (8 posed frames: 40,500 -> 20,300 cycles, a 1280x720 frame 7,300 -> 5,600)
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
-    int cur = -1;
-    tr_points<kPosed, U>(a, fm, T, [&](const TrPoints<U>& t) {
+    int cur = 0;
+    tr_lanes<kPosed, 4, true>(a, fm, T, [&](uint32_t, const TrLanePoints<4>& t) {
+      if (t.f != cur) {
+        tr_fold_extent(mn, mx, fm.ext + 6 * cur);
+        cur = t.f;
+      }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (F > 1 && t.f[u] != cur) {
-          if (cur >= 0) tr_flush_extent(mn, mx, a.fs, cur, sm);
-          cur = t.f[u];
-        }
-        if (point_valid(t.q[u][0], t.q[u][1], t.q[u][2])) {
+      for (int j = 0; j < 4; ++j) {
+        if (!point_valid(t.q[j][0], t.q[j][1], t.q[j][2])) continue;
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            mn[c] = fminf(mn[c], t.q[u][c]);
-            mx[c] = fmaxf(mx[c], t.q[u][c]);
-          }
+        for (int c = 0; c < 3; ++c) {
+          mn[c] = fminf(mn[c], t.q[j][c]);
+          mx[c] = fmaxf(mx[c], t.q[j][c]);
         }
       }
     });
-    tr_flush_extent(mn, mx, a.fs, cur < 0 ? 0 : cur, sm);
+    tr_fold_extent(mn, mx, fm.ext + 6 * cur);
+    __syncthreads();
+    for (int i = threadIdx.x; i < 6 * F; i += kTrThreads) {
+      const uint32_t v = fm.ext[i];
+      const int c = i % 6;
+      FrameState& f = a.fs[i / 6];
+      if (v) atomicMax(c < 3 ? &f.ord_min_inv[c] : &f.ord_max[c - 3], v);
+    }
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
   }
 
