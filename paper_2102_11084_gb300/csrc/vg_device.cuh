@@ -139,6 +139,11 @@ __device__ __forceinline__ bool point_index(float x, float y, float z, const flo
   if (!sure) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) fi[a] = floorf(__fdiv_rn(t[a], leaf));
+    // (a NaN of the origin ends here too, and would convert to index 0)
+    if (!(fi[0] >= 0.0f && fi[1] >= 0.0f && fi[2] >= 0.0f)) {
+      *range_bad = true;
+      return false;
+    }
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) ijk[a] = static_cast<uint32_t>(__float2int_rz(fi[a]));
