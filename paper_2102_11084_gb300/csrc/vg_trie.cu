@@ -675,7 +675,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
         const uint32_t s0 =
             j == 1 ? static_cast<uint32_t>(key >> (sh + 2 * kTrDigitBits)) : pslot[i];
         if (s0 < lv.ns) {
-          v[u] = __ldcg(lv.bits + s0 * kTrWords + (id[u] >> (kTrDigitBits + 5)));
+          v[u] = __ldcg(lv.bits + trie_word(s0, id[u] >> kTrDigitBits));
           r[u] = __ldcg(lv.rec + s0);
         }
       }
@@ -690,12 +690,13 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
           in[u] = false;
           continue;
         }
-        id[u] = (s << kTrDigitBits) | (id[u] & kTrDigit);
-        seen[u] = __ldcg(nbits + (id[u] >> 5));
+        v[u] = 1u << (id[u] & 31u);  // (the bit and, below, its word)
+        id[u] = trie_word(s, id[u] & kTrDigit);
+        seen[u] = __ldcg(nbits + id[u]);
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u)
-        tr_set(nbits, id[u] >> 5, in[u] ? (1u << (id[u] & 31u)) & ~seen[u] : 0u);
+        tr_set(nbits, id[u], in[u] ? v[u] & ~seen[u] : 0u);
     }
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
     lv = TrLevel{nbits, reinterpret_cast<uint2*>(nb + size_t(cap) * (kTrWords * 4)), n1};
@@ -751,7 +752,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
       e[u] = run[i];
       const uint32_t s0 = levels == 1 ? e[u].x >> kTrDigitBits : pslot[i];
       if (s0 < lv.ns) {
-        v[u] = __ldcg(lv.bits + s0 * kTrWords + ((e[u].x >> 5) & (kTrWords - 1u)));
+        v[u] = __ldcg(lv.bits + trie_word(s0, e[u].x & kTrDigit));
         r[u] = __ldcg(lv.rec + s0);
       }
     }

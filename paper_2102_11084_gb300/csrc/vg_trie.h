@@ -11,6 +11,9 @@ constexpr int kTrWords = (1 << kTrDigitBits) / 32;
 constexpr size_t kTrSlotBytes = kTrWords * 4 + 8;  // bits and record
 constexpr size_t kTrRowBytes = 32;                 // sums, carries and key
 static_assert(kTrWords == 4, "a slot's bits are one 16-byte word, its record three prefixes");
+// Word of a slot's child d among the words of its level.  (The number of the child's bit, slot
+// x 2^7 + d, passes 32 bits from 2^25 slots on; the word's does not.)
+constexpr uint32_t trie_word(uint32_t slot, uint32_t d) { return slot * kTrWords + (d >> 5); }
 constexpr int kTrMaxGrid = 1024;    // blocks of the launch at most
 // Bits of the first level at most (one bit per key prefix).  Up to kTrMidPoints points 2^26,
 // 2^24 of which (2 MB) every call of at most kTrMaxPoints clears while the extents are found
@@ -37,6 +40,12 @@ constexpr int64_t kTrCellShare = 4;
 constexpr uint32_t kTrMidBits = 27;
 constexpr uint32_t kTrSame = 2, kTrSameOf = 5;
 
+// Slots of a further level, and rows, that a call's buffers hold.
+constexpr int64_t trie_slots(int64_t n) { return n <= kTrMidPoints ? n : n / kTrCellShare; }
+static_assert(trie_word(static_cast<uint32_t>(trie_slots(kMaxPoints)) - 1u, kTrDigit) ==
+                  uint64_t(trie_slots(kMaxPoints) - 1) * kTrWords + (kTrDigit >> 5),
+              "32-bit word numbers for the largest call");
+
 constexpr int trie_root_bits(int64_t n) {
   return n <= kTrMidPoints ? kTrRootBits : kTrRootBitsLarge;
 }
@@ -62,7 +71,7 @@ constexpr TrieLayout trie_layout(int64_t n, int frames, size_t base, size_t att_
   TrieLayout L{};
   const int64_t nn = n < 1 ? 1 : n;
   const int root_bits = trie_root_bits(nn);
-  L.slots = nn <= kTrMidPoints ? nn : nn / kTrCellShare;
+  L.slots = trie_slots(nn);
   const size_t places = size_t(max_chunks(nn, frames)) * kChunk;
   size_t off = align_up(base, 256);
   L.root = off;
