@@ -546,7 +546,7 @@ constexpr uint32_t kLocalBatch = 4096;
 constexpr uint32_t kLocalHeads = 4096;  // lists (a power of two): a cell's by its low bits
 constexpr int kLocalAtOnce = 2;  // deleted points a warp tests at a time
 struct LocalSmem {
-  float4 node[kLocalBatch + 1];  // place (negated); w = the next rank of the list; a far point
+  float4 node[kLocalBatch + 1];  // place (negated); w = the next rank of the list; last, a NaN
   uint32_t cell[kLocalBatch];
   uint32_t head[kLocalHeads];
 };
@@ -644,8 +644,8 @@ __global__ __launch_bounds__(kLoopThreads, 1) void thin_local_kernel(const LoopA
     a.gone[k] = 0;
     a.rank[e] = static_cast<uint32_t>(k);
   }
-  if (threadIdx.x == 0)  // (at no finite distance)
-    sm.node[kLocalBatch] = make_float4(INFINITY, INFINITY, INFINITY, __uint_as_float(kListEnd));
+  if (threadIdx.x == 0)  // (NaN: within no radius, also where its square overflows)
+    sm.node[kLocalBatch] = make_float4(NAN, NAN, NAN, __uint_as_float(kListEnd));
   LocalGroup mine{};  // (no entries: no count is above the threshold)
   mine.nb = kNoCell;
   if (gw < groups) local_group_load(a, gw, mine);
