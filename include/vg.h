@@ -325,8 +325,9 @@ VG_API vg_status vg_map_extract(vg_map* map, uint64_t* out_keys, float* out_cent
  *   out_passes     host int32 or NULL: passes of the loop.
  * Workspace: vg_thin_workspace_bytes(n) bytes.  The call synchronises the stream twice:
  * all passes run in one cooperative launch that keeps every point's neighbour count.  Where
- * the points are so dense, or the batch so large, that counting afresh is cheaper, it
- * synchronises once per pass and once per round of the batch selection (8 bits a round).
+ * the points are so dense, or the batch so large, that counting afresh is cheaper (or the
+ * device cannot hold that launch), it synchronises once per pass and once per round of the
+ * batch selection (8 bits a round).
  */
 VG_API size_t vg_thin_workspace_bytes(int64_t n_points);
 VG_API vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float radius,
@@ -476,6 +477,11 @@ VG_API vg_status vg_debug_grid_barrier_timeout(uint32_t* scratch_words, uint32_t
 /* Test hook: limit of every chained-scan wait in later calls (0 restores the default
  * of about a second).  A wait that reaches it records VG_ERR_TIMEOUT and returns. */
 VG_API void vg_debug_set_spin_limit(uint32_t limit);
+
+/* Test hook: later calls take a cooperative launch of more than `blocks` blocks for one that
+ * the device cannot hold, as where SMs are withheld from the process (0 restores the device's
+ * own limit).  Such calls take their other routes: same results. */
+VG_API void vg_debug_set_cooperative_blocks(int blocks);
 
 #ifdef __cplusplus
 }

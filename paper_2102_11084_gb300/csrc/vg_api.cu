@@ -18,6 +18,7 @@ namespace vg {
 
 namespace {
 std::atomic<uint32_t> g_spin_limit{0};
+std::atomic<int> g_coop_limit{0};
 void** g_events = nullptr;
 int g_max_events = 0;
 bool g_events_paused = false;
@@ -90,6 +91,16 @@ int persistent_grid(const void* kernel, int threads, size_t dyn_smem, int64_t wo
   const int64_t cap = int64_t(blocks) * num_sms();
   const int64_t g = work_tiles < cap ? work_tiles : cap;
   return static_cast<int>(g < 1 ? 1 : g);
+}
+
+cudaError_t launch_cooperative(const void* kernel, int64_t blocks, int threads, void** args,
+                               size_t dyn_smem, cudaStream_t stream) {
+  const int limit = g_coop_limit.load(std::memory_order_relaxed);
+  if (limit > 0 && blocks > limit) return cudaErrorCooperativeLaunchTooLarge;
+  const cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(static_cast<unsigned>(blocks)),
+                                                    dim3(threads), args, dyn_smem, stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge) (void)cudaGetLastError();
+  return e;
 }
 
 namespace {
@@ -225,8 +236,7 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
         for (int k = 1; k < 1 + 1 + 1 + 3 + kMaxPasses + 1; ++k) mark(stage + k, stream);
         return cuda_status(et);
       }
-      (void)cudaGetLastError();  // (SMs withheld from this process: the sort path)
-    }
+    }  // (too large: the sort path)
     const bool try_trie = trie && n > kTrMaxPoints;
 
     // (the frame path needs only the state and frame state cleared: its last kernel
@@ -263,10 +273,7 @@ vg_status run_frames(const float* xyz, const FramesArg& fr, bool from_min, const
     mark(stage++, stream);
     if (e == cudaSuccess && try_trie) {
       e = launch_trie(xyz, frn, st, fs, ws, TL, out, spins, err, stream);
-      if (e == cudaErrorCooperativeLaunchTooLarge) {  // (SMs withheld from this process)
-        (void)cudaGetLastError();
-        e = cudaSuccess;
-      }
+      if (e == cudaErrorCooperativeLaunchTooLarge) e = cudaSuccess;
     }
     if (e == cudaSuccess && !frame_path)
       e = launch_keys_any(xyz, frn, have_extent, st, fs, keys0, k32_0, pay_0, err, stream);
@@ -398,6 +405,10 @@ int vg_set_stage_events(void** events, int max_events) {
 
 void vg_debug_set_spin_limit(uint32_t limit) {
   g_spin_limit.store(limit, std::memory_order_relaxed);
+}
+
+void vg_debug_set_cooperative_blocks(int blocks) {
+  g_coop_limit.store(blocks, std::memory_order_relaxed);
 }
 
 vg_status vg_debug_wait_timeout(uint32_t* scratch_words, uint32_t limit, int32_t* out_error,

@@ -270,6 +270,11 @@ uint32_t spin_limit();
 // Grid of a persistent kernel: all its blocks resident at once (occupancy x SMs), at most
 // one block per unit of work.  Sets the dynamic shared-memory limit when needed.
 int persistent_grid(const void* kernel, int threads, size_t dyn_smem, int64_t work_tiles);
+// A cooperative launch, or cudaErrorCooperativeLaunchTooLarge (and no pending error) where its
+// blocks cannot all be resident -- SMs withheld from the process, or the test hook's limit --
+// so that the caller takes its other route.
+cudaError_t launch_cooperative(const void* kernel, int64_t blocks, int threads, void** args,
+                               size_t dyn_smem, cudaStream_t stream);
 // Runs the occupancy queries of every persistent kernel on the current device (so that a
 // later CUDA-graph capture makes none).
 void warm_launch_config();

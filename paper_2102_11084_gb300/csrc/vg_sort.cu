@@ -333,10 +333,9 @@ cudaError_t launch_sort(State* st, uint64_t* keys0, uint32_t* idx0, uint64_t* ke
              compact_input ? 1 : 0, spin_limit, err};
   int first = 0, last = max_passes;
   void* args[] = {&a, &first, &last};
-  cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(onesweep_kernel),
-                                              dim3(tiles), dim3(kSortThreads), args, 0, stream);
+  const cudaError_t e = launch_cooperative(reinterpret_cast<const void*>(onesweep_kernel), tiles,
+                                           kSortThreads, args, 0, stream);
   if (e != cudaErrorCooperativeLaunchTooLarge) return e;
-  (void)cudaGetLastError();  // (SMs withheld from this process: a launch a pass)
   for (int p = 0; p < max_passes; ++p)
     onesweep_kernel<<<tiles, kSortThreads, 0, stream>>>(a, p, p + 1);
   return cudaGetLastError();

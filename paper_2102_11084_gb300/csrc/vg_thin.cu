@@ -24,7 +24,8 @@
 //              neighbour of a deleted point.  No pass reads the other points again and none
 //              goes through the host.
 //   recounted  where the points are so dense, or the batch so large, that the deleted points
-//              meet more candidates than a fresh count (which stops at the threshold):
+//              meet more candidates than a fresh count (which stops at the threshold), or the
+//              device cannot hold the cooperative launch:
 //              thin_count_kernel counts and marks every pass, the host reads the number
 //              marked and finds the batch by a radix select on 256-bin histograms
 //              (thin_hist_kernel), thin_delete_kernel removes it.
@@ -780,6 +781,22 @@ __global__ __launch_bounds__(256) void thin_count_kernel(
   if ((threadIdx.x & 31) == 0 && marked) atomicAdd(marked_count, marked);
 }
 
+// The arrays of this form that the kept counts' cells, groups and flags have overwritten.
+__global__ __launch_bounds__(256) void thin_refill_kernel(const State* st,
+                                                          const float4* __restrict__ pos,
+                                                          const uint32_t* __restrict__ prio,
+                                                          uint32_t* sprio, uint32_t* sidx,
+                                                          uint8_t* state, const int* err) {
+  if (error_raised(err)) return;
+  const int64_t m = st->nitems;
+  for (int64_t i = blockIdx.x * int64_t(256) + threadIdx.x; i < m; i += int64_t(gridDim.x) * 256) {
+    const uint32_t p = __float_as_uint(pos[i].w);
+    sprio[i] = prio[p];
+    sidx[i] = p;
+    state[i] = kAlive;
+  }
+}
+
 __device__ __forceinline__ uint64_t select_key(const uint32_t* sprio, const uint32_t* sidx,
                                                int64_t i) {
   return (uint64_t(sprio[i]) << 32) | sidx[i];
@@ -1042,9 +1059,8 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
       la.off = reinterpret_cast<uint32_t*>(keys0);
       la.gone = reinterpret_cast<uint8_t*>(la.off + align_up(size_t(n), 4));
       la.rank = entry;
-      e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(thin_local_kernel),
-                                      dim3(local_grid), dim3(kLoopThreads), args,
-                                      sizeof(LocalSmem), stream);
+      e = launch_cooperative(reinterpret_cast<const void*>(thin_local_kernel), local_grid,
+                             kLoopThreads, args, sizeof(LocalSmem), stream);
     } else {
       // the deleted lists' heads (a cell each) and nodes (16 bytes a point of the batch, in
       // the 16 bytes a point from keys1 to the end of idx1), or `sel`
@@ -1053,18 +1069,22 @@ vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float 
       la.sel = reinterpret_cast<uint32_t*>(keys0);
       la.head = reinterpret_cast<unsigned long long*>(keys0);
       la.node = reinterpret_cast<float4*>(keys1);
-      e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(thin_loop_kernel),
-                                      dim3(loop_grid), dim3(kLoopThreads), args, 0, stream);
+      e = launch_cooperative(reinterpret_cast<const void*>(thin_loop_kernel), loop_grid,
+                             kLoopThreads, args, 0, stream);
     }
-    if (e != cudaSuccess) return VG_ERR_CUDA;
-    thin_keep_kernel<<<g, 256, 0, stream>>>(st, pos, cnt, state, thr, out_keep, ctr + kCtrKept,
-                                            err);
-    thin_finish_kernel<<<1, 1, 0, stream>>>(ctr + kCtrKept, out_num_kept);
-    uint32_t run = 0;
-    e = cudaMemcpyAsync(&run, ctr + kCtrPasses, sizeof(run), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (out_passes) *out_passes = static_cast<int32_t>(run);
-    return thin_status(e == cudaSuccess ? cudaGetLastError() : e);
+    if (e == cudaSuccess) {
+      thin_keep_kernel<<<g, 256, 0, stream>>>(st, pos, cnt, state, thr, out_keep, ctr + kCtrKept,
+                                              err);
+      thin_finish_kernel<<<1, 1, 0, stream>>>(ctr + kCtrKept, out_num_kept);
+      uint32_t run = 0;
+      e = cudaMemcpyAsync(&run, ctr + kCtrPasses, sizeof(run), cudaMemcpyDeviceToHost, stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+      if (out_passes) *out_passes = static_cast<int32_t>(run);
+      return thin_status(e == cudaSuccess ? cudaGetLastError() : e);
+    }
+    if (e != cudaErrorCooperativeLaunchTooLarge) return VG_ERR_CUDA;
+    thin_refill_kernel<<<g, 256, 0, stream>>>(st, pos, priority, sprio, sidx, state, err);
+    e = cudaSuccess;  // (the launch does not fit: counted afresh every pass)
   }
   for (; n > 0 && passes < max_passes; ++passes) {
     uint32_t marked = 0;

@@ -969,9 +969,7 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   }
   void* args[] = {&a};
   const void* fn = reinterpret_cast<const void*>(trie_kernel_of(posed(fr), a.large != 0));
-  return cudaLaunchCooperativeKernel(fn, dim3(static_cast<unsigned>(g)), dim3(kTrThreads), args,
-                                     
-                                     tr_frames_bytes(fr.nframes, posed(fr)), stream);
+  return launch_cooperative(fn, g, kTrThreads, args, tr_frames_bytes(fr.nframes, posed(fr)), stream);
 }
 
 }  // namespace vg

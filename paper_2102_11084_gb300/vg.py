@@ -73,6 +73,7 @@ _SIGS = {
                        ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                        ctypes.c_size_t, ctypes.c_int, ctypes.c_void_p], ctypes.c_int),
     "vg_debug_set_spin_limit": ([ctypes.c_uint32], None),
+    "vg_debug_set_cooperative_blocks": ([ctypes.c_int], None),
     "vg_downsample_noalloc": ([ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p, ctypes.c_float,
                                ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64,
                                ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int,
