@@ -10,6 +10,7 @@
 
 #include "../../include/vg.h"
 #include "vg_api_internal.h"
+#include "vg_device_int.h"
 #include "vg_internal.h"
 #include "vg_frame.h"
 #include "vg_trie.h"
@@ -22,7 +23,7 @@ std::atomic<int> g_coop_limit{0};
 void** g_events = nullptr;
 int g_max_events = 0;
 bool g_events_paused = false;
-int g_sms[64] = {0};
+DeviceInt g_sms;
 constexpr int kMaxStages = 20;
 }  // namespace
 
@@ -33,14 +34,12 @@ uint32_t spin_limit() {
 
 int num_sms() {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 132;
-  if (g_sms[dev] == 0) {
+  if (cudaGetDevice(&dev) != cudaSuccess) return 132;
+  const int sms = g_sms.get(dev, [dev] {
     int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-      v = 132;
-    g_sms[dev] = v;
-  }
-  return g_sms[dev];
+    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? v : 0;
+  });
+  return sms > 0 ? sms : 132;
 }
 
 void pause_stage_events(bool paused) { g_events_paused = paused; }

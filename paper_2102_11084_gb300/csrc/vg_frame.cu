@@ -30,6 +30,7 @@
 #include <cstddef>
 
 #include "vg_device.cuh"
+#include "vg_device_int.h"
 #include "vg_internal.h"
 #include "vg_frame.h"
 #include "vg_rows.cuh"
@@ -1050,11 +1051,10 @@ static_assert(kFrSmem + 1024 <= 227 * 1024, "bin block shared memory");
 namespace {
 // Blocks of the one-launch kernel resident on an SM (0: it cannot run), per device.
 int fused_blocks_per_sm(bool posed) {
-  static int cache[64][2];
+  static DeviceInt cache[2];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  int& b = cache[dev][posed ? 1 : 0];
-  if (b == 0) {
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  return cache[posed ? 1 : 0].get(dev, [posed] {
     const void* fn = posed ? reinterpret_cast<const void*>(frame_fused_kernel<true>)
                            : reinterpret_cast<const void*>(frame_fused_kernel<false>);
     int v = 0;
@@ -1063,9 +1063,8 @@ int fused_blocks_per_sm(bool posed) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, fn, kFzThreads, kFzSmem) != cudaSuccess)
       v = 0;
     (void)cudaGetLastError();
-    b = v > 0 ? v : -1;
-  }
-  return b > 0 ? b : 0;
+    return v;
+  });
 }
 
 int fused_grid(bool posed) {

@@ -43,6 +43,7 @@
 #include <cstddef>
 
 #include "vg_device.cuh"
+#include "vg_device_int.h"
 #include "vg_internal.h"
 #include "vg_rows.cuh"
 #include "vg_stream.cuh"
@@ -905,11 +906,10 @@ TrKernel trie_kernel_of(bool posed, bool large) {
   return large ? trie_kernel<false, kTrLaneLarge> : trie_kernel<false, kTrLane>;
 }
 int trie_blocks_per_sm(bool posed, bool large) {
-  static int cache[64][2][2];
+  static DeviceInt cache[2][2];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  int& b = cache[dev][posed ? 1 : 0][large ? 1 : 0];
-  if (b == 0) {
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  return cache[posed ? 1 : 0][large ? 1 : 0].get(dev, [posed, large] {
     const void* fn = reinterpret_cast<const void*>(trie_kernel_of(posed, large));
     int v = 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -917,9 +917,8 @@ int trie_blocks_per_sm(bool posed, bool large) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, fn, kTrThreads, kTrSmem) != cudaSuccess)
       v = 0;
     (void)cudaGetLastError();
-    b = v > 0 ? v : -1;
-  }
-  return b > 0 ? b : 0;
+    return v;
+  });
 }
 
 }  // namespace
