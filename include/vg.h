@@ -130,7 +130,9 @@ VG_API const char* vg_status_string(int status);
 /* Library ABI version (major * 100 + minor). */
 VG_API int vg_version(void);
 
-/* Bytes of device workspace vg_downsample needs for a cloud of n_points with `flags`.
+/* Bytes of device workspace vg_downsample needs for clouds of up to n_points with `flags` (this
+ * and the other queries never fall as n_points grows: a workspace for the largest cloud holds
+ * what every smaller one takes).
  * Pure host function; returns 0 for a negative n_points. */
 VG_API size_t vg_downsample_workspace_bytes(int64_t n_points, int flags);
 

@@ -160,6 +160,23 @@ size_t frames_workspace_bytes(int64_t n, int frames, int flags) {
   return a > b ? a : b;
 }
 
+namespace {
+// The largest need(m) of clouds of m <= n points: a workspace asked for n holds the smaller ones
+// too.  (AUTO's need falls at two sizes, from where on the trie's buffers hold a share of the
+// points, or not the attributes; at every other step it grows.)
+template <typename Need>
+size_t most_up_to(int64_t n, Need need) {
+  size_t most = need(n);
+  for (const int64_t m : {kTrMidPoints, kTrieAttrPoints})
+    if (m < n) most = need(m) > most ? need(m) : most;
+  return most;
+}
+}  // namespace
+
+size_t frames_workspace_query(int64_t n, int frames, int flags) {
+  return most_up_to(n, [&](int64_t m) { return frames_workspace_bytes(m, frames, flags); });
+}
+
 vg_status check_outputs(int64_t n, const float* xyz, uint64_t* out_keys, float* out_centroids,
                         uint32_t* out_counts, int64_t cap, const int64_t* num_voxels,
                         const int32_t* p2v, const int32_t* out_error, const void* workspace) {
@@ -437,14 +454,14 @@ vg_status vg_debug_grid_barrier_timeout(uint32_t* scratch_words, uint32_t limit,
 }
 
 size_t vg_downsample_workspace_bytes(int64_t n_points, int flags) {
-  return frames_workspace_bytes(n_points, 1, flags);
+  return frames_workspace_query(n_points, 1, flags);
 }
 
 int64_t vg_frame_one_launch_points(int posed) { return frame_fused_max_points(posed != 0); }
 
 size_t vg_batch_workspace_bytes(int64_t n_total, int n_frames, int flags) {
   if (n_frames < 1 || n_frames > kMaxFrames) return 0;
-  return frames_workspace_bytes(n_total, n_frames, flags);
+  return frames_workspace_query(n_total, n_frames, flags);
 }
 
 vg_status vg_downsample(const float* xyz, int64_t n, float* origin, float leaf,
@@ -509,9 +526,11 @@ static size_t ex_base(int64_t n, int frames, int flags, bool attrs) {
 size_t vg_downsample_ex_workspace_bytes(int64_t n_total, int n_frames, int flags,
                                         const vg_voxel_extras* extras) {
   if (n_total < 0 || n_frames < 1 || n_frames > kMaxFrames) return 0;
-  const size_t base = ex_base(n_total, n_frames, flags, extras && extras->attrs);
-  if (!extras || extras->min_count <= 1) return base;
-  return filter_layout(n_total, base).total;
+  const bool attrs = extras && extras->attrs, filtered = extras && extras->min_count > 1;
+  return most_up_to(n_total, [&](int64_t m) {
+    const size_t base = ex_base(m, n_frames, flags, attrs);
+    return filtered ? filter_layout(m, base).total : base;
+  });
 }
 
 vg_status vg_downsample_frames_ex(const float* xyz, int64_t n_total,
@@ -575,7 +594,9 @@ vg_status vg_downsample_frames_ex(const float* xyz, int64_t n_total,
 size_t vg_pyramid_workspace_bytes(int64_t n_points, int levels, int flags) {
   (void)flags;
   if (n_points < 0 || levels < 1 || levels > kMaxLevels) return 0;
-  return pyramid_layout(n_points, levels, frames_workspace_bytes(n_points, 1, VG_METHOD_AUTO)).total;
+  return most_up_to(n_points, [&](int64_t m) {
+    return pyramid_layout(m, levels, frames_workspace_bytes(m, 1, VG_METHOD_AUTO)).total;
+  });
 }
 
 vg_status vg_pyramid(const float* xyz, int64_t n, float* origin, float leaf, int levels,

@@ -18,7 +18,6 @@
 #include "../../include/vg.h"
 #include "vg_api_internal.h"
 #include "vg_internal.h"
-#include "vg_trie.h"
 
 struct vg_plan {
   int device = 0;
@@ -85,14 +84,10 @@ vg_status vg_plan_create(vg_plan** out, int max_frames, int64_t max_points, int 
     return VG_ERR_INVALID_ARG;
   }
   // room for every grouping a later configure may pick
-  const size_t a = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_SORT | VG_SORT_FRAME);
-  const size_t b = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_HASH);
-  const size_t small = vg::frames_workspace_bytes(
-      max_points < vg::kTrMidPoints ? max_points : vg::kTrMidPoints, max_frames, VG_METHOD_AUTO);
-  const size_t large = vg::frames_workspace_bytes(max_points, max_frames, VG_METHOD_AUTO);
-  p->ws_bytes = 0;
-  for (const size_t w : {a, b, small, large})
+  for (const int f : {VG_METHOD_SORT | VG_SORT_FRAME, VG_METHOD_HASH, VG_METHOD_AUTO}) {
+    const size_t w = vg::frames_workspace_query(max_points, max_frames, f);
     if (w > p->ws_bytes) p->ws_bytes = w;
+  }
   if (cudaMalloc(&p->ws, p->ws_bytes) != cudaSuccess) {
     delete p;
     return VG_ERR_CUDA;
