@@ -52,8 +52,23 @@ class _Request(NamedTuple):
     future: Future
 
 
+def slot_workspaces(n_slots: int, other: int, full: int, least: int,
+                    mem_budget: Optional[int]) -> list:
+    """Workspace bytes of each slot a budget holds (always one): as many slots as fit, up to
+    n_slots, with the least workspace the method accepts, then the full one -- what its
+    fastest grouping takes -- in as many of them as the rest of the budget holds.  ``other``: a
+    slot's other device bytes."""
+    if mem_budget is None:
+        return [full] * max(1, n_slots)
+    n = min(max(1, n_slots), max(1, mem_budget // (other + least)))
+    more = max(0, mem_budget - n * (other + least))
+    wide = n if full <= least else min(n, more // (full - least))
+    return [full] * wide + [least] * (n - wide)
+
+
 class _Slot:
-    def __init__(self, device, max_points: int, max_frames: int, method: str):
+    def __init__(self, device, max_points: int, max_frames: int, method: str,
+                 workspace_bytes: int):
         self.stream = torch.cuda.Stream(device=device)
         self.max_points = max_points
         self.max_frames = max_frames
@@ -69,8 +84,7 @@ class _Slot:
         self.counts = torch.empty(cap, dtype=torch.int32, device=d)
         self.out_offsets = torch.zeros(max_frames + 1, dtype=torch.int64, device=d)
         self.error = torch.zeros(1, dtype=torch.int32, device=d)
-        nbytes = int(vg.lib().vg_batch_workspace_bytes(cap, max_frames, self.flags))
-        self.workspace = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=d)
+        self.workspace = torch.empty(max(workspace_bytes, 256), dtype=torch.uint8, device=d)
         self.h_xyz = torch.empty((cap, 3), dtype=torch.float32).pin_memory()
         self.h_off_in = torch.zeros(max_frames + 1, dtype=torch.int64).pin_memory()
         self.h_leaf_in = torch.ones(max_frames, dtype=torch.float32).pin_memory()
@@ -86,6 +100,13 @@ class _Slot:
         self.batch: list = []
         self.busy = False
         self.copying = False
+
+    @staticmethod
+    def other_bytes(max_points: int, max_frames: int) -> int:
+        """Device bytes of a slot beside its workspace."""
+        points = 12 + 8 + 12 + 4           # cloud; keys, centroids, counts
+        frames = 8 + 4 + 12 + 8            # offsets, leaves, origins, row offsets
+        return max(max_points, 1) * points + max_frames * frames + 2 * 8 + 4
 
     def device_bytes(self) -> int:
         ts = [self.xyz, self.offsets, self.leaves, self.origins, self.keys, self.centroids,
@@ -211,7 +232,8 @@ class Server:
     max_frames   most requests in one batch.
     n_slots      device slots (>= 2 lets a batch's copies overlap another's decimation; with
                  3, one batch can be copied in and another copied out while a third runs).
-    mem_budget   device bytes the slots may hold; fewer slots are made if needed.
+    mem_budget   device bytes the slots may hold; where it is short, "auto" slots get the sort
+                 path's smaller workspace, then fewer slots are made.
     """
 
     def __init__(self, *, max_points: int = 8 * 307_200, max_frames: int = 16, n_slots: int = 3,
@@ -224,15 +246,14 @@ class Server:
             self._t0 = torch.cuda.Event(enable_timing=True)
             self._t0.record(torch.cuda.current_stream(dev))
             self._t0.synchronize()
-        self.slots = []
-        used = 0
-        for _ in range(max(1, n_slots)):
-            s = _Slot(dev, max_points, max_frames, method)
-            if mem_budget is not None and self.slots and used + s.device_bytes() > mem_budget:
-                del s
-                break
-            used += s.device_bytes()
-            self.slots.append(s)
+        # AUTO runs in the sort path's workspace as well, with the same results
+        flags = vg.method_flag(method)
+        least = vg.METHOD_SORT if flags == vg.METHOD_AUTO else flags
+        query = lambda f: int(vg.lib().vg_batch_workspace_bytes(max(max_points, 1), max_frames, f))
+        self.slots = [_Slot(dev, max_points, max_frames, method, w) for w in slot_workspaces(
+            n_slots, _Slot.other_bytes(max_points, max_frames), query(flags), query(least),
+            mem_budget)]
+        used = sum(s.device_bytes() for s in self.slots)
         self.device_bytes = used
         self.max_points = max_points
         self.max_frames = max_frames
