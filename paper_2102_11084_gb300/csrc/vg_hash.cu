@@ -9,8 +9,9 @@
 // centroid formula as the sort path, so both paths give identical bits.
 //
 //   hash_insert_kernel   key per point; runs of equal keys within 32 consecutive points (eight
-//                        threads' four) merged and queued by warp; 32 queued runs at a time
-//                        claim or find their slots and add to them
+//                        threads' four) merged and queued by warp; 32 queued runs at a time,
+//                        in a crowded cloud merged once more, claim or find their slots and
+//                        add to them
 //   hash_insert_p2v_kernel  the same for calls that want point_to_voxel: points of a warp with
 //                        equal keys are merged (match.any) and their leader claims/updates one
 //                        slot, which every point of the group records
@@ -27,6 +28,12 @@
 // The insert is bound by instruction issue (keys, offsets) and by L2's atomics: 64 posed
 // frames (29M points) 417 us; runs within a thread's four points only, 475; merging by
 // match.any lane group by lane group with four atomics a group, 954.
+// In a crowded cloud without order (few cells, or one cell with a tenth of the points) the atomics
+// meet on a few addresses, at 1.3 cycles a lane each: the queue's runs of one key are merged
+// first (queue_merge).  50M shuffled points of 2 cells 16.9 -> 1.7 ms, of 10 cells 6.7 -> 3.6 (merging
+// every point's group by match.any, as the point_to_voxel form does: 5.2 and 5.3); half of the
+// points in one of 1M cells 27.5 -> 9.0.  The merge is out of line and behind a test of two ballots:
+// in line it spilled, and the 64 frames took 5 % longer; tested by up to four keys of every drain, 7 %.
 #include "vg_device.cuh"
 #include "vg_internal.h"
 #include "vg_stream.cuh"
@@ -152,8 +159,44 @@ struct InsertQueue {
   unsigned long long key[kQueue];
   unsigned long long xy[kQueue];  // sum x | sum y << 32
   uint32_t zn[kQueue];            // sum z | points << 26
+  unsigned long long hot;         // a key that came back, or the last drain's first
 };
 constexpr size_t kInsertSmem = (kStreamThreads / 32) * sizeof(InsertQueue);
+
+// A crowded cloud's drain (below): merges the warp's runs of one key where three or more meet;
+// the first one's lane keeps their sums, the others nothing (kNoKey).
+struct QueueRun {
+  uint64_t key;
+  unsigned long long a, b;  // as table_add's va, vb
+};
+__device__ __noinline__ QueueRun queue_merge(QueueRun r, unsigned long long* hot_key) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t mine = r.key, hot = *hot_key;
+  uint32_t untried = __ballot_sync(kFullMask, mine != kNoKey);
+  uint64_t k = __any_sync(kFullMask, mine == hot) ? hot : __shfl_sync(kFullMask, mine, 0);
+  for (int misses = 0; untried && misses < 4;) {
+    const uint32_t same = __ballot_sync(kFullMask, mine == k) & untried;
+    if (__popc(same) >= 3) {
+      const bool in = (same >> lane) & 1u, first = int(lane) == __ffs(same) - 1;
+      uint32_t w[4] = {uint32_t(r.a), uint32_t(r.a >> 32), uint32_t(r.b), uint32_t(r.b >> 32)};
+#pragma unroll
+      for (int c = 0; c < 4; ++c)  // (32 runs of 26 bits: below 2^32)
+        w[c] = __reduce_add_sync(kFullMask, in ? w[c] : 0u);
+      if (first) {
+        r.a = w[0] | ((unsigned long long)w[1] << 32);
+        r.b = w[2] | ((unsigned long long)w[3] << 32);
+        *hot_key = k;
+      } else if (in) {
+        r.key = kNoKey;
+      }
+    } else {
+      ++misses;
+    }
+    untried &= ~same;
+    k = __shfl_sync(kFullMask, mine, __ffs(untried) - 1);
+  }
+  return r;
+}
 
 template <bool kPosed>
 __global__ __launch_bounds__(kStreamThreads, 3) void hash_insert_kernel(
@@ -165,6 +208,8 @@ __global__ __launch_bounds__(kStreamThreads, 3) void hash_insert_kernel(
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   InsertQueue& q = reinterpret_cast<InsertQueue*>(hi_smem)[warp];
   uint32_t qn = 0;  // queued runs (the same in every lane)
+  if (lane == 0) q.hot = kNoKey;
+  __syncwarp();
   const uint32_t T = build_chunk_map(fr, sm.off, sm.cstart, sm.tmp, err);
   const uint32_t key_shift = frame_prologue(fr, have_extent != 0, st, fs, T, sm, err);
   // a warp takes every W-th piece of 128 points: no block waits for its slowest warp, and the
@@ -244,11 +289,22 @@ __global__ __launch_bounds__(kStreamThreads, 3) void hash_insert_kernel(
     while (qn > left) {
       const uint32_t take = min(qn, 32u);
       qn -= take;
+      QueueRun r{kNoKey, 0ull, 0ull};
       if (uint32_t(lane) < take) {
         const uint32_t b = q.zn[qn + lane];
-        (void)table_add(tab, q.key[qn + lane], q.xy[qn + lane],
-                        (b & 0x3ffffffu) | ((unsigned long long)(b >> 26) << 32), spin_limit, err);
+        r = QueueRun{q.key[qn + lane], q.xy[qn + lane],
+                     (b & 0x3ffffffu) | ((unsigned long long)(b >> 26) << 32)};
       }
+      // crowded: a quarter of the runs have lane 0's key, or two have one that the warp has
+      // met before (pieces of a scan lie apart: theirs do not come back)
+      const uint64_t lead = __shfl_sync(kFullMask, r.key, 0), hot = q.hot;
+      const int again = __popc(__ballot_sync(kFullMask, r.key == hot && hot != kNoKey));
+      if (again >= 2 || __popc(__ballot_sync(kFullMask, r.key == lead)) >= 8)
+        r = queue_merge(r, &q.hot);
+      else if (again == 0 && lane == 0)
+        q.hot = lead;
+      if (r.key != kNoKey) (void)table_add(tab, r.key, r.a, r.b, spin_limit, err);
+      __syncwarp();
     }
     __syncwarp();
   }
