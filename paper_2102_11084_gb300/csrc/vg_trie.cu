@@ -30,8 +30,9 @@
 //             merges anything (a camera frame's warp meets few words, a shuffled cloud's many);
 //   count, rank
 //   add       a run's points and sums at its row, with two 64-bit atomics whose returned
-//             values tell the carries out of their 32-bit halves; attribute sums and, through
-//             the runs, point_to_voxel here too;
+//             values tell the carries out of their 32-bit halves (rows that many runs meet
+//             first in the block's shared memory); attribute sums and, through the runs,
+//             point_to_voxel here too;
 //   rows      one thread a row: the centroid, by the formula and from the integer sums of every
 //             other grouping, so the rows are theirs bit for bit.
 // Bound by the latency of the passes and barriers (1.2 us each) for a camera frame, by
@@ -52,7 +53,6 @@
 namespace vg {
 namespace {
 
-constexpr int kTrAdd = 1;  // runs a lane adds at a time
 // Consecutive points of a lane in the marking pass: calls of up to kTrMaxPoints points, larger
 // ones.
 constexpr int kTrLane = 2, kTrLaneLarge = 4;
@@ -76,6 +76,7 @@ struct TrArgs {
   uint32_t* stat;      // per level (8): the blocks' totals
   SegOut out;
   int64_t slots;       // slots and rows the buffers hold
+  uint32_t hot;        // entries of a block's table of hot rows (a power of two)
   uint32_t chunks;     // chunks of points at most
   int root_bits;
   int large;           // after the extent kernel; the call may be left to the sort path
@@ -88,6 +89,7 @@ struct TrSmem {
   uint32_t bits[kTrThreads / 32];
   uint32_t first;
   uint32_t nruns;
+  uint32_t hot;  // some entry of the table of hot rows is taken
 };
 
 // Tables of a call's frames (dynamic shared memory).
@@ -374,6 +376,58 @@ struct TrRows {
   int64_t cap;
   uint32_t rows;
 };
+
+// A run's sums at a row: x + y 2^32 and z + points 2^32, and the carries that the old values
+// tell (and those the sums themselves hold beyond 64 and 32 bits).
+__device__ __forceinline__ void tr_add(const TrRows& R, uint32_t row, unsigned long long va,
+                                       unsigned long long vb, uint32_t hx = 0u, uint32_t hy = 0u,
+                                       uint32_t hz = 0u) {
+  const unsigned long long oa = atomicAdd(R.A + row, va), ob = atomicAdd(R.B + row, vb);
+  // carries out of a 32-bit half: x into y, A out of 64 bits, z into the points
+  const unsigned long long cx = hx + (((oa & 0xffffffffull) + (va & 0xffffffffull)) >> 32);
+  const unsigned long long cy = hy + (oa + va < oa ? 1ull : 0ull);
+  const unsigned long long cz = hz + (((ob & 0xffffffffull) + (vb & 0xffffffffull)) >> 32);
+  if (cx | cy | cz) atomicAdd(R.C + row, cx | (cy << 21) | (cz << 42));
+}
+
+// Rows that many of a block's runs meet, summed in its shared memory before the rows are
+// touched: in a crowded cloud without order the atomics of all blocks meet on a few sectors of
+// L2.  Entry `row` mod the entries, first come, first kept.  Where there are fewer rows than
+// entries, and runs for them, every row has its own; else a row takes one once a warp has met
+// it again, or eight times in 32 runs.  Shuffled points, before -> after (and the radix sort): 2.5M
+// of 10 cells 1255 -> 102 us (289), of 1000 cells 351 -> 118 (258), a quarter in one of 100,000
+// cells 551 -> 156 (362); 4M of 100 cells 879 -> 190 (302).  The tests of a run cost clouds that
+// are not crowded nothing that shows (2.5M points of 2.16M cells 216 and 217 us).
+struct TrHot {
+  uint32_t *tag, *x, *y, *z, *n, *carry;  // (carries of the sums, 10 bits each)
+  uint32_t* att;                          // sums of 4 channels an entry
+  uint32_t mask;
+};
+constexpr uint32_t kTrHotWords = 6, kTrHotAttWords = 4;
+constexpr uint32_t kTrNoRow = 0xffffffffu;
+constexpr uint32_t kTrHotPlaces = 1u << 21;  // points of a block whose carries fit 10 bits
+static_assert((uint64_t(kTrHotPlaces) * 0x1fffffu) >> 32 < 1024, "10-bit carries");
+__device__ __forceinline__ TrHot tr_hot(uint32_t* mem, uint32_t entries) {
+  TrHot h;
+  h.tag = mem;
+  h.x = h.tag + entries;
+  h.y = h.x + entries;
+  h.z = h.y + entries;
+  h.n = h.z + entries;
+  h.carry = h.n + entries;
+  h.att = h.carry + entries;
+  h.mask = entries - 1u;
+  return h;
+}
+// Adds to an entry; true for the entry's first run.
+__device__ __forceinline__ bool tr_hot_add(const TrHot& h, uint32_t e, uint32_t x, uint32_t y,
+                                           uint32_t z, uint32_t n) {
+  const uint32_t ox = atomicAdd(h.x + e, x), oy = atomicAdd(h.y + e, y), oz = atomicAdd(h.z + e, z);
+  const uint32_t c = (ox + x < x ? 1u : 0u) | (oy + y < y ? 1u << 10 : 0u) |
+                     (oz + z < z ? 1u << 20 : 0u);
+  if (c) atomicAdd(h.carry + e, c);
+  return atomicAdd(h.n + e, n) == 0u;
+}
 
 template <bool kPosed, int K>
 __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
@@ -721,6 +775,17 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
       R.att[i + cap] = 0ull;
     }
   }
+  const uint32_t hot_entries = places <= kTrHotPlaces ? a.hot : 0u;  // (the same in every thread)
+  const TrHot hot = tr_hot(reinterpret_cast<uint32_t*>(tr_smem + tr_frames_bytes(F, kPosed)), a.hot);
+  const bool all_hot = rows <= hot_entries && nruns / 2u >= rows;
+  for (uint32_t e = threadIdx.x; e < hot_entries; e += kTrThreads) {
+    hot.tag[e] = all_hot && e < rows ? e : kTrNoRow;
+    hot.x[e] = hot.y[e] = hot.z[e] = hot.n[e] = hot.carry[e] = 0u;
+  }
+  if (with_attrs)
+    for (uint32_t e = threadIdx.x; e < kTrHotAttWords * hot_entries; e += kTrThreads)
+      hot.att[e] = 0u;
+  if (threadIdx.x == 0) sm.hot = all_hot ? 1u : 0u;
   if (blockIdx.x == 0) {
     if (threadIdx.x == 0) {
       // more cells than output rows: recorded once, here; the first cap rows are written
@@ -738,66 +803,88 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
 
   // ---- every run's points and sums at its row ----
-  for (uint32_t i0 = 0; i0 < nruns; i0 += kTrThreads * kTrAdd) {
-    uint4 e[kTrAdd];
-    uint2 r[kTrAdd];
-    uint32_t v[kTrAdd], row[kTrAdd];
-    unsigned long long oa[kTrAdd], ob[kTrAdd], va[kTrAdd], vb[kTrAdd];
-#pragma unroll
-    for (int u = 0; u < kTrAdd; ++u) {
-      const uint32_t i = i0 + kTrThreads * u + threadIdx.x;
-      v[u] = 0u;
-      r[u] = make_uint2(~0u, 0u);
-      e[u] = zero4;
-      if (i >= nruns) continue;
-      e[u] = run[i];
-      const uint32_t s0 = levels == 1 ? e[u].x >> kTrDigitBits : pslot[i];
+  uint32_t met = kTrNoRow;  // a row that the warp has met, looked for again
+  for (uint32_t i0 = 0; i0 < nruns; i0 += kTrThreads) {
+    const uint32_t i = i0 + threadIdx.x;
+    uint4 e = zero4;
+    uint32_t row = kTrNoRow;
+    if (i < nruns) {
+      e = run[i];
+      const uint32_t s0 = levels == 1 ? e.x >> kTrDigitBits : pslot[i];
       if (s0 < lv.ns) {
-        v[u] = __ldcg(lv.bits + trie_word(s0, e[u].x & kTrDigit));
-        r[u] = __ldcg(lv.rec + s0);
+        const uint32_t v = __ldcg(lv.bits + trie_word(s0, e.x & kTrDigit));
+        row = tr_rank(__ldcg(lv.rec + s0), v, e.x & kTrDigit);
       }
-    }
-#pragma unroll
-    for (int u = 0; u < kTrAdd; ++u) {
-      const uint32_t i = i0 + kTrThreads * u + threadIdx.x;
-      row[u] = ~0u;
-      oa[u] = ob[u] = va[u] = vb[u] = 0ull;
-      if (i >= nruns) continue;
-      if (r[u].x != ~0u) row[u] = tr_rank(r[u], v[u], e[u].x & kTrDigit);
-      if (row[u] >= rows) {
+      if (row >= rows) {
         set_error(err, kErrInvalidArg);
-        row[u] = ~0u;
-      } else {
-        uint64_t key = e[u].x;
-        if (kb > 32u) key |= uint64_t(runhi[i]) << 32;
-        R.key[row[u]] = key;  // (every run of the row stores the same key)
-        va[u] = e[u].y | ((unsigned long long)e[u].z << 32);
-        vb[u] = (e[u].w & 0x3ffffffu) | ((unsigned long long)(e[u].w >> 26) << 32);
-        oa[u] = atomicAdd(R.A + row[u], va[u]);
-        ob[u] = atomicAdd(R.B + row[u], vb[u]);
-        if (with_attrs) {
-          const uint2 t = runatt[i];
-          atomicAdd(R.att + row[u],
-                    (unsigned long long)(t.x & 0xffffu) | ((unsigned long long)(t.x >> 16) << 32));
-          if (a.out.channels > 2)
-            atomicAdd(R.att + cap + row[u], (unsigned long long)(t.y & 0xffffu) |
-                                                ((unsigned long long)(t.y >> 16) << 32));
+        row = kTrNoRow;
+      }
+      if (a.out.p2v) pslot[i] = row;
+    }
+    bool in_hot = false;
+    if (hot_entries) {
+      if (!all_hot) {
+        const uint32_t lead = __shfl_sync(kFullMask, row, 0);
+        const uint32_t again = __ballot_sync(kFullMask, row == met && row != kTrNoRow);
+        const bool many = __popc(__ballot_sync(kFullMask, row == lead)) >= 8;
+        if (many || __popc(again) >= 2) {
+          const uint32_t r = many ? lead : met;
+          if (lane == 0 && r != kTrNoRow &&
+              atomicCAS(hot.tag + (r & hot.mask), kTrNoRow, r) == kTrNoRow)
+            sm.hot = 1u;
+        } else if (again == 0u) {
+          met = lead;
         }
       }
-      if (a.out.p2v) pslot[i] = row[u];
+      in_hot = row != kTrNoRow && *reinterpret_cast<volatile uint32_t*>(&sm.hot) != 0u &&
+               *reinterpret_cast<volatile uint32_t*>(hot.tag + (row & hot.mask)) == row;
     }
+    if (row == kTrNoRow) continue;
+    const uint2 at = with_attrs ? runatt[i] : make_uint2(0u, 0u);
+    bool first = true;
+    if (in_hot) {
+      const uint32_t h = row & hot.mask;
+      first = tr_hot_add(hot, h, e.y, e.z, e.w & 0x3ffffffu, e.w >> 26);
+      if (with_attrs) {
 #pragma unroll
-    for (int u = 0; u < kTrAdd; ++u) {
-      if (row[u] == ~0u) continue;
-      // carries out of a 32-bit half: x into y, A out of 64 bits, z into the points
-      const unsigned long long cx = ((oa[u] & 0xffffffffull) + (va[u] & 0xffffffffull)) >> 32;
-      const unsigned long long cy = oa[u] + va[u] < oa[u] ? 1ull : 0ull;
-      const unsigned long long cz = ((ob[u] & 0xffffffffull) + (vb[u] & 0xffffffffull)) >> 32;
-      if (cx | cy | cz) atomicAdd(R.C + row[u], cx | (cy << 21) | (cz << 42));
+        for (int c = 0; c < 4; ++c)
+          if (c < a.out.channels)
+            atomicAdd(hot.att + kTrHotAttWords * h + c, ((c >> 1 ? at.y : at.x) >> (16 * (c & 1))) & 0xffffu);
+      }
+    } else {
+      tr_add(R, row, e.y | ((unsigned long long)e.z << 32),
+             (e.w & 0x3ffffffu) | ((unsigned long long)(e.w >> 26) << 32));
+      if (with_attrs) {
+        atomicAdd(R.att + row,
+                  (unsigned long long)(at.x & 0xffffu) | ((unsigned long long)(at.x >> 16) << 32));
+        if (a.out.channels > 2)
+          atomicAdd(R.att + cap + row, (unsigned long long)(at.y & 0xffffu) |
+                                           ((unsigned long long)(at.y >> 16) << 32));
+      }
+    }
+    if (first) {
+      uint64_t key = e.x;
+      if (kb > 32u) key |= uint64_t(runhi[i]) << 32;
+      R.key[row] = key;  // (every run of the row stores the same key)
     }
   }
+  __syncthreads();
+  if (sm.hot)
+    for (uint32_t h = threadIdx.x; h < hot_entries; h += kTrThreads) {
+      const uint32_t n = hot.n[h], row = hot.tag[h];
+      if (n == 0u) continue;
+      const uint32_t c = hot.carry[h], cx = c & 1023u, cy = (c >> 10) & 1023u, cz = c >> 20;
+      // x + y 2^32 of sums beyond 32 bits: the carries of x add to y
+      const unsigned long long y = hot.y[h] + (unsigned long long)cx;
+      tr_add(R, row, hot.x[h] | (y << 32), hot.z[h] | ((unsigned long long)(n + cz) << 32), cx,
+             cy + uint32_t(y >> 32), cz);
+      if (with_attrs) {
+        const uint32_t* t = hot.att + kTrHotAttWords * h;
+        atomicAdd(R.att + row, t[0] | ((unsigned long long)t[1] << 32));
+        if (a.out.channels > 2) atomicAdd(R.att + cap + row, t[2] | ((unsigned long long)t[3] << 32));
+      }
+    }
   if (a.out.p2v) {  // a point's row is its run's: that of the next point to end one
-    __syncthreads();
     tr_lanes<kPosed, K, false>(a, fm, T, [&](uint32_t part, const TrLanePoints<K>& t) {
       uint32_t row[K], tails[K], m = 0u, valid = 0u, first = ~0u;
 #pragma unroll
@@ -895,8 +982,14 @@ __global__ __launch_bounds__(1024) void trie_clear_kernel(uint32_t* st, uint32_t
   if (threadIdx.x == 0) *err = 0;
 }
 
-// Dynamic shared memory of a block at most: the tables of kMaxFrames frames.
-constexpr size_t kTrSmem = tr_frames_bytes(kMaxFrames, true);
+// Entries of the table of hot rows, and their bytes.
+constexpr uint32_t tr_hot_entries(bool attrs) { return attrs ? 2048u : 4096u; }
+constexpr size_t tr_hot_bytes(bool attrs) {
+  return size_t(tr_hot_entries(attrs)) * (kTrHotWords + (attrs ? kTrHotAttWords : 0u)) * 4u;
+}
+// Dynamic shared memory of a block at most: the tables of kMaxFrames frames and the hot rows.
+constexpr size_t kTrSmem = tr_frames_bytes(kMaxFrames, true) + tr_hot_bytes(false);
+static_assert(tr_hot_bytes(true) <= tr_hot_bytes(false), "the larger table");
 static_assert(kTrSmem + sizeof(TrSmem) <= 227 * 1024, "block shared memory");
 
 // Blocks an SM holds of the kernel (0: it cannot run there), per device.
@@ -952,6 +1045,8 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   a.first = reinterpret_cast<uint32_t*>(ws + L.first);
   a.stat = reinterpret_cast<uint32_t*>(ws + L.stat);
   a.out = out;
+  const bool attrs = out.attrs_in != nullptr;
+  a.hot = tr_hot_entries(attrs);
   a.slots = L.slots;
   a.spin_limit = spin_limit;
   a.err = err;
@@ -968,7 +1063,8 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   }
   void* args[] = {&a};
   const void* fn = reinterpret_cast<const void*>(trie_kernel_of(posed(fr), a.large != 0));
-  return launch_cooperative(fn, g, kTrThreads, args, tr_frames_bytes(fr.nframes, posed(fr)), stream);
+  return launch_cooperative(fn, g, kTrThreads, args,
+                            tr_frames_bytes(fr.nframes, posed(fr)) + tr_hot_bytes(attrs), stream);
 }
 
 }  // namespace vg

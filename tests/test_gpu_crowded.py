@@ -1,6 +1,7 @@
 """Crowded clouds without order: few cells, or one cell with much of the cloud, points shuffled.
-The hash insert merges the queued runs of keys that come back; its rows, and a voxel map's, are
-the radix sort's bit for bit."""
+The hash insert merges the queued runs of keys that come back, the occupancy trie sums the rows
+that many runs meet in each block first; their rows, and a voxel map's, are the radix sort's
+bit for bit."""
 import numpy as np
 import pytest
 import torch
@@ -48,3 +49,32 @@ def test_hash_and_map(n, cells, hot):
         if part.shape[0]:
             m.insert(part.contiguous())
     same(m.extract(), ref)
+
+
+@pytest.mark.parametrize("p2v", [False, True])
+@pytest.mark.parametrize("n,cells,hot", CLOUDS + [(900_001, 4095, 0.0), (900_001, 4096, 0.0),
+                                                  (900_001, 4097, 0.0), (2_600_000, 70_000, 0.2)])
+def test_auto(n, cells, hot, p2v):
+    # rows up to a block's table of them and one more; rows that take an entry once met again
+    x = crowd(n, cells, hot)
+    o = torch.zeros(3, device="cuda")
+    ref = vg.downsample(x, LEAF, o, method="sort_lsd", point_to_voxel=p2v)
+    got = vg.downsample(x, LEAF, o, point_to_voxel=p2v)
+    same(got, ref)
+    if p2v:
+        assert torch.equal(got.point_to_voxel, ref.point_to_voxel)
+
+
+@pytest.mark.parametrize("channels", [1, 2, 3, 4])
+@pytest.mark.parametrize("n,cells,hot", [(200_003, 3, 0.0), (900_001, 2049, 0.0),
+                                         (900_001, 2048, 0.0), (900_001, 60_000, 0.4)])
+def test_auto_attributes(n, cells, hot, channels):
+    x = crowd(n, cells, hot)
+    r = np.random.Generator(np.random.PCG64(channels))
+    at = torch.from_numpy(r.integers(0, 256, (n, channels), np.uint8)).cuda()
+    at[: n // 2] = 255
+    o = torch.zeros(3, device="cuda")
+    ref = vg.downsample(x, LEAF, o, method="sort_lsd", attrs=at)
+    got = vg.downsample(x, LEAF, o, attrs=at)
+    same(got, ref)
+    assert torch.equal(got.attrs, ref.attrs)
