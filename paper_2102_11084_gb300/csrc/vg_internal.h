@@ -112,6 +112,9 @@ struct FrameState {
 // has written the rows: nothing is left to do for the sort path's kernels.
 constexpr uint32_t kRowsWritten = 2;
 
+// Distance of consecutive points, in leaves on every axis, that tells a scan's order.
+constexpr float kNearLeaves = 32.0f;
+
 // Per-call device state, at the start of the workspace.  Zeroed by the call.
 struct alignas(256) State {
   unsigned long long maxkey;  // largest sort key
@@ -137,8 +140,8 @@ struct alignas(256) State {
   uint32_t sort_bar;          // radix passes: grid-barrier arrivals
   uint32_t fz_bar;            // one-launch frame grouping: grid-barrier arrivals
   uint32_t fz_rows;           // one-launch frame grouping: rows (occupied cells)
-  unsigned long long smp;     // sampled pairs of consecutive points: valid ones, and (upper
-                              // 32 bits) those of one cell
+  unsigned long long smp;     // sampled pairs of consecutive points, 21 bits each: valid ones,
+                              // those of one cell, those within kNearLeaves leaves
   uint32_t ctot[64];          // entries of every 1024 consecutive buckets
   uint32_t nztot[64];         // non-empty buckets of every 1024 consecutive buckets
   uint32_t vtot[64];          // cells of every 1024 consecutive non-empty buckets

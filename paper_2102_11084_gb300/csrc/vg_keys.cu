@@ -54,11 +54,12 @@ __device__ __forceinline__ void flush_extent(float mn[3], float mx[3], FrameStat
   }
 }
 
-// Pairs of consecutive points among a warp's 128 (4 a thread in v, NaN rows invalid) and those
-// of one cell, added to st->smp (lattice through 0: the origin is not known yet).
+// Pairs of consecutive points among a warp's 128 (4 a thread in v, NaN rows invalid), those of
+// one cell and those near each other, added to st->smp (lattice through 0: the origin is not
+// known yet).
 __device__ __forceinline__ void sample_pairs(const float v[12], float leaf, State* st) {
   const float r = __fdiv_rn(1.0f, leaf);
-  uint32_t pairs = 0, same = 0;
+  uint32_t pairs = 0, same = 0, near = 0;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     const float* a = v + 3 * j;
@@ -66,11 +67,14 @@ __device__ __forceinline__ void sample_pairs(const float v[12], float leaf, Stat
     ++pairs;
     same += floorf(a[0] * r) == floorf(a[3] * r) && floorf(a[1] * r) == floorf(a[4] * r) &&
             floorf(a[2] * r) == floorf(a[5] * r);
+    near += fabsf(a[0] - a[3]) * r < kNearLeaves && fabsf(a[1] - a[4]) * r < kNearLeaves &&
+            fabsf(a[2] - a[5]) * r < kNearLeaves;
   }
   pairs = __reduce_add_sync(kFullMask, pairs);
   same = __reduce_add_sync(kFullMask, same);
+  near = __reduce_add_sync(kFullMask, near);
   if ((threadIdx.x & 31) == 0 && pairs)
-    atomicAdd(&st->smp, (unsigned long long)pairs | ((unsigned long long)same << 32));
+    atomicAdd(&st->smp, pairs | ((unsigned long long)same << 21) | ((unsigned long long)near << 42));
 }
 
 // a1: per-frame minimum and maximum over the valid points.  With st, the first 128 points of

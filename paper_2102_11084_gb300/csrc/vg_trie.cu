@@ -455,10 +455,12 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   // (barriers below come before their first use)
   if (threadIdx.x == 0) sm.nruns = 0u;
   for (int i = threadIdx.x; i < 6 * F; i += kTrThreads) fm.ext[i] = 0u;
-  bool few = true;  // (the same in every block)
+  bool few = true, ordered = true;  // (the same in every block)
   if (a.large) {
     const unsigned long long smp = a.st->smp;
-    few = kTrSameOf * uint32_t(smp >> 32) >= kTrSame * uint32_t(smp);
+    const uint32_t pairs = uint32_t(smp) & 0x1fffffu;
+    few = kTrSameOf * (uint32_t(smp >> 21) & 0x1fffffu) >= kTrSame * pairs;
+    ordered = 2u * uint32_t(smp >> 42) >= pairs;
     if (!few && a.fr.n > kTrMidPoints) return;
   }
   // ---- extents; the first level's bits cleared ----
@@ -586,7 +588,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     }
     return;
   }
-  if (!few && kb > kTrMidBits && kb <= 32u) return;
+  if (!few && kb > kTrMidBits && (kb <= 32u || !ordered)) return;
   const bool wide = local_bits > 32u;
   // levels, and the key bits below level 1
   const uint32_t root_bits = static_cast<uint32_t>(a.root_bits);

@@ -32,8 +32,9 @@ constexpr int kTrRootBitsLarge = 28;
 //     frames at 5 mm to 0.1 m: 2 of 5 come with cells for at most a quarter of the points, 1
 //     of 5 with more than half); above kTrMidPoints they must fit a quarter of the points;
 //   * up to kTrMidPoints points, whose keys have at most 27 bits (one level or a nearly empty
-//     second: 4M points of 26-bit keys 210 us, the radix sort 316) or more than 32 (the radix
-//     sort's wide layout: a scan of 4M points 401 us against 450).
+//     second: 4M points of 26-bit keys 210 us, the radix sort 316), or more than 32 where half
+//     of the sampled pairs lie within 32 leaves (a scan of 4M points in its order 428 us, the
+//     radix sort's wide layout 480; shuffled, every level's accesses miss: 874 against 486).
 constexpr int64_t kTrMaxPoints = int64_t(5) << 19;
 constexpr int64_t kTrMidPoints = int64_t(1) << 22;
 constexpr int64_t kTrCellShare = 4;
