@@ -777,7 +777,8 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
       R.att[i + cap] = 0ull;
     }
   }
-  const uint32_t hot_entries = places <= kTrHotPlaces ? a.hot : 0u;  // (the same in every thread)
+  // (the same in every thread of the block; few runs are not worth clearing the table)
+  const uint32_t hot_entries = places <= kTrHotPlaces && nruns >= kTrThreads ? a.hot : 0u;
   const TrHot hot = tr_hot(reinterpret_cast<uint32_t*>(tr_smem + tr_frames_bytes(F, kPosed)), a.hot);
   const bool all_hot = rows <= hot_entries && nruns / 2u >= rows;
   for (uint32_t e = threadIdx.x; e < hot_entries; e += kTrThreads) {
@@ -984,14 +985,19 @@ __global__ __launch_bounds__(1024) void trie_clear_kernel(uint32_t* st, uint32_t
   if (threadIdx.x == 0) *err = 0;
 }
 
-// Entries of the table of hot rows, and their bytes.
-constexpr uint32_t tr_hot_entries(bool attrs) { return attrs ? 2048u : 4096u; }
-constexpr size_t tr_hot_bytes(bool attrs) {
-  return size_t(tr_hot_entries(attrs)) * (kTrHotWords + (attrs ? kTrHotAttWords : 0u)) * 4u;
+// Entries of the table of hot rows, and their bytes.  Smaller calls have none: clearing and
+// looking costs them 0.4 us, and even ten cells of 100,000 points take 81 us without (38 with,
+// the radix sort 116).
+constexpr int64_t kTrHotPoints = int64_t(1) << 17;
+constexpr uint32_t tr_hot_entries(bool attrs, int64_t n) {
+  return n < kTrHotPoints ? 0u : (attrs ? 2048u : 4096u);
+}
+constexpr size_t tr_hot_bytes(bool attrs, int64_t n) {
+  return size_t(tr_hot_entries(attrs, n)) * (kTrHotWords + (attrs ? kTrHotAttWords : 0u)) * 4u;
 }
 // Dynamic shared memory of a block at most: the tables of kMaxFrames frames and the hot rows.
-constexpr size_t kTrSmem = tr_frames_bytes(kMaxFrames, true) + tr_hot_bytes(false);
-static_assert(tr_hot_bytes(true) <= tr_hot_bytes(false), "the larger table");
+constexpr size_t kTrSmem = tr_frames_bytes(kMaxFrames, true) + tr_hot_bytes(false, kMaxPoints);
+static_assert(tr_hot_bytes(true, kMaxPoints) <= tr_hot_bytes(false, kMaxPoints), "the larger table");
 static_assert(kTrSmem + sizeof(TrSmem) <= 227 * 1024, "block shared memory");
 
 // Blocks an SM holds of the kernel (0: it cannot run there), per device.
@@ -1048,7 +1054,7 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   a.stat = reinterpret_cast<uint32_t*>(ws + L.stat);
   a.out = out;
   const bool attrs = out.attrs_in != nullptr;
-  a.hot = tr_hot_entries(attrs);
+  a.hot = tr_hot_entries(attrs, fr.n);
   a.slots = L.slots;
   a.spin_limit = spin_limit;
   a.err = err;
@@ -1066,7 +1072,8 @@ cudaError_t launch_trie(const float* xyz, const FramesArg& fr, State* st, FrameS
   void* args[] = {&a};
   const void* fn = reinterpret_cast<const void*>(trie_kernel_of(posed(fr), a.large != 0));
   return launch_cooperative(fn, g, kTrThreads, args,
-                            tr_frames_bytes(fr.nframes, posed(fr)) + tr_hot_bytes(attrs), stream);
+                            tr_frames_bytes(fr.nframes, posed(fr)) + tr_hot_bytes(attrs, fr.n),
+                            stream);
 }
 
 }  // namespace vg

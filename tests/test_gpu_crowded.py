@@ -52,7 +52,8 @@ def test_hash_and_map(n, cells, hot):
 
 
 @pytest.mark.parametrize("p2v", [False, True])
-@pytest.mark.parametrize("n,cells,hot", CLOUDS + [(900_001, 4095, 0.0), (900_001, 4096, 0.0),
+@pytest.mark.parametrize("n,cells,hot", CLOUDS + [(131_071, 7, 0.0), (131_072, 7, 0.0),
+                                                  (900_001, 4095, 0.0), (900_001, 4096, 0.0),
                                                   (900_001, 4097, 0.0), (2_600_000, 70_000, 0.2)])
 def test_auto(n, cells, hot, p2v):
     # rows up to a block's table of them and one more; rows that take an entry once met again
