@@ -41,6 +41,10 @@ constexpr int64_t kTrCellShare = 4;
 constexpr uint32_t kTrMidBits = 27;
 constexpr uint32_t kTrSame = 2, kTrSameOf = 5;
 
+// Points a prefix, on average, up to which a further level is marked unseen (8: a 1280x720 frame
+// at 0.01 m, whose runs meet again, 2 % slower).
+constexpr int64_t kTrSparse = 4;
+
 // Slots of a further level, and rows, that a call's buffers hold.
 constexpr int64_t trie_slots(int64_t n) { return n <= kTrMidPoints ? n : n / kTrCellShare; }
 static_assert(trie_word(static_cast<uint32_t>(trie_slots(kMaxPoints)) - 1u, kTrDigit) ==

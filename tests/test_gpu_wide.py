@@ -44,3 +44,34 @@ def check(x, leaf, **kw):
 @pytest.mark.parametrize("n", [2_621_441, 4_194_304])
 def test_above_what_the_trie_always_takes(n, leaf, shuffled):
     check(scan(n, 3, shuffled), leaf)
+
+
+def uniform(n, seed, cells, leaf):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    i = torch.randint(0, cells, (n, 3), generator=g, device="cuda")
+    return ((i + 0.25 * torch.randint(0, 4, (n, 3), generator=g, device="cuda")).float() * leaf)
+
+
+# prefixes nearly as many as the points from the first level on, or a few points each
+@pytest.mark.parametrize("n", [33, 30_001, 1_000_003, 2_621_440])
+@pytest.mark.parametrize("bits", [12, 14, 17, 21])
+def test_sparse_cells(n, bits):
+    leaf = 2.0 ** -bits
+    x = uniform(n, bits, 2 ** bits, leaf)  # (dyadic: indices exact)
+    x[: n // 8] = x[n // 2: n // 2 + n // 8]     # cells of two and more points, far apart
+    x[n // 3] = float("nan")
+    check(x.contiguous(), leaf, origin=torch.zeros(3, device="cuda"))
+
+
+def test_frames_of_sparse_cells():
+    leaf = 2.0 ** -16
+    x = uniform(900_000, 4, 2 ** 16, leaf)
+    offs = [0, 0, 300_001, 300_001, 750_000, 900_000]
+    rgb = (torch.arange(3 * x.shape[0], device="cuda") * 37 % 256).to(torch.uint8).reshape(-1, 3)
+    for kw in ({}, {"point_to_voxel": True}, {"attrs": rgb, "min_count": 2}):
+        a = vg.downsample_frames((x, offs), [leaf] * 5, **kw)
+        b = vg.downsample_frames((x, offs), [leaf] * 5, method="sort_lsd", **kw)
+        assert a.offsets == b.offsets
+        same(a, b)
+        assert a.attrs is None or torch.equal(a.attrs, b.attrs)
