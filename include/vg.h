@@ -352,7 +352,8 @@ VG_API vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell,
  * host-synchronising) and keeps the fastest; out_ms (12 floats or NULL) receives
  * sort@4,8,16, sort_lsd@4,8,16, frame@4,8,16 then hash@4,8,16 in ms per batch, -1 for a
  * grouping not timed (frame with several frames) or one whose runs recorded a device
- * error (frame with keys wider than 32 bits; the error word is cleared again).  A plan's
+ * error (frame with keys wider than 32 bits; the error word is cleared again).  AUTO is
+ * timed as well, unreported, and kept where it is faster than all of those.  A plan's
  * method (vg_plan_create flags, vg_plan_configure, vg_plan_get) is one of those four or
  * VG_METHOD_AUTO (the library's choice by cloud size, the default of a new plan).
  */

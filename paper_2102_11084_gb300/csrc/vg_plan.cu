@@ -181,9 +181,12 @@ vg_status vg_plan_tune(vg_plan* p, const float* xyz, int64_t n_total,
                        float* out_ms) {
   if (!p || reps < 1) return VG_ERR_INVALID_ARG;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-  const int methods[4] = {VG_METHOD_SORT, VG_METHOD_SORT | VG_SORT_LSD,
-                          VG_METHOD_SORT | VG_SORT_FRAME, VG_METHOD_HASH};
+  // the four groupings of out_ms, then AUTO (one grid, not reported), which is kept where it is
+  // faster than all of them
+  const int methods[5] = {VG_METHOD_SORT, VG_METHOD_SORT | VG_SORT_LSD,
+                          VG_METHOD_SORT | VG_SORT_FRAME, VG_METHOD_HASH, VG_METHOD_AUTO};
   const int grids[3] = {4, 8, 16};
+  constexpr int kReported = 12;
   // the device error word of the tuning runs: a grouping that records an error (the bin
   // grouping of keys wider than 32 bits) is not a candidate
   const int32_t* errw = out_error ? out_error : &reinterpret_cast<const vg::State*>(p->ws)->error;
@@ -193,8 +196,9 @@ vg_status vg_plan_tune(vg_plan* p, const float* xyz, int64_t n_total,
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return VG_ERR_CUDA;
   vg_status result = VG_OK;
   int slot = 0;
-  for (int mi = 0; mi < 4 && result == VG_OK; ++mi) {
+  for (int mi = 0; mi < 5 && result == VG_OK; ++mi) {
     for (int gi = 0; gi < 3 && result == VG_OK; ++gi, ++slot) {
+      if (methods[mi] == VG_METHOD_AUTO && grids[gi] != 8) continue;
       if ((methods[mi] & VG_SORT_FRAME) != 0 && n_frames != 1) {  // several frames: SORT
         if (out_ms) out_ms[slot] = -1.0f;
         continue;
@@ -230,7 +234,7 @@ vg_status vg_plan_tune(vg_plan* p, const float* xyz, int64_t n_total,
           break;
         }
       }
-      if (out_ms) out_ms[slot] = ms;
+      if (out_ms && slot < kReported) out_ms[slot] = ms;
       if (ms < 0.0f) continue;
       if (ms < best) {
         best = ms;

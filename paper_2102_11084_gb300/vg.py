@@ -695,8 +695,9 @@ class Plan:
     def tune(self, xyz, frame_offsets, n_frames, origins, leaves, out_keys, out_centroids,
              out_counts, out_frame_offsets, out_error, *, origin_from_min=True, reps=5,
              stream: Optional[torch.cuda.Stream] = None):
-        """vg_plan_tune: time sort/sort_lsd/frame/hash x grids {4,8,16}; keeps the fastest
-        (-1: not timed, or the grouping recorded a device error)."""
+        """vg_plan_tune: time sort/sort_lsd/frame/hash x grids {4,8,16}, and auto; keeps the
+        fastest.  Returns the twelve times (-1: not timed, or the grouping recorded a device
+        error)."""
         ms = (ctypes.c_float * 12)()
         flags = ORIGIN_FROM_MIN if origin_from_min else 0
         st = lib().vg_plan_tune(
