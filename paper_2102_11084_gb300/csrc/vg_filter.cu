@@ -5,14 +5,14 @@
 // drop sparsely occupied voxels; here that is a stable compaction of the V rows (keys,
 // counts, centroids, attribute means) with a chained scan over tiles of 1024 rows:
 //   filter_kernel   a tile reads its rows, ranks the kept ones, waits (bounded) for the
-//                   kept-row count of all earlier tiles (the whole block looks back 256 tiles
-//                   at a time: bound by latency, 146K rows of 8 colour frames 20 us
-//                   where one thread's walk took 28), then writes its kept rows at their new
-//                   place.  Tiles start in ticket order and a tile's prefix is
-//                   complete only once every earlier tile has read its rows, so the
-//                   in-place writes (always to rows at or before the tile's own) never
-//                   overwrite a row not yet read.  Every row also gets its remap word:
-//                   bit 31 = kept, bits 0-30 = kept rows before it.
+//                   kept-row count of all earlier tiles (a warp looks back 32 tiles at a
+//                   time: bound by latency, 146K rows of 8 colour frames 20 us where one
+//                   thread's walk took 28), then writes its kept rows at their new place.
+//                   Tiles start in ticket order and a tile's prefix is complete only once
+//                   every earlier tile has read its rows, so the in-place writes (always to
+//                   rows at or before the tile's own) never overwrite a row not yet read.
+//                   Every row also gets its remap word: bit 31 = kept, bits 0-30 = kept rows
+//                   before it.
 //   filter_fix      one block: the new voxel count and per-frame row offsets.
 //   filter_p2v      point_to_voxel through the remap (-1 for removed voxels).
 #include "vg_device.cuh"
@@ -31,7 +31,7 @@ __global__ __launch_bounds__(kFiltThreads) void filter_kernel(
     uint32_t* counts, float* centroids, float* attrs, int channels, uint32_t* remap,
     uint32_t* status, uint32_t* ticket, uint32_t spin_limit, int* err) {
   __shared__ uint32_t s_tmp[kFiltThreads / 32];
-  __shared__ uint32_t s_look[kFiltThreads / 32][2];
+  __shared__ uint32_t s_look;
   __shared__ int s_tile;
   const int t = threadIdx.x;
   const int64_t V = *num_voxels < cap ? *num_voxels : cap;  // rows beyond cap were not written
@@ -68,7 +68,7 @@ __global__ __launch_bounds__(kFiltThreads) void filter_kernel(
     uint32_t tile_kept;
     const uint32_t rank = block_excl_scan(mine, &tile_kept, s_tmp);
     if (t == 0) st_relaxed(status + tile, (tile ? kFlagAggregate : kFlagPrefix) | tile_kept);
-    const uint32_t excl = block_lookback(status, tile, spin_limit, err, s_look);
+    const uint32_t excl = block_lookback(status, tile, spin_limit, err, &s_look);
     if (t == 0 && tile) st_relaxed(status + tile, kFlagPrefix | ((excl + tile_kept) & kValueMask));
     uint32_t dst = excl + rank;
 #pragma unroll
