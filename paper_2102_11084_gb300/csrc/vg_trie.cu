@@ -972,12 +972,20 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
       put_row(rc, a.out, row, key, r, err);
     if (with_attrs) {
       const unsigned long long t[2] = {__ldcg(R.att + row), __ldcg(R.att + cap + row)};
+      // The exact sum over the points, divided in FP64 and rounded to float32.  Where both are
+      // exact in binary32 its own division gives the same bits (FP64 has more than twice its
+      // digits, so rounding a quotient twice changes nothing), without the few FP64 units: 2.5M
+      // shuffled points with 4 channels 584 -> 398 us (the radix sort 487).
 #pragma unroll
-      for (int c = 0; c < 4; ++c)  // exact sums, one FP64 division each
-        if (c < a.out.channels)
-          a.out.attrs_out[size_t(row) * a.out.channels + c] = __double2float_rn(
-              __ddiv_rn(static_cast<double>(uint32_t(t[c >> 1] >> (32 * (c & 1)))),
-                        static_cast<double>(r.n)));
+      for (int c = 0; c < 4; ++c)
+        if (c < a.out.channels) {
+          const uint32_t sum = uint32_t(t[c >> 1] >> (32 * (c & 1)));
+          a.out.attrs_out[size_t(row) * a.out.channels + c] =
+              (sum | r.n) < (1u << 24)
+                  ? __fdiv_rn(__uint2float_rn(sum), __uint2float_rn(r.n))
+                  : __double2float_rn(
+                        __ddiv_rn(static_cast<double>(sum), static_cast<double>(r.n)));
+        }
     }
   }
 }
