@@ -325,11 +325,11 @@ VG_API vg_status vg_map_extract(vg_map* map, uint64_t* out_keys, float* out_cent
  *   out_keep       uint8 [n] (device): 1 for the points that remain, 0 otherwise
  *                  (invalid points included); *out_num_kept (device int64) their number.
  *   out_passes     host int32 or NULL: passes of the loop.
- * Workspace: vg_thin_workspace_bytes(n) bytes.  The call synchronises the stream twice:
- * all passes run in one cooperative launch that keeps every point's neighbour count.  Where
- * the points are so dense, or the batch so large, that counting afresh is cheaper (or the
- * device cannot hold that launch), it synchronises once per pass and once per round of the
- * batch selection (8 bits a round).
+ * Workspace: vg_thin_workspace_bytes(n) bytes.  The call synchronises the stream two
+ * or three times: all passes run in one cooperative launch that keeps every point's neighbour
+ * count.  Where the points are so dense, or the batch so large, that counting afresh is
+ * cheaper (or the device cannot hold that launch), it synchronises once per pass and once per
+ * round of the batch selection (8 bits a round).
  */
 VG_API size_t vg_thin_workspace_bytes(int64_t n_points);
 VG_API vg_status vg_thin(const float* xyz, int64_t n, float* origin, float cell, float radius,
