@@ -30,6 +30,7 @@
 //              marked and finds the batch by a radix select on 256-bin histograms
 //              (thin_hist_kernel), thin_delete_kernel removes it.
 //   output     keep flag per input point and the number kept.
+#include <algorithm>
 #include <cmath>
 
 #include "../../include/vg.h"
@@ -888,17 +889,26 @@ int thin_local_grid() {
   return v > 0 ? num_sms() : 0;
 }
 
-// Whether the loop keeps counts, by estimated microseconds.  Kept: every candidate pair is
-// tested about twice in all (the count, then the deletions; 1.5e12 tests a second) and a pass
-// takes 10 us.  Recounted: a pass takes 100 us of host round trips and about 100 ps a point and
-// neighbour it looks for (640x480 frame, threshold 20: 570 us).  Passes: where the candidates
-// of a point are many times the threshold, most points are deleted.
+// Whether the loop keeps counts, by estimated microseconds beside what both forms share.  Kept:
+// 100 for its launches, every candidate pair once, a deleted point 4.5 ns and 1.5 more for each
+// 1000 candidates, and 10 a pass.  Recounted: a pass takes 130 of host round trips and, a point,
+// 0.3 ns, 1.2 for each 1000 candidates up to 1500 (threads of crowded cells end last) and 0.25
+// beyond, and 0.5 for 1000 tested until the threshold is passed.  Passes: where the candidates of
+// a point are many times the threshold, most points are deleted.  Measured both ways, kept
+// against recounted: 640x480 frame (3600 candidates a point), threshold 20, batches of half the
+// points 2944 and 1683 us, of an eighth 4063 and 6666; 1M points of 53 candidates, threshold
+// 2, half 4102 and 1185, a sixteenth 4981 and 4623; 200,000 of 675, threshold 20, half 883 and
+// 593, a quarter 993 and 1074.
 bool keep_counts(int64_t n, unsigned long long pairs, int64_t batch, int64_t threshold) {
   if (n <= 0) return false;
   const double nn = double(n), pp = double(pairs), want = double(threshold) + 1.0;
-  const double gone = pp > 0.0 ? 1.0 - 3.0 * want * nn / pp : 0.0;
-  const double passes = gone > 0.0 && gone * nn > double(batch) ? gone * nn / double(batch) : 1.0;
-  return 2.0 * pp / 1.5e6 + 10.0 * passes <= passes * (100.0 + nn * want * 1e-4);
+  const double c = pp / nn;  // candidates of a point
+  const double gone = pp > 0.0 ? std::max(0.0, 1.0 - 3.0 * want / c) * nn : 0.0;
+  const double passes = std::max(1.0, gone / double(batch));
+  const double kept = 100.0 + pp / 1.4e6 + (4.5e-3 + 1.5e-6 * c) * gone + 10.0 * passes;
+  const double point = 3e-4 + 1.2e-6 * std::min(c, 1500.0) + 2.5e-7 * std::max(c - 1500.0, 0.0) +
+                       5e-7 * std::min(c, 6.5 * want);
+  return kept <= passes * (130.0 + point * nn);
 }
 
 // Whether a pass is thin_local_kernel's, by estimated cycles: 6000 and, for every round of the
