@@ -463,14 +463,60 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* ctr, uint32_t& target, ui
   return __syncthreads_or(late) == 0;
 }
 
+// The chained-scan wait of lookback_u32 with the whole block (256 threads): thread t reads
+// the t-th predecessor of the window, so a window of 256 tiles costs one round trip, where
+// one thread's walk costs one a tile (200 to 400 tiles that start together: most of 150 us against 2).
+// status + i: tile i's word.  Returns the exclusive prefix of `tile` in every thread.  Contains
+// __syncthreads; `tmp` holds 2 * 8 words.
+__device__ __forceinline__ uint32_t block_lookback(const uint32_t* status, int tile,
+                                                   uint32_t spin_limit, int* err,
+                                                   uint32_t (*tmp)[2]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t excl = 0;
+  for (int end = tile; end > 0; end -= 256) {
+    const int j = end - 1 - int(threadIdx.x);
+    uint32_t s = kFlagPrefix;  // before the first tile: nothing
+    if (j >= 0) {
+      uint32_t spins = 0;
+      while (((s = ld_relaxed(status + j)) & ~kValueMask) == 0) {
+        if (++spins > spin_limit) {
+          set_error(err, kErrTimeout);
+          s = kFlagPrefix;
+          break;
+        }
+        if (spins > 64) __nanosleep(64);
+      }
+    }
+    // the values up to the warp's nearest prefix, and whether it has one
+    const uint32_t pre = __ballot_sync(kFullMask, (s & ~kValueMask) == kFlagPrefix);
+    const int last = pre ? __ffs(pre) - 1 : 31;
+    const uint32_t sum = __reduce_add_sync(kFullMask, lane <= last ? s & kValueMask : 0u);
+    __syncthreads();  // earlier readers of tmp are done
+    if (lane == 0) {
+      tmp[warp][0] = sum;
+      tmp[warp][1] = pre;
+    }
+    __syncthreads();
+    bool found = false;
+#pragma unroll
+    for (int w = 0; w < 8; ++w)
+      if (!found) {
+        excl += tmp[w][0];
+        found = tmp[w][1] != 0;
+      }
+    if (found) break;
+  }
+  return excl;
+}
+
 // The chained-scan wait of lookback_u32 with one warp of the block: a lane reads a predecessor, so
 // that a window of 32 tiles costs one round trip, where one thread's walk costs one a tile (200 to
-// 400 tiles that start together: most of 150 us against 2).  No more: with 128 or all 256
-// words a round the blocks' polls wait on one another at the few sectors that hold them (the
-// minimum-count filter of 7M rows 266 us with 32, 338 with 128, 370 with 256).  status + i:
-// tile i's word.  Returns the exclusive prefix of `tile` in every thread.  Contains
+// 400 tiles that start together: most of 150 us against 2).  For scans of thousands of tiles: with
+// 128 words a round, or the whole block's 256, the blocks' polls wait on one another at the few
+// sectors that hold them (the minimum-count filter of 7M rows 266 us with 32, 338, 370).
+// status + i: tile i's word.  Returns the exclusive prefix of `tile` in every thread.  Contains
 // __syncthreads; `out` is one word of shared memory.
-__device__ __forceinline__ uint32_t block_lookback(const uint32_t* status, int tile,
+__device__ __forceinline__ uint32_t warp_lookback(const uint32_t* status, int tile,
                                                    uint32_t spin_limit, int* err,
                                                    uint32_t* out) {
   const int lane = threadIdx.x & 31;

@@ -68,7 +68,7 @@ __global__ __launch_bounds__(kFiltThreads) void filter_kernel(
     uint32_t tile_kept;
     const uint32_t rank = block_excl_scan(mine, &tile_kept, s_tmp);
     if (t == 0) st_relaxed(status + tile, (tile ? kFlagAggregate : kFlagPrefix) | tile_kept);
-    const uint32_t excl = block_lookback(status, tile, spin_limit, err, &s_look);
+    const uint32_t excl = warp_lookback(status, tile, spin_limit, err, &s_look);
     if (t == 0 && tile) st_relaxed(status + tile, kFlagPrefix | ((excl + tile_kept) & kValueMask));
     uint32_t dst = excl + rank;
 #pragma unroll

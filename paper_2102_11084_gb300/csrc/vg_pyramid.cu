@@ -12,7 +12,7 @@
 //
 // One kernel per level, tiles of 1024 rows (ticketed): the tile's run heads are found with
 // coalesced loads (a ballot word per warp and step), ranked by a bounded chained scan that
-// one warp of the block waits in, and compacted, so that consecutive threads take consecutive
+// the whole block waits in, and compacted, so that consecutive threads take consecutive
 // parents.  Bound by latency (one wait and three dependent loads a level).  A 1280x720 frame
 // at 0.01 m (390K rows, three merges): 152 us a level with eight rows a thread and one
 // thread walking the chained scan, 12 us now.
@@ -22,6 +22,7 @@
 namespace vg {
 namespace {
 
+static_assert(kMergeThreads == 256, "block_lookback");
 constexpr int kMergeWarps = kMergeThreads / 32;
 
 __global__ __launch_bounds__(kMergeThreads) void pyramid_merge_kernel(
@@ -32,7 +33,7 @@ __global__ __launch_bounds__(kMergeThreads) void pyramid_merge_kernel(
   __shared__ uint32_t s_bits[kMergeItems * kMergeWarps];  // heads among 32 consecutive rows
   __shared__ uint32_t s_before[kMergeItems * kMergeWarps];
   __shared__ uint32_t s_total;
-  __shared__ uint32_t s_lb;
+  __shared__ uint32_t s_lb[kMergeWarps][2];
   __shared__ uint16_t s_head[kMergeTile];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   // An earlier step failed: take no ticket.  Every ticket taken is processed, so no tile
@@ -97,7 +98,7 @@ __global__ __launch_bounds__(kMergeThreads) void pyramid_merge_kernel(
       s_head[s_before[j * kMergeWarps + warp] + __popc(b & ((1u << lane) - 1u))] =
           static_cast<uint16_t>(j * kMergeThreads + t);
   }
-  const uint32_t excl = block_lookback(lb, tile, spin_limit, err, &s_lb);
+  const uint32_t excl = block_lookback(lb, tile, spin_limit, err, s_lb);
   if (t == 0) {
     if (tile > 0) st_relaxed(lb + tile, kFlagPrefix | ((excl + total) & kValueMask));
     if (base + kMergeTile >= vprev) level_offsets[level + 1] = off_cur + excl + total;

@@ -1,5 +1,6 @@
-"""The chained scans that a warp looks back in, 32 tiles of 1024 rows a time (the minimum-count
-filter and the pyramid's merges): sizes at the edges of that window."""
+"""The chained scans over tiles of 1024 rows, looked back by a warp 32 tiles at a time (the
+minimum-count filter) or by the whole block (the pyramid's merges): sizes at the edges of the
+warp's window."""
 import pytest
 
 from tests import test_gpu_filter_tiles as filter_tiles
