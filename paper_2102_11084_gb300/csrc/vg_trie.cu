@@ -89,7 +89,9 @@ struct TrSmem {
   uint32_t bits[kTrThreads / 32];
   uint32_t first;
   uint32_t nruns;
-  uint32_t hot;  // some entry of the table of hot rows is taken
+  uint32_t hot;     // some entry of the table of hot rows is taken
+  uint32_t look;    // rows that the block's runs meet again are looked for
+  uint32_t single;  // its runs are hardly more than points
 };
 
 // Tables of a call's frames (dynamic shared memory).
@@ -453,7 +455,10 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
 
   // (barriers below come before their first use)
-  if (threadIdx.x == 0) sm.nruns = 0u;
+  if (threadIdx.x == 0) {
+    sm.nruns = 0u;
+    sm.look = 1u;
+  }
   for (int i = threadIdx.x; i < 6 * F; i += kTrThreads) fm.ext[i] = 0u;
   bool few = true, ordered = true;  // (the same in every block)
   if (a.large) {
@@ -461,6 +466,8 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     const uint32_t pairs = uint32_t(smp) & 0x1fffffu;
     few = kTrSameOf * (uint32_t(smp >> 21) & 0x1fffffu) >= kTrSame * pairs;
     ordered = 2u * uint32_t(smp >> 42) >= pairs;
+    // (camera frames: the ballots took 64 of them 0.6 % longer)
+    if (few && threadIdx.x == 0) sm.look = 0u;
     if (!few && a.fr.n > kTrMidPoints) return;
   }
   // ---- extents; the first level's bits cleared ----
@@ -691,6 +698,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
   if (__any_sync(kFullMask, range_bad) && lane == 0) set_error(err, kErrRange);
   if (!grid_barrier(bar, target, a.spin_limit, err)) return;
   const uint32_t nruns = min(sm.nruns, places);
+  if (threadIdx.x == 0) sm.single = nruns >= places - places / 4u ? 1u : 0u;
 
   // ---- every level ranked, the next one marked ----
   uint32_t rows = 0;
@@ -714,10 +722,11 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     for (uint32_t i = gt; i < n1; i += gthreads) reinterpret_cast<uint4*>(nbits)[i] = zero4;
     if (!grid_barrier(bar, target, a.spin_limit, err)) return;
     const uint32_t sh = below - uint32_t(j) * kTrDigitBits;  // key bits below the next level
-    // Where the prefixes are many for the points, few runs would see their bit set: it is not
-    // looked for, one of four accesses a run (2.5M shuffled points of 60-bit keys 738 -> 631 us,
-    // of 45 bits 425 -> 390; 1M points of a scan in its order 2 % less).
-    const bool sparse = int64_t(n1) * kTrSparse >= a.fr.n;
+    // Where the prefixes are many for the points, and the runs hardly more than points, few runs
+    // would see their bit set: it is not looked for, one of four accesses a run (2.5M shuffled
+    // points of 60-bit keys 738 -> 631 us, of 45 bits 425 -> 390; 1M points of a scan in its
+    // order 2 % less; a 1280x720 frame at 0.01 m, whose runs meet again, would take 3 % more).
+    const bool sparse = int64_t(n1) * kTrSparse >= a.fr.n && sm.single;  // (a block's own)
     for (uint32_t i0 = 0; i0 < nruns; i0 += 2 * kTrThreads) {
       uint32_t id[2], seen[2], v[2];
       uint2 r[2];
@@ -830,7 +839,7 @@ __global__ __launch_bounds__(kTrThreads, 1) void trie_kernel(const TrArgs a) {
     }
     bool in_hot = false;
     if (hot_entries) {
-      if (!all_hot) {
+      if (!all_hot && sm.look) {
         const uint32_t lead = __shfl_sync(kFullMask, row, 0);
         const uint32_t again = __ballot_sync(kFullMask, row == met && row != kTrNoRow);
         const bool many = __popc(__ballot_sync(kFullMask, row == lead)) >= 8;

@@ -41,8 +41,7 @@ constexpr int64_t kTrCellShare = 4;
 constexpr uint32_t kTrMidBits = 27;
 constexpr uint32_t kTrSame = 2, kTrSameOf = 5;
 
-// Points a prefix, on average, up to which a further level is marked unseen (8: a 1280x720 frame
-// at 0.01 m, whose runs meet again, 2 % slower).
+// Points a prefix, on average, up to which a further level is marked unseen.
 constexpr int64_t kTrSparse = 4;
 
 // Slots of a further level, and rows, that a call's buffers hold.
