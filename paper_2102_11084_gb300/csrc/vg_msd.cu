@@ -894,7 +894,7 @@ __device__ __forceinline__ void slot_window(BkSmem& sm, const Bufs& bf, const Jo
 //      per-axis sums (shared-memory atomics; integers, so the order does not matter);
 //   4. one thread per cell writes its row and clears its counter and sums.
 // Four barriers a job; counters, sums and bitmaps are left clean for the next one.
-// Bound by shared-memory wavefronts (64 % of their rate) and issue (54 %).  A job's bitmap is 2048
+// Bound by issue (55 %) and shared-memory wavefronts (52 % of their rate).  A job's bitmap is 2048
 // words where its bucket spans 2^16 keys, whatever its entries (some 500 of a 14M-point map at
 // 0.02 m), so a thread reads, ranks and clears its four words with one access each, where
 // scalar ones took four wavefronts for one: 50M points 580 -> 532 us, the 14M map 331 -> 287.
