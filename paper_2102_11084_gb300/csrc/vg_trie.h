@@ -25,9 +25,11 @@ constexpr int kTrRootClear = 24;
 constexpr int kTrRootBits = 26;
 constexpr int kTrRootBitsLarge = 28;
 // Up to kTrMaxPoints points every call takes the trie.  Above, its accesses miss L2 where the
-// cells are many: a shuffled cloud takes 213 to 237 us at 2.5M points (0.05 to 0.02 m), the
-// radix sort 236; at 3.5M 308 to 386 against 293.  So the kernel looks, on the device, and
-// takes the calls
+// cells are many: a shuffled map takes 238 to 255 us at 2,621,440 points (0.05 to 0.02 m), the
+// radix sort 258; at 3.5M 308 to 386 against 293.  (Shuffled keys wider than 33 bits lose below
+// the line too: from 1.08 times the sort's time at 1.6M points of random keys to 1.49 at 2.62M.  The
+// sort path behind every call of that size, to leave them to, costs 22 us a call.)  So the
+// kernel looks, on the device, and takes the calls
 //   * whose cells are few: 2 of 5 sampled pairs of consecutive points share a cell (camera
 //     frames at 5 mm to 0.1 m: 2 of 5 come with cells for at most a quarter of the points, 1
 //     of 5 with more than half); above kTrMidPoints they must fit a quarter of the points;
